@@ -304,20 +304,62 @@ __device__ __forceinline__ void cs_release_successor()
 #endif
 }
 
+// A chained launch; cluster > 1 makes every `cluster` consecutive CTAs a thread-block cluster.  The caller reads the
+// error with cs_check_launch().
 template <class... KArgs, class... Args>
-static inline void cs_launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+static inline void cs_launch_chained_clusters(void (*kernel)(KArgs...), dim3 grid, uint32_t cluster, dim3 block, size_t smem,
+                                              cudaStream_t s, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = CS_USE_PDL;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster ? 2 : 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <class... KArgs, class... Args>
+static inline void cs_launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+{
+    cs_launch_chained_clusters(kernel, grid, 0u, block, smem, s, args...);
+}
+
+// Largest cluster (a power of two, at most `most`) of which `clusters_needed` fit the current device at once with this
+// block size and dynamic shared memory, -1 when not even single CTAs do.  Raises the function's limits for it.
+template <class Kernel>
+static inline int cs_probe_cluster(Kernel kernel, int most, int threads, size_t smem, int clusters_needed)
+{
+    if ((smem && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return -1;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    (void)cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);       // the caller reads the error with cs_check_launch()
+    for (int cl = most; cl >= 1; cl >>= 1) {
+        cfg.gridDim = dim3(clusters_needed * cl);
+        attr[0].val.clusterDim.x = cl;
+        int n_clusters = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n_clusters, kernel, &cfg);
+        if (e == cudaSuccess && n_clusters >= clusters_needed) return cl;
+        (void)cudaGetLastError();
+    }
+    return -1;
 }
 
 // Recency factor of Eq. 9 as every kernel computes it: fp64 exp and add, rounded once to fp32.

@@ -433,34 +433,6 @@ struct CselDevice {
 static std::mutex g_csel_mu;
 static CselDevice g_csel_dev[CSEL_MAX_DEVICES];
 
-template <class Kernel>
-static int csel_probe(Kernel kernel, size_t smem, int clusters_needed)
-{
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return -1;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.blockDim = dim3(CSEL_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    for (int cl = CSEL_MAX_CLUSTER; cl >= 1; cl >>= 1) {
-        cfg.gridDim = dim3(clusters_needed * cl);
-        attr[0].val.clusterDim.x = cl;
-        int n_clusters = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&n_clusters, kernel, &cfg);
-        if (e == cudaSuccess && n_clusters >= clusters_needed) return cl;
-        (void)cudaGetLastError();
-    }
-    return -1;
-}
-
 // Returns the device's entry (set up on first use, with `device` current), or nullptr for a device index out of range.
 static const CselDevice *csel_device(int device)
 {
@@ -469,9 +441,9 @@ static const CselDevice *csel_device(int device)
     CselDevice &d = g_csel_dev[device];
     if (!d.ready) {
         const size_t smem_max = csel_smem_bytes(CS_MAX_AGENTS, CS_GTAB_MAX);
-        d.max_v = csel_probe(cs_select_cluster_kernel<false>, smem_max, 1);
-        d.max_pf = csel_probe(cs_select_cluster_kernel<true>, smem_max, 1);
-        d.max_step = csel_probe(cs_select_step_kernel, smem_max, 3);
+        d.max_v = cs_probe_cluster(cs_select_cluster_kernel<false>, CSEL_MAX_CLUSTER, CSEL_THREADS, smem_max, 1);
+        d.max_pf = cs_probe_cluster(cs_select_cluster_kernel<true>, CSEL_MAX_CLUSTER, CSEL_THREADS, smem_max, 1);
+        d.max_step = cs_probe_cluster(cs_select_step_kernel, CSEL_MAX_CLUSTER, CSEL_THREADS, smem_max, 3);
         d.ready = 1;
     }
     return &d;

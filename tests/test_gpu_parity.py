@@ -633,6 +633,32 @@ def test_small_batches_ride_with_the_refresh(A, chains, all_sources):
     assert cn["transitions_counted"] == int(o.C.sum())
 
 
+@pytest.mark.parametrize("A,chains,sizes", [(12, 64, (257, 1024, 1025, 20_000)), (64, 1, (16_384, 16_385)), (65, 3000, (5_000, 33_000)),
+                                            (300, 7, (2_047, 2_049))])
+def test_long_batches_across_the_cluster(A, chains, sizes):
+    """Batches above 256 events: one and several CTAs, one round and several, a chain whose events are far apart or all
+    in one share, chains that occur once, counts in shared memory (up to 64 agents) and not; 10 % warm-up events, bad
+    ids, an all-skipped batch, and a stretch of skipped events longer than a CTA's share."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=chains)
+    c, o = make_ctx(cfg, 64, r_min=0.0)
+    rng = synth.rng_for(cfg, 17)
+    for size in sizes:
+        chain = rng.integers(0, chains, size).astype(np.uint32)
+        if chains > 8:
+            chain[rng.random(size) < 0.3] = 5                    # one busy chain
+        agent = rng.integers(0, A, size).astype(np.uint16)
+        flags = (rng.random(size) < 0.1).astype(np.uint8)
+        agent[size // 3] = A
+        chain[size // 2] = chains + 3
+        flags[size // 4: size // 4 + min(1500, size // 3)] = 1
+        for f in (flags, None, np.ones(size, np.uint8)):
+            c.observe_invocations(dev(chain), dev(agent), None if f is None else dev(f))
+            o.observe(chain, agent, np.zeros(size, np.uint8) if f is None else f)
+            H.compare_model(c, o)
+    assert c.get_status() == (cs.CS_ST_BAD_AGENT | cs.CS_ST_BAD_CHAIN)
+    assert c.counters()["transitions_counted"] == int(o.C.sum())
+
+
 @pytest.mark.parametrize("A,stride", [(40, 1), (300, 1), (300, 7), (512, 1), (512, 33), (544, 1), (96, 5)])
 def test_bfs_on_deep_path_graphs(A, stride):
     """A workflow that is one long path (agent i is followed by agent i + stride mod A, over and over): the BFS from

@@ -614,92 +614,143 @@ cs_survival_kernel(cs_workspace ws, uint32_t A, uint32_t W, const uint16_t *__re
 }
 
 // ---------------------------------------------------------------------------------------------
-// Exact survival probability of Eq. 6 for every agent: one CTA per target agent a.  The unit
-// mass at the current agent a0 is pushed through K steps of the chain with column a removed
-// (mass that reaches a leaves the vector); what is left after K steps never visited a:
+// Exact survival probability of Eq. 6 for every agent.  The unit mass at the current agent a0 is pushed through K steps
+// of the chain with column a removed (mass that reaches a leaves the vector); what is left after K steps never visited a:
 //     v_0 = e_{a0};  v_{t+1}[j] = sum_i v_t[i] P[i][j] (j != a), v_{t+1}[a] = 0;
 //     p = sum_t sum_i v_t[i] P[i][a]  (= 1 - sum_j v_K[j]).
-// fp64 accumulation over the canonical fp32 matrix, terms added in index order.  The paper
-// treats this as too expensive for its per-request runtime and uses the hop proxy of Eq. 8;
-// here it is an alternative scorer (A^3 K multiply-adds, off the critical path).
+// The probability is accumulated as the mass absorbed at the target step by step (no 1 - x cancellation, so small
+// probabilities keep full relative accuracy), in fp64 over the canonical fp32 matrix.  The paper treats this as too
+// expensive for its per-request runtime and uses the hop proxy of Eq. 8; here it is an alternative scorer.
+//
+// A step for all targets is a product V (targets x agents) * P with another column zeroed in every row, so it is tiled
+// like one: a cluster advances 8 targets together and splits the columns among its CTAs (every CTA keeps the whole of V
+// for its targets in shared memory, [agent][target], and its columns of the new V go to every CTA of the cluster through
+// distributed shared memory); inside a CTA a warp owns 64 columns (two per lane, 16 accumulators) and a slice of the
+// agents summed over, so that 16 warps stay busy however few the columns; the slices' partial sums meet in shared memory.
+// P comes from global memory; a CTA's columns stay in its L1 for the later steps.  The last step needs column a only: one
+// dot product per target, one warp each.
+//
+// Bound by the fp64 pipe for many agents (2 A^3 (K - 2) operations), by latency for few.  256 agents, K = 4: 62.7 us with
+// one CTA per 8 targets that walked the matrix column by column (32 CTAs, one serial chain of 256 loads per step),
+// 13.7 us per call like this (128 CTAs).
 // ---------------------------------------------------------------------------------------------
-#define XS_MAX_TARGETS 8
-__global__ void __launch_bounds__(ROW_THREADS)
-cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t K, uint32_t n_tgt, float delta,
+#define XS_TARGETS 8u
+#define XS_THREADS 512u
+#define XS_WARPS (XS_THREADS / 32u)
+#define XS_PART_ROW 68u                  // 64 columns of one target, padded: the reduction reads without bank conflicts
+#define XS_MAX_CLUSTER 8u                // the portable limit
+static size_t xs_smem_bytes(uint32_t A)
+{
+    return (2 * (size_t)A * XS_TARGETS + XS_WARPS * XS_TARGETS * XS_PART_ROW) * sizeof(double);
+}
+
+__global__ void __launch_bounds__(XS_THREADS, 1)
+cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t K, uint32_t n_cols, float delta,
                          float *__restrict__ psurv_out, float *__restrict__ fsurv_out)
 {
-    // A CTA advances n_tgt target agents together, so that every element of the matrix it reads
-    // feeds n_tgt accumulators (the matrix is the only sizeable traffic: A^2 floats per step).
-    extern __shared__ double s_vec[];                 // v[n_tgt][A], w[n_tgt][A]
-    double *v = s_vec, *w = s_vec + (size_t)n_tgt * A;
-    const uint32_t tid = threadIdx.x;
+    extern __shared__ __align__(16) double s_xs[];
+    double *const v_all = s_xs;                                    // [2][A][XS_TARGETS]
+    double *const part = s_xs + 2 * (size_t)A * XS_TARGETS;        // [XS_WARPS][XS_TARGETS][XS_PART_ROW]
+    __shared__ double s_hit[XS_TARGETS];
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t base = (blockIdx.x / CL) * XS_TARGETS;          // this cluster's targets
+    const uint32_t col0 = rank * n_cols, col1 = min(col0 + n_cols, A);
+    const float *__restrict__ P = ws.P;
+    cs_wait_for_predecessor();
+    cs_release_successor();
     const uint32_t a0 = a0_arg == CS_AGENT_NONE ? ws.sc->last_agent : a0_arg;
-    for (uint32_t base = blockIdx.x * n_tgt; base < A; base += gridDim.x * n_tgt) {
-        // The probability is accumulated as the mass absorbed at the target step by step (no 1 - x
-        // cancellation, so small probabilities keep full relative accuracy).  Column (base + m) of
-        // target m is owned by one thread, which does the adding for that target.
-        double hit[XS_MAX_TARGETS];
+    const bool any = a0 < A && K > 0;
+    auto owner = [&](uint32_t a) { return a >= col0 && a < col1; };  // this CTA holds column a
+    if (tid < XS_TARGETS) s_hit[tid] = (any && base + tid < A) ? (double)P[(size_t)a0 * A + base + tid] : 0.0;
+    if (any) {
+        // step 1: every target starts from the unit mass at a0, i.e. from row a0 of the matrix
+        for (uint32_t e = tid; e < A * XS_TARGETS; e += XS_THREADS) {
+            const uint32_t j = e / XS_TARGETS, m = e % XS_TARGETS;
+            v_all[e] = j == base + m ? 0.0 : (double)P[(size_t)a0 * A + j];
+        }
+        cluster.sync();                                            // (also: every CTA has started before its memory is written)
+        const uint32_t col_warps = (n_cols + 63u) / 64u, slices = XS_WARPS / col_warps;
+        const uint32_t cw = warp % col_warps, sl = warp / col_warps;
+        uint32_t cur = 0;
+        for (uint32_t t = 1; t + 1 < K; ++t) {
+            const double *v = v_all + (size_t)cur * A * XS_TARGETS;
+            if (sl < slices) {
+                const uint32_t j0 = col0 + cw * 64u + lane, j1 = j0 + 32u;
+                const float *p0 = P + (j0 < col1 ? j0 : 0u), *p1 = P + (j1 < col1 ? j1 : 0u);    // (columns past the end: unused)
+                const uint32_t i_end = (uint32_t)((unsigned long long)(sl + 1u) * A / slices);
+                double acc0[XS_TARGETS], acc1[XS_TARGETS];
 #pragma unroll
-        for (int m = 0; m < XS_MAX_TARGETS; ++m) hit[m] = 0.0;
-        if (a0 < A && K > 0) {
-            __syncthreads();
-            // step 1: every target starts from the unit mass at a0, i.e. from row a0 of the matrix
-            for (uint32_t j = tid; j < A; j += ROW_THREADS) {
-                const double p = (double)ws.P[a0 * A + j];
+                for (uint32_t m = 0; m < XS_TARGETS; ++m) acc0[m] = acc1[m] = 0.0;
+#pragma unroll 8
+                for (uint32_t i = (uint32_t)((unsigned long long)sl * A / slices); i < i_end; ++i) {
+                    const double x0 = (double)__ldg(p0 + (size_t)i * A), x1 = (double)__ldg(p1 + (size_t)i * A);
+                    const double2 *vi = (const double2 *)(v + (size_t)i * XS_TARGETS);
 #pragma unroll
-                for (int m = 0; m < XS_MAX_TARGETS; ++m) {
-                    if ((uint32_t)m < n_tgt) {
-                        const bool own = (j == base + m);
-                        if (own) hit[m] += p;
-                        v[(size_t)m * A + j] = own ? 0.0 : p;
+                    for (uint32_t h = 0; h < XS_TARGETS / 2; ++h) {
+                        const double2 y = vi[h];
+                        acc0[2 * h] = fma(y.x, x0, acc0[2 * h]);
+                        acc0[2 * h + 1] = fma(y.y, x0, acc0[2 * h + 1]);
+                        acc1[2 * h] = fma(y.x, x1, acc1[2 * h]);
+                        acc1[2 * h + 1] = fma(y.y, x1, acc1[2 * h + 1]);
                     }
                 }
+                double *o = part + (size_t)warp * XS_TARGETS * XS_PART_ROW + lane;
+#pragma unroll
+                for (uint32_t m = 0; m < XS_TARGETS; ++m) { o[m * XS_PART_ROW] = acc0[m]; o[m * XS_PART_ROW + 32u] = acc1[m]; }
             }
             __syncthreads();
-            for (uint32_t t = 1; t < K; ++t) {
-                for (uint32_t j = tid; j < A; j += ROW_THREADS) {
-                    double s[XS_MAX_TARGETS];
-#pragma unroll
-                    for (int m = 0; m < XS_MAX_TARGETS; ++m) s[m] = 0.0;
-                    for (uint32_t i = 0; i < A; ++i) {
-                        const double p = (double)ws.P[i * A + j];
-#pragma unroll
-                        for (int m = 0; m < XS_MAX_TARGETS; ++m)
-                            if ((uint32_t)m < n_tgt) s[m] = fma(v[(size_t)m * A + i], p, s[m]);
-                    }
-#pragma unroll
-                    for (int m = 0; m < XS_MAX_TARGETS; ++m) {
-                        if ((uint32_t)m < n_tgt) {
-                            const bool own = (j == base + m);
-                            if (own) hit[m] += s[m];
-                            w[(size_t)m * A + j] = own ? 0.0 : s[m];
-                        }
-                    }
-                }
-                __syncthreads();
-                double *tmp = v; v = w; w = tmp;
+            double *nxt = v_all + (size_t)(cur ^ 1u) * A * XS_TARGETS;
+            for (uint32_t e = tid; e < (col1 > col0 ? col1 - col0 : 0u) * XS_TARGETS; e += XS_THREADS) {
+                const uint32_t jc = e / XS_TARGETS, m = e % XS_TARGETS, j = col0 + jc;
+                const double *q = part + (size_t)(jc / 64u) * XS_TARGETS * XS_PART_ROW + m * XS_PART_ROW + jc % 64u;
+                double sum = 0.0;
+                for (uint32_t u = 0; u < slices; ++u) sum += q[(size_t)u * col_warps * XS_TARGETS * XS_PART_ROW];
+                if (j == base + m) { s_hit[m] += sum; sum = 0.0; }   // (one thread per target)
+                for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)j * XS_TARGETS + m] = sum;
             }
+            cluster.sync();                                        // the new V is complete everywhere; `part` is free again
+            cur ^= 1u;
         }
+        if (K > 1 && warp < XS_TARGETS && base + warp < A && owner(base + warp)) {
+            const double *v = v_all + (size_t)cur * A * XS_TARGETS + warp;
+            double sum = 0.0;
+            for (uint32_t i = lane; i < A; i += 32u) sum = fma(v[(size_t)i * XS_TARGETS], (double)__ldg(P + (size_t)i * A + base + warp), sum);
 #pragma unroll
-        for (int m = 0; m < XS_MAX_TARGETS; ++m) {
-            const uint32_t a = base + m;
-            if ((uint32_t)m < n_tgt && a < A && tid == (a % ROW_THREADS)) {
-                if (psurv_out) psurv_out[a] = (float)hit[m];
-                if (fsurv_out) fsurv_out[a] = (float)(hit[m] + (double)delta);
-            }
+            for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, d);
+            if (lane == 0) s_hit[warp] += sum;
         }
+    }
+    __syncthreads();
+    if (tid < XS_TARGETS && base + tid < A && owner(base + tid)) {
+        if (psurv_out) psurv_out[base + tid] = (float)s_hit[tid];
+        if (fsurv_out) fsurv_out[base + tid] = (float)(s_hit[tid] + (double)delta);
     }
 }
 
 int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_out, float *fsurv_out, cudaStream_t s)
 {
     const cs_params &p = ctx->p;
-    uint32_t n_tgt = 2048u / p.n_agents;               // 2 * n_tgt * A doubles of shared memory <= 32 KiB
-    if (n_tgt > XS_MAX_TARGETS) n_tgt = XS_MAX_TARGETS;
-    if (n_tgt < 1) n_tgt = 1;
-    const uint32_t grid = (p.n_agents + n_tgt - 1) / n_tgt;
-    cs_exact_survival_kernel<<<grid, ROW_THREADS, 2 * (size_t)n_tgt * p.n_agents * sizeof(double), s>>>(
-        ctx->ws, p.n_agents, a0, K, n_tgt, p.delta, psurv_out, fsurv_out);
+    static std::mutex mu;
+    static bool opted[64];                                  // shared-memory opt-in, once per process and device
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (ctx->device < 0 || ctx->device >= 64) return CS_EINVAL;
+        if (!opted[ctx->device]) {
+            const cudaError_t e = cudaFuncSetAttribute(cs_exact_survival_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)xs_smem_bytes(CS_MAX_AGENTS));
+            if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
+            opted[ctx->device] = true;
+        }
+    }
+    // as many CTAs per cluster as give each at least 64 columns and still fit one wave
+    const uint32_t n_clusters = (p.n_agents + XS_TARGETS - 1) / XS_TARGETS;
+    uint32_t cl = 1;
+    while (cl < XS_MAX_CLUSTER && p.n_agents > 64u * cl && 2u * cl * n_clusters <= (uint32_t)ctx->sm_count) cl *= 2;
+    const uint32_t n_cols = (p.n_agents + cl - 1) / cl;
+    cs_launch_chained_clusters(cs_exact_survival_kernel, n_clusters * cl, cl, XS_THREADS, xs_smem_bytes(p.n_agents), s, ctx->ws,
+                               p.n_agents, a0, K, n_cols, p.delta, psurv_out, fsurv_out);
     return cs_check_launch(ctx);
 }
 

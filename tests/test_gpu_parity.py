@@ -550,6 +550,23 @@ def test_exact_survival_parity_and_select(name, K):
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("A,Ks", [(1, (0, 1, 3)), (2, (2, 5)), (9, (3, 6)), (64, (4,)), (65, (2, 4)), (130, (3, 4)), (296, (4,)), (700, (4,)),
+                                  (1024, (3,))])
+def test_exact_survival_table_shapes(A, Ks):
+    """Agent counts on both sides of the target groups (8), the column tiles (64) and every cluster size, with the step
+    counts that take no product (0, 1, 2) and several; both outputs.  Bound: the oracle multiplies K entries of the fp64
+    matrix, the kernel of its canonical fp32 form, three roundings (3 * 2^-24) each; the sums are fp64 on both sides and
+    the result is rounded to fp32 once (2^-24); the floor of Eq. 9 adds one rounding more."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, transitions=("sparse", min(8, A - 1)) if A > 1 else ("dirichlet", 1.0))
+    c, o = warm_state(cfg, 3000, 64, r_min=0.0)
+    for K in Ks:
+        ps, fs = c.exact_survival(K)
+        want = o.exact_survival(K)
+        assert np.all(np.abs(ps.cpu().numpy().astype(np.float64) - want) <= (3 * K + 1) * 2.0 ** -24 * want + 1e-15), (A, K)
+        d64 = float(np.float32(o.p.delta))
+        assert np.all(np.abs(fs.cpu().numpy().astype(np.float64) - (want + d64)) <= (3 * K + 2) * 2.0 ** -24 * (want + d64)), (A, K)
+
+
 def test_select_with_other_tier_copy_preference():
     """cs_params.prefer_other_copy = 1: (score, has no copy, last_access, id), both select paths."""
     cfg = synth.CONFIGS["llama8b"]

@@ -80,15 +80,12 @@ struct cs_scalars {
     float R;                // Eq. 2
     uint32_t gate;          // Eq. 11: R >= r_min
     uint32_t n_transitions; // sum of all counts
-    uint32_t ticket0;       // "last CTA done" counter of the learner refresh
     uint32_t gtab_monotone; // the recency table covers every unsaturated age and never increases with age
     uint32_t status_read;   // cs_get_status(): the value swapped out of `status`
     uint32_t val_le, val_elig, val_ticket;   // cs_validate_selection(): keys at or below the last one, eligible entries, ticket
-    uint32_t adjT_cur;      // which copy of the transposed adjacency the last refresh filled
     uint32_t sel_hint[4];   // bin up to which the next select of each kind (GPU victims, host victims, prefetch)
                             // collects ahead of its own threshold, chosen from the previous call's histogram;
                             // ~0 = none; slot 3 is never written: calls that must not speculate read it
-    unsigned long long qbase;   // Eq. 2 column sums: what every column gets from the rows' zero-count entries (see qfix)
 #ifdef CS_PHASE_STAMPS
     unsigned long long stamps[CS_N_PHASE_STAMPS];   // %globaltimer at phase boundaries of the latest call (profiling builds)
 #endif
@@ -126,12 +123,8 @@ struct cs_workspace {
     uint16_t *cur;        // [n_chains]
     float *P;             // [A*A] Eq. 3
     uint16_t *amax;       // [A]
-    double *rowH;         // [A] sum_j P_ij ln P_ij
-    unsigned long long *qfix;   // [A] column sums of Eq. 2 in 2^-60 fixed point, WITHOUT the part that is the same for every
-                                // column (sc->qbase); zero between refreshes
-    uint32_t *adj;        // [A*W] Eq. 7 adjacency, one bit per edge, W = ceil(A/32)
-    uint32_t *adjT;       // [2][A*W] its transpose (row v = the predecessors of v), two copies used in turn: a refresh
-                          // fills one with atomics and clears the other for the refresh after it
+    uint32_t *adjT;       // [W][A] transpose of the Eq. 7 adjacency, W = ceil(A/32): bit b of word w of column v = an edge from
+                          // agent 32 w + b to agent v (word by word, so that one thread per agent reads it coalesced)
     uint16_t *hops;       // [A]
     float *fsurv;         // [A] p~ + delta for the cached source
     uint16_t *hops_tmp;   // [A] same, for cs_score_blocks() with explicit sources

@@ -4,6 +4,7 @@
 // (Eq. 8).  The model is tiny (A <= 1024), so these kernels are latency-bound: the design
 // goal is few launches and no host round trip, not bandwidth.
 #include <mutex>
+#include <stddef.h>
 
 #include <cooperative_groups.h>
 
@@ -14,7 +15,7 @@ namespace cg = cooperative_groups;
 #define OBS_THREADS 1024
 #define ROW_THREADS 256
 #define OBS_FUSED_MAX 256u     // events up to which a batch is applied inside the refresh launch (one per thread)
-static_assert(OBS_FUSED_MAX == ROW_THREADS, "the refresh kernel stages one event per thread");
+static_assert(OBS_FUSED_MAX <= 256, "the refresh kernel stages one event per thread");
 
 // ---------------------------------------------------------------------------------------------
 // Initial state of Algorithm 1: zero counts, no current agent; plus the recency table.
@@ -24,7 +25,7 @@ __global__ void cs_init_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, u
 {
     const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     for (uint32_t i = tid; i < A * A; i += nth) ws.C[i] = 0;
-    for (uint32_t i = tid; i < A; i += nth) { ws.rowsum[i] = 0; ws.qfix[i] = 0; }
+    for (uint32_t i = tid; i < A; i += nth) ws.rowsum[i] = 0;
     for (uint32_t i = tid; i < n_chains; i += nth) ws.cur[i] = CS_AGENT_NONE;
     for (uint32_t i = tid; i < CS_HIST_BINS; i += nth) ws.hist[i] = 0;
     for (uint32_t i = tid; i <= CS_MAX_SPLITTERS; i += nth) CS_BCOUNT(ws, i) = 0;
@@ -235,102 +236,58 @@ cs_observe_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, const uint32_t
 }
 
 // ---------------------------------------------------------------------------------------------
-// BFS over the bit-matrix graph from a set of source bits, then Eq. 8.  Runs inside one CTA.
-// s_front: 64 words (two frontiers, used in turn), s_visit / s_next: 32 words each, s_hops: one entry per agent.
-//
-// Up to one agent per thread the search PULLS: thread v holds row v of the TRANSPOSED adjacency matrix (the
-// predecessors of v; kept up to date in global memory by the refresh, fetched ahead of time into registers) and at
-// every level ANDs it with the frontier.  A level is then W broadcast loads and ANDs per node, all nodes in
-// parallel, one ballot per warp for the next frontier and ONE barrier -- whatever the frontier size, with no
-// atomics and no divergent loops.  (A push over the frontier's nodes by one warp was tried: lanes that walk
-// different frontier words run one after the other, 80 cycles per node.  So was a transpose built in shared memory
-// by this CTA: 3 us of shared-memory atomics.)
-// More agents take the level-synchronous push from global memory: a node of the current frontier ORs its adjacency
-// row into the next frontier (shared-memory atomics), two barriers per level.
+// BFS over the bit-matrix graph from a set of source bits, then Eq. 8, by the first W warps of a CTA (all of their threads
+// call; W = words of a row, KW = words it is compiled for).  The search PULLS: thread v holds row v of the TRANSPOSED
+// adjacency matrix (the predecessors of v; row[], zero for a thread without a node) in registers and at every level ANDs it
+// with the frontier.  A level is then W broadcast loads and ANDs per node, all nodes in parallel, one ballot per warp
+// for the next frontier and ONE barrier -- whatever the frontier size, with no atomics and no divergent loops; up to 32
+// agents one warp does it without any barrier.  (A push over the frontier's nodes, each ORing its adjacency row into the next
+// frontier, was tried: one warp at it takes 80 cycles per node; a CTA at it from global memory, one dependent trip to L2 per
+// word of every row, took most of the 92 us of a refresh of 1,024 agents.)
+// s_front: 2 * PULL_MAX_WORDS words, the first half the source bits, ordered before this call.  Uses hardware barrier 1.
 // ---------------------------------------------------------------------------------------------
-#define BFS_ROW_WORDS 8u                   // words of a row when the search pulls (one agent per thread: 256 agents)
-struct BfsRow { uint32_t w[BFS_ROW_WORDS]; };
-__device__ __forceinline__ bool cs_bfs_pulls(uint32_t A) { return A <= ROW_THREADS; }
-
-// Row threadIdx.x of the transposed adjacency matrix, fetched so that the trip to global memory overlaps whatever
-// the caller does in between (zero where the search will not pull, or for a thread without a node).
-__device__ __forceinline__ void cs_bfs_load_row(const uint32_t *adjT, uint32_t A, uint32_t W, BfsRow &row)
+#define PULL_MAX_WORDS (CS_MAX_AGENTS / 32u)
+template <int KW>
+__device__ __forceinline__ void cs_bfs_pull(const uint32_t (&row)[KW], uint32_t A, uint32_t W, uint32_t *s_front,
+                                            uint16_t *hops, float *fsurv, uint32_t e_max, float delta)
 {
-    if (!cs_bfs_pulls(A)) {
-#pragma unroll
-        for (uint32_t w = 0; w < BFS_ROW_WORDS; ++w) row.w[w] = 0u;
-        return;
-    }
-    const bool mine = threadIdx.x < A;
-    const uint32_t *r = adjT + (mine ? threadIdx.x * W : 0u);          // (always a valid address; unused words are masked)
-#pragma unroll
-    for (uint32_t w = 0; w < BFS_ROW_WORDS; ++w) row.w[w] = cs_ld_cg_pinned(r + (w < W ? w : 0u));
-#pragma unroll
-    for (uint32_t w = 0; w < BFS_ROW_WORDS; ++w)
-        if (!mine || w >= W) row.w[w] = 0u;
-}
-
-__device__ __forceinline__ void cs_bfs_survival(const uint32_t *__restrict__ adj, uint32_t A, uint32_t W, const BfsRow &rowT,
-                                                uint32_t *s_front, uint32_t *s_visit, uint32_t *s_next, uint16_t *s_hops,
-                                                uint16_t *hops, float *fsurv, uint32_t e_max, float delta)
-{
-    // on entry s_front[0 .. 32) holds the source bits and s_front[32 .. 64) zeroes (synchronised by the caller)
-    const uint32_t tid = threadIdx.x;
-    if (cs_bfs_pulls(A)) {
-        const uint32_t v = tid;                                       // blockDim.x >= A
-        bool seen = v >= A || ((s_front[v >> 5] >> (v & 31)) & 1u);
-        uint32_t my_hops = (v < A && seen) ? 0u : CS_HOP_NONE;
+    const uint32_t v = threadIdx.x, lane = v & 31;
+    uint32_t my_hops = CS_HOP_NONE;
+    if (KW == 1) {
+        uint32_t front = s_front[0], seen = front;
+        if ((seen >> lane) & 1u) my_hops = 0;
+        for (uint32_t level = 1; front; ++level) {
+            const bool fresh = (row[0] & front) != 0u && !((seen >> lane) & 1u);
+            front = __ballot_sync(0xFFFFFFFFu, fresh);
+            seen |= front;
+            if (fresh) my_hops = level;
+        }
+    } else {
+        bool seen = v >= A || ((s_front[v >> 5] >> lane) & 1u);
+        if (v < A && seen) my_hops = 0;
         for (uint32_t level = 1; level <= A; ++level) {
-            const uint32_t *cur = s_front + ((level & 1u) ? 0u : 32u);
-            uint32_t *nxt = s_front + ((level & 1u) ? 32u : 0u);
+            const uint32_t *cur = s_front + ((level & 1u) ? 0u : PULL_MAX_WORDS);
+            uint32_t *nxt = s_front + ((level & 1u) ? PULL_MAX_WORDS : 0u);
             uint32_t hit = 0;
 #pragma unroll
-            for (uint32_t w = 0; w < BFS_ROW_WORDS; ++w) hit |= rowT.w[w] & cur[w];
+            for (int w = 0; w < KW; ++w) hit |= row[w] & cur[w];          // (words past W: zero rows)
             const bool fresh = hit != 0u && !seen;
             const uint32_t word = __ballot_sync(0xFFFFFFFFu, fresh);
-            if ((tid & 31u) == 0) nxt[tid >> 5] = word;
+            if (lane == 0) nxt[v >> 5] = word;
             if (fresh) { seen = true; my_hops = level; }
-            if (!__syncthreads_or(fresh)) break;
-        }
-        if (v < A) s_hops[v] = (uint16_t)my_hops;
-    } else {
-        for (uint32_t a = tid; a < A; a += blockDim.x)
-            s_hops[a] = ((s_front[a >> 5] >> (a & 31)) & 1u) ? 0 : CS_HOP_NONE;
-        if (tid < W) { s_visit[tid] = s_front[tid]; s_next[tid] = 0; }
-        __syncthreads();
-        for (uint32_t level = 1; level <= A; ++level) {
-            for (uint32_t node = tid; node < A; node += blockDim.x) {
-                if ((s_front[node >> 5] >> (node & 31)) & 1u) {
-                    for (uint32_t w = 0; w < W; ++w) {
-                        const uint32_t v = __ldcg(&adj[node * W + w]);
-                        if (v) atomicOr(&s_next[w], v);
-                    }
-                }
-            }
-            __syncthreads();
-            uint32_t acc = 0;
-            if (tid < W) {
-                acc = s_next[tid] & ~s_visit[tid];
-                s_next[tid] = 0;
-                s_front[tid] = acc;
-                s_visit[tid] |= acc;
-                uint32_t bits = acc;
-                while (bits) {
-                    const uint32_t b2 = tid * 32 + (__ffs(bits) - 1);
-                    bits &= bits - 1;
-                    if (b2 < A) s_hops[b2] = (uint16_t)level;
-                }
-            }
-            if (!__syncthreads_or(acc != 0)) break;
+            uint32_t any;
+            asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                         : "=r"(any)
+                         : "r"((uint32_t)fresh), "r"(W * 32u)
+                         : "memory");
+            if (!any) break;
         }
     }
-    __syncthreads();
-    for (uint32_t a = tid; a < A; a += blockDim.x) {
-        const uint32_t h = s_hops[a];
-        const uint32_t m = h < e_max ? h : e_max;          // CS_HOP_NONE > e_max by construction
+    if (v < A) {
+        const uint32_t m = my_hops < e_max ? my_hops : e_max;             // CS_HOP_NONE > e_max by construction
         const double ptilde = 1.0 - (double)m / (double)e_max;
-        hops[a] = (uint16_t)h;
-        fsurv[a] = (float)(ptilde + (double)delta);
+        hops[v] = (uint16_t)my_hops;
+        fsurv[v] = (float)(ptilde + (double)delta);
     }
 }
 
@@ -350,141 +307,267 @@ __device__ T cs_block_sum(T v, T *s_red)
     return r;
 }
 
-__device__ void cs_block_sum2(double &a, double &b, double *s_red)
-{
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        a += __shfl_xor_sync(0xFFFFFFFFu, a, d);
-        b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
-    }
-    __syncthreads();
-    if (lane == 0) { s_red[warp] = a; s_red[32 + warp] = b; }
-    __syncthreads();
-    a = s_red[0];
-    b = s_red[32];
-    for (uint32_t w = 1; w < n_warps; ++w) { a += s_red[w]; b += s_red[32 + w]; }
-}
+// ---------------------------------------------------------------------------------------------
+// The refresh of everything derived from the counts: Eq. 3 in canonical fp32 (one rounding per operation, no FMA), every
+// row's arg-max, adjacency bits (Eq. 7) and entropy term, then Eq. 2 / Eq. 11 over all rows and the cached search of
+// Eq. 7 / 8.  One thread-block cluster, one warp per row.
+//
+// A refresh is a chain of dependent steps on a few hundred kilobytes, so what counts is the number of trips to L2 and of
+// barriers between its first load and its last store -- and, once a row has a warp of its own, the instructions an SM has to
+// issue for its rows (about a thousand per row: 32 rows per CTA were slower than 16).  Every warp fetches its row, the row's
+// sum and -- redundantly per CTA -- the batch of events at once, and what has to meet (column sums of Eq. 2, the transposed
+// adjacency matrix for the search, entropies, arg-max) does so through distributed shared memory:
+//   * up to 32 agents: one CTA;
+//   * up to 256 (KW = 8): 8 or 16 rows per CTA, every CTA adds up its rows' share of all columns and adds it to the first CTA's;
+//   * more (KW = 32): a column's sum and its row of the transposed matrix belong to one CTA of the cluster, which the others
+//     reach with atomics (only entries that have a count, or an edge); that CTA passes the sums on to the first one and the
+//     matrix rows to global memory, from where the first CTA fetches them.
+// The first CTA then runs the search on some of its warps and the sums of Eq. 2 on others.
+//
+// Rows are sparse: entries with a zero count all have the same P = eps / n_i, so one logarithm stands for all of them, the
+// entries with a count are compacted (one per lane), and their share of the column sums is one number per row with the
+// differences on top.  A row no event of a small batch starts at keeps its P and arg-max; only what depends on the total
+// number of transitions is recomputed.  Column sums are 2^-60 fixed point: integer addition commutes, so they are
+// bit-identical from run to run whatever the order of the atomics.
+//
+// Measured (back to back in a CUDA graph, us per refresh) against one CTA per row with a "last CTA done" epilogue over
+// global atomics and, above 256 agents, a search that pushed from global memory:
+//   agents / events      4/1   12/5   12/256   30/8   64/64   128/64   256/64   256/256   400/64   1,024/64
+//   before               7.7   8.4    14.8     8.7    12.3    11.9     10.9     21.9      35.8     93.4
+//   now                  4.6   4.8    7.5      6.0    6.8     7.2      9.2      11.1      17.2     35.2
+// ---------------------------------------------------------------------------------------------
+#define RF_OWN_COLS 128u                                  // KW = 32: columns a CTA owns in a cluster of 8 (64 in one of 16)
+template <int KW> struct RfShape {                        // KW: words of an adjacency row the kernel is compiled for
+    static constexpr uint32_t COLS = KW * 32u;
+    static constexpr uint32_t ROWS = KW == 8 ? 16u : 32u;                            // most rows a CTA works on at a time, one per warp
+    static constexpr uint32_t CTAS = KW == 1 ? 1u : 16u;                             // most CTAs of the cluster
+    static constexpr int CHUNK = KW < 8 ? KW : 8;                                    // words of a row in registers at a time
+    static constexpr uint32_t T_COLS = KW == 32 ? RF_OWN_COLS : COLS;                // columns of the transposed matrix kept here
+};
+template <int KW> struct RfShared {
+    unsigned long long q[RfShape<KW>::COLS];                        // column sums: this CTA's, in the first one everybody's
+    unsigned long long base[RfShape<KW>::CTAS];                     // what every column gets from a CTA's zero-count entries
+    double hc[RfShape<KW>::CTAS];                                   // sum over a CTA's rows of n_i * (row entropy)
+    double row_hc[32];
+    unsigned long long row_base[32];
+    double red[32];
+    unsigned long long own_q[KW == 32 ? RF_OWN_COLS : 1];
+    __align__(16) uint32_t ev_chain[OBS_FUSED_MAX];                 // the batch: chain of event e (read as 16-byte words),
+    uint16_t ev_agent[OBS_FUSED_MAX];                               // its agent (CS_AGENT_NONE: skipped),
+    uint16_t ev_prev[OBS_FUSED_MAX];                                // and the agent it follows when that is a counted transition
+    uint32_t adj[KW == 32 ? 1 : RfShape<KW>::COLS];                 // bit i: this CTA's row i has an edge to the column
+    uint32_t adjT[KW][RfShape<KW>::T_COLS];                         // transposed matrix, word by word
+    uint32_t nz_v[RfShape<KW>::ROWS][32];                           // per warp: entries of its row that have a count, gathered
+    uint16_t nz_j[RfShape<KW>::ROWS][32];                           // so that every lane works on one
+    uint16_t amax[RfShape<KW>::COLS];
+    uint32_t front[2 * PULL_MAX_WORDS];
+    int last_live;
+    uint8_t succ[OBS_FUSED_MAX];                                    // 1: a later live event of the batch has the same chain
+};
+static_assert(sizeof(RfShared<8>) <= 48 * 1024 && sizeof(RfShared<32>) <= 48 * 1024, "the default shared-memory limit");
+static_assert(offsetof(RfShared<1>, ev_chain) % 16 == 0 && offsetof(RfShared<8>, ev_chain) % 16 == 0 &&
+              offsetof(RfShared<32>, ev_chain) % 16 == 0, "read as 16-byte words");
 
-// ---------------------------------------------------------------------------------------------
-// One CTA per row i: Eq. 3 in canonical fp32 (one rounding per operation, no FMA), the row's
-// arg-max, its adjacency bits (Eq. 7) and its entropy term.  The last CTA to finish then
-// computes Eq. 2 / Eq. 11 over all rows and refreshes the cached BFS / Eq. 8 tables.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(ROW_THREADS)
-cs_normalise_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max,
-                    float delta, uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain,
-                    const uint16_t *__restrict__ ev_agent, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
-                    const uint32_t *__restrict__ n_events_dev)
+__device__ __forceinline__ double cs_xlogx(double x) { return x * log(x); }
+
+// blockDim.x / 32 rows at a time per CTA: 8, 16 or 32, all of them (KW = 1), 8 or 16 (KW = 8), 32 (KW = 32).
+template <int KW>
+__global__ void __launch_bounds__(RfShape<KW>::ROWS * 32u)
+cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
+                  uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
+                  const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
+                  const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
 {
-    __shared__ uint32_t s_evc[OBS_FUSED_MAX];        // the batch: chain of event e,
-    __shared__ uint16_t s_eva[OBS_FUSED_MAX];        // its agent (CS_AGENT_NONE: skipped),
-    __shared__ uint16_t s_evp[OBS_FUSED_MAX];        // and the agent it follows when that is a counted transition
-    __shared__ uint8_t s_succ[OBS_FUSED_MAX];        // 1: a later live event of the batch has the same chain
-    __shared__ uint32_t s_add[CS_MAX_AGENTS];        // what the batch adds to the row being worked on
-    __shared__ int s_last_live;
-    __shared__ double s_red[64];
-    __shared__ float s_bestv[ROW_THREADS / 32];
-    __shared__ uint32_t s_besti[ROW_THREADS / 32];
-    __shared__ uint32_t s_front[64], s_visit[32], s_next[32];
-    __shared__ uint16_t s_hops[CS_MAX_AGENTS];
-    __shared__ bool s_is_last;
-    const uint32_t tid = threadIdx.x;
+    constexpr uint32_t COLS = RfShape<KW>::COLS, T_COLS = RfShape<KW>::T_COLS, ADJ = KW == 32 ? 1u : COLS, OWN = KW == 32 ? RF_OWN_COLS : 1u;
+    constexpr int CHUNK = RfShape<KW>::CHUNK;
+    __shared__ RfShared<KW> sm;
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_threads = blockDim.x, rows = n_threads >> 5;
+    const uint32_t own = KW == 32 ? COLS / CL : 1u;           // columns per CTA
     CS_STAMP(ws, CS_PS_REFRESH_ENTRY, blockIdx.x == 0 && tid == 0);
+    if (KW == 32) {
+        for (uint32_t x = tid; x < KW * T_COLS; x += n_threads) (&sm.adjT[0][0])[x] = 0;
+        if (tid < OWN) sm.own_q[tid] = 0;
+    } else if (tid < COLS) {
+        sm.q[tid] = 0;
+        sm.adj[tid % ADJ] = 0;
+#pragma unroll
+        for (int w = 0; w < KW; ++w) sm.adjT[w][tid % T_COLS] = 0;         // (bits past the last row)
+    }
+    if (tid == 0) sm.last_live = -1;
+    if (tid < OBS_FUSED_MAX) sm.succ[tid] = 0;
+    if (tid < 2 * PULL_MAX_WORDS) sm.front[tid] = 0;
+    if (KW > 1) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");             // waited for below
     cs_wait_for_predecessor();
     CS_STAMP(ws, CS_PS_REFRESH_WAITED, blockIdx.x == 0 && tid == 0);
     cs_release_successor();
 
-    // ---- a small batch of events is applied here, by every CTA to the rows it owns, instead of by a launch of its
-    // own: each CTA stages the batch, finds every event's predecessor (in the batch, else the chain's current agent)
-    // exactly as cs_observe_kernel does, and adds the transitions that start at row i to row i.  What is shared --
-    // cur[], the last agent, the totals and the counters -- is written by the last CTA, after every CTA has read it.
-    if (n_events_dev) n_events = min(n_events, *n_events_dev);
+    // ---- everything that depends on nothing, in one trip ---------------------------------------------------------
+    if (n_events_dev) n_events = min(n_events, cs_ld_cg_pinned(n_events_dev));
+    uint32_t c[CHUNK], n_i = 0;
+    auto load_chunk = [&](uint32_t row, uint32_t col0) {
+#pragma unroll
+        for (int k = 0; k < CHUNK; ++k) {
+            const uint32_t j = col0 + lane + 32u * k;
+            c[k] = 0;
+            if (row < A && j < A) c[k] = cs_ld_cg_pinned(ws.C + row * A + j);
+        }
+        if (col0 == 0) n_i = cs_ld_cg_pinned(ws.rowsum + (row < A ? row : 0u));
+    };
+    load_chunk(rank * rows + warp, 0u);
+    uint32_t n_total = cs_ld_cg_pinned(&ws.sc->n_transitions);
+    uint32_t la = cs_ld_cg_pinned(&ws.sc->last_agent);
+
+    // ---- a small batch of events is applied here, by every CTA to its own rows: each CTA finds every event's predecessor
+    // (in the batch, else the chain's current agent) as cs_observe_kernel does.  What is shared -- cur[], the last agent,
+    // the totals and the counters -- is written by the first CTA behind the cluster barrier, after every CTA has read it.
     uint32_t n_new = 0, n_skipped = 0;
     if (n_events) {
-        uint32_t c = 0, a = CS_AGENT_NONE;
-        if (tid == 0) s_last_live = -1;
+        uint32_t ch = OBS_NO_CHAIN, a = CS_AGENT_NONE, before = CS_AGENT_NONE;
         if (tid < n_events) {
-            c = ev_chain[tid];
-            a = ev_agent[tid];
+            ch = ev_chain_in[tid];
+            a = ev_agent_in[tid];
             const bool warm = ev_flags && (ev_flags[tid] & CS_EV_WARMUP);
             uint32_t bad = 0;
             if (!warm && a >= A) bad |= CS_ST_BAD_AGENT;
-            if (!warm && c >= n_chains) bad |= CS_ST_BAD_CHAIN;
-            if (bad && blockIdx.x == 0) atomicOr(&ws.sc->status, bad);
-            if (warm || bad) a = CS_AGENT_NONE;
+            if (!warm && ch >= n_chains) bad |= CS_ST_BAD_CHAIN;
+            if (bad && rank == 0) atomicOr(&ws.sc->status, bad);
+            if (warm || bad) { a = CS_AGENT_NONE; ch = OBS_NO_CHAIN; }
+            else before = cs_ld_cg_pinned(ws.cur + ch);        // in flight during the search below
         }
-        s_evc[tid] = c;
-        s_eva[tid] = (uint16_t)a;
-        s_succ[tid] = 0;
+        const bool live = a != CS_AGENT_NONE;
+        if (tid < OBS_FUSED_MAX) { sm.ev_chain[tid] = ch; sm.ev_agent[tid] = (uint16_t)a; }
+        uint32_t same = 0;
+        int newest = -1;
+        if (32u * warp < n_events) {                           // (whole warps)
+            newest = __reduce_max_sync(0xFFFFFFFFu, live ? (int)tid : -1);
+            same = __match_any_sync(0xFFFFFFFFu, ch) & ((1u << lane) - 1u);
+        }
         __syncthreads();
-        const bool live = tid < n_events && a != CS_AGENT_NONE;
-        uint32_t prev = CS_AGENT_NONE;
+        if (lane == 0 && newest >= 0) atomicMax(&sm.last_live, newest);
+        bool counted = false;
         if (live) {
-            int j = (int)tid - 1;
-            for (; j >= 0; --j)
-                if (s_evc[j] == c && s_eva[j] != CS_AGENT_NONE) { prev = s_eva[j]; break; }
-            if (j < 0) prev = ws.cur[c];
-            else s_succ[j] = 1;                                // event j is not the last of its chain in this batch
-            atomicMax(&s_last_live, (int)tid);
+            int p = same ? (int)(warp * 32u) + 31 - __clz(same) : -1;
+            for (int w = (int)warp - 1; w >= 0 && p < 0; --w) {          // earlier warps, nearest first
+                const uint4 *q = (const uint4 *)(sm.ev_chain + 32 * w);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {                            // the last match is the one wanted
+                    const uint4 v = q[u];
+                    if (v.x == ch) p = 32 * w + 4 * u;
+                    if (v.y == ch) p = 32 * w + 4 * u + 1;
+                    if (v.z == ch) p = 32 * w + 4 * u + 2;
+                    if (v.w == ch) p = 32 * w + 4 * u + 3;
+                }
+            }
+            if (p >= 0) { before = sm.ev_agent[p]; sm.succ[p] = 1; }
+            counted = before != CS_AGENT_NONE && before != a;
         }
-        const bool counted = live && prev != CS_AGENT_NONE && prev != a;
-        s_evp[tid] = (uint16_t)(counted ? prev : CS_AGENT_NONE);
+        if (tid < OBS_FUSED_MAX) sm.ev_prev[tid] = (uint16_t)(counted ? before : CS_AGENT_NONE);
         n_new = (uint32_t)__syncthreads_count(counted);
-        n_skipped = (uint32_t)__syncthreads_count(tid < n_events && a == CS_AGENT_NONE);
+        if (rank == 0) n_skipped = (uint32_t)__syncthreads_count(tid < n_events && !live);
+    } else {
+        __syncthreads();
     }
-    // Column sums q_j = sum_i pi_i P_ij of Eq. 2 are accumulated by the row CTAs in 2^-60 fixed
-    // point with integer atomics: integer addition commutes, so the sum is bit-identical from run
-    // to run whatever order the CTAs finish in (a float atomic would not be).
-    const uint32_t n_total = ws.sc->n_transitions + n_new;
-    const uint32_t fill = ws.sc->adjT_cur ^ 1u;              // every CTA reads this before the last one flips it
-    uint32_t *adjT_fill = ws.adjT + (size_t)fill * A * W, *adjT_clear = ws.adjT + (size_t)(fill ^ 1u) * A * W;
+    n_total += n_new;
+    if (KW > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");                // every CTA has started and cleared its sums
+
+    auto add_edge = [&](uint32_t i, uint32_t j) {
+        if (KW == 32) atomicOr(cluster.map_shared_rank(&sm.adjT[0][0], j / own) + (i >> 5) * T_COLS + j % own, 1u << (i & 31u));
+        else atomicOr(&sm.adj[j % ADJ], 1u << warp);                                       // (KW < 32: one row per warp)
+    };
+    // ---- this warp's rows (more than one only where the cluster holds fewer than A of them) -------------------------
+    double row_hc = 0.0;
+    unsigned long long row_base = 0;
     const double inv_total = n_total ? 1.0 / (double)n_total : 0.0;
-    for (uint32_t i = blockIdx.x; i < A; i += gridDim.x) {
-        uint32_t n_i = ws.rowsum[i];
-        // transitions of the batch that start at agent i
-        const bool mine = n_events && tid < n_events && s_evp[tid] == i;
-        const uint32_t row_new = n_events ? (uint32_t)__syncthreads_count(mine) : 0u;
-        if (row_new) {
-            for (uint32_t j = tid; j < A; j += ROW_THREADS) s_add[j] = 0;
-            __syncthreads();
-            if (mine) atomicAdd(&s_add[s_eva[tid]], 1u);
-            __syncthreads();
-            n_i += row_new;
-            if (tid == 0) ws.rowsum[i] = n_i;
-        }
+    for (uint32_t i = rank * rows + warp; i < A; i += CL * rows) {
+        if (i >= CL * rows) load_chunk(i, 0u);
+        uint32_t n_add = 0;
+        if (n_new)
+            for (uint32_t e0 = 0; e0 < n_events; e0 += 32u)
+                n_add += __popc(__ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i));
+        n_i += n_add;
+        const bool write = every_row || n_add;
         const double pi_fix = (double)n_i * inv_total * 1152921504606846976.0;      // pi_i * 2^60
         const float den = __fadd_rn((float)n_i, __fmul_rn((float)A, eps));
-        // Most entries of a row have a zero count and therefore the same P = eps / den: their contribution to the
-        // column sums is one number per row, added once to a scalar instead of A times to A columns; a column with a
-        // count gets the difference on top.  Integer arithmetic, so the sums are bit for bit what A atomics per row gave.
-        const long long base_fix = __double2ll_rn(pi_fix * (double)__fdiv_rn(__fadd_rn(0.0f, eps), den));
-        if (tid == 0 && n_i) atomicAdd(&ws.sc->qbase, (unsigned long long)base_fix);
+        const float p0 = __fdiv_rn(__fadd_rn(0.0f, eps), den);              // every entry with a zero count
+        const bool p0_edge = p0 >= tau;
+        const long long base_fix = __double2ll_rn(pi_fix * (double)p0);
         float bestv = -1.0f;
-        uint32_t besti = 0xFFFFFFFFu;
+        uint32_t besti = 0xFFFFFFFFu, n_nz = 0, n_list = 0;
         double h = 0.0;
-        for (uint32_t j0 = 0; j0 < A; j0 += ROW_THREADS) {       // A is padded to whole warps for the ballot
-            const uint32_t j = j0 + tid;
-            bool edge = false;
-            if (j < A) {
-                uint32_t cij = ws.C[i * A + j];
-                if (row_new && s_add[j]) { cij += s_add[j]; ws.C[i * A + j] = cij; }
-                const float p = __fdiv_rn(__fadd_rn((float)cij, eps), den);
-                ws.P[i * A + j] = p;
-                if (p > bestv) { bestv = p; besti = j; }         // strict: the lowest j among equals stays
-                const double pd = (double)p;
-                h += pd * log(pd);
-                edge = p >= tau;
-                if (n_i && cij) atomicAdd(&ws.qfix[j], (unsigned long long)(__double2ll_rn(pi_fix * pd) - base_fix));
+        uint32_t *lv = sm.nz_v[warp];
+        uint16_t *lj = sm.nz_j[warp];
+        // up to 32 entries that have a count, one per lane; in the lane behind them, the last time, those that have none
+        auto take = [&](uint32_t n, bool last) {
+            __syncwarp();
+            const bool mine = lane < n;
+            const uint32_t v = mine ? lv[lane] : 0u, j = mine ? lj[lane] : 0u;
+            const float p = mine ? __fdiv_rn(__fadd_rn((float)v, eps), den) : p0;
+            const double pd = (double)p, t = cs_xlogx(pd);
+            if (mine) {
+                if (write) {
+                    ws.P[(size_t)i * A + j] = p;
+                    ws.C[(size_t)i * A + j] = v;
+                }
+                if (p > bestv) { bestv = p; besti = j; }                       // strict: the lowest j among equals stays
+                if (p >= tau) add_edge(i, j);
+                if (n_i) {
+                    unsigned long long *q = KW == 32 ? cluster.map_shared_rank(sm.own_q, j / own) + j % own : &sm.q[j];
+                    atomicAdd(q, (unsigned long long)(__double2ll_rn(pi_fix * pd) - base_fix));
+                }
+                h += t;
+            } else if (last && lane == n) {
+                h += (double)(A - n_nz) * t;
             }
-            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, edge);
-            if ((tid & 31) == 0 && (j >> 5) < W) ws.adj[i * W + (j >> 5)] = bits;
-            if (edge) atomicOr(&adjT_fill[j * W + (i >> 5)], 1u << (i & 31));      // the transpose: i precedes j
+            __syncwarp();
+        };
+        for (uint32_t col0 = 0; col0 < A; col0 += 32u * CHUNK) {
+            if (col0) load_chunk(i, col0);
+            if (n_add) {
+                for (uint32_t e0 = 0; e0 < n_events; e0 += 32u) {
+                    uint32_t hits = __ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i);
+                    for (; hits; hits &= hits - 1u) {
+                        const uint32_t j = sm.ev_agent[e0 + __ffs(hits) - 1] - col0;
+#pragma unroll
+                        for (int k = 0; k < CHUNK; ++k)
+                            if (j == lane + 32u * k) ++c[k];
+                    }
+                }
+            }
+            // the entries that have a count go to the list, a word of 32 columns at a time; the rest is uniform
+            uint32_t words = 0;
+#pragma unroll
+            for (int k = 0; k < CHUNK; ++k) {
+                if (col0 + 32u * k >= A) break;
+                const uint32_t j = col0 + lane + 32u * k;
+                if (__any_sync(0xFFFFFFFFu, c[k] != 0u)) words |= 1u << k;
+                if (write && j < A) ws.P[(size_t)i * A + j] = p0;
+                if (p0_edge && j < A && c[k] == 0u) add_edge(i, j);
+            }
+            __syncwarp();                                                      // (an entry's P is written again by another lane)
+#pragma unroll 1
+            for (; words; words &= words - 1u) {
+                const uint32_t k = __ffs(words) - 1u;
+                uint32_t v = c[0];
+#pragma unroll
+                for (int u = 1; u < CHUNK; ++u) v = k == (uint32_t)u ? c[u] : v;
+                const uint32_t b = __ballot_sync(0xFFFFFFFFu, v != 0u), n_b = __popc(b);
+                if (n_list + n_b > 32u) { take(n_list, false); n_list = 0; }
+                if (v) {
+                    const uint32_t at = n_list + __popc(b & ((1u << lane) - 1u));
+                    lv[at] = v;
+                    lj[at] = (uint16_t)(col0 + lane + 32u * k);
+                }
+                n_list += n_b;
+                n_nz += n_b;
+            }
         }
-        for (uint32_t w = tid; w < W; w += ROW_THREADS) adjT_clear[i * W + w] = 0;  // for the refresh after this one
-        // arg-max (max value, then min index) and the entropy term: a butterfly inside each warp, then the warp results
-        // combined in warp order by thread 0
-        const uint32_t lane = tid & 31, warp = tid >> 5;
+#pragma unroll 1
+        do {                                                                   // (twice when the list is full: the last lane has to be free)
+            take(n_list, n_list < 32u);
+            n_list = n_list == 32u ? 0u : 33u;
+        } while (n_list != 33u);
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
             const float v = __shfl_xor_sync(0xFFFFFFFFu, bestv, d);
@@ -492,53 +575,67 @@ cs_normalise_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float ta
             if (v > bestv || (v == bestv && x < besti)) { bestv = v; besti = x; }
             h += __shfl_xor_sync(0xFFFFFFFFu, h, d);
         }
-        __syncthreads();                                         // the partials of the row before have been read
-        if (lane == 0) { s_bestv[warp] = bestv; s_besti[warp] = besti; s_red[warp] = h; }
-        __syncthreads();
-        if (tid == 0) {
-            float bv = s_bestv[0];
-            uint32_t bi = s_besti[0];
-            double hs = s_red[0];
-            for (uint32_t w = 1; w < ROW_THREADS / 32; ++w) {
-                if (s_bestv[w] > bv || (s_bestv[w] == bv && s_besti[w] < bi)) { bv = s_bestv[w]; bi = s_besti[w]; }
-                hs += s_red[w];
-            }
-            ws.amax[i] = (uint16_t)bi;
-            ws.rowH[i] = hs;
+        const uint32_t am = bestv > p0 ? besti : 0u;          // no entry above the zero-count ones: all are equal, the lowest wins
+        if (lane == 0) {
+            if (write) ws.amax[i] = (uint16_t)am;
+            if (n_add) ws.rowsum[i] = n_i;
+            cluster.map_shared_rank(sm.amax, 0)[i] = (uint16_t)am;
         }
+        row_hc += (double)n_i * h;
+        row_base += n_i ? (unsigned long long)base_fix : 0ull;
     }
-
+    if (lane == 0) { sm.row_hc[warp] = row_hc; sm.row_base[warp] = row_base; }
+    __syncthreads();
     CS_STAMP(ws, CS_PS_REFRESH_ROWS_DONE, blockIdx.x == 0 && tid == 0);
-    // ---- last CTA done: global quantities ---------------------------------------------------------
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const uint32_t t = atomicAdd(&ws.sc->ticket0, 1u);
-        s_is_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_is_last) return;
-    __threadfence();
-    CS_STAMP(ws, CS_PS_REFRESH_LAST_CTA, tid == 0);
 
-    BfsRow rowT;                                                         // in flight during the sums
-    cs_bfs_load_row(adjT_fill, A, W, rowT);
-    // the operands of Eq. 2 (the first ROW_THREADS of each array) travel with it, so that the sums below start on data
-    // that has arrived instead of on a trip of their own
-    const uint32_t t0_ = tid < A ? tid : 0u;
-    const uint32_t pre_rowsum = cs_ld_cg_pinned(ws.rowsum + t0_);
-    const unsigned long long pre_rowH = cs_ld_cg_pinned((const unsigned long long *)ws.rowH + t0_);
-    const unsigned long long pre_qfix = cs_ld_cg_pinned(ws.qfix + t0_);
-    const unsigned long long qbase = cs_ld_cg_pinned(&ws.sc->qbase);
-    uint32_t la = cs_ld_cg_pinned(&ws.sc->last_agent);
-    if (n_events) {
-        // the batch's effect on what all CTAs share (every other CTA is done reading it)
-        const uint32_t a = tid < n_events ? s_eva[tid] : CS_AGENT_NONE;
-        if (a != CS_AGENT_NONE) {
-            if (!s_succ[tid]) ws.cur[s_evc[tid]] = (uint16_t)a;       // the chain's last live event of the batch
+    // ---- everything meets in the first CTA -----------------------------------------------------------------------------
+    RfShared<KW> *first = cluster.map_shared_rank(&sm, 0);
+    if (KW != 32 && tid < A) {
+        const uint32_t bits = sm.adj[tid % ADJ];
+        if (KW == 8 && rank && sm.q[tid % COLS]) atomicAdd(&first->q[tid % COLS], sm.q[tid % COLS]);
+        // this CTA's rows are 32, 16 or 8 bits of a word
+        if (rows == 32u) first->adjT[0][tid % T_COLS] = bits;
+        else if (rows == 16u) ((uint16_t *)&first->adjT[rank / 2u % KW][tid % T_COLS])[rank & 1u] = (uint16_t)bits;
+        else ((uint8_t *)&first->adjT[rank / 4u % KW][tid % T_COLS])[rank & 3u] = (uint8_t)bits;
+    }
+    if (warp == rows - 1u) {
+        double s = lane < rows ? sm.row_hc[lane] : 0.0;
+        unsigned long long b = lane < rows ? sm.row_base[lane] : 0ull;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+            b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
         }
-        if (all_chains) __threadfence();                      // (cur[] is read back below when every chain is a source)
-        if (s_last_live >= 0) la = s_eva[s_last_live];
+        if (lane == 0) { first->hc[rank] = s; first->base[rank] = b; }
+    }
+    if (KW > 1) cluster.sync();
+    else __syncthreads();
+    if (KW == 32) {
+        // owned columns are complete: sums to the first CTA, rows of the transposed matrix to global memory
+        for (uint32_t x = tid; x < own * W; x += n_threads) {
+            const uint32_t w = x / own, jc = x - w * own, j = rank * own + jc;
+            if (j < A) ws.adjT[(size_t)w * A + j] = (&sm.adjT[0][0])[w * T_COLS + jc];
+        }
+        if (tid < own) first->q[(rank * own + tid) % COLS] = sm.own_q[tid % OWN];
+        cluster.sync();
+    }
+    if (rank != 0) return;
+    CS_STAMP(ws, CS_PS_REFRESH_LAST_CTA, tid == 0);
+    uint32_t row[KW];                                         // thread v: the predecessors of agent v
+#pragma unroll
+    for (int w = 0; w < KW; ++w) {
+        row[w] = 0;
+        if ((uint32_t)w < W && tid < A) {
+            row[w] = KW == 32 ? cs_ld_cg_pinned(ws.adjT + (size_t)w * A + tid) : sm.adjT[w][tid % T_COLS];
+            if (KW != 32) ws.adjT[(size_t)w * A + tid] = row[w];          // for searches from explicit sources
+        }
+    }
+
+    if (n_events) {
+        // the batch's effect on what all CTAs share
+        const uint32_t a = tid < n_events ? sm.ev_agent[tid] : CS_AGENT_NONE;
+        if (a != CS_AGENT_NONE && !sm.succ[tid]) ws.cur[sm.ev_chain[tid]] = (uint16_t)a;   // the chain's last live event of the batch
+        if (sm.last_live >= 0) la = sm.ev_agent[sm.last_live];
         if (tid == 0) {
             ws.sc->last_agent = la;
             ws.sc->n_transitions = n_total;
@@ -547,70 +644,74 @@ cs_normalise_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float ta
             if (n_new) atomicAdd((unsigned long long *)&ws.cnt->transitions_counted, (unsigned long long)n_new);
         }
     }
-    if (tid < 64) s_front[tid] = (tid < 32 && !all_chains && la < A && (la >> 5) == tid) ? (1u << (la & 31)) : 0u;
-    // Eq. 10's arg-max successor of the (now final) last agent: asked for here, used by thread 0 after the sums
-    const uint32_t a_star_pre = (tid == 0 && la < A) ? (uint32_t)cs_ld_cg_pinned(ws.amax + la) : 0xFFFFFFFFu;
-    const uint32_t N = n_total;
-    double Hc = 0.0, Hm = 0.0;
-    if (N > 0) {
-        const double invN = 1.0 / (double)N;
-        for (uint32_t i = tid; i < A; i += ROW_THREADS) {
-            const uint32_t rs = i == tid ? pre_rowsum : __ldcg(&ws.rowsum[i]);
-            const double rh = i == tid ? __longlong_as_double((long long)pre_rowH) : __ldcg(&ws.rowH[i]);
-            Hc -= ((double)rs * invN) * rh;
-        }
-        for (uint32_t j = tid; j < A; j += ROW_THREADS) {
-            const unsigned long long qf = j == tid ? pre_qfix : __ldcg(&ws.qfix[j]);
-            const double q = (double)(qf + qbase) * (1.0 / 1152921504606846976.0);
-            if (q > 0.0) Hm -= q * log(q);
-        }
-    }
-    for (uint32_t j = tid; j < A; j += ROW_THREADS) ws.qfix[j] = 0;      // ready for the next refresh
-    __syncthreads();                                                     // (every thread has read qbase)
-    if (tid == 0) ws.sc->qbase = 0;
-    cs_block_sum2(Hc, Hm, s_red);
-    CS_STAMP(ws, CS_PS_REFRESH_SUMS_DONE, tid == 0);                                        // (its barriers also order s_front's zeroes)
-    if (tid == 0) {
-        double R = 0.0;
-        if (N > 0 && Hm > 0.0) R = 1.0 - Hc / Hm;
-        const float Rf = (float)R;
-        ws.sc->R = Rf;
-        ws.sc->gate = (Rf >= r_min) ? 1u : 0u;
-        ws.sc->a_star = a_star_pre;                           // Eq. 10, for the prefetch ranking
-        ws.sc->adjT_cur = fill;
-        ws.sc->ticket0 = 0;
-    }
     if (all_chains) {
         // sources: the current agent of every chain that has one (all live sessions)
-        for (uint32_t ch = tid; ch < n_chains; ch += ROW_THREADS) {
-            const uint32_t a = __ldcg(&ws.cur[ch]);
-            if (a < A) atomicOr(&s_front[a >> 5], 1u << (a & 31));
+        __syncthreads();
+        for (uint32_t x = tid; x < n_chains; x += n_threads) {
+            const uint32_t a = __ldcg(&ws.cur[x]);
+            if (a < A) atomicOr(&sm.front[a >> 5], 1u << (a & 31));
         }
+        __syncthreads();
     }
-    __syncthreads();
-    cs_bfs_survival(ws.adj, A, W, rowT, s_front, s_visit, s_next, s_hops, ws.hops, ws.fsurv, e_max, delta);
+    // The search by the first W warps; the sums of Eq. 2 by the warps behind them, side by side, where the CTA has enough of
+    // them, else by the same warps first.
+    const uint32_t sum0 = 2u * W * 32u <= n_threads ? W * 32u : 0u;       // first thread of the sums
+    if (tid >= sum0 && tid < sum0 + W * 32u) {
+        const uint32_t j = tid - sum0;
+        double Hm = 0.0;
+        if (n_total && j < A) {
+            unsigned long long qf = sm.q[j % COLS];
+            for (uint32_t r = 0; r < CL; ++r) qf += sm.base[r];
+            const double q = (double)qf * (1.0 / 1152921504606846976.0);
+            if (q > 0.0) Hm = -cs_xlogx(q);
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) Hm += __shfl_xor_sync(0xFFFFFFFFu, Hm, d);
+        if (lane == 0) sm.red[j >> 5] = Hm;
+        asm volatile("bar.sync 2, %0;" ::"r"(W * 32u) : "memory");
+        if (j == 0) {
+            double Hc = 0.0, Hs = 0.0;
+            for (uint32_t r = 0; r < CL; ++r) Hc -= sm.hc[r];
+            for (uint32_t w = 0; w < W; ++w) Hs += sm.red[w];
+            double R = 0.0;
+            if (n_total && Hs > 0.0) R = 1.0 - Hc / (double)n_total / Hs;
+            const float Rf = (float)R;
+            ws.sc->R = Rf;
+            ws.sc->gate = (Rf >= r_min) ? 1u : 0u;
+            ws.sc->a_star = la < A ? (uint32_t)sm.amax[la] : 0xFFFFFFFFu;    // Eq. 10, for the prefetch ranking
+        }
+        CS_STAMP(ws, CS_PS_REFRESH_SUMS_DONE, j == 0);
+    }
+    if (tid < 32u * W) {
+        if (!all_chains) {
+            if (tid == 0 && la < A) sm.front[la >> 5] = 1u << (la & 31);
+            asm volatile("bar.sync 1, %0;" ::"r"(W * 32u) : "memory");
+        }
+        cs_bfs_pull<KW>(row, A, W, sm.front, ws.hops, ws.fsurv, e_max, delta);
+    }
     CS_STAMP(ws, CS_PS_REFRESH_END, tid == 0);
 }
 
-// BFS + Eq. 8 from explicit sources into the temporary tables (cs_score_blocks with sources).
-__global__ void __launch_bounds__(ROW_THREADS)
+// BFS + Eq. 8 from explicit sources into the temporary tables (cs_score_blocks with sources): one thread per agent.
+template <int KW>
+__global__ void __launch_bounds__(KW * 32)
 cs_survival_kernel(cs_workspace ws, uint32_t A, uint32_t W, const uint16_t *__restrict__ sources, uint32_t n_sources,
                    uint32_t e_max, float delta)
 {
-    __shared__ uint32_t s_front[64], s_visit[32], s_next[32];
-    __shared__ uint16_t s_hops[CS_MAX_AGENTS];
+    __shared__ uint32_t s_front[2 * PULL_MAX_WORDS];
     const uint32_t tid = threadIdx.x;
-    BfsRow rowT;
-    cs_bfs_load_row(ws.adjT + (size_t)ws.sc->adjT_cur * A * W, A, W, rowT);
-    if (tid < 64) s_front[tid] = 0;
+    uint32_t row[KW];
+#pragma unroll
+    for (int w = 0; w < KW; ++w) row[w] = ((uint32_t)w < W && tid < A) ? cs_ld_cg_pinned(ws.adjT + (size_t)w * A + tid) : 0u;
+    for (uint32_t i = tid; i < 2 * PULL_MAX_WORDS; i += blockDim.x) s_front[i] = 0;
     __syncthreads();
-    for (uint32_t s = tid; s < n_sources; s += ROW_THREADS) {
+    for (uint32_t s = tid; s < n_sources; s += blockDim.x) {
         const uint32_t a = sources[s];
         if (a < A) atomicOr(&s_front[a >> 5], 1u << (a & 31));
         else atomicOr(&ws.sc->status, CS_ST_BAD_SOURCE);
     }
     __syncthreads();
-    cs_bfs_survival(ws.adj, A, W, rowT, s_front, s_visit, s_next, s_hops, ws.hops_tmp, ws.fsurv_tmp, e_max, delta);
+    cs_bfs_pull<KW>(row, A, W, s_front, ws.hops_tmp, ws.fsurv_tmp, e_max, delta);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -811,16 +912,30 @@ int cs_launch_init(cs_ctx *ctx, cudaStream_t s)
     return cs_launch_observe(ctx, nullptr, nullptr, nullptr, 0, s);
 }
 
-// Largest cluster (a power of two) the observe kernel can run as on a device; asked once per process and device, with
-// that device current.
+// Largest cluster (a power of two) a kernel can run as on a device; asked once per process and device, with that device
+// current.
+struct ClusterLimit {
+    std::mutex mu;
+    int known[64];                                            // 0: not asked yet
+    template <class Kernel> int get(int device, Kernel kernel, int most, int threads)
+    {
+        if (device < 0 || device >= 64) return 1;
+        std::lock_guard<std::mutex> lock(mu);
+        if (!known[device]) known[device] = cs_probe_cluster(kernel, most, threads, 0, 1);
+        return known[device];
+    }
+};
 static int obs_cluster_limit(int device)
 {
-    static std::mutex mu;
-    static int known[64];                                     // 0: not asked yet
-    if (device < 0 || device >= 64) return 1;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!known[device]) known[device] = cs_probe_cluster(cs_observe_kernel, OBS_MAX_CLUSTER, OBS_THREADS, 0, 1);
-    return known[device];
+    static ClusterLimit limit;
+    return limit.get(device, cs_observe_kernel, OBS_MAX_CLUSTER, OBS_THREADS);
+}
+static int refresh_cluster_limit(int device)
+{
+    static ClusterLimit l8, l32;                              // both kernels need their opt-in to clusters beyond 8
+    const int a = l8.get(device, cs_refresh_kernel<8>, RfShape<8>::CTAS, RfShape<8>::ROWS * 32);
+    const int b = l32.get(device, cs_refresh_kernel<32>, RfShape<32>::CTAS, RfShape<32>::ROWS * 32);
+    return a < b ? a : b;
 }
 
 int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent, const uint8_t *evflags,
@@ -839,18 +954,37 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
         int rc = cs_check_launch(ctx);
         if (rc != CS_OK) return rc;
     }
-    const uint32_t grid = p.n_agents < 2u * (uint32_t)ctx->sm_count ? p.n_agents : 2u * (uint32_t)ctx->sm_count;
-    cs_launch_chained(cs_normalise_kernel, grid, ROW_THREADS, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min,
-                      p.e_max, p.delta, ctx->source_mode == CS_SOURCES_ALL_CHAINS ? 1u : 0u, p.n_chains,
-                      fused ? chain : (const uint32_t *)nullptr, fused ? agent : (const uint16_t *)nullptr,
-                      fused ? evflags : (const uint8_t *)nullptr, fused ? n_events : 0u,
-                      fused ? (const uint32_t *)ctx->step_n_events_dev : (const uint32_t *)nullptr);
+    const uint32_t all_chains = ctx->source_mode == CS_SOURCES_ALL_CHAINS ? 1u : 0u;
+    if (!fused) chain = nullptr, agent = nullptr, evflags = nullptr;
+    const uint32_t n_fused = fused ? n_events : 0u;
+    const uint32_t *n_fused_dev = fused ? ctx->step_n_events_dev : nullptr;
+    const uint32_t every_row = n_fused ? 0u : 1u;            // a row keeps its P when no event of a small batch starts at it
+    const auto launch = [&](auto kernel, uint32_t cl, uint32_t rows) {
+        cs_launch_chained_clusters(kernel, cl, cl, rows * 32u, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min, p.e_max,
+                                   p.delta, all_chains, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
+    };
+    const uint32_t most = (uint32_t)refresh_cluster_limit(ctx->device);
+    if (p.n_agents <= 32) {
+        // one CTA of as many warps as there are rows, at least one thread per event of a small batch
+        launch(cs_refresh_kernel<1>, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));
+    } else if (p.n_agents <= RfShape<8>::COLS && p.n_agents <= RfShape<8>::ROWS * most) {
+        // few rows per CTA (64 agents: 8.8 us with 32, 7.4 with 16, 6.8 with 8), as far as the cluster goes
+        const uint32_t rows = p.n_agents <= 8u * most ? 8u : RfShape<8>::ROWS;
+        uint32_t cl = 2;
+        while (cl * rows < p.n_agents) cl <<= 1;
+        launch(cs_refresh_kernel<8>, cl, rows);
+    } else {
+        launch(cs_refresh_kernel<32>, most >= 16u ? 16u : 8u, 32u);
+    }
     return cs_check_launch(ctx);
 }
 
 int cs_launch_survival(cs_ctx *ctx, const uint16_t *sources, uint32_t n_sources, cudaStream_t s)
 {
     const cs_params &p = ctx->p;
-    cs_survival_kernel<<<1, ROW_THREADS, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
+    const dim3 block(32u * ctx->W);
+    if (ctx->W == 1) cs_survival_kernel<1><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
+    else if (ctx->W <= 8) cs_survival_kernel<8><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
+    else cs_survival_kernel<32><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
     return cs_check_launch(ctx);
 }

@@ -650,6 +650,33 @@ def test_small_batches_ride_with_the_refresh(A, chains, all_sources):
     assert cn["transitions_counted"] == int(o.C.sum())
 
 
+@pytest.mark.parametrize("A", [1, 2, 31, 32, 33, 64, 65, 129, 255, 256, 257, 511, 513, 1024])
+@pytest.mark.parametrize("tau,eps", [(0.05, 0.01), (0.001, 0.5)])
+def test_refresh_shapes(A, tau, eps):
+    """The learner refresh at the edges of its forms (one CTA up to 32 agents, clusters of several sizes up to 256, columns
+    owned by CTAs above, more than one row per warp above 512), with batches that touch one row, many rows and none, rows
+    with more counts than a warp has lanes, cold rows whose every entry is an edge (a small tau), and a state imported in
+    between."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=5)
+    c, o = make_ctx(cfg, 64, r_min=0.1, tau=tau, eps=eps)
+    rng = synth.rng_for(cfg, 23)
+    H.compare_model(c, o)
+    for size in (1, 1, 40, 256, 256, 255, 33, 3000, 7):
+        chain = rng.integers(0, 5, size).astype(np.uint32)
+        hub = rng.random(size) < 0.5                              # half of the transitions start at or lead to one agent
+        agent = np.where(hub, A // 2, rng.integers(0, A, size)).astype(np.uint16)
+        c.observe_invocations(dev(chain), dev(agent), None)
+        o.observe(chain, agent)
+        H.compare_model(c, o)
+    m = c.get_model()
+    c.import_state(dev(m["C"].astype(np.uint32).ravel()), dev(m["cur"]), m["last_agent"])
+    H.compare_model(c, o)
+    c.observe_invocations(dev(np.zeros(1, np.uint32)), dev(np.array([A - 1], np.uint16)), dev(np.ones(1, np.uint8)))    # warm-up only
+    o.observe(np.zeros(1, np.uint32), np.array([A - 1], np.uint16), np.ones(1, np.uint8))
+    H.compare_model(c, o)
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("A,chains,sizes", [(12, 64, (257, 1024, 1025, 20_000)), (64, 1, (16_384, 16_385)), (65, 3000, (5_000, 33_000)),
                                             (300, 7, (2_047, 2_049))])
 def test_long_batches_across_the_cluster(A, chains, sizes):

@@ -107,10 +107,6 @@ struct cs_sel_state {
     uint32_t c_spec;        // candidates appended by the fast pass; 0 between calls
     uint32_t n_above;       // eligible entries the fast pass found above the remembered bin; 0 between calls
     uint32_t spec;          // 1: the fast pass's candidates cover the k winners, the histogram and collect passes are skipped
-    uint32_t cc[2];         // candidate counters of the cluster kernel: a call uses one and clears the other for the
-                            // next call, so that the counter is zero on entry without a barrier
-    uint32_t toggle;        // which of the two the next call uses; flipped by every call on the device, so that a
-                            // captured sequence of calls stays consistent when it is replayed
 };
 
 // Device pointers into the caller's workspace.

@@ -1011,6 +1011,33 @@ void cs_fill_sel_args(const cs_ctx *ctx, const cs_block_index *idx, uint32_t now
     a.now_dev = ctx->step_now_dev ? ctx->step_now_dev : ctx->clock_dev;
     a.sort_cap = 0;
     a.region_cap_max = ctx->region_cap_max;
+    a.bin_lo = 0;
+    a.bin_shift = 20;
+}
+
+// The scores of Eq. 9 lie between delta^2 (one token) and (1 + delta)^2 |b|: the bins of the cluster select divide that range.
+// A survival table of the caller's own, or a block with more tokens, may leave it; the bins clamp.
+void cs_fill_sel_bins(const cs_ctx *ctx, SelArgs &a, int prefetch)
+{
+    const float d = ctx->p.delta, lo_f = 0.99f * d * d, hi_f = 1.01f * (1.0f + d) * (1.0f + d) * (float)ctx->p.block_tokens;
+    uint32_t lo, hi;
+    memcpy(&lo, &lo_f, 4);
+    memcpy(&hi, &hi_f, 4);
+    if (!(lo_f > 0.0f) || lo >= 0x7F800000u) lo = 0;                // delta^2 underflows
+    if (hi > 0x7F800000u || hi <= lo) hi = 0x7F800000u;
+    if (prefetch) {                                                 // primary = ~bits without the sign: high scores first
+        const uint32_t t = 0x7FFFFFFFu - hi;
+        hi = 0x7FFFFFFFu - lo;
+        lo = t;
+    } else if (a.prefer_copy) {                                     // one bit more below the score
+        lo <<= 1;
+        hi = (hi << 1) | 1u;
+    }
+    const uint32_t bins = (prefetch ? CS_HIST_BINS / 2 : CS_HIST_BINS) - 1u;
+    uint32_t shift = 0;
+    while (((hi - lo) >> shift) >= bins) ++shift;
+    a.bin_lo = lo;
+    a.bin_shift = shift;
 }
 
 uint32_t cs_scan_grid(const cs_ctx *ctx, uint32_t n, uint32_t per_cta, uint32_t ctas_per_sm)
@@ -1073,6 +1100,7 @@ static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, ui
     a.kind = prefetch ? 2u : tier;
     a.sort_cap = ctx->p.max_blocks;          // keys the sort region of this select holds
     if (ctx->select_path != CS_SELECT_MULTI && idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) {
+        cs_fill_sel_bins(ctx, a, prefetch);
         const int rc1 = cs_launch_select_cluster(ctx, &a, &ws, prefetch, ids_out, n_out, s);
         if (rc1 != CS_ENOTIMPL) return rc1;          // no usable cluster on this device: fall through
     }
@@ -1143,6 +1171,7 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
             a[i].k = ks[q];
             a[i].hint_slot = ctx->no_speculation ? 3u : (uint32_t)q;
             a[i].kind = (uint32_t)q;
+            cs_fill_sel_bins(ctx, a[i], q == 2);
             j_ids[i] = ids[q];
             j_cnt[i] = cnt[q];
             pf[i] = q == 2 ? 1u : 0u;

@@ -24,10 +24,12 @@ struct SelArgs {
     const uint32_t *now_dev;      // when set, the clock is read from device memory at execution time (graph replay)
     uint32_t sort_cap;            // keys the sort region holds (0: buckets never get fixed regions)
     uint32_t region_cap_max;      // cap on a bucket's own region (0: none)
+    uint32_t bin_lo, bin_shift;   // histogram bins of the cluster select: (primary - bin_lo) >> bin_shift, set per list kind
 };
 
 // host helpers defined in cs_select.cu
 void cs_fill_sel_args(const cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const float *fsurv, SelArgs &a);
+void cs_fill_sel_bins(const cs_ctx *ctx, SelArgs &a, int prefetch);
 uint32_t cs_scan_grid(const cs_ctx *ctx, uint32_t n, uint32_t per_cta, uint32_t ctas_per_sm = 2);
 size_t cs_table_smem(const cs_ctx *ctx);
 

@@ -186,6 +186,23 @@ def test_select_massive_ties_and_lru_case():
     assert np.all(np.diff(idx.last_access[rest].astype(np.int64)) >= 0)
 
 
+@pytest.mark.parametrize("n,ks", [(127, (1, 64, 127)), (128, (65,)), (4095, (181, 182, 700, 4095)), (8193, (63, 64, 1025, 4096, 4097)),
+                                  (65537, (16, 724, 2000, 9000, 40_000)), (262_144, (300, 12_000, 30_000))])
+@pytest.mark.parametrize("ties", ["ages", "one_age", "two_ages"])
+def test_select_ordering_routes(n, ks, ties):
+    """The ways candidates are put in order inside a cluster -- all against all, ranges of a sample, buckets, a second sample
+    after a first cut, the sample sort through global memory -- with few ties, with every key of an agent tied down to the id,
+    and with two classes of which one lies wholly inside the threshold bin."""
+    cfg = synth.CONFIGS["llama8b"]
+    c, o = warm_state(cfg, 1000, max(n, max(ks)), r_min=0.02)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    if ties != "ages":
+        idx.last_access[:] = 90_000
+        if ties == "two_ages":
+            idx.last_access[::3] = 90_001
+    assert run_selects(c, o, idx, 100_000, ks, tiers=(0,) if n > 100_000 else (0, 1)) == 0
+
+
 def test_select_gate_closed_and_cold_start():
     cfg = synth.CONFIGS["tiny"]
     idx = synth.make_block_index(cfg, n=2560)

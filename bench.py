@@ -1146,18 +1146,16 @@ def run_reference(args):
 
 
 PHASE_NAMES = {0: "refresh: entry", 1: "refresh: dependency wait over", 2: "refresh: rows of CTA 0 done (events applied, Eq. 3, arg-max, adjacency)",
-               3: "refresh: last CTA starts", 4: "refresh: cur[] / last agent written, Eq. 2 done", 5: "refresh: BFS and Eq. 8 done",
-               8: "scan: entry", 9: "scan: tables, thresholds, histogram set up", 10: "scan: dependency wait over",
-               11: "scan: index read, queues worked off (CTA 0)", 12: "scan: candidates and histogram flushed (CTA 0)",
-               13: "scan: last CTA starts", 14: "scan: threshold found, splitters published",
-               24: "bucket: dependency wait over (histogram and collect launches returned)", 25: "bucket: CTA 0 done",
-               26: "scatter: dependency wait over", 27: "rank: dependency wait over", 28: "rank: CTA 0 done",
-               29: "bucket: state, splitters and keys arrived (CTA 0)", 30: "bucket: buckets found (CTA 0)",
-               31: "bucket: slots taken (CTA 0)",
-               40: "rank: bucket offsets known (CTA 0)", 41: "rank: bucket 0 in the tile", 42: "rank: bucket 0 sorted",
-               56: "scan: per-call tables loaded [victims]", 57: "scan: age cuts built [victims]",
+               3: "refresh: rows of the cluster have met in the first CTA", 4: "refresh: Eq. 2 done", 5: "refresh: BFS and Eq. 8 done",
+               8: "scan: entry", 9: "scan: recency table copied", 10: "scan: dependency wait over",
+               11: "scan: index read, queues worked off (CTA 0)", 12: "scan: candidates flushed (CTA 0)",
+               13: "scan: last CTA starts", 14: "scan: verdict written",
+               24: "sample: dependency wait over (histogram and collect launches returned)", 25: "sample: CTA 0 done",
+               26: "place: dependency wait over", 27: "place: CTA 0 done", 28: "finish: dependency wait over",
+               29: "finish: bucket 0 ranked",
+               56: "scan: per-call tables loaded [victims]", 57: "scan: cuts built [victims]",
                58: "scan: index tiles walked, whole rounds of the queue worked off (CTA 0) [victims]",
-               60: "scan: per-call tables loaded [prefetch]", 61: "scan: age cuts built [prefetch]",
+               60: "scan: per-call tables loaded [prefetch]", 61: "scan: cuts built [prefetch]",
                62: "scan: index tiles walked, whole rounds of the queue worked off (CTA 0) [prefetch]"}
 
 

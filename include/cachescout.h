@@ -182,7 +182,7 @@ int cs_select_prefetch(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uin
  * GPU to its KV pool at start-up, a hook that runs while the host application forbids
  * allocation, or a process with a fixed memory budget can own inputs and outputs but cannot
  * provide a workspace.  This call needs neither a cs_ctx nor a workspace: the scratch of the
- * select kernels lives in a static device array inside the library (2 MiB + 40 KiB on every
+ * select kernels lives in a static device array inside the library (2 MiB + 60 KiB on every
  * GPU that loads the library, held until the process exits), and the call itself allocates
  * nothing, on the host or on the device.
  *   p      : the method's constants (n_chains and max_blocks are ignored).
@@ -363,13 +363,13 @@ typedef struct cs_counters {
     uint64_t selects[3];            /* selects completed, per kind */
     uint64_t eligible[3];           /* eligible entries the latest select of the kind saw */
     uint64_t selected[3];           /* ids emitted, per kind */
-    uint64_t candidates[3];         /* keys the latest select of the kind had to order (k winners + ties of the threshold bin) */
-    uint64_t fast_hits[3];          /* selects whose remembered threshold held: the index was read once, mostly without keys */
+    uint64_t candidates[3];         /* keys the latest select of the kind had to order (the list, and what was collected beyond it) */
+    uint64_t fast_hits[3];          /* large selects whose remembered key held: the index was read once, mostly without keys */
     uint64_t blocks_moved[3];       /* blocks copied, per direction */
     uint64_t bytes_moved[3];        /* their bytes (block_bytes each) */
     uint64_t blocks_skipped;        /* mover list entries skipped: CS_ID_NONE or slot out of range */
     uint64_t region_selects[3];     /* multi-launch selects whose sample-sort buckets were filled in place (cs_set_select_bucket_regions) */
-    uint64_t region_overflows[3];   /* of those: a bucket outgrew its region and the buckets were grouped by a launch of their own */
+    uint64_t region_overflows[3];   /* of those: a bucket outgrew its region and was gathered again out of all candidates */
 } cs_counters;
 
 /* Synchronises `stream` and copies the counters to *out (host memory); reset != 0 clears them afterwards. */
@@ -411,7 +411,7 @@ int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream
 /* Phase stamps of the latest calls (profiling builds only: a library compiled with -DCS_PHASE_STAMPS makes its kernels
  * store the GPU's global nanosecond timer at phase boundaries -- refresh: entry, dependency wait over, rows done, last
  * CTA starts, sums done, end; scans: entry, set-up done, wait over, index read, flushed, last CTA starts, tail done;
- * ordering: bucket wait over / done, scatter wait over, rank wait over / done -- slots as in the CS_PS_* list of
+ * ordering: sample, place and finish wait over / done each -- slots as in the CS_PS_* list of
  * csrc/cs_common.cuh, the prefetch select's eight slots above the victims').  Synchronises the device and copies the
  * CS_PHASE_STAMP_SLOTS stamps to `out` (host).  An ordinary build returns CS_ENOTIMPL and stores nothing. */
 #define CS_PHASE_STAMP_SLOTS 64
@@ -459,26 +459,24 @@ int cs_use_survival_table(cs_ctx *ctx, const float *fsurv);
 
 /* Implementation of the two select calls: CS_SELECT_AUTO (= the single-launch cluster kernel up
  * to 262,144 index entries, the multi-launch path above), CS_SELECT_CLUSTER, CS_SELECT_MULTI
- * (fast pass / histogram / collect / bucket / scatter / rank as six grid-wide launches).  Both give the
+ * (fast pass / histogram / collect / sample / place / finish as six grid-wide launches).  Both give the
  * same lists. */
 #define CS_SELECT_AUTO 0u
 #define CS_SELECT_CLUSTER 1u
 #define CS_SELECT_MULTI 2u
 int cs_set_select_path(cs_ctx *ctx, uint32_t path);
 
-/* The multi-launch select remembers the threshold bin each kind of call (GPU victims, host victims,
- * prefetch) ended with, and the next call of that kind collects candidates up to that bin while it
- * builds its histogram; when the new threshold is not above the remembered one the index is read
- * once instead of twice.  The result never depends on it.  enabled = 0 turns the speculation off. */
+/* The multi-launch select remembers a key somewhat above the one each kind of call (GPU victims, host victims,
+ * prefetch) ended with, and the next call of that kind collects the entries at or below it in one scan; when the list
+ * lies within them the index is read once instead of three times.  The result never depends on it.  enabled = 0
+ * turns the speculation off. */
 int cs_set_select_speculation(cs_ctx *ctx, uint32_t enabled);
 
-/* The multi-launch select orders its candidates by a sample sort into <= 256 buckets.  When the candidates are few
- * for the size of the workspace (8 c <= max_blocks) every bucket owns a fixed region of the sort arrays --
- * max_blocks / (buckets) keys, at most 2048 -- which the bucket launch fills directly; a bucket that outgrows its
- * region makes the call fall back to grouping the buckets in a launch of its own.  max_keys caps that region
- * (0 = no cap, the default; 1 = every bucket with two keys or more takes the fallback).  The result never depends
- * on it: the setting exists so that both routes can be exercised and compared.  Host-side, takes effect from the
- * next select call. */
+/* The multi-launch select orders its candidates by a sample sort into up to 512 buckets.  Every bucket owns a fixed region
+ * of the sort arrays -- max_blocks / (buckets) keys -- which the place launch fills; a bucket that outgrows its region is
+ * gathered a second time out of all candidates.  max_keys caps that region (0 = no cap, the default; 1 = every bucket
+ * with two keys or more takes the fallback).  The result never depends on it: the setting exists so that both routes can
+ * be exercised and compared.  Host-side, takes effect from the next select call. */
 int cs_set_select_bucket_regions(cs_ctx *ctx, uint32_t max_keys);
 
 /* Clock source for CUDA-graph replay (the paper's runtime reads now() when a block is touched, Algorithm 1;

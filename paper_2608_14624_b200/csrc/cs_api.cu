@@ -70,9 +70,9 @@ size_t cs_layout_workspace(const cs_params *p, uint32_t gtab_len, void *base, cs
     TAKE(cand_slot, uint32_t, N);
     TAKE(sort_km, unsigned long long, N);
     TAKE(sort_id, uint32_t, N);
-    TAKE(spl_km, unsigned long long, CS_MAX_SPLITTERS + 1);
-    TAKE(spl_id, uint32_t, CS_MAX_SPLITTERS + 1);
-    TAKE(bcount, uint32_t, (CS_MAX_SPLITTERS + 1) * CS_BCOUNT_STRIDE);
+    TAKE(spl_km, unsigned long long, CS_SAMPLE);
+    TAKE(spl_id, uint32_t, CS_SAMPLE);
+    TAKE(bcount, uint32_t, CS_BUCKETS * CS_BCOUNT_STRIDE);
     // Private select state, histogram and candidate / sort regions for the second and third select of a step,
     // which run beside the first one.  Full size up to CS_CONCURRENT_MAX_BLOCKS entries; beyond that only the
     // single-launch cluster select (at most CS_SELECT_CLUSTER_MAX_BLOCKS entries) runs selects side by side.
@@ -90,9 +90,9 @@ size_t cs_layout_workspace(const cs_params *p, uint32_t gtab_len, void *base, cs
         TAKE(cand_slot, uint32_t, Nc);
         TAKE(sort_km, unsigned long long, Nc);
         TAKE(sort_id, uint32_t, Nc);
-        TAKE(spl_km, unsigned long long, CS_MAX_SPLITTERS + 1);
-        TAKE(spl_id, uint32_t, CS_MAX_SPLITTERS + 1);
-        TAKE(bcount, uint32_t, (CS_MAX_SPLITTERS + 1) * CS_BCOUNT_STRIDE);
+        TAKE(spl_km, unsigned long long, CS_SAMPLE);
+        TAKE(spl_id, uint32_t, CS_SAMPLE);
+        TAKE(bcount, uint32_t, CS_BUCKETS * CS_BCOUNT_STRIDE);
             ws = all;
     }
 #undef TAKE

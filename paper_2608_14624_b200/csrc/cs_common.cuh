@@ -37,11 +37,12 @@ struct cs_nvtx_range {
 #define CS_HIST_BINS 4096u        // first radix digit of the select: top 12 bits of the primary key
 #define CS_MAX_SPLITTERS 255u     // bucket sort of the candidates: up to 256 buckets
 #define CS_SAMPLE 1024u           // candidates sampled to choose the splitters
+#define CS_BUCKETS 512u           // buckets of the grid-wide ordering
 #define CS_GTAB_MAX 4096u          // largest recency table kept in shared memory (ages below saturation)
 
 // Scalars the kernels share, one 256-byte line in the workspace.
 #define CS_BCOUNT_STRIDE 8u                                      // words between bucket counters
-#define CS_BCOUNT(ws, b) ((ws).bcount[(size_t)(b) * CS_BCOUNT_STRIDE])
+#define CS_BCOUNT(ws, b) ((ws).bcount[(size_t)(b) * CS_BCOUNT_STRIDE])          // candidates of a bucket
 // Phase stamps (builds with -DCS_PHASE_STAMPS only; cs_debug_phase_stamps() reads them).  A call's kernels are chains
 // of dependent steps whose cost is latency, not work, so "where does the time go" is answered by the GPU's global
 // nanosecond timer read at the boundaries: CS_STAMP(ws, slot, cond) stores it into slot `slot` when `cond` holds
@@ -52,12 +53,9 @@ enum {
     CS_PS_REFRESH_END,
     CS_PS_SCAN_ENTRY = 8,       // + 8 for the prefetch select: entry, set-up done, waited, index read, flushed, last CTA, tail done
     CS_PS_SCAN_SETUP, CS_PS_SCAN_WAITED, CS_PS_SCAN_READ, CS_PS_SCAN_FLUSHED, CS_PS_SCAN_LAST_CTA, CS_PS_SCAN_TAIL_DONE,
-    CS_PS_BUCKET_WAITED = 24,   // + 8 for the prefetch select: bucket waited / done, scatter waited, rank waited / done
-    CS_PS_BUCKET_DONE, CS_PS_SCATTER_WAITED, CS_PS_RANK_WAITED, CS_PS_RANK_DONE, CS_PS_BUCKET_STAGED, CS_PS_BUCKET_SEARCHED,
-    CS_PS_BUCKET_SLOTS,
-    CS_PS_RANK_OFFSETS = 40,    // + 8 for the prefetch select: bucket offsets known, bucket in the tile, tile sorted (CTA 0)
-    CS_PS_RANK_LOADED, CS_PS_RANK_SORTED,
-    CS_PS_SCAN_TABLES = 56,     // + 4 for the prefetch select: per-call tables loaded, age cuts built, index tiles walked (CTA 0)
+    CS_PS_SAMPLE_WAITED = 24,   // + 8 for the prefetch select: sample waited / done, place waited / done, finish waited / done
+    CS_PS_SAMPLE_DONE, CS_PS_PLACE_WAITED, CS_PS_PLACE_DONE, CS_PS_FINISH_WAITED, CS_PS_FINISH_DONE,
+    CS_PS_SCAN_TABLES = 56,     // + 4 for the prefetch select: per-call tables loaded, cuts built, index tiles walked (CTA 0)
     CS_PS_SCAN_CUTS, CS_PS_SCAN_WALKED
 };
 #ifdef CS_PHASE_STAMPS
@@ -83,8 +81,8 @@ struct cs_scalars {
     uint32_t gtab_monotone; // the recency table covers every unsaturated age and never increases with age
     uint32_t status_read;   // cs_get_status(): the value swapped out of `status`
     uint32_t val_le, val_elig, val_ticket;   // cs_validate_selection(): keys at or below the last one, eligible entries, ticket
-    uint32_t sel_hint[4];   // bin up to which the next select of each kind (GPU victims, host victims, prefetch)
-                            // collects ahead of its own threshold, chosen from the previous call's histogram;
+    unsigned long long sel_T[4];   // key (primary, secondary) up to which the next large select of each kind (GPU victims,
+                            // host victims, prefetch) collects in its one scan, chosen by the previous call of the kind;
                             // ~0 = none; slot 3 is never written: calls that must not speculate read it
 #ifdef CS_PHASE_STAMPS
     unsigned long long stamps[CS_N_PHASE_STAMPS];   // %globaltimer at phase boundaries of the latest call (profiling builds)
@@ -94,18 +92,15 @@ struct cs_scalars {
 // State of one select in flight, rewritten by every call.  The selects of a step that run side by side each
 // have their own (with their own histogram, candidate and sort regions).
 struct cs_sel_state {
-    // what the bucket launch reads first, as one 16-byte word
-    uint32_t c;             // candidates collected (first digit <= b0)
-    uint32_t n_spl;         // splitters in use
-    uint32_t placed;        // 1: every bucket has a fixed region of `cap` keys in the sort arrays, filled by the bucket launch
-    uint32_t cap;           // keys per bucket region
+    uint32_t c;             // candidates collected
     uint32_t n_out;         // min(k, eligible)
-    uint32_t overflow;      // 1: a bucket outgrew its region; the scatter launch groups the buckets instead
-    uint32_t b0;            // threshold bin of the first digit
     uint32_t n_elig;        // eligible entries
-    uint32_t ticket[6];     // "last CTA done" counters, one per kernel that has an epilogue
+    uint32_t b0;            // threshold bin of the histogram (after a miss)
+    unsigned long long bound;      // key up to which the candidates were collected
+    unsigned long long ahead;      // key up to which about cs_ahead(k) candidates lie, ~0: fewer were collected
+    uint32_t ticket[4];     // "last CTA done" counters, one per kernel that has an epilogue
     uint32_t c_spec;        // candidates appended by the fast pass; 0 between calls
-    uint32_t n_above;       // eligible entries the fast pass found above the remembered bin; 0 between calls
+    uint32_t n_above;       // eligible entries the fast pass found above the remembered key; 0 between calls
     uint32_t spec;          // 1: the fast pass's candidates cover the k winners, the histogram and collect passes are skipped
 };
 
@@ -133,8 +128,8 @@ struct cs_workspace {
     uint32_t *cand_slot;  // [max_blocks]
     unsigned long long *sort_km;    // [max_blocks] candidates grouped by bucket
     uint32_t *sort_id;    // [max_blocks]
-    unsigned long long *spl_km;     // [CS_MAX_SPLITTERS+1]
-    uint32_t *spl_id;     // [CS_MAX_SPLITTERS+1]
+    unsigned long long *spl_km;     // [CS_SAMPLE] the ranked sample; the splitters of the general route
+    uint32_t *spl_id;     // [CS_SAMPLE]
     uint32_t *bcount;     // bucket counters, one per 32-byte sector (CS_BCOUNT): atomics on counters that share a sector
                           // queue up behind one another in L2 (measured: 3.6 us for 16,000 of them on adjacent words,
                           // 0.8 us on separate sectors; separate 128-byte lines are no faster and cost the readers more)

@@ -35,7 +35,7 @@ __global__ void cs_init_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, u
         memset(&z, 0, sizeof(z));
         z.last_agent = CS_AGENT_NONE;
         z.a_star = 0xFFFFFFFFu;
-        z.sel_hint[0] = z.sel_hint[1] = z.sel_hint[2] = z.sel_hint[3] = 0xFFFFFFFFu;
+        z.sel_T[0] = z.sel_T[1] = z.sel_T[2] = z.sel_T[3] = ~0ull;
         *ws.sc = z;
     }
 }

@@ -12,21 +12,19 @@
 //
 // This file holds the multi-launch path, used for indexes above 262,144 entries (smaller ones take
 // the single-launch cluster kernel of cs_select_cluster.cu).  Six launches, none of which waits
-// on another CTA:
-//   0 fast pass : one scan against the threshold bin remembered from the last call of this kind; when the k
-//                 winners lie within it (the usual case) the candidates are complete and launches 1 and 2
-//                 return at once.  Its last CTA searches the threshold and sorts the splitter sample side by side.
-//   1 histogram : 4096-bin histogram of the top 12 primary bits; the last CTA to finish finds
+// on another CTA outside its own cluster:
+//   0 fast pass : one scan against a key remembered from the last call of this kind; when the k
+//                 winners lie at or below it (the usual case) the candidates are complete and launches 1 and 2
+//                 return at once.
+//   1 histogram : 4096-bin histogram of the primary keys; the last CTA to finish finds
 //                 the threshold bin b0 (first bin whose running count reaches k).
 //   2 collect   : every eligible entry whose bin <= b0 is appended to the candidate buffer
-//                 (c >= min(k, eligible) keys); the last CTA samples <= 1024 candidates,
-//                 sorts them in shared memory and publishes <= 255 splitters.
-//   3 bucket    : each candidate finds its bucket by a search over the splitters and takes a slot in it; with few
-//                 candidates the key goes straight into the bucket's own fixed-size region.
-//   4 scatter   : otherwise the candidates of the needed buckets are grouped by bucket (every CTA derives the
-//                 bucket offsets from the 256 counters itself).
-//   5 rank      : every needed bucket is sorted by one CTA in a shared-memory tile; bucket offset
-//                 + position in the bucket is the position in the output list.
+//                 (c >= min(k, eligible) keys).
+//   3 sample    : 1,024 of the candidates, ranked.
+//   4 place     : what lies beyond the output's share of the sample is dropped; the rest goes to up to 512 buckets of
+//                 consecutive samples, each with a fixed region of the sort arrays.
+//   5 finish    : every bucket's keys are ranked by one CTA, which stores their ids.  Chooses the key that the next call of
+//                 this kind gets.
 // Keys are unique (the id is part of the key), so the order is total and the output does not
 // depend on the order in which atomics were served.
 #include "cs_common.cuh"
@@ -70,80 +68,26 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_score_kernel(SelArgs a, cs_wor
     }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Sample sort set-up, run by one CTA (or half of one) once every candidate is in the buffer: sort P <= 1024 sampled
-// keys in shared memory, publish <= 255 splitters, clear the bucket counters, and decide where the buckets will
-// live.  When the candidates are few for the size of the sort region (8 c <= its capacity), every bucket gets a
-// fixed region of `cap` keys -- at least eight times the mean bucket -- that the bucket launch fills directly.
-// P: power of two, 64 <= P <= min(CS_SAMPLE, 2 * threads of the group).
-// ---------------------------------------------------------------------------------------------
 #define RANK_TILE 2048u                 // keys of the shared-memory tile a bucket is sorted in
-#define CS_SPLIT_SAMPLE_MAX 32768u      // up to this many candidates half a CTA sorts a 512-key sample (fast pass)
-__device__ __forceinline__ void publish_splitters(const cs_workspace &ws, unsigned long long *s_km, uint32_t *s_id,
-                                                  uint32_t c, uint32_t sort_cap, uint32_t region_cap_max, uint32_t P,
-                                                  const CtaPart &cp)
-{
-    const uint32_t n_samp = c < P ? c : P;
-    {
-        // a group sorts two keys per thread: both are fetched before either is stored
-        const uint32_t i0 = cp.t, i1 = cp.t + cp.n;
-        unsigned long long k0 = ~0ull, k1 = ~0ull;
-        uint32_t d0 = 0xFFFFFFFFu, d1 = 0xFFFFFFFFu;
-        if (i0 < n_samp) {
-            const uint32_t pos = (uint32_t)(((unsigned long long)i0 * c) / n_samp);
-            k0 = __ldcg(&ws.cand_km[pos]);
-            d0 = __ldcg(&ws.cand_id[pos]);
-        }
-        if (i1 < n_samp) {
-            const uint32_t pos = (uint32_t)(((unsigned long long)i1 * c) / n_samp);
-            k1 = __ldcg(&ws.cand_km[pos]);
-            d1 = __ldcg(&ws.cand_id[pos]);
-        }
-        if (i0 < P) { s_km[i0] = k0; s_id[i0] = d0; }
-        if (i1 < P) { s_km[i1] = k1; s_id[i1] = d1; }
-    }
-    part_sync(cp);
-    bitonic_sort_fast(s_km, s_id, P, cp);
-    uint32_t n_spl = c / 64;
-    if (n_spl > CS_MAX_SPLITTERS) n_spl = CS_MAX_SPLITTERS;
-    for (uint32_t j = cp.t; j <= CS_MAX_SPLITTERS; j += cp.n) {
-        if (j < n_spl) {
-            const uint32_t q = (uint32_t)(((unsigned long long)(j + 1) * n_samp) / (n_spl + 1));
-            ws.spl_km[j] = s_km[q];
-            ws.spl_id[j] = s_id[q];
-        }
-        CS_BCOUNT(ws, j) = 0;
-    }
-    if (cp.t == 0) {
-        uint32_t cap = sort_cap / (n_spl + 1u);
-        if (cap > RANK_TILE) cap = RANK_TILE;
-        if (region_cap_max && cap > region_cap_max) cap = region_cap_max;
-        ws.sel->n_spl = n_spl;
-        ws.sel->placed = (c && 8ull * c <= sort_cap) ? 1u : 0u;
-        ws.sel->cap = cap;
-        ws.sel->overflow = 0;
-    }
-}
 
 // ---------------------------------------------------------------------------------------------
-// 0 fast pass (remembered threshold)
+// 0 fast pass (remembered key)
 //
-// The threshold bin moves little from one call to the next, so each kind of call (GPU victims, host
-// victims, prefetch) remembers a bin H at or a little above the one it ended with.  With H known, almost
-// every eligible entry can be dismissed without its key, in two steps:
-//   a  by age alone.  For victims (low scores = old blocks) an entry younger than a cut A_c cannot reach
-//      H whatever its agent and size: fl(f_min * g(age)) is already on the far side of the largest per-size
-//      threshold X (build_x_thresholds), g never increases with age, and IEEE products are monotone.  That is
-//      ONE integer compare on last_access per entry.  For prefetch candidates (high scores = young blocks)
-//      the same holds with the roles swapped, for entries of agents other than a*.
-//   b  what is left (a few per cent) is queued per warp as entry ids and worked off with all 32 lanes
-//      busy: two table look-ups, one multiply and one compare against X decide exactly whether the entry's
-//      first key digit is <= H; only then is the key built, binned and appended to the candidate buffer.
-// Dismissed entries are only counted.  The last CTA has the exact histogram of bins <= H plus the number
-// of entries above: if the k-th smallest key lies within H the candidates are complete, the sample sort is
-// set up right here, and the index has been read ONCE at a fraction of the instructions of a full-key
-// scan.  Otherwise (the threshold rose above H, or nothing is remembered yet) the pass reports a miss and
-// the full histogram and collect passes below run.  The result never depends on H.
+// The k-th smallest key moves little from one call to the next, so each kind of call (GPU victims, host
+// victims, prefetch) remembers a key T somewhat above the one it ended with (cs_ahead()).  With T known, almost
+// every eligible entry is dismissed by ONE compare of its last_access:
+//   a  for a fixed agent and the common block size the key never decreases with last_access (victims: younger blocks score
+//      higher, equal scores order by last_access; IEEE products are monotone, and g never increases with age) or never
+//      increases (prefetch), so "key <= T" is a half-line of last_access.  Its end is found once per agent and CTA by
+//      binary search over ages -- exactly, the part of a tie in score that lies below T's last_access included.  (A cut
+//      by score alone let every entry tied with T through: 70,000 of 1,000,000 for k = 10,000, 990,000 of 9,400,000 for
+//      k = 203, where a fifth of the ages are past the point at which the recency factor saturates.)
+//   b  what is left (the candidates, and blocks of another size) is queued per warp as entry ids and worked off with all 32
+//      lanes busy: the key is built and compared with T; candidates are appended to the buffer.
+// Dismissed entries are only counted.  If at least k candidates were found, or nothing eligible lies above T, the
+// candidates are complete and the index has been read ONCE.  Otherwise (the threshold rose above T, or nothing is
+// remembered yet) the pass reports a miss and the full histogram and collect passes below run.  The result never depends
+// on T.
 // ---------------------------------------------------------------------------------------------
 #define FQ_CAP 544u                 // per-warp queue: at most 31 left over + the 512 entries of one warp tile
 
@@ -155,93 +99,86 @@ __device__ __forceinline__ uint32_t max_halves(const uint4 &a, const uint4 &b)
     return max(m & 0xFFFFu, m >> 16);
 }
 
+// End of the half-line of last_access that an agent's blocks of the common size need for a key at or below T: victims
+// la <= cut, prefetch la >= cut.  (Entries on the line's side of it that fail after all are sorted out by the exact test.)
 template <bool PF>
-__global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_workspace ws)
+__device__ __forceinline__ uint32_t la_cut(const SelArgs &a, const Tables &T, uint32_t agent, u64 bound)
 {
-    extern __shared__ float smem[];                 // tables, then the per-warp queues (reused by the epilogue)
-    __shared__ __align__(16) uint32_t s_hist[CS_HIST_BINS];   // bins of the candidates (the threshold bin is dense: global
-                                                              // atomics on one address per candidate would serialise)
-    __shared__ uint32_t s_xt[2 * XT_TOK];
-    __shared__ uint32_t s_part[SEL_THREADS];
-    __shared__ uint32_t s_b0, s_ahead, s_above;
+    const uint32_t Tp = (uint32_t)(bound >> 32), Ts = (uint32_t)bound;
+    const uint32_t flip = (PF && agent != T.a_star) ? 0x80000000u : 0u;
+    // smallest possible primary key at an age (a copy on the other tier would make it that; the exact test tells)
+    auto primary = [&](uint32_t age) {
+        const uint32_t bits = __float_as_uint(score_from_age(a, T, agent, age, a.block_tokens));
+        return PF ? (flip | (~bits & 0x7FFFFFFFu)) : (a.prefer_copy ? bits << 1 : bits);
+    };
+    // victims: primary falls with age: n_le = first age with primary <= Tp, n_lt = first with primary < Tp (age_sat + 1: none);
+    // prefetch: it rises: n_le = first age with primary > Tp, n_lt = first with primary >= Tp
+    uint32_t lo0 = 0, hi0 = a.age_sat + 1, lo1 = 0, hi1 = a.age_sat + 1;
+    while (lo0 < hi0 || lo1 < hi1) {
+        const uint32_t m0 = lo0 + ((hi0 - lo0) >> 1), m1 = lo1 + ((hi1 - lo1) >> 1);
+        const uint32_t p0 = primary(m0 < a.age_sat ? m0 : a.age_sat), p1 = primary(m1 < a.age_sat ? m1 : a.age_sat);
+        if (lo0 < hi0) { if (PF ? p0 > Tp : p0 <= Tp) hi0 = m0; else lo0 = m0 + 1; }
+        if (lo1 < hi1) { if (PF ? p1 >= Tp : p1 < Tp) hi1 = m1; else lo1 = m1 + 1; }
+    }
+    const uint32_t n_le = lo0, n_lt = lo1;
+    if (!PF) {
+        if (n_le > a.age_sat) return 0u;                                   // no age qualifies
+        // la <= now - n_lt for the ages below T's score; at T's score (n_le <= age < n_lt) also la <= Ts.  Age 0 stands for
+        // every last_access from now on.
+        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt : 0u));
+        const uint32_t at_score = min(n_le == 0 ? 0xFFFFFFFFu : (a.now >= n_le ? a.now - n_le : 0u), Ts);
+        return max(by_score, at_score);
+    } else {
+        if (n_le == 0) return 0xFFFFFFFFu;                                 // not even age 0
+        // la > now - n_lt for the ages above T's score; at T's score (n_lt <= age < n_le) also ~la <= Ts
+        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt + 1u : 0u));
+        const uint32_t at_score = max(n_le > a.age_sat ? 0u : (a.now >= n_le ? a.now - n_le + 1u : 0u), ~Ts);
+        return min(by_score, at_score);
+    }
+}
+
+template <bool PF>
+__global__ void __launch_bounds__(SEL_THREADS, 2) cs_sel_fast_kernel(SelArgs a, cs_workspace ws)
+{
+    extern __shared__ float smem[];                 // tables, per-warp queues, per-warp candidate staging, cuts
+    __shared__ uint32_t s_above;
     __shared__ bool s_flag;
     constexpr int PS = PF ? 8 : 0;                  // phase-stamp slots of this kind of scan (profiling builds)
+    (void)PS;
     CS_STAMP(ws, CS_PS_SCAN_ENTRY + PS, blockIdx.x == 0 && threadIdx.x == 0);
     cs_release_successor();
-    // Before waiting for the predecessor grid: everything that depends only on the context's constants and on the
-    // remembered bin (a stale bin would cost time, never correctness: the result does not depend on H).
-    const uint32_t H = ws.sc->sel_hint[a.hint_slot];        // ~0: nothing remembered
+    // Before waiting for the predecessor grid: what depends only on the context's constants.
     Tables T;
     const size_t table_words = ((size_t)(a.A + a.gtab_len) * 4 + (size_t)a.A * 2 + 15) / 16 * 4;
     uint32_t *queues = (uint32_t *)smem + table_words;
-    const size_t cut_off_words = table_words + (size_t)(SEL_THREADS / 32) * (FQ_CAP + STAGE_CAP * 3) + 4;     // after queues and staging
-    if (H != 0xFFFFFFFFu) {
-        load_tables_static(a, ws, smem, T);
-        build_x_thresholds<PF>(a, H, s_xt);
-        for (uint32_t i = threadIdx.x; i < CS_HIST_BINS; i += blockDim.x) s_hist[i] = 0;
-        if (threadIdx.x == 0) s_above = 0;
-    }
+    uint32_t *s_cut = queues + (size_t)(SEL_THREADS / 32) * (FQ_CAP + STAGE_CAP * 3) + 4;     // after queues and staging
+    load_tables_static(a, ws, smem, T);
+    if (threadIdx.x == 0) s_above = 0;
     CS_STAMP(ws, CS_PS_SCAN_SETUP + PS, blockIdx.x == 0 && threadIdx.x == 0);
     cs_wait_for_predecessor();
     CS_STAMP(ws, CS_PS_SCAN_WAITED + PS, blockIdx.x == 0 && threadIdx.x == 0);
-    if (H == 0xFFFFFFFFu) {                                   // every CTA sees the same word
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    const uint32_t n_tiles = a.n / TILE, n_warps = nth >> 5;
+    // the first tile travels with the tables
+    const u64 bound = cs_ld_cg_pinned(&ws.sc->sel_T[a.hint_slot]);      // ~0: nothing remembered
+    Group G;
+    if ((gtid >> 5) < n_tiles) load_group<PF>(a, gtid >> 5, lane, G);
+    resolve_now(a);
+    load_tables_dynamic(a, ws, T, PF && a.anchor);
+    if (bound == ~0ull) {                                     // every CTA sees the same word
         if (blockIdx.x == 0 && threadIdx.x == 0) ws.sel->spec = 0;
         return;
     }
-    resolve_now(a);
-    load_tables_dynamic(a, ws, T, PF && a.anchor);
     __syncthreads();
     CS_STAMP(ws, CS_PS_SCAN_TABLES + PS / 2, blockIdx.x == 0 && threadIdx.x == 0);
-    // ---- the age cuts, one per agent, for blocks of the common size ----------------------------------------
-    // victims: s_cut[agent] = number of ages (0, 1, ..) that are dismissed, i.e. for which fl(f g(age)) >= X;
-    // prefetch: s_cut[agent] = first age that is dismissed, i.e. fl(f g(age)) < X of the agents other than a*.
-    // Both rely on g never increasing with age (checked when the table was built) and on the table covering every
-    // unsaturated age; otherwise nothing is dismissed by age and every eligible entry takes the exact test.
-    const uint32_t Tb = a.block_tokens;
-    uint32_t *s_cut = (uint32_t *)smem + cut_off_words;
-    {
-        const bool usable = ws.sc->gtab_monotone && a.gtab_len == a.age_sat;
-        const uint32_t X = s_xt[(PF ? XT_TOK : 0u) + Tb];
-        for (uint32_t e = threadIdx.x; e < a.A; e += blockDim.x) {
-            const float f = T.fsurv[e];
-            auto dismissed = [&](uint32_t age) {
-                const uint32_t xb = __float_as_uint(__fmul_rn(f, recency_of_age(a, T, age)));
-                return PF ? (xb < X) : (xb >= X);
-            };
-            uint32_t cut;
-            if (!PF) {
-                cut = 0;                                            // none
-                if (usable && X != XT_NONE && dismissed(0)) {
-                    if (dismissed(a.age_sat)) cut = 0xFFFFFFFFu;    // every age
-                    else {
-                        uint32_t lo = 0, hi = a.age_sat;            // largest dismissed age
-                        while (lo < hi) {
-                            const uint32_t mid = lo + ((hi - lo + 1) >> 1);
-                            if (dismissed(mid)) lo = mid;
-                            else hi = mid - 1;
-                        }
-                        cut = lo + 1;
-                    }
-                }
-            } else {
-                cut = 0xFFFFFFFFu;                                  // none
-                if (usable && (X == XT_NONE || dismissed(0))) cut = 0;          // every age
-                else if (usable && dismissed(a.age_sat)) {
-                    uint32_t lo = 0, hi = a.age_sat;                // smallest dismissed age
-                    while (lo < hi) {
-                        const uint32_t mid = lo + ((hi - lo) >> 1);
-                        if (dismissed(mid)) hi = mid;
-                        else lo = mid + 1;
-                    }
-                    cut = lo;
-                }
-            }
-            s_cut[e] = cut;
-        }
-    }
+    // the cuts rely on g never increasing with age (checked when the table was built) and on the table covering every
+    // unsaturated age; otherwise nothing is dismissed and every eligible entry takes the exact test
+    const bool usable = ws.sc->gtab_monotone && a.gtab_len == a.age_sat;
+    for (uint32_t e = threadIdx.x; e < a.A; e += blockDim.x) s_cut[e] = usable ? la_cut<PF>(a, T, e, bound) : (PF ? 0u : 0xFFFFFFFFu);
     __syncthreads();
     CS_STAMP(ws, CS_PS_SCAN_CUTS + PS / 2, blockIdx.x == 0 && threadIdx.x == 0);
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t Tb = a.block_tokens;
     uint32_t *q = queues + warp * FQ_CAP;
     uint32_t qn = 0;                                           // queued ids of this warp (same value in every lane)
     WarpStage st;
@@ -258,29 +195,15 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
         for (uint32_t r = 0; r < rounds; ++r) {
             const uint32_t i = r * 32u + lane;
             bool cand = false;
-            uint32_t id = 0, ag = 0, la = 0, tok = a.block_tokens, dp = 0, fl = 0;
+            uint32_t id = 0, pr = 0, se = 0;
             if (i < qn) {
                 id = q[i];
-                ag = __ldg(a.agent + id);
-                la = __ldg(a.la + id);
-                fl = __ldg(a.flags + id);                        // (needed by the key of a candidate: one round trip, not two)
-                if (a.ntok) tok = __ldg(a.ntok + id);
-                if (PF && a.anchor) dp = __ldg(a.depth + id);
-                bool elig = true;
-                if (ag >= a.A) { atomicOr(&ws.sc->status, CS_ST_BAD_AGENT); elig = false; }
-                else if (PF && a.anchor && !(dp < T.anchor[ag])) elig = false;
-                if (elig) {
-                    const uint32_t age = la <= a.now ? a.now - la : 0u;
-                    const uint32_t xb = __float_as_uint(__fmul_rn(T.fsurv[ag], recency_of_age(a, T, age)));
-                    const uint32_t X = s_xt[((PF && ag != T.a_star) ? XT_TOK : 0u) + tok];
-                    cand = PF ? (xb >= X) : (xb < X);
+                const uint32_t ag = __ldg(a.agent + id), la = __ldg(a.la + id), fl = __ldg(a.flags + id);
+                const uint32_t tok = a.ntok ? __ldg(a.ntok + id) : Tb, dp = (PF && a.anchor) ? __ldg(a.depth + id) : 0u;
+                if (entry_key_rest<PF>(a, T, &ws.sc->status, ag, dp, fl, la, tok, pr, se)) {
+                    cand = (((u64)pr << 32) | se) <= bound;
                     if (!cand) ++n_above;
                 }
-            }
-            uint32_t pr = 0, se = 0;
-            if (cand) {
-                entry_key_rest<PF>(a, T, &ws.sc->status, ag, dp, fl, la, tok, pr, se);
-                atomicAdd(&s_hist[pr >> 20], 1u);
             }
             // candidates gather in the warp's slice of shared memory and leave it 32 or more at a time
             stage_push(st, cand, pr, se, id, &ws.sel->c_spec, ws.cand_km, ws.cand_id);
@@ -299,49 +222,43 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
     };
 
     if (enabled) {
-        const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-        const uint32_t n_tiles = a.n / TILE, n_warps = nth >> 5;
         const uint32_t n_iter = (n_tiles + n_warps - 1) / n_warps;     // whole warps stay in the shuffles
         for (uint32_t it = 0; it < n_iter; ++it) {
             const uint32_t t = it * n_warps + (gtid >> 5);
             uint32_t rem = 0;                                          // entries that need the exact test
             if (t < n_tiles) {
-                Group G;
-                load_group<PF>(a, t, lane, G);
+                if (it) load_group<PF>(a, t, lane, G);
                 const uint32_t em = group_elig<PF>(a, G);
+                uint32_t near = 0;                                     // on the cut's side of last_access, or of another size
                 if (!PF) {
-                    uint32_t dm = 0;                                   // dismissed by age: young, of the common size
                     if (max_halves(G.ag0, G.ag1) < a.A) {              // (a bad agent id anywhere: everything takes the exact test)
 #pragma unroll
-                        for (int j = 0; j < GRP; ++j) {
-                            const uint32_t la = grp_u32(G, j), age = max(a.now, la) - la;
-                            dm |= (age < s_cut[grp_u16(G.ag0, G.ag1, j)] ? 1u : 0u) << j;
-                        }
+                        for (int j = 0; j < GRP; ++j) near |= (grp_u32(G, j) <= s_cut[grp_u16(G.ag0, G.ag1, j)] ? 1u : 0u) << j;
                         if (a.ntok) {
-                            uint32_t same = 0;
 #pragma unroll
                             for (int w = 0; w < 4; ++w)
-                                same |= nibble_of_flags(zero_bytes(u4_word(G.tk, w) ^ (0x01010101u * Tb))) << (4 * w);
-                            dm &= same;
+                                near |= (~nibble_of_flags(zero_bytes(u4_word(G.tk, w) ^ (0x01010101u * Tb))) & 0xFu) << (4 * w);
                         }
+                    } else {
+                        near = 0xFFFFu;
                     }
-                    n_above += __popc(em & dm);
-                    rem = em & ~dm;
+                    n_above += __popc(em & ~near);
+                    rem = em & near;
                 } else {
 #pragma unroll
                     for (int j = 0; j < GRP; ++j) {
                         if (!((em >> j) & 1u)) continue;
                         const uint32_t ag = grp_u16(G.ag0, G.ag1, j);
                         const uint32_t tok = a.ntok ? grp_u8(G.tk, j) : Tb;
-                        if (ag >= a.A || ag == T.a_star || tok != Tb) { rem |= 1u << j; continue; }
+                        if (ag >= a.A || tok != Tb) { rem |= 1u << j; continue; }
                         if (a.anchor && !(grp_u16(G.dp0, G.dp1, j) < T.anchor[ag])) continue;      // not eligible
-                        const uint32_t la = grp_u32(G, j), age = max(a.now, la) - la;
-                        if (age >= s_cut[ag]) ++n_above;
-                        else rem |= 1u << j;
+                        if (grp_u32(G, j) >= s_cut[ag]) rem |= 1u << j;
+                        else ++n_above;
                     }
                 }
             }
             // queue the remaining entries of the warp (ids only), then work off whole rounds
+            if (!__any_sync(0xFFFFFFFFu, rem != 0u)) continue;
             const uint32_t cnt = __popc(rem);
             uint32_t incl = cnt;
 #pragma unroll
@@ -350,7 +267,6 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
                 if (lane >= d) incl += v;
             }
             const uint32_t total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-            if (total == 0) continue;
             uint32_t pos = qn + incl - cnt;
             while (rem) {
                 const int j = __ffs(rem) - 1;
@@ -366,13 +282,12 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
         stage_flush(st, &ws.sel->c_spec, ws.cand_km, ws.cand_id);
         CS_STAMP(ws, CS_PS_SCAN_READ + PS, blockIdx.x == 0 && threadIdx.x == 0);
         const uint32_t t0 = n_tiles * TILE;
-        if (gtid < a.n - t0) {                                // ragged tail, one entry per thread, through the key
+        if (gtid < a.n - t0) {                                // ragged tail, one entry per thread
             const uint32_t i = t0 + gtid;
             uint32_t pr, se;
-            const uint32_t tok = a.ntok ? a.ntok[i] : a.block_tokens;
+            const uint32_t tok = a.ntok ? a.ntok[i] : Tb;
             if (entry_key<PF>(a, T, &ws.sc->status, a.agent[i], a.depth[i], a.ref[i], a.flags[i], a.la[i], tok, pr, se)) {
-                if ((pr >> 20) <= H) {
-                    atomicAdd(&s_hist[pr >> 20], 1u);
+                if ((((u64)pr << 32) | se) <= bound) {
                     const uint32_t pos = atomicAdd(&ws.sel->c_spec, 1u);
                     ws.cand_km[pos] = ((unsigned long long)pr << 32) | se;
                     ws.cand_id[pos] = i;
@@ -382,94 +297,27 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
             }
         }
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) n_above += __shfl_xor_sync(0xFFFFFFFFu, n_above, d);
+    n_above = __reduce_add_sync(0xFFFFFFFFu, n_above);
     if (lane == 0 && n_above) atomicAdd(&s_above, n_above);
     __syncthreads();
-    {
-        const uint32_t h_end = H < CS_HIST_BINS ? H + 1u : CS_HIST_BINS;          // bins above H stay empty
-        for (uint32_t i = threadIdx.x; i < h_end; i += blockDim.x) {
-            const uint32_t v = s_hist[i];
-            if (v) atomicAdd(&ws.hist[i], v);
-        }
-    }
     if (threadIdx.x == 0 && s_above) atomicAdd(&ws.sel->n_above, s_above);
     CS_STAMP(ws, CS_PS_SCAN_FLUSHED + PS, blockIdx.x == 0 && threadIdx.x == 0);
     if (!last_cta_done(&ws.sel->ticket[0], &s_flag)) return;
     CS_STAMP(ws, CS_PS_SCAN_LAST_CTA + PS, threadIdx.x == 0);
-
-    // ---- last CTA -----------------------------------------------------------------------------------------
-    // Two things are left and neither needs the other: whether the k-th smallest key lies within the remembered
-    // bin (a scan of the histogram), and the splitters for ordering the candidates (a sort of a sample of them).
-    // With few candidates half of the CTA is enough for the sample, so the two halves do one each, side by side;
-    // the sample sort is then wasted on a miss, which costs nothing on the critical path.
-    constexpr uint32_t HALF = SEL_THREADS / 2;
-    const uint32_t c_spec = __ldcg(&ws.sel->c_spec);
-    const uint32_t c_use = a.k ? c_spec : 0u;
-    const bool small = c_use <= CS_SPLIT_SAMPLE_MAX;
-    unsigned long long *s_km = (unsigned long long *)(((uintptr_t)queues + 7) & ~(uintptr_t)7);   // the queues are idle now
-    uint32_t *s_id = (uint32_t *)(s_km + CS_SAMPLE);
-    if (threadIdx.x >= HALF) {
-        if (small) {
-            // a sample of at least twice the splitters (c / 64 of them): 128, 256 or 512 keys
-            const uint32_t P = c_use <= 4096u ? 128u : (c_use <= 8192u ? 256u : CS_SAMPLE / 2);
-            publish_splitters(ws, s_km, s_id, c_use, a.sort_cap, a.region_cap_max, P, CtaPart{threadIdx.x - HALF, HALF, 2u});
-        }
-    } else {
-        const CtaPart cp{threadIdx.x, HALF, 1u};
-        constexpr uint32_t PER = CS_HIST_BINS / HALF;
-        uint32_t loc[PER], sum = 0;
-        {
-            uint4 *h4 = (uint4 *)(ws.hist + threadIdx.x * PER);
-#pragma unroll
-            for (uint32_t qq = 0; qq < PER / 4; ++qq) {
-                const uint4 v = __ldcg(h4 + qq);
-                h4[qq] = make_uint4(0u, 0u, 0u, 0u);             // ready for the next pass or call
-                loc[4 * qq] = v.x; loc[4 * qq + 1] = v.y; loc[4 * qq + 2] = v.z; loc[4 * qq + 3] = v.w;
-                sum += v.x + v.y + v.z + v.w;
-            }
-        }
-        if (threadIdx.x == 0) s_b0 = 0xFFFFFFFFu;
-        uint32_t below;                                          // eligible entries at or below H
-        const uint32_t before = sel_block_scan(sum, s_part, below, cp);
-        const uint32_t total = below + __ldcg(&ws.sel->n_above);
-        if (a.k && below >= a.k && before < a.k && a.k <= before + sum) {
-            uint32_t run = before;
-#pragma unroll
-            for (uint32_t qq = 0; qq < PER; ++qq) {
-                run += loc[qq];
-                if (run >= a.k) { s_b0 = threadIdx.x * PER + qq; break; }
-            }
-        }
-        part_sync(cp);
-        // complete when the k winners lie at or below H, when fewer than k entries are eligible and all of them do, or when k = 0
-        const bool hit = a.k == 0 || below >= a.k || below == total;
-        const uint32_t b0 = a.k == 0 ? 0xFFFFFFFFu : (s_b0 != 0xFFFFFFFFu ? s_b0 : (H < CS_HIST_BINS ? H : CS_HIST_BINS - 1));
-        uint32_t ahead = 0;
-        const bool have_b0 = a.k && below >= a.k;
-        if (hit && have_b0) {
-            ahead = collect_ahead_limit<PER>(loc, threadIdx.x * PER, before, a.k, b0, &s_ahead, cp);
-            if (ahead > H) ahead = H;                             // nothing is known about the bins above H
-        }
-        if (threadIdx.x == 0) {
-            s_flag = hit;
-            if (hit) {
-                ws.sel->b0 = b0;
-                ws.sel->n_elig = total;
-                ws.sel->n_out = total < a.k ? total : a.k;
-                ws.sel->c = c_use;
-                count_select(ws, a.kind, total, total < a.k ? total : a.k);
-                count_candidates(ws, a.kind, c_use, true);
-                // fewer eligible entries than k: keep H; otherwise tighten it to what the histogram allows
-                if (have_b0) remember_threshold(ws.sc, a.hint_slot, true, ahead);
-            }
-        }
-    }
-    __syncthreads();
-    const bool hit = s_flag;
-    if (hit && !small) publish_splitters(ws, s_km, s_id, c_use, a.sort_cap, a.region_cap_max, CS_SAMPLE, whole_cta());
     if (threadIdx.x == 0) {
+        const uint32_t c = __ldcg(&ws.sel->c_spec), above = __ldcg(&ws.sel->n_above), total = c + above;
+        // complete when the k winners lie at or below T, when fewer than k entries are eligible and all of them do, or when k = 0
+        const bool hit = a.k == 0 || c >= a.k || above == 0;
         ws.sel->spec = hit ? 1u : 0u;
+        if (hit) {
+            const uint32_t n_out = total < a.k ? total : a.k;
+            ws.sel->c = c;
+            ws.sel->n_out = n_out;
+            ws.sel->n_elig = total;
+            ws.sel->bound = bound;
+            count_select(ws, a.kind, total, n_out);
+            count_candidates(ws, a.kind, a.k ? c : 0u, true);
+        }
         ws.sel->c_spec = 0;
         ws.sel->n_above = 0;
         ws.sel->ticket[0] = 0;
@@ -480,8 +328,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_fast_kernel(SelArgs a, cs_
 // ---------------------------------------------------------------------------------------------
 // 1 histogram (runs when the fast pass missed or had nothing to go by)
 //
-// Full keys of all eligible entries into a 4096-bin histogram; the last CTA finds the threshold bin and
-// chooses how far ahead of it the next call of this kind may look.
+// Full keys of all eligible entries into a 4096-bin histogram; the last CTA finds the threshold bin.
 // ---------------------------------------------------------------------------------------------
 template <bool PF>
 __global__ void __launch_bounds__(SEL_THREADS) cs_sel_hist_kernel(SelArgs a, cs_workspace ws)
@@ -489,7 +336,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_hist_kernel(SelArgs a, cs_
     extern __shared__ float smem[];
     __shared__ __align__(16) uint32_t s_hist[CS_HIST_BINS];
     __shared__ uint32_t s_part[SEL_THREADS];
-    __shared__ uint32_t s_b0, s_ahead;
+    __shared__ uint32_t s_b0;
     __shared__ bool s_flag;
     cs_wait_for_predecessor();
     cs_release_successor();
@@ -502,7 +349,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_hist_kernel(SelArgs a, cs_
     if (!PF || prefetch_enabled(ws, a.A)) {
         uint32_t run_bin = 0xFFFFFFFFu, run_cnt = 0;                    // adjacent entries often share a bin
         for_each_eligible<PF>(a, T, &ws.sc->status, [&](uint32_t, uint32_t pr, uint32_t) {
-            const uint32_t bin = pr >> 20;
+            const uint32_t bin = bin_of<PF>(a, pr);
             if (bin == run_bin) { ++run_cnt; return; }
             if (run_cnt) atomicAdd(&s_hist[run_bin], run_cnt);
             run_bin = bin;
@@ -547,21 +394,19 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_hist_kernel(SelArgs a, cs_
     }
     __syncthreads();
     const uint32_t b0 = s_b0;
-    const bool have_b0 = a.k && total >= a.k;
-    const uint32_t ahead = have_b0 ? collect_ahead_limit<PER>(loc, threadIdx.x * PER, before, a.k, b0, &s_ahead, whole_cta()) : 0u;
     if (threadIdx.x == 0) {
         ws.sel->b0 = b0;
         ws.sel->n_elig = total;
         ws.sel->n_out = total < a.k ? total : a.k;
+        ws.sel->bound = b0 == 0xFFFFFFFFu ? 0ull : (primary_limit<PF>(a, b0) << 32) - 1ull;
         count_select(ws, a.kind, total, total < a.k ? total : a.k);
         ws.sel->c = 0;
-        remember_threshold(ws.sc, a.hint_slot, have_b0, ahead);
         ws.sel->ticket[1] = 0;
     }
 }
 
 // ---------------------------------------------------------------------------------------------
-// 2 collect (+ splitters)
+// 2 collect
 // ---------------------------------------------------------------------------------------------
 // Age limits.  For a fixed agent and block size the score never increases with age (the recency
 // table is checked to be monotone, IEEE multiplication is), so "first digit <= b0" is an interval
@@ -576,43 +421,28 @@ __device__ __forceinline__ uint32_t age_limit_of(const SelArgs &a, const Tables 
                                                  uint32_t b0)
 {
     const uint32_t n_age = a.age_sat;                        // ages >= age_sat all score like age_sat
-    if (!PF) {
-        // candidate <=> score bits < lim_bits, i.e. (bits [<< 1 | copy bit]) >> 20 <= b0
-        const unsigned long long lim_bits = (unsigned long long)(b0 + 1u) << (a.prefer_copy ? 19 : 20);
-        uint32_t lo = 0, hi = n_age + 1;                      // first age with bits < lim_bits; n_age + 1 = none
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            const unsigned long long bits = __float_as_uint(score_from_age(a, T, agent, mid, tok));
-            if (bits < lim_bits) hi = mid;
-            else lo = mid + 1;
-        }
-        return lo > n_age ? 0xFFFFFFFFu : lo;                 // 0xFFFFFFFF: no age qualifies (ages are clamped below it)
-    } else {
-        const bool star = agent == T.a_star;
-        if (!star && b0 < 2048u) return 0u;                   // the whole non-a* class lies above the threshold bin
-        if (star && b0 >= 2048u) return 0xFFFFFFFFu;          // every a* entry is a candidate
-        const uint32_t x = star ? b0 : b0 - 2048u;            // (~bits & 0x7FFFFFFF) >> 20 <= x  <=>  bits >= lim_bits
-        const uint32_t lim_bits = (0x7FFu - x) << 20;
-        uint32_t lo = 0, hi = n_age + 1;                      // first age with bits < lim_bits
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (__float_as_uint(score_from_age(a, T, agent, mid, tok)) < lim_bits) hi = mid;
-            else lo = mid + 1;
-        }
-        return lo > n_age ? 0xFFFFFFFFu : lo;                 // candidate <=> age + 1 <= lo  (lo = 0: none)
+    const u64 limit = primary_limit<PF>(a, b0);              // candidate <=> primary key < limit
+    const uint32_t flip = (PF && agent != T.a_star) ? 0x80000000u : 0u;
+    uint32_t lo = 0, hi = n_age + 1;                          // victims: first age that qualifies; prefetch: first that does not
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        const uint32_t bits = __float_as_uint(score_from_age(a, T, agent, mid, tok));
+        const uint32_t pr = PF ? (flip | (~bits & 0x7FFFFFFFu)) : (a.prefer_copy ? bits << 1 : bits);
+        if ((pr < limit) != PF) hi = mid;
+        else lo = mid + 1;
     }
+    return lo > n_age ? 0xFFFFFFFFu : lo;                     // victims: 0xFFFFFFFF: no age qualifies (ages are clamped below it);
+                                                              // prefetch: candidate <=> age + 1 <= lo  (0: none, 0xFFFFFFFF: all)
 }
 
 template <bool PF>
 __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, cs_workspace ws)
 {
     extern __shared__ float smem[];
-    __shared__ unsigned long long s_km[CS_SAMPLE];
-    __shared__ uint32_t s_id[CS_SAMPLE];
     __shared__ bool s_flag;
     cs_wait_for_predecessor();
     cs_release_successor();
-    if (ws.sel->spec) return;          // the histogram pass already collected the candidates
+    if (ws.sel->spec) return;          // the fast pass already collected the candidates
     resolve_now(a);
     Tables T;
     load_tables(a, ws, smem, T, PF && a.anchor);
@@ -661,7 +491,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, 
                     }
                     uint32_t prj;
                     if (entry_key_rest<PF>(a, T, &ws.sc->status, ag, dp, grp_u8(G.fl, j), grp_u32(G, j), tok, prj, se) &&
-                        (prj >> 20) <= b0)
+                        bin_of<PF>(a, prj) <= b0)
                         mask |= 1u << j;
                 }
             }
@@ -684,7 +514,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, 
                     const uint32_t tok = a.ntok ? grp_u8(G.tk, j) : a.block_tokens;
                     const uint32_t dp = (PF && a.anchor) ? grp_u16(G.dp0, G.dp1, j) : 0u;
                     const bool ok = entry_key_rest<PF>(a, T, &ws.sc->status, grp_u16(G.ag0, G.ag1, j), dp, grp_u8(G.fl, j),
-                                                       grp_u32(G, j), tok, prj, se) && (prj >> 20) <= b0;
+                                                       grp_u32(G, j), tok, prj, se) && bin_of<PF>(a, prj) <= b0;
                     // (a slot was reserved from the prefilter's verdict; should the exact key ever disagree,
                     //  the slot gets a key that sorts behind every real candidate and is never emitted)
                     ws.cand_km[pos] = ok ? (((unsigned long long)prj << 32) | se) : ~0ull;
@@ -699,7 +529,7 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, 
             uint32_t p, se;
             const uint32_t tok = a.ntok ? a.ntok[i] : a.block_tokens;
             if (entry_key<PF>(a, T, &ws.sc->status, a.agent[i], a.depth[i], a.ref[i], a.flags[i], a.la[i], tok, p, se) &&
-                (p >> 20) <= b0) {
+                bin_of<PF>(a, p) <= b0) {
                 const uint32_t pos = atomicAdd(&ws.sel->c, 1u);
                 ws.cand_km[pos] = ((unsigned long long)p << 32) | se;
                 ws.cand_id[pos] = i;
@@ -708,8 +538,6 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, 
     }
     if (!last_cta_done(&ws.sel->ticket[2], &s_flag)) return;
 
-    // ---- last CTA: sample, sort the sample (bitonic, shared memory), publish splitters -----------
-    publish_splitters(ws, s_km, s_id, __ldcg(&ws.sel->c), a.sort_cap, a.region_cap_max, CS_SAMPLE, whole_cta());
     if (threadIdx.x == 0) { ws.sel->ticket[2] = 0; count_candidates(ws, a.kind, __ldcg(&ws.sel->c), false); }
 }
 
@@ -746,241 +574,256 @@ __device__ __forceinline__ void sort_tile(unsigned long long *t_km, uint32_t *t_
 }
 
 // ---------------------------------------------------------------------------------------------
-// Exclusive prefix sum of the bucket sizes, computed by every CTA that needs it (256 counters, L2-resident):
-// s_off[b] = first output position of bucket b, s_off[256] = candidates in all buckets.  Also returns the last
-// bucket that holds one of the n_out winners (0 when n_out = 0).  Whole CTA of 256 threads.
+// 3 - 5 ordering the candidates
+//
+// The n_out smallest of c candidates, in order, by ranks of a sample: 1,024 candidates at even distances are ranked against
+// each other (counting smaller ones: 96-bit compares spread over 64 CTAs), and J of them cover the output with four
+// standard deviations to spare.  Everything beyond the J-th is dropped; the rest is split at the samples into nb buckets of a few dozen
+// keys, which are small enough to be ranked by counting as well.  Whole-GPU launches, because the work is comparisons:
+// one cluster of 16 SMs took 36 us for 35,000 candidates, k = 10,000 (8 us the sample, 14 us the buckets, 8 us the ranks).
+// A bucket has a fixed region of the sort arrays; one that outgrows it is gathered again from the candidates by its CTA.
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t bucket_offsets(const cs_workspace &ws, uint32_t n_spl, uint32_t n_out, uint32_t *s_off,
-                                                   uint32_t *s_tmp)
+#define SAMPLE_CTAS 64u
+struct OrderPlan { uint32_t S, J, nb, cap; };
+__device__ __forceinline__ OrderPlan order_plan(uint32_t c, uint32_t n_out, uint32_t max_blocks, uint32_t region_max)
 {
-    const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t mine = t <= n_spl ? __ldcg(&CS_BCOUNT(ws, t)) : 0u;
-    uint32_t incl = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= d) incl += v;
-    }
-    if (t == 0) s_tmp[8] = 0;
-    if (lane == 31) s_tmp[warp] = incl;
-    __syncthreads();
-    uint32_t before = 0;
-#pragma unroll
-    for (uint32_t w = 0; w < 8; ++w) before += w < warp ? s_tmp[w] : 0u;
-    const uint32_t excl = before + incl - mine;
-    s_off[t] = excl;
-    if (t == 255) s_off[256] = excl + mine;
-    if (n_out && mine && excl <= n_out - 1 && n_out - 1 < excl + mine) s_tmp[8] = t;
-    __syncthreads();
-    return s_tmp[8];
+    OrderPlan P;
+    P.S = c < CS_SAMPLE ? c : CS_SAMPLE;
+    const float e = (float)n_out * (float)P.S / (float)c;
+    const uint32_t want = (uint32_t)(e + 4.0f * sqrtf(e)) + 3u;
+    P.J = want < P.S ? want : P.S;
+    P.nb = P.J < CS_BUCKETS ? P.J : CS_BUCKETS;
+    P.cap = max_blocks / P.nb;
+    if (region_max && P.cap > region_max) P.cap = region_max;
+    return P;
 }
 
-// ---------------------------------------------------------------------------------------------
-// 3 bucket
-//
-// Each candidate finds its bucket by binary search over the splitters and takes a slot in it.
-// Roomy case (few candidates for the size of the sort region): the slot comes straight from one atomic on the
-// bucket's counter and the key is written to slot `slot` of the bucket's own fixed-size region, so that the
-// buckets are ready for the rank launch and the scatter launch has nothing to do.  A bucket that outgrows its
-// region sets `overflow`: bucket and slot of every candidate are recorded as well, and the scatter and rank
-// launches then take the general route.
-// General case: per round a CTA takes 1024 candidates, counts them per bucket in shared memory and reserves the
-// CTA's range in each non-empty bucket with one global atomic; bucket and slot are recorded for the scatter launch.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) cs_sel_bucket_kernel(cs_workspace ws, uint32_t sort_cap, uint32_t kind)
+__global__ void __launch_bounds__(512) cs_sel_sample_kernel(SelArgs a, cs_workspace ws, uint32_t *__restrict__ ids_out,
+                                                            uint32_t *__restrict__ n_out_dev)
 {
-    __shared__ unsigned long long s_km[CS_MAX_SPLITTERS + 1];
-    __shared__ uint32_t s_id[CS_MAX_SPLITTERS + 1];
-    __shared__ uint32_t s_cnt[CS_MAX_SPLITTERS + 1], s_base[CS_MAX_SPLITTERS + 1];
-    constexpr int ITEMS = 4;                                  // candidates per thread and round
-    const int PS = kind == 2 ? 8 : 0;                         // phase-stamp slots (profiling builds)
+    __shared__ u64 s_km[CS_SAMPLE];
+    __shared__ uint32_t s_id[CS_SAMPLE];
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     cs_wait_for_predecessor();
-    CS_STAMP(ws, CS_PS_BUCKET_WAITED + PS, blockIdx.x == 0 && threadIdx.x == 0);
+    CS_STAMP(ws, CS_PS_SAMPLE_WAITED + (a.kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
     cs_release_successor();
-    // Everything the first round needs is asked for at once -- the select's state, the splitters and the round's keys
-    // (addresses bounded by the capacity of the buffers; what lies beyond the live counts is ignored below) -- so that
-    // the launch starts with one trip to L2 instead of three.
-    unsigned long long km[ITEMS];
-    uint32_t id[ITEMS], bkt[ITEMS], loc[ITEMS];
-    // Item u of a round lies one grid-wide sweep (sweep = 256 keys per CTA) after item u - 1, so that few candidates
-    // spread over all CTAs with one live key per thread instead of filling a few CTAs with four.
-    const uint32_t sweep = gridDim.x * 256u, lane0 = blockIdx.x * 256u + threadIdx.x;
-    const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_spl, placed, cap
+    const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);      // c, n_out, n_elig, b0
+    const uint32_t c = st.x, n_out = st.y;
+    for (uint32_t i = n_out + blockIdx.x * blockDim.x + tid; i < a.k; i += gridDim.x * blockDim.x) ids_out[i] = CS_ID_NONE;
+    if (blockIdx.x == 0) {
+        CS_BCOUNT(ws, tid) = 0;
+        if (tid == 0) *n_out_dev = n_out;
+    }
+    if (n_out == 0) return;
+    const uint32_t S = c < CS_SAMPLE ? c : CS_SAMPLE, ahead = cs_ahead(a.k);
+    {
+        u64 km[2];
+        uint32_t id[2];
+#pragma unroll
+        for (uint32_t u = 0; u < 2; ++u) {
+            const uint32_t s = tid + u * 512u, at = s < S ? (uint32_t)((u64)s * c / S) : 0u;
+            km[u] = cs_ld_cg_pinned(ws.cand_km + at);
+            id[u] = cs_ld_cg_pinned(ws.cand_id + at);
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 2; ++u) {
+            const uint32_t s = tid + u * 512u;
+            s_km[s] = s < S ? km[u] : ~0ull;
+            s_id[s] = s < S ? id[u] : 0xFFFFFFFFu;
+        }
+    }
+    if (blockIdx.x == 0 && tid == 0 && c <= ahead) ws.sel->ahead = ~0ull;
+    __syncthreads();
+    for (uint32_t s = blockIdx.x * 16u + warp; s < S; s += gridDim.x * 16u) {       // a warp per sample
+        const u64 my = s_km[s];
+        const uint32_t mine = s_id[s];
+        uint32_t r = 0;
+#pragma unroll 8
+        for (uint32_t q = lane; q < CS_SAMPLE; q += 32u) count_less(r, s_km[q], s_id[q], my, mine);
+        r = __reduce_add_sync(0xFFFFFFFFu, r);
+        if (lane == 0) {
+            ws.spl_km[r] = my;
+            ws.spl_id[r] = mine;
+            if (c > ahead && r == (uint32_t)((u64)ahead * S / c)) ws.sel->ahead = my;
+        }
+    }
+    CS_STAMP(ws, CS_PS_SAMPLE_DONE + (a.kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
+}
+
+__global__ void __launch_bounds__(256) cs_sel_place_kernel(cs_workspace ws, uint32_t max_blocks, uint32_t region_max, uint32_t kind)
+{
+    __shared__ u64 s_km[CS_SAMPLE];
+    __shared__ uint32_t s_id[CS_SAMPLE];
+    constexpr int ITEMS = 4;                                  // candidates per thread and round
+    const uint32_t tid = threadIdx.x;
+    cs_wait_for_predecessor();
+    CS_STAMP(ws, CS_PS_PLACE_WAITED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
+    (void)kind;
+    cs_release_successor();
+    // Everything the first round needs is asked for at once -- the select's state, the ranked sample and the round's keys
+    // (addresses bounded by the capacity of the buffers; what lies beyond the live counts is ignored below).  Item u of a
+    // round lies a grid-wide sweep after item u - 1, so that few candidates spread over all CTAs.
+    const uint32_t sweep = gridDim.x * 256u, lane0 = blockIdx.x * 256u + tid;
+    const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_out, n_elig, b0
+    u64 km[ITEMS], sk[4];
+    uint32_t id[ITEMS], si[4];
 #pragma unroll
     for (int u = 0; u < ITEMS; ++u) {
-        const uint32_t i = u * sweep + lane0, ii = i < sort_cap ? i : 0u;
+        const uint32_t i = u * sweep + lane0, ii = i < max_blocks ? i : 0u;
         km[u] = cs_ld_cg_pinned(ws.cand_km + ii);
         id[u] = cs_ld_cg_pinned(ws.cand_id + ii);
     }
-    const unsigned long long my_spl_km = cs_ld_cg_pinned(ws.spl_km + threadIdx.x);
-    const uint32_t my_spl_id = cs_ld_cg_pinned(ws.spl_id + threadIdx.x);
-    const uint32_t c = st.x, n_spl = st.y, placed = st.z, cap = st.w;
-    // splitters past the last one sort behind every key, so that the search below always takes eight steps
-    s_km[threadIdx.x] = threadIdx.x < n_spl ? my_spl_km : ~0ull;
-    s_id[threadIdx.x] = threadIdx.x < n_spl ? my_spl_id : 0xFFFFFFFFu;
-    s_cnt[threadIdx.x] = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { sk[u] = cs_ld_cg_pinned(ws.spl_km + tid + 256 * u); si[u] = cs_ld_cg_pinned(ws.spl_id + tid + 256 * u); }
+    const uint32_t c = st.x, n_out = st.y;
+    if (n_out == 0) return;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { s_km[tid + 256 * u] = sk[u]; s_id[tid + 256 * u] = si[u]; }
+    const OrderPlan P = order_plan(c, n_out, max_blocks, region_max);
     __syncthreads();
-    CS_STAMP(ws, CS_PS_BUCKET_STAGED + PS, blockIdx.x == 0 && threadIdx.x == 0);
+    const u64 cut_km = s_km[P.J - 1];
+    const uint32_t cut_id = s_id[P.J - 1];
     for (uint32_t base = 0; base < c; base += sweep * ITEMS) {
         if (base != 0) {
 #pragma unroll
-            for (int u = 0; u < ITEMS; ++u) {                 // all of the round's keys are fetched before any is used
+            for (int u = 0; u < ITEMS; ++u) {
                 const uint32_t i = base + u * sweep + lane0, ii = i < c ? i : 0u;
                 km[u] = cs_ld_cg_pinned(ws.cand_km + ii);
                 id[u] = cs_ld_cg_pinned(ws.cand_id + ii);
             }
         }
-        // bucket = number of splitters <= key: a branch-free descent over the 255 (padded) splitters, the round's four
-        // keys side by side
-        uint32_t pos[ITEMS];
 #pragma unroll
-        for (int u = 0; u < ITEMS; ++u) pos[u] = 0;
+        for (int u = 0; u < ITEMS; ++u) {
+            const uint32_t i = base + u * sweep + lane0;
+            // keys from the cut up are dropped when there are samples beyond it
+            if (i >= c || (P.J < P.S && !less96(km[u], id[u], cut_km, cut_id))) continue;
+            uint32_t b = 0;                                   // splitters at or below the key; splitter j (from 1) = sample rank j J / nb
 #pragma unroll 1
-        for (uint32_t step = 128; step > 0; step >>= 1) {
-            unsigned long long sk[ITEMS];
-            uint32_t si[ITEMS];
-#pragma unroll
-            for (int u = 0; u < ITEMS; ++u) {                 // the step's eight loads first, ...
-                const uint32_t probe = pos[u] + step - 1u;
-                sk[u] = s_km[probe];
-                si[u] = s_id[probe];
+            for (uint32_t step = CS_BUCKETS / 2; step > 0; step >>= 1) {
+                const uint32_t j = b + step, at = (j < P.nb ? j : 0u) * P.J / P.nb;
+                if (j < P.nb && !less96(km[u], id[u], s_km[at], s_id[at])) b = j;
             }
-#pragma unroll
-            for (int u = 0; u < ITEMS; ++u) {                 // ... then the compares, with no short-circuit branch
-                const bool lt = (km[u] < sk[u]) | ((km[u] == sk[u]) & (id[u] < si[u]));
-                pos[u] += lt ? 0u : step;
+            const uint32_t slot = atomicAdd(&CS_BCOUNT(ws, b), 1u);
+            if (slot < P.cap) {
+                ws.sort_km[(size_t)b * P.cap + slot] = km[u];
+                ws.sort_id[(size_t)b * P.cap + slot] = id[u];
             }
         }
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const uint32_t i = base + u * sweep + lane0;
-            bkt[u] = 0xFFFFFFFFu;
-            if (i < c) {
-                bkt[u] = pos[u] < n_spl ? pos[u] : n_spl;    // (a key equal to the padding stays in the last bucket)
-                if (!placed) loc[u] = atomicAdd(&s_cnt[bkt[u]], 1u);
-            }
-        }
-        CS_STAMP(ws, CS_PS_BUCKET_SEARCHED + PS, blockIdx.x == 0 && threadIdx.x == 0 && base == 0);
-        if (placed) {
-#pragma unroll
-            for (int u = 0; u < ITEMS; ++u)                   // the round's atomics are in flight together
-                if (bkt[u] != 0xFFFFFFFFu) loc[u] = atomicAdd(&CS_BCOUNT(ws, bkt[u]), 1u);
-            CS_STAMP(ws, CS_PS_BUCKET_SLOTS + PS, blockIdx.x == 0 && threadIdx.x == 0 && base == 0 && loc[0] != 0xFFFFFFF1u);
-#pragma unroll
-            for (int u = 0; u < ITEMS; ++u) {
-                const uint32_t i = base + u * sweep + lane0;
-                if (bkt[u] == 0xFFFFFFFFu) continue;
-                ws.cand_bkt[i] = bkt[u];
-                ws.cand_slot[i] = loc[u];
-                if (loc[u] < cap) {
-                    ws.sort_km[(size_t)bkt[u] * cap + loc[u]] = km[u];
-                    ws.sort_id[(size_t)bkt[u] * cap + loc[u]] = id[u];
-                } else {
-                    ws.sel->overflow = 1;
-                }
-            }
-            continue;
-        }
-        __syncthreads();
-        {
-            const uint32_t n_b = s_cnt[threadIdx.x];
-            if (n_b) s_base[threadIdx.x] = atomicAdd(&CS_BCOUNT(ws, threadIdx.x), n_b);
-            s_cnt[threadIdx.x] = 0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const uint32_t i = base + u * sweep + lane0;
-            if (bkt[u] != 0xFFFFFFFFu) {
-                ws.cand_bkt[i] = bkt[u];
-                ws.cand_slot[i] = s_base[bkt[u]] + loc[u];
-            }
-        }
-        __syncthreads();
     }
-    CS_STAMP(ws, CS_PS_BUCKET_DONE + PS, blockIdx.x == 0 && threadIdx.x == 0);
-    (void)PS;
+    CS_STAMP(ws, CS_PS_PLACE_DONE + (kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
 }
 
-// ---------------------------------------------------------------------------------------------
-// 4 scatter (general case only: candidates of the needed buckets are grouped by bucket)
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) cs_sel_scatter_kernel(cs_workspace ws, uint32_t kind)
+// The key the next call of this kind gets: the one it had while the candidates it gave were enough and not too many; where
+// they were too many, the key below which cs_ahead(k) of them lay; where they were few, as much beyond it as the
+// candidates above the list's last entry say that cs_ahead(k) would need.
+__device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u64 kth)
 {
-    __shared__ uint32_t s_off[CS_MAX_SPLITTERS + 2];
-    __shared__ uint32_t s_tmp[16];
-    cs_wait_for_predecessor();
-    CS_STAMP(ws, CS_PS_SCATTER_WAITED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
-    (void)kind;
-    cs_release_successor();
-    if (ws.sel->placed && !ws.sel->overflow) return;         // the buckets are in their regions already
-    const uint32_t c = ws.sel->c, n_out = ws.sel->n_out;
-    if (n_out == 0) return;
-    const uint32_t b_last = bucket_offsets(ws, ws.sel->n_spl, n_out, s_off, s_tmp);
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < c; i += gridDim.x * blockDim.x) {
-        const uint32_t b = ws.cand_bkt[i];
-        if (b > b_last) continue;
-        const uint32_t pos = s_off[b] + ws.cand_slot[i];
-        ws.sort_km[pos] = ws.cand_km[i];
-        ws.sort_id[pos] = ws.cand_id[i];
-    }
+    const u64 none = ~0ull, all = ~0ull - 1ull;
+    if (st.n_elig <= k) return all;                           // everything eligible is wanted
+    const uint32_t ahead = cs_ahead(k);
+    if (st.ahead != none && (!st.spec || st.c > 2ull * ahead)) return st.ahead < all ? st.ahead : all;
+    if (st.c >= 2ull * k + 1024ull || st.c >= st.n_elig || st.bound >= all || st.bound < kth) return st.bound < all ? st.bound : all;
+    const u64 gap = st.bound - kth, per = (ahead - st.c) / (st.c - k + 1u);
+    const u64 more = (gap < (1ull << 40) ? gap : (1ull << 40)) * (per < 8ull ? per : 8ull) + 64ull;
+    return more < all - st.bound ? st.bound + more : all;
 }
 
-// ---------------------------------------------------------------------------------------------
-// 5 rank and emit
-// ---------------------------------------------------------------------------------------------
-// Each needed bucket is ordered by one CTA: a bitonic sort of the bucket in a shared-memory tile
-// (O(m log^2 m), so an unlucky large bucket costs little more than an average one), after which
-// position i of the bucket is position offset + i of the output list.
+// Bucket b of CTA b: ranked by counting while it is small, sorted in the tile (bitonic, O(m log^2 m)) when it is large.
+#define FINISH_COUNT_MAX 256u
 __global__ void __launch_bounds__(256)
-cs_sel_rank_kernel(cs_workspace ws, uint32_t k, uint32_t kind, uint32_t *__restrict__ ids_out, uint32_t *__restrict__ n_out_dev)
+cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t region_max, uint32_t kind, uint32_t hint_slot,
+                     uint32_t *__restrict__ ids_out)
 {
-    __shared__ unsigned long long t_km[RANK_TILE];
+    __shared__ u64 t_km[RANK_TILE];
     __shared__ uint32_t t_id[RANK_TILE];
-    __shared__ uint32_t s_off[CS_MAX_SPLITTERS + 2];
-    __shared__ uint32_t s_tmp[16];
+    __shared__ uint32_t s_off, s_max, s_n;
+    const uint32_t tid = threadIdx.x, b = blockIdx.x;
+    if (tid == 0) { s_off = 0; s_max = 0; s_n = 0; }
+    __syncthreads();
     cs_wait_for_predecessor();
-    CS_STAMP(ws, CS_PS_RANK_WAITED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
+    CS_STAMP(ws, CS_PS_FINISH_WAITED + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
     cs_release_successor();
-    const uint32_t n_out = ws.sel->n_out, cap = ws.sel->cap;
-    const bool in_regions = ws.sel->placed && !ws.sel->overflow;
-    const uint32_t gtid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
-    for (uint32_t i = n_out + gtid; i < k; i += nth) ids_out[i] = CS_ID_NONE;
-    if (gtid == 0) {
-        *n_out_dev = n_out;
-        if (ws.sel->placed && kind < 3) {                     // work counters: how the buckets got to their places
-            atomicAdd((unsigned long long *)&ws.cnt->region_selects[kind], 1ull);
-            if (ws.sel->overflow) atomicAdd((unsigned long long *)&ws.cnt->region_overflows[kind], 1ull);
-        }
-    }
+    const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_out, n_elig, b0
+    const uint32_t n0 = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid)), n1 = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid + 256u));
+    uint32_t m = cs_ld_cg_pinned(&CS_BCOUNT(ws, b));
+    const uint32_t c = st.x, n_out = st.y;
     if (n_out == 0) return;
-    const uint32_t b_last = bucket_offsets(ws, ws.sel->n_spl, n_out, s_off, s_tmp);
-    CS_STAMP(ws, CS_PS_RANK_OFFSETS + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
-    for (uint32_t b = blockIdx.x; b <= b_last; b += gridDim.x) {
-        const uint32_t beg = s_off[b], end = s_off[b + 1], m = end - beg;
-        const size_t src = in_regions ? (size_t)b * cap : (size_t)beg;      // where the bucket's keys are
-        __syncthreads();
-        if (m <= RANK_TILE) {
-            for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-                t_km[i] = ws.sort_km[src + i];
-                t_id[i] = ws.sort_id[src + i];
-            }
-            CS_STAMP(ws, CS_PS_RANK_LOADED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0 && t_km[0] != 1ull);
-            sort_tile(t_km, t_id, m);
-            CS_STAMP(ws, CS_PS_RANK_SORTED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
-            for (uint32_t i = threadIdx.x; i < m; i += blockDim.x)
-                if (beg + i < n_out) ids_out[beg + i] = t_id[i];
-        } else {                                              // larger than the tile: rank straight from global memory
-            for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-                const unsigned long long km = ws.sort_km[src + i];
-                const uint32_t id = ws.sort_id[src + i];
-                uint32_t rank = 0;
-                for (uint32_t q = 0; q < m; ++q) rank += key_less(ws.sort_km[src + q], ws.sort_id[src + q], km, id) ? 1u : 0u;
-                if (beg + rank < n_out) ids_out[beg + rank] = id;
+    const OrderPlan P = order_plan(c, n_out, max_blocks, region_max);
+    if (b >= P.nb) return;
+    const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, (tid < b ? n0 : 0u) + (tid + 256u < b ? n1 : 0u));
+    if ((tid & 31) == 0 && before) atomicAdd(&s_off, before);
+    if (b == 0) {                                             // work counters, and whether any bucket outgrew its region
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n0 > n1 ? n0 : n1);
+        if ((tid & 31) == 0) atomicMax(&s_max, most);
+    }
+    __syncthreads();
+    const uint32_t off = s_off;
+    if (b == 0 && tid == 0 && kind < 3) {
+        atomicAdd((unsigned long long *)&ws.cnt->region_selects[kind], 1ull);
+        if (s_max > P.cap) atomicAdd((unsigned long long *)&ws.cnt->region_overflows[kind], 1ull);
+    }
+    // (should the sample have misled, the last bucket takes everything from its start on)
+    const bool rest = b == P.nb - 1u && P.J < P.S && off + m < n_out;
+    if (rest) m = c - off;
+    if (off >= n_out || m == 0) return;
+    const u64 *src_km = ws.sort_km + (size_t)b * P.cap;
+    const uint32_t *src_id = ws.sort_id + (size_t)b * P.cap;
+    // one id of the list; whoever places the last one knows the k-th key and chooses the next call's
+    auto emit = [&](uint32_t r, u64 km, uint32_t id) {
+        const uint32_t pos = off + r;
+        if (pos >= n_out) return;
+        ids_out[pos] = id;
+        if (pos == n_out - 1 && hint_slot < 3) ws.sc->sel_T[hint_slot] = next_bound(*ws.sel, k, km);
+    };
+    if (m > P.cap || rest) {
+        // the region was too small: the bucket's keys once more, out of all candidates
+        const uint32_t at_lo = b * P.J / P.nb, at_hi = (b + 1u) * P.J / P.nb;
+        const u64 lo_km = b ? ws.spl_km[at_lo] : 0ull, hi_km = b + 1u < P.nb ? ws.spl_km[at_hi] : (P.J < P.S && !rest ? ws.spl_km[P.J - 1] : ~0ull);
+        const uint32_t lo_id = b ? ws.spl_id[at_lo] : 0u, hi_id = b + 1u < P.nb ? ws.spl_id[at_hi] : (P.J < P.S && !rest ? ws.spl_id[P.J - 1] : 0xFFFFFFFFu);
+        const bool fits = m <= RANK_TILE;
+        for (uint32_t i = tid; i < c; i += 256u) {
+            const u64 km = __ldcg(ws.cand_km + i);
+            const uint32_t id = __ldcg(ws.cand_id + i);
+            if (less96(km, id, lo_km, lo_id) || !less96(km, id, hi_km, hi_id)) continue;
+            if (fits) {
+                const uint32_t at = atomicAdd(&s_n, 1u);
+                t_km[at] = km;
+                t_id[at] = id;
+            } else {                                          // nor does the tile hold them: each against all candidates
+                uint32_t r = 0;
+                for (uint32_t q = 0; q < c; ++q) {
+                    const u64 qk = __ldcg(ws.cand_km + q);
+                    const uint32_t qi = __ldcg(ws.cand_id + q);
+                    if (!less96(qk, qi, lo_km, lo_id)) count_less(r, qk, qi, km, id);
+                }
+                emit(r, km, id);
             }
         }
+        if (!fits) return;
+        __syncthreads();
+    } else if (m <= RANK_TILE) {
+        for (uint32_t i = tid; i < m; i += 256u) {
+            t_km[i] = __ldcg(src_km + i);
+            t_id[i] = __ldcg(src_id + i);
+        }
+        __syncthreads();
+    } else {                                                  // larger than the tile: ranked straight from global memory
+        for (uint32_t i = tid; i < m; i += 256u) {
+            const u64 km = __ldcg(src_km + i);
+            const uint32_t id = __ldcg(src_id + i);
+            uint32_t r = 0;
+            for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(src_km + q), __ldcg(src_id + q), km, id);
+            emit(r, km, id);
+        }
+        return;
     }
-    CS_STAMP(ws, CS_PS_RANK_DONE + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
+    if (m <= FINISH_COUNT_MAX) {
+        rank_keys(t_km, t_id, m, t_km, t_id, m, emit);
+    } else {
+        sort_tile(t_km, t_id, m);
+        for (uint32_t i = tid; i < m; i += 256u) emit(i, t_km[i], t_id[i]);
+    }
+    CS_STAMP(ws, CS_PS_FINISH_DONE + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1009,8 +852,8 @@ void cs_fill_sel_args(const cs_ctx *ctx, const cs_block_index *idx, uint32_t now
     a.hint_slot = 0;
     a.kind = 0;
     a.now_dev = ctx->step_now_dev ? ctx->step_now_dev : ctx->clock_dev;
-    a.sort_cap = 0;
     a.region_cap_max = ctx->region_cap_max;
+    a.max_blocks = ctx->p.max_blocks;
     a.bin_lo = 0;
     a.bin_shift = 20;
 }
@@ -1098,14 +941,13 @@ static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, ui
     a.k = k;
     a.hint_slot = ctx->no_speculation ? 3u : (prefetch ? 2u : tier);
     a.kind = prefetch ? 2u : tier;
-    a.sort_cap = ctx->p.max_blocks;          // keys the sort region of this select holds
+    cs_fill_sel_bins(ctx, a, prefetch);
     if (ctx->select_path != CS_SELECT_MULTI && idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) {
-        cs_fill_sel_bins(ctx, a, prefetch);
         const int rc1 = cs_launch_select_cluster(ctx, &a, &ws, prefetch, ids_out, n_out, s);
         if (rc1 != CS_ENOTIMPL) return rc1;          // no usable cluster on this device: fall through
     }
     const uint32_t grid = cs_scan_grid(ctx, idx->n_blocks, SEL_THREADS * GRP);
-    const uint32_t grid_c = cs_scan_grid(ctx, idx->n_blocks, 256);
+    const uint32_t grid_c = cs_scan_grid(ctx, idx->n_blocks, 1024);
     const size_t sm = cs_table_smem(ctx);
     int rc;
     const size_t sm_fast = (sm + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
@@ -1129,11 +971,11 @@ static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, ui
     if (prefetch) cs_launch_chained(cs_sel_collect_kernel<true>, grid, SEL_THREADS, sm_collect, s, a, ws);
     else cs_launch_chained(cs_sel_collect_kernel<false>, grid, SEL_THREADS, sm_collect, s, a, ws);
     if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_bucket_kernel, grid_c, 256, 0, s, ws, (uint32_t)ctx->p.max_blocks, a.kind);
+    cs_launch_chained(cs_sel_sample_kernel, SAMPLE_CTAS, 512, 0, s, a, ws, ids_out, n_out);
     if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_scatter_kernel, grid_c, 256, 0, s, ws, a.kind);
+    cs_launch_chained(cs_sel_place_kernel, grid_c, 256, 0, s, ws, a.max_blocks, a.region_cap_max, a.kind);
     if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_rank_kernel, CS_MAX_SPLITTERS + 1, 256, 0, s, ws, k, a.kind, ids_out, n_out);
+    cs_launch_chained(cs_sel_finish_kernel, CS_BUCKETS, 256, 0, s, ws, k, a.max_blocks, a.region_cap_max, a.kind, a.hint_slot, ids_out);
     return cs_check_launch(ctx);
 }
 
@@ -1220,9 +1062,9 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
 #define CS_SO_GTAB (CS_SO_SEL + CS_STATIC_ALIGN(sizeof(cs_sel_state)))
 #define CS_SO_HIST (CS_SO_GTAB + CS_GTAB_MAX * 4u)
 #define CS_SO_SPLKM (CS_SO_HIST + CS_HIST_BINS * 4u)
-#define CS_SO_SPLID (CS_SO_SPLKM + CS_STATIC_ALIGN((CS_MAX_SPLITTERS + 1u) * 8u))
-#define CS_SO_BCOUNT (CS_SO_SPLID + CS_STATIC_ALIGN((CS_MAX_SPLITTERS + 1u) * 4u))
-#define CS_SO_CANDKM (CS_SO_BCOUNT + CS_STATIC_ALIGN((CS_MAX_SPLITTERS + 1u) * CS_BCOUNT_STRIDE * 4u))
+#define CS_SO_SPLID (CS_SO_SPLKM + CS_STATIC_ALIGN(CS_SAMPLE * 8u))
+#define CS_SO_BCOUNT (CS_SO_SPLID + CS_STATIC_ALIGN(CS_SAMPLE * 4u))
+#define CS_SO_CANDKM (CS_SO_BCOUNT + CS_STATIC_ALIGN(CS_BUCKETS * CS_BCOUNT_STRIDE * 4u))
 #define CS_SO_SORTKM (CS_SO_CANDKM + CS_STATIC_MAX_BLOCKS * 8u)
 #define CS_SO_CANDID (CS_SO_SORTKM + CS_STATIC_MAX_BLOCKS * 8u)
 #define CS_SO_CANDBKT (CS_SO_CANDID + CS_STATIC_MAX_BLOCKS * 4u)
@@ -1231,7 +1073,7 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
 #define CS_SO_CNT (CS_SO_SORTID + CS_STATIC_MAX_BLOCKS * 4u)
 #define CS_STATIC_BYTES (CS_SO_CNT + CS_STATIC_ALIGN(sizeof(cs_counters)))
 
-static __device__ __align__(256) unsigned char cs_static_scratch[CS_STATIC_BYTES];   // 2 MiB + 40 KiB
+static __device__ __align__(256) unsigned char cs_static_scratch[CS_STATIC_BYTES];   // 2 MiB + 60 KiB
 
 static std::mutex g_static_mu;
 static unsigned char *g_static_ptr[CS_STATIC_MAX_DEVICES];     // device address of the array, per device
@@ -1250,7 +1092,7 @@ __global__ void cs_static_prepare_kernel(cs_workspace ws, uint32_t gtab_len, flo
         memset(&z, 0, sizeof(z));
         z.last_agent = CS_AGENT_NONE;
         z.a_star = 0xFFFFFFFFu;
-        z.sel_hint[0] = z.sel_hint[1] = z.sel_hint[2] = z.sel_hint[3] = 0xFFFFFFFFu;
+        z.sel_T[0] = z.sel_T[1] = z.sel_T[2] = z.sel_T[3] = ~0ull;
         *ws.sc = z;
         cs_sel_state zs;
         memset(&zs, 0, sizeof(zs));

@@ -10,9 +10,9 @@
 //     range that scores can have, not the 32 bits of the key: a bin is 1/128 of an octave instead of 1/8;
 //   2 CTA r sums bins [r*B/CL, (r+1)*B/CL) over all CTAs through DSMEM and writes the sums into
 //     every CTA's copy of the total histogram; each CTA then finds the threshold bin b0;
-//   3 the entries with bin <= b0 (c >= min(k, eligible) keys) go to the CTA's list in shared memory;
-//   4 c <= 4096: order_small() places them straight out of the cluster's lists; more: order_global() (cs_select_order.cuh),
-//     and for lists too long for its buckets a sample sort through global memory.
+//   3 the entries with bin <= b0 (c >= min(k, eligible) keys) go to the candidate buffer (a single CTA keeps them in shared
+//     memory);
+//   4 they are put in order (cs_select_order.cuh); where buckets overflow there, by a sample sort through global memory.
 //
 // Bound by latency: trips to L2, barriers, and the instructions of one warp's entries.  The three selects of
 // a step, back to back in a CUDA graph: 2,560 entries, k = 32 / 64: 26.8 us when the index was scanned twice, bins were an
@@ -29,18 +29,14 @@ __host__ __device__ inline size_t csel_table_bytes(uint32_t A, uint32_t gtab_len
 {
     return (((size_t)(A + gtab_len) * 4 + (size_t)A * 2) + 15) / 16 * 16;
 }
-// Lists and buckets no longer than the index needs.
-static void csel_caps(uint32_t n, uint32_t &list_cap, uint32_t &reg_cap)
+// Candidates a CTA holds at once: no more than the index has entries.
+static uint32_t csel_cap(uint32_t n)
 {
-    list_cap = n < OR_LIST ? (n + 255u) / 256u * 256u : OR_LIST;
-    if (list_cap == 0) list_cap = 256u;
-    reg_cap = n <= OR_LIST ? list_cap : OR_REGION;
+    return n < 256u ? 256u : (n < OR_ALL ? (n + 255u) / 256u * 256u : OR_ALL);
 }
 static size_t csel_smem_bytes(uint32_t A, uint32_t gtab_len, uint32_t n)
 {
-    uint32_t lc, rc;
-    csel_caps(n, lc, rc);
-    return csel_table_bytes(A, gtab_len) + 2 * CS_HIST_BINS * 4 + order_smem_bytes(lc, rc);
+    return csel_table_bytes(A, gtab_len) + 2 * CS_HIST_BINS * 4 + order_smem_bytes(csel_cap(n));
 }
 
 // Four consecutive entries per lane, as they come from memory.
@@ -61,18 +57,6 @@ __device__ __forceinline__ void load_quad(const SelArgs &a, uint32_t q, Quad &Q)
     if (PF && a.anchor) Q.dp = __ldg((const uint2 *)a.depth + q);
 }
 
-// Histogram bin of a primary key: the range of possible scores divided evenly over the bins (of both classes of a prefetch
-// list), clamped at its ends, which keeps the order whatever the survival table holds.
-template <bool PF>
-__device__ __forceinline__ uint32_t bin_of(const SelArgs &a, uint32_t pr)
-{
-    const uint32_t v = PF ? pr & 0x7FFFFFFFu : pr;
-    const uint32_t x = (v > a.bin_lo ? v - a.bin_lo : 0u) >> a.bin_shift;
-    constexpr uint32_t PER_CLASS = PF ? CS_HIST_BINS / 2 : CS_HIST_BINS;
-    const uint32_t b = x < PER_CLASS - 1u ? x : PER_CLASS - 1u;
-    return PF ? b + ((pr >> 31) ? PER_CLASS : 0u) : b;
-}
-
 // Ordering through global memory, for candidates the cluster's buckets cannot hold: a 1,024-key sample is sorted, every
 // candidate finds its bucket, the needed buckets are grouped and each is sorted in a shared-memory tile.
 __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const OrderSmem &O, uint32_t c, uint32_t n_out,
@@ -81,8 +65,8 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank(), tid = threadIdx.x;
     const uint32_t cthreads = CL * CSEL_THREADS, ctid = rank * CSEL_THREADS + tid;
-    u64_key *km_s = O.g_km;
-    uint32_t *id_s = O.g_id;
+    u64 *km_s = O.s_km;
+    uint32_t *id_s = O.s_id;
     uint32_t *s_off = O.off;
     cluster.sync();
     if (rank == 0) {
@@ -108,7 +92,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
     if (tid == 0) O.misc[OM_IN] = 0;
     __syncthreads();
     for (uint32_t i = ctid; i < c; i += cthreads) {
-        const u64_key km = __ldcg(&ws.cand_km[i]);
+        const u64 km = __ldcg(&ws.cand_km[i]);
         const uint32_t id = __ldcg(&ws.cand_id[i]);
         uint32_t lo = 0, hi = CS_MAX_SPLITTERS;
         while (lo < hi) {
@@ -155,7 +139,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
                 if (beg + i < n_out) ids_out[beg + i] = id_s[i];
         } else {                                     // a large bucket: ranked straight from global memory
             for (uint32_t i = tid; i < m; i += CSEL_THREADS) {
-                const u64_key km = __ldcg(&ws.sort_km[beg + i]);
+                const u64 km = __ldcg(&ws.sort_km[beg + i]);
                 const uint32_t id = __ldcg(&ws.sort_id[beg + i]);
                 uint32_t r = 0;
                 for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(&ws.sort_km[beg + q]), __ldcg(&ws.sort_id[beg + q]), km, id);
@@ -169,7 +153,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
 // clusters of one launch can run different selects at once.
 template <bool PF>
 __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uint32_t *__restrict__ ids_out,
-                                          uint32_t *__restrict__ n_out_dev, unsigned char *dsm, uint32_t list_cap, uint32_t reg_cap)
+                                          uint32_t *__restrict__ n_out_dev, unsigned char *dsm, uint32_t cap)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
@@ -182,7 +166,7 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
     OrderSmem O;
     uint32_t *hist = (uint32_t *)(dsm + csel_table_bytes(a.A, a.gtab_len));       // [4096] this CTA's histogram
     uint32_t *tot = hist + CS_HIST_BINS;                                          // [4096] the cluster's (same in every CTA)
-    order_carve((unsigned char *)(tot + CS_HIST_BINS), list_cap, reg_cap, O);
+    order_carve((unsigned char *)(tot + CS_HIST_BINS), cap, O);
     Tables T;
     load_tables_static(a, ws, (float *)dsm, T);
     for (uint32_t i = tid; i < CS_HIST_BINS / 4; i += CSEL_THREADS) ((uint4 *)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -219,7 +203,11 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
     }
     uint32_t pr[4 * CSEL_UNITS], em = 0;                          // primary keys; bit 4 q + r: entry r of unit q is eligible
     uint32_t b0 = 0xFFFFFFFFu, n_out = 0, c = 0;
-    bool small = true;
+    // candidates: in shared memory when one CTA is all there is and they fit, else in L2, numbered by the first CTA
+    uint32_t *counter = cluster.map_shared_rank(O.misc, 0) + OM_LIST;
+    u64 *to_km = ws.cand_km;
+    uint32_t *to_id = ws.cand_id;
+    bool here = false;
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
         // phase 0 counts the keys, phase 1 puts those at or below the threshold bin away
@@ -262,15 +250,13 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
                 if (lane >= d) incl += v;
             }
             uint32_t base = 0;
-            if (lane == 31 && incl) base = atomicAdd(small ? &O.misc[OM_LIST] : cluster.map_shared_rank(O.misc, 0) + OM_GLOBAL, incl);
+            if (lane == 31 && incl) base = atomicAdd(counter, incl);
             uint32_t pos = __shfl_sync(0xFFFFFFFFu, base, 31) + incl - cnt;
-            u64_key *to_km = small ? O.list_km : ws.cand_km;
-            uint32_t *to_id = small ? O.list_id : ws.cand_id;
 #pragma unroll
             for (int e = 0; e < 4 * CSEL_UNITS; ++e) {
                 if (!((mask >> e) & 1u)) continue;
                 const uint32_t la = u4_word(Q[e >> 2].la, e & 3);
-                to_km[pos] = ((u64_key)pr[e] << 32) | (PF ? ~la : la);
+                to_km[pos] = ((u64)pr[e] << 32) | (PF ? ~la : la);
                 to_id[pos] = (u0 + (uint32_t)(e >> 2) * n_warps + gw) * CSEL_UNIT + 4u * lane + (uint32_t)(e & 3);
                 ++pos;
             }
@@ -327,34 +313,37 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
             count_candidates(ws, a.kind, n_out ? c : 0u, false);
         }
         if (n_out == 0) return;                                     // nothing eligible or nothing asked for (same in every CTA)
-        small = c <= OR_LIST && c <= list_cap && c <= reg_cap;
+        here = CL == 1 && c <= cap;
+        if (here) { to_km = O.all_km; to_id = O.all_id; }
     }
     if (tail && bin_of<PF>(a, tail_pr) <= b0) {
-        const uint32_t pos = atomicAdd(small ? &O.misc[OM_LIST] : cluster.map_shared_rank(O.misc, 0) + OM_GLOBAL, 1u);
-        (small ? O.list_km : ws.cand_km)[pos] = ((u64_key)tail_pr << 32) | tail_se;
-        (small ? O.list_id : ws.cand_id)[pos] = tail_id;
+        const uint32_t pos = atomicAdd(counter, 1u);
+        to_km[pos] = ((u64)tail_pr << 32) | tail_se;
+        to_id[pos] = tail_id;
     }
     CS_STAMP(ws, CS_PS_SCAN_LAST_CTA + PS, stamp);
-    if (small) {
-        if (CL > 1) cluster.sync();
-        else __syncthreads();
-        order_small(O, n_out, ids_out, nullptr);
+    if (here) {
+        __syncthreads();
+        order_few(O, nullptr, nullptr, c, n_out, ids_out);
     } else {
         __threadfence();
         cluster.sync();
-        const OrderResult res = order_global(O, ws.cand_km, ws.cand_id, c, n_out, ids_out, nullptr, 0u, nullptr, 0u);
-        if (!res.done) csel_order_general(ws, O, c, n_out, ids_out);
+        OrderBufs B = order_bufs(ws, a.max_blocks);
+        const OrderResult res = order_candidates(O, B, c, n_out, ids_out);
+        if (!res.done) {
+            order_restore(B, ws.cand_km, ws.cand_id, c);
+            csel_order_general(ws, O, c, n_out, ids_out);
+        }
     }
     CS_STAMP(ws, CS_PS_SCAN_TAIL_DONE + PS, stamp);
 }
 
 template <bool PF>
 __global__ void __launch_bounds__(CSEL_THREADS, 1)
-cs_select_cluster_kernel(SelArgs a, cs_workspace ws, uint32_t *__restrict__ ids_out, uint32_t *__restrict__ n_out_dev, uint32_t list_cap,
-                         uint32_t reg_cap)
+cs_select_cluster_kernel(SelArgs a, cs_workspace ws, uint32_t *__restrict__ ids_out, uint32_t *__restrict__ n_out_dev, uint32_t cap)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
-    csel_body<PF>(a, ws, ids_out, n_out_dev, dsm, list_cap, reg_cap);
+    csel_body<PF>(a, ws, ids_out, n_out_dev, dsm, cap);
 }
 
 // The three selects of a step in one launch: cluster q of the grid runs select q (GPU-tier victims,
@@ -365,19 +354,19 @@ struct SelJob {
     uint32_t *ids_out, *n_out;
     uint32_t prefetch;
 };
-struct SelJobs { SelJob j[3]; uint32_t list_cap, reg_cap; };     // the grid holds one cluster per job in use
+struct SelJobs { SelJob j[3]; uint32_t cap; };     // the grid holds one cluster per job in use
 
 __global__ void __launch_bounds__(CSEL_THREADS, 1) cs_select_step_kernel(const __grid_constant__ SelJobs jobs)
 {
     extern __shared__ __align__(16) unsigned char dsm[];
     const uint32_t q = blockIdx.x / cg::this_cluster().num_blocks();
     const SelJob &J = jobs.j[q];
-    if (J.prefetch) csel_body<true>(J.a, J.ws, J.ids_out, J.n_out, dsm, jobs.list_cap, jobs.reg_cap);
-    else csel_body<false>(J.a, J.ws, J.ids_out, J.n_out, dsm, jobs.list_cap, jobs.reg_cap);
+    if (J.prefetch) csel_body<true>(J.a, J.ws, J.ids_out, J.n_out, dsm, jobs.cap);
+    else csel_body<false>(J.a, J.ws, J.ids_out, J.n_out, dsm, jobs.cap);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Per-device set-up of the three cluster kernels, done once per process and device.  The dynamic shared-memory
+// Per-device set-up of the cluster kernels, done once per process and device.  The dynamic shared-memory
 // opt-in is an attribute of the FUNCTION (on a device), not of a context, so it is raised once to the fixed
 // maximum any parameter set can ask for (CS_MAX_AGENTS agents, the longest recency table) and never lowered:
 // contexts of different shape and the static-scratch entry point can then share the kernels.  The largest
@@ -446,10 +435,8 @@ static int launch_cluster(cs_ctx *ctx, const SelArgs &a, const cs_workspace &ws,
     if (max_cl < 1) return CS_ENOTIMPL;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
-    uint32_t lc, rc;
-    csel_caps(a.n, lc, rc);
     csel_config(ctx, cfg, attr, csel_cluster_size(a.n, a.k, max_cl), 1, csel_smem_bytes(a.A, a.gtab_len, a.n), s);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, cs_select_cluster_kernel<PF>, a, ws, ids_out, n_out, lc, rc);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, cs_select_cluster_kernel<PF>, a, ws, ids_out, n_out, csel_cap(a.n));
     ctx->n_launches++;
     if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
     return CS_OK;
@@ -467,11 +454,12 @@ int cs_launch_select_clusters(cs_ctx *ctx, int n_jobs, const void *sel_args, con
     uint32_t k = 0;
     for (int q = 0; q < n_jobs; ++q) k = aj[q].k > k ? aj[q].k : k;
     SelJobs jobs;
-    csel_caps(aj[0].n, jobs.list_cap, jobs.reg_cap);
+    jobs.cap = csel_cap(aj[0].n);
     csel_config(ctx, cfg, attr, csel_cluster_size(aj[0].n, k, max_cl), n_jobs, csel_smem_bytes(aj[0].A, aj[0].gtab_len, aj[0].n), s);
     for (int q = 0; q < n_jobs; ++q) {
         jobs.j[q].a = aj[q];
         jobs.j[q].ws = q == 0 ? ctx->ws : ctx->ws_job[q - 1];
+        if (q && !ctx->concurrent_selects) jobs.j[q].a.max_blocks = CS_SELECT_CLUSTER_MAX_BLOCKS;      // (as the workspace is laid out)
         jobs.j[q].ids_out = ids_out[q];
         jobs.j[q].n_out = n_out[q];
         jobs.j[q].prefetch = prefetch[q];

@@ -3,6 +3,8 @@
 #pragma once
 #include "cs_common.cuh"
 
+typedef unsigned long long u64;
+
 #define SEL_THREADS 512
 #define GRP 16                    // index entries per thread and iteration
 
@@ -19,12 +21,12 @@ struct SelArgs {
     float lambda, delta;
     uint32_t tier, k, prefer_copy;
     uint32_t use_age_limits;      // collect pass may prefilter by per-(agent, size) age limits (large indexes)
-    uint32_t hint_slot;           // which remembered threshold bin this call may speculate on
+    uint32_t hint_slot;           // which remembered key (cs_scalars.sel_T) this call may speculate on
     uint32_t kind;                // 0 GPU-tier victims, 1 host-tier victims, 2 prefetch candidates (work counters)
     const uint32_t *now_dev;      // when set, the clock is read from device memory at execution time (graph replay)
-    uint32_t sort_cap;            // keys the sort region holds (0: buckets never get fixed regions)
-    uint32_t region_cap_max;      // cap on a bucket's own region (0: none)
-    uint32_t bin_lo, bin_shift;   // histogram bins of the cluster select: (primary - bin_lo) >> bin_shift, set per list kind
+    uint32_t region_cap_max;      // cap on the keys of a bucket (0: none)
+    uint32_t max_blocks;          // keys the candidate and sort buffers hold
+    uint32_t bin_lo, bin_shift;   // histogram bins: (primary - bin_lo) >> bin_shift, set per list kind
 };
 
 // host helpers defined in cs_select.cu
@@ -43,41 +45,10 @@ __device__ __forceinline__ void part_sync(const CtaPart &p)
     asm volatile("bar.sync %0, %1;" ::"r"(p.bar), "r"(p.n) : "memory");
 }
 
-// What the next call of this kind may collect ahead of its own threshold.  The threshold bin of consecutive
-// calls moves little, so the next call's first scan appends every entry up to a remembered bin.  That bin is
-// chosen from this call's exact histogram: the furthest bin whose cumulative population stays within
-// 3 k + 1024 entries, at least the threshold bin itself and at most CS_SPEC_MAX_AHEAD bins beyond it.  Sparse
-// bins (a prefetch list whose best entries leave the tier every call, so its threshold jumps) get several bins
-// of slack for a few thousand extra candidates; dense bins get none.  Only the amount of work depends on this,
-// never the result.  `loc` are the calling thread's bins [first, first + PER), `before` the population below
-// them; every thread of the group calls; s_lim is a shared word.
-#define CS_SPEC_MAX_AHEAD 8u
-template <uint32_t PER>
-__device__ __forceinline__ uint32_t collect_ahead_limit(const uint32_t (&loc)[PER], uint32_t first, uint32_t before,
-                                                        uint32_t k, uint32_t b0, uint32_t *s_lim, const CtaPart &cp)
-{
-    if (cp.t == 0) *s_lim = 0;
-    part_sync(cp);
-    const unsigned long long cap = 3ull * k + 1024ull;
-    unsigned long long run = before;
-    uint32_t best = 0xFFFFFFFFu;
-#pragma unroll
-    for (uint32_t q = 0; q < PER; ++q) {
-        run += loc[q];
-        if (run <= cap) best = first + q;
-    }
-    if (best != 0xFFFFFFFFu) atomicMax(s_lim, best);
-    part_sync(cp);
-    uint32_t lim = *s_lim;
-    if (lim < b0) lim = b0;
-    if (lim > b0 + CS_SPEC_MAX_AHEAD) lim = b0 + CS_SPEC_MAX_AHEAD;
-    return lim < CS_HIST_BINS ? lim : CS_HIST_BINS - 1;
-}
-
-__device__ __forceinline__ void remember_threshold(cs_scalars *sc, uint32_t slot, bool valid, uint32_t limit)
-{
-    if (slot < 3) sc->sel_hint[slot] = valid ? limit : 0xFFFFFFFFu;
-}
+// How many candidates the next large select of a kind should find at or below the key it is given: enough that an index
+// which loses its k best entries between calls, or whose survival table shifts, still has k of them; few enough that
+// collecting and ordering them costs little.
+__host__ __device__ __forceinline__ uint32_t cs_ahead(uint32_t k) { return k < 0x10000000u ? 3u * k + 4096u : 0x40000000u; }
 
 // Work counters of one finished select (called by one thread).
 __device__ __forceinline__ void count_select(const cs_workspace &ws, uint32_t kind, uint32_t n_elig, uint32_t n_out)
@@ -151,53 +122,6 @@ __device__ __forceinline__ float score_from_age(const SelArgs &a, const Tables &
     return __fmul_rn(__fmul_rn(T.fsurv[agent], recency_of_age(a, T, age)), (float)tok);      // two roundings, never an FMA
 }
 
-// ---------------------------------------------------------------------------------------------
-// Threshold test without the key.  The score is fl(fl(f * g) * |b|) and IEEE multiplication by a positive
-// constant never decreases when its operand grows, so "the first key digit is at most H" is, for a fixed
-// block size, an interval of x = fl(f * g): victims  x < X[|b|],  prefetch candidates  x >= X[class][|b|]
-// (class 0: blocks of a*, class 1: the rest).  X is found once per CTA by binary search over the bit
-// patterns of positive floats; an entry then costs two table look-ups, one multiply and one compare, and only
-// the few entries that pass get a key.  Exact: it is the same product the key is made of.
-// ---------------------------------------------------------------------------------------------
-#define XT_TOK 256u                // |b| is a u8
-#define XT_NONE 0x7F800001u        // above every finite pattern
-
-// smallest bit pattern x in [0, +inf] with bits(fl(x * tok)) >= lim; XT_NONE when there is none
-__device__ __forceinline__ uint32_t first_x_reaching(unsigned long long lim, uint32_t tok)
-{
-    uint32_t lo = 0, hi = 0x7F800001u;
-    const float t = (float)tok;
-    while (lo < hi) {
-        const uint32_t mid = lo + ((hi - lo) >> 1);
-        const unsigned long long bits = __float_as_uint(__fmul_rn(__uint_as_float(mid), t));
-        if (bits >= lim) hi = mid;
-        else lo = mid + 1;
-    }
-    return lo;
-}
-
-// Fills xt[2][XT_TOK] for the remembered bin H (every thread of the CTA calls; synchronise afterwards).
-template <bool PF>
-__device__ __forceinline__ void build_x_thresholds(const SelArgs &a, uint32_t H, uint32_t *xt)
-{
-    for (uint32_t e = threadIdx.x; e < 2 * XT_TOK; e += blockDim.x) {
-        const uint32_t cls = e / XT_TOK, tok = e % XT_TOK;
-        uint32_t x;
-        if (!PF) {
-            // bin = bits >> 20 (bits >> 19 with the copy-preference bit below the score): candidate <=> bits < lim
-            const unsigned long long lim = (unsigned long long)(H + 1u) << (a.prefer_copy ? 19 : 20);
-            x = first_x_reaching(lim, tok);                                  // candidate <=> x bits < this
-        } else if (cls == 0) {
-            // a*: bin = (0x7FFFFFFF - bits) >> 20 <= H  <=>  bits >= 0x80000000 - ((H + 1) << 20)
-            x = H >= 2047u ? 0u : first_x_reaching(0x80000000ull - ((unsigned long long)(H + 1u) << 20), tok);
-        } else {
-            // the rest: bin = 2048 + ((0x7FFFFFFF - bits) >> 20)
-            x = H < 2048u ? XT_NONE : (H >= 4095u ? 0u : first_x_reaching(0x80000000ull - ((unsigned long long)(H - 2047u) << 20), tok));
-        }
-        xt[e] = x;                                                           // prefetch: candidate <=> x bits >= this
-    }
-}
-
 __device__ __forceinline__ float score_of(const SelArgs &a, const Tables &T, uint32_t agent, uint32_t la,
                                           uint32_t tok)
 {
@@ -207,6 +131,29 @@ __device__ __forceinline__ float score_of(const SelArgs &a, const Tables &T, uin
     else if (age >= a.age_sat) g = T.g_sat;
     else g = cs_recency(a.lambda, a.delta, age);
     return __fmul_rn(__fmul_rn(T.fsurv[agent], g), (float)tok);      // two roundings, never an FMA
+}
+
+// Histogram bin of a primary key: the range of possible scores divided evenly over the bins (of both classes of a prefetch
+// list), clamped at its ends, which keeps the order whatever the survival table holds.
+template <bool PF>
+__device__ __forceinline__ uint32_t bin_of(const SelArgs &a, uint32_t pr)
+{
+    const uint32_t v = PF ? pr & 0x7FFFFFFFu : pr;
+    const uint32_t x = (v > a.bin_lo ? v - a.bin_lo : 0u) >> a.bin_shift;
+    constexpr uint32_t PER_CLASS = PF ? CS_HIST_BINS / 2 : CS_HIST_BINS;
+    const uint32_t b = x < PER_CLASS - 1u ? x : PER_CLASS - 1u;
+    return PF ? b + ((pr >> 31) ? PER_CLASS : 0u) : b;
+}
+
+// "bin <= b0" as a limit on the primary key: candidate <=> primary < limit.
+template <bool PF>
+__device__ __forceinline__ u64 primary_limit(const SelArgs &a, uint32_t b0)
+{
+    constexpr uint32_t PER_CLASS = PF ? CS_HIST_BINS / 2 : CS_HIST_BINS;
+    const uint32_t b = b0 % PER_CLASS;
+    const u64 cls = PF && b0 >= PER_CLASS ? 0x80000000ull : 0ull, end = PF ? 0x80000000ull : 0x100000000ull;
+    const u64 lim = (u64)a.bin_lo + ((u64)(b + 1u) << a.bin_shift);
+    return cls + (b == PER_CLASS - 1u || lim > end ? end : lim);     // (a class's last bin holds the rest of it)
 }
 
 // Key of an entry already known to pass the flag / ref_count rules: the agent range check, the
@@ -463,6 +410,44 @@ __device__ __forceinline__ uint32_t sel_block_scan(uint32_t v, uint32_t *s_part,
     total = s_part[32 + n_warps - 1];
     const uint32_t before = warp ? s_part[32 + warp - 1] : 0;
     return before + incl - v;
+}
+
+// Adds 1 to `count` where (ka, ia) < (kb, ib): the borrow of a 96-bit subtraction.
+__device__ __forceinline__ void count_less(uint32_t &count, u64 ka, uint32_t ia, u64 kb, uint32_t ib)
+{
+    uint32_t r;
+    asm("{\n\t.reg .u32 x;\n\tsub.cc.u32 x, %1, %2;\n\tsubc.cc.u32 x, %3, %4;\n\tsubc.cc.u32 x, %5, %6;\n\tsubc.u32 %0, 0, 0;\n\t}"
+        : "=r"(r)
+        : "r"(ia), "r"(ib), "r"((uint32_t)ka), "r"((uint32_t)kb), "r"((uint32_t)(ka >> 32)), "r"((uint32_t)(kb >> 32)));
+    count -= r;
+}
+__device__ __forceinline__ bool less96(u64 ka, uint32_t ia, u64 kb, uint32_t ib)
+{
+    uint32_t n = 0;
+    count_less(n, ka, ia, kb, ib);
+    return n != 0;
+}
+
+// Ranks m keys against c keys, both in shared memory: emit(rank, km, id) for each.  Whole CTA; up to 32 neighbouring
+// lanes share a key.
+template <class Emit>
+__device__ __forceinline__ void rank_keys(const u64 *km, const uint32_t *id, uint32_t m, const u64 *all_km, const uint32_t *all_id,
+                                          uint32_t c, Emit emit)
+{
+    uint32_t parts = 1;
+    while (parts < 32u && 2u * parts * m <= blockDim.x) parts <<= 1;
+    const uint32_t sub = threadIdx.x & (parts - 1u), step = blockDim.x / parts;
+    for (uint32_t k0 = 0; k0 < m; k0 += step) {                     // (uniform: whole warps stay in the shuffles)
+        const uint32_t k = k0 + threadIdx.x / parts;
+        const bool have = k < m;
+        const u64 my = have ? km[k] : 0ull;
+        const uint32_t mine = have ? id[k] : 0u;
+        uint32_t r = 0;
+#pragma unroll 4
+        for (uint32_t q = sub; q < c; q += parts) count_less(r, all_km[q], all_id[q], my, mine);
+        for (uint32_t d = parts >> 1; d > 0; d >>= 1) r += __shfl_xor_sync(0xFFFFFFFFu, r, d);
+        if (have && sub == 0) emit(r, my, mine);
+    }
 }
 
 __device__ __forceinline__ bool key_less(unsigned long long km_a, uint32_t id_a, unsigned long long km_b,

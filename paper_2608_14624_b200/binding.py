@@ -149,10 +149,19 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+def _current_stream() -> int:
+    """Handle of torch's current stream on the current device.  (torch.cuda.current_stream() wraps it in a new Stream
+    object: 3.4 us, a third of what a small call costs the host; the raw handle takes 0.2 us.)"""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch._C._cuda_getDevice())
+
+
 def _stream(s) -> Optional[int]:
     if s is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(s, int):
         return s
     return s.cuda_stream

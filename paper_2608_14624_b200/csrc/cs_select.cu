@@ -162,6 +162,8 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) cs_sel_fast_kernel(SelArgs a, 
     const uint32_t n_tiles = a.n / TILE, n_warps = nth >> 5;
     // the first tile travels with the tables
     const u64 bound = cs_ld_cg_pinned(&ws.sc->sel_T[a.hint_slot]);      // ~0: nothing remembered
+    const uint32_t monotone = cs_ld_cg_pinned(&ws.sc->gtab_monotone);
+    const bool enabled = !PF || prefetch_enabled(ws, a.A);
     Group G;
     if ((gtid >> 5) < n_tiles) load_group<PF>(a, gtid >> 5, lane, G);
     resolve_now(a);
@@ -174,7 +176,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) cs_sel_fast_kernel(SelArgs a, 
     CS_STAMP(ws, CS_PS_SCAN_TABLES + PS / 2, blockIdx.x == 0 && threadIdx.x == 0);
     // the cuts rely on g never increasing with age (checked when the table was built) and on the table covering every
     // unsaturated age; otherwise nothing is dismissed and every eligible entry takes the exact test
-    const bool usable = ws.sc->gtab_monotone && a.gtab_len == a.age_sat;
+    const bool usable = monotone && a.gtab_len == a.age_sat;
     for (uint32_t e = threadIdx.x; e < a.A; e += blockDim.x) s_cut[e] = usable ? la_cut<PF>(a, T, e, bound) : (PF ? 0u : 0xFFFFFFFFu);
     __syncthreads();
     CS_STAMP(ws, CS_PS_SCAN_CUTS + PS / 2, blockIdx.x == 0 && threadIdx.x == 0);
@@ -187,7 +189,6 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) cs_sel_fast_kernel(SelArgs a, 
         stage_init(st, stage_km, (uint32_t *)(stage_km + (SEL_THREADS / 32) * STAGE_CAP));
     }
     uint32_t n_above = 0;
-    const bool enabled = !PF || prefetch_enabled(ws, a.A);
 
     // Works off whole rounds of 32 queued entries (all of them when `all`), every lane busy.
     auto drain = [&](bool all) {
@@ -584,7 +585,13 @@ __device__ __forceinline__ void sort_tile(unsigned long long *t_km, uint32_t *t_
 // A bucket has a fixed region of the sort arrays; one that outgrows it is gathered again from the candidates by its CTA.
 // ---------------------------------------------------------------------------------------------
 #define SAMPLE_CTAS 64u
-struct OrderPlan { uint32_t S, J, nb, cap; };
+struct OrderPlan {
+    uint32_t S, J;            // samples; of those, how many cover the output
+    uint32_t gaps;            // gap g lies between samples g - 1 and g (the first from the smallest key, the last to the largest
+                              // key when no sample lies beyond the output)
+    uint32_t sub, join;       // buckets per gap, gaps per bucket; one of them is 1
+    uint32_t nb, cap;         // buckets, and keys a bucket's region holds
+};
 __device__ __forceinline__ OrderPlan order_plan(uint32_t c, uint32_t n_out, uint32_t max_blocks, uint32_t region_max)
 {
     OrderPlan P;
@@ -592,10 +599,29 @@ __device__ __forceinline__ OrderPlan order_plan(uint32_t c, uint32_t n_out, uint
     const float e = (float)n_out * (float)P.S / (float)c;
     const uint32_t want = (uint32_t)(e + 4.0f * sqrtf(e)) + 3u;
     P.J = want < P.S ? want : P.S;
-    P.nb = P.J < CS_BUCKETS ? P.J : CS_BUCKETS;
+    P.gaps = P.J + (P.J == P.S ? 1u : 0u);
+    P.sub = P.gaps <= CS_BUCKETS ? CS_BUCKETS / P.gaps : 1u;
+    P.join = (P.gaps + CS_BUCKETS - 1u) / CS_BUCKETS;
+    P.nb = P.join > 1u ? (P.gaps + P.join - 1u) / P.join : P.gaps * P.sub;
     P.cap = max_blocks / P.nb;
     if (region_max && P.cap > region_max) P.cap = region_max;
     return P;
+}
+// Smallest key of bucket j.  A gap that is several buckets is divided evenly: locally the keys of a tie in score are spread
+// evenly over last_access, and the largest of a few hundred gaps is six times the mean one.
+__device__ __forceinline__ void bucket_start(const OrderPlan &P, const u64 *s_km, const uint32_t *s_id, uint32_t j, u64 &km, uint32_t &id)
+{
+    const uint32_t g = P.join > 1u ? j * P.join : j / P.sub, f = P.join > 1u ? 0u : j - g * P.sub;
+    km = g ? s_km[g - 1] : 0ull;
+    id = g ? s_id[g - 1] : 0u;
+    if (j >= P.nb) {
+        km = ~0ull;
+        id = 0xFFFFFFFFu;
+    } else if (f) {
+        const u64 step = ((g < P.J ? s_km[g] : ~0ull) - km) / P.sub;
+        if (step) id = 0u;                                    // (a gap inside a tie down to the id is not divided)
+        km += step * f;
+    }
 }
 
 __global__ void __launch_bounds__(512) cs_sel_sample_kernel(SelArgs a, cs_workspace ws, uint32_t *__restrict__ ids_out,
@@ -652,8 +678,8 @@ __global__ void __launch_bounds__(512) cs_sel_sample_kernel(SelArgs a, cs_worksp
 
 __global__ void __launch_bounds__(256) cs_sel_place_kernel(cs_workspace ws, uint32_t max_blocks, uint32_t region_max, uint32_t kind)
 {
-    __shared__ u64 s_km[CS_SAMPLE];
-    __shared__ uint32_t s_id[CS_SAMPLE];
+    __shared__ u64 s_km[CS_SAMPLE], b_km[CS_BUCKETS];         // the sample, and where the buckets start
+    __shared__ uint32_t s_id[CS_SAMPLE], b_id[CS_BUCKETS];
     constexpr int ITEMS = 4;                                  // candidates per thread and round
     const uint32_t tid = threadIdx.x;
     cs_wait_for_predecessor();
@@ -683,6 +709,8 @@ __global__ void __launch_bounds__(256) cs_sel_place_kernel(cs_workspace ws, uint
     __syncthreads();
     const u64 cut_km = s_km[P.J - 1];
     const uint32_t cut_id = s_id[P.J - 1];
+    for (uint32_t j = tid; j < CS_BUCKETS; j += 256u) bucket_start(P, s_km, s_id, j, b_km[j], b_id[j]);
+    __syncthreads();
     for (uint32_t base = 0; base < c; base += sweep * ITEMS) {
         if (base != 0) {
 #pragma unroll
@@ -697,12 +725,10 @@ __global__ void __launch_bounds__(256) cs_sel_place_kernel(cs_workspace ws, uint
             const uint32_t i = base + u * sweep + lane0;
             // keys from the cut up are dropped when there are samples beyond it
             if (i >= c || (P.J < P.S && !less96(km[u], id[u], cut_km, cut_id))) continue;
-            uint32_t b = 0;                                   // splitters at or below the key; splitter j (from 1) = sample rank j J / nb
-#pragma unroll 1
-            for (uint32_t step = CS_BUCKETS / 2; step > 0; step >>= 1) {
-                const uint32_t j = b + step, at = (j < P.nb ? j : 0u) * P.J / P.nb;
-                if (j < P.nb && !less96(km[u], id[u], s_km[at], s_id[at])) b = j;
-            }
+            uint32_t b = 0;                                   // the last bucket that starts at or below the key
+#pragma unroll
+            for (uint32_t step = CS_BUCKETS / 2; step > 0; step >>= 1)
+                b += less96(km[u], id[u], b_km[b + step], b_id[b + step]) ? 0u : step;
             const uint32_t slot = atomicAdd(&CS_BCOUNT(ws, b), 1u);
             if (slot < P.cap) {
                 ws.sort_km[(size_t)b * P.cap + slot] = km[u];
@@ -721,7 +747,7 @@ __device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u6
     const u64 none = ~0ull, all = ~0ull - 1ull;
     if (st.n_elig <= k) return all;                           // everything eligible is wanted
     const uint32_t ahead = cs_ahead(k);
-    if (st.ahead != none && (!st.spec || st.c > 2ull * ahead)) return st.ahead < all ? st.ahead : all;
+    if (st.ahead != none && (!st.spec || st.c > ahead + ahead / 4u)) return st.ahead < all ? st.ahead : all;
     if (st.c >= 2ull * k + 1024ull || st.c >= st.n_elig || st.bound >= all || st.bound < kth) return st.bound < all ? st.bound : all;
     const u64 gap = st.bound - kth, per = (ahead - st.c) / (st.c - k + 1u);
     const u64 more = (gap < (1ull << 40) ? gap : (1ull << 40)) * (per < 8ull ? per : 8ull) + 64ull;
@@ -729,8 +755,10 @@ __device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u6
 }
 
 // Bucket b of CTA b: ranked by counting while it is small, sorted in the tile (bitonic, O(m log^2 m)) when it is large.
-#define FINISH_COUNT_MAX 256u
-__global__ void __launch_bounds__(256)
+#define FINISH_THREADS 512u
+#define FINISH_COUNT_MAX 512u
+static_assert(FINISH_THREADS == CS_BUCKETS, "one bucket size per thread");
+__global__ void __launch_bounds__(FINISH_THREADS)
 cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t region_max, uint32_t kind, uint32_t hint_slot,
                      uint32_t *__restrict__ ids_out)
 {
@@ -744,16 +772,16 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
     CS_STAMP(ws, CS_PS_FINISH_WAITED + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
     cs_release_successor();
     const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_out, n_elig, b0
-    const uint32_t n0 = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid)), n1 = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid + 256u));
+    const uint32_t n_t = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid));
     uint32_t m = cs_ld_cg_pinned(&CS_BCOUNT(ws, b));
     const uint32_t c = st.x, n_out = st.y;
     if (n_out == 0) return;
     const OrderPlan P = order_plan(c, n_out, max_blocks, region_max);
     if (b >= P.nb) return;
-    const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, (tid < b ? n0 : 0u) + (tid + 256u < b ? n1 : 0u));
+    const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, tid < b ? n_t : 0u);
     if ((tid & 31) == 0 && before) atomicAdd(&s_off, before);
     if (b == 0) {                                             // work counters, and whether any bucket outgrew its region
-        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n0 > n1 ? n0 : n1);
+        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n_t);
         if ((tid & 31) == 0) atomicMax(&s_max, most);
     }
     __syncthreads();
@@ -777,11 +805,13 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
     };
     if (m > P.cap || rest) {
         // the region was too small: the bucket's keys once more, out of all candidates
-        const uint32_t at_lo = b * P.J / P.nb, at_hi = (b + 1u) * P.J / P.nb;
-        const u64 lo_km = b ? ws.spl_km[at_lo] : 0ull, hi_km = b + 1u < P.nb ? ws.spl_km[at_hi] : (P.J < P.S && !rest ? ws.spl_km[P.J - 1] : ~0ull);
-        const uint32_t lo_id = b ? ws.spl_id[at_lo] : 0u, hi_id = b + 1u < P.nb ? ws.spl_id[at_hi] : (P.J < P.S && !rest ? ws.spl_id[P.J - 1] : 0xFFFFFFFFu);
+        u64 lo_km, hi_km;
+        uint32_t lo_id, hi_id;
+        bucket_start(P, ws.spl_km, ws.spl_id, b, lo_km, lo_id);
+        bucket_start(P, ws.spl_km, ws.spl_id, b + 1u, hi_km, hi_id);
+        if (b == P.nb - 1u && P.J < P.S && !rest) { hi_km = ws.spl_km[P.J - 1]; hi_id = ws.spl_id[P.J - 1]; }
         const bool fits = m <= RANK_TILE;
-        for (uint32_t i = tid; i < c; i += 256u) {
+        for (uint32_t i = tid; i < c; i += FINISH_THREADS) {
             const u64 km = __ldcg(ws.cand_km + i);
             const uint32_t id = __ldcg(ws.cand_id + i);
             if (less96(km, id, lo_km, lo_id) || !less96(km, id, hi_km, hi_id)) continue;
@@ -802,13 +832,13 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
         if (!fits) return;
         __syncthreads();
     } else if (m <= RANK_TILE) {
-        for (uint32_t i = tid; i < m; i += 256u) {
+        for (uint32_t i = tid; i < m; i += FINISH_THREADS) {
             t_km[i] = __ldcg(src_km + i);
             t_id[i] = __ldcg(src_id + i);
         }
         __syncthreads();
     } else {                                                  // larger than the tile: ranked straight from global memory
-        for (uint32_t i = tid; i < m; i += 256u) {
+        for (uint32_t i = tid; i < m; i += FINISH_THREADS) {
             const u64 km = __ldcg(src_km + i);
             const uint32_t id = __ldcg(src_id + i);
             uint32_t r = 0;
@@ -821,7 +851,7 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
         rank_keys(t_km, t_id, m, t_km, t_id, m, emit);
     } else {
         sort_tile(t_km, t_id, m);
-        for (uint32_t i = tid; i < m; i += 256u) emit(i, t_km[i], t_id[i]);
+        for (uint32_t i = tid; i < m; i += FINISH_THREADS) emit(i, t_km[i], t_id[i]);
     }
     CS_STAMP(ws, CS_PS_FINISH_DONE + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
 }
@@ -930,53 +960,80 @@ static int scan_opt_in(cs_ctx *ctx)
     return CS_OK;
 }
 
-// One select through the grid-wide kernels (or one single-launch cluster select), on the scratch of `job`.
+// One select through the grid-wide kernels, on the scratch of one job: the arguments, and its six launches one by one, so
+// that several selects' launches can be issued in turn.
+#define SELECT_STAGES 6
+struct SelectChain {
+    SelArgs a;
+    const cs_workspace *ws;
+    uint32_t prefetch, *ids_out, *n_out;
+    cudaStream_t s;
+};
+
+static void prepare_chain(const cs_ctx *ctx, int job, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier, uint32_t k,
+                          uint32_t *ids_out, uint32_t *n_out, cudaStream_t s, SelectChain &c)
+{
+    c.ws = job == 0 ? &ctx->ws : &ctx->ws_job[job - 1];
+    c.prefetch = prefetch ? 1u : 0u;
+    c.ids_out = ids_out;
+    c.n_out = n_out;
+    c.s = s;
+    cs_fill_sel_args(ctx, idx, now, ctx->fsurv_override ? ctx->fsurv_override : ctx->ws.fsurv, c.a);
+    c.a.tier = tier;
+    c.a.k = k;
+    c.a.hint_slot = ctx->no_speculation ? 3u : (prefetch ? 2u : tier);
+    c.a.kind = prefetch ? 2u : tier;
+    cs_fill_sel_bins(ctx, c.a, prefetch);
+}
+
+static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage)
+{
+    const uint32_t grid = cs_scan_grid(ctx, c.a.n, SEL_THREADS * GRP), grid_c = cs_scan_grid(ctx, c.a.n, 1024), A = ctx->p.n_agents;
+    const size_t sm = cs_table_smem(ctx);
+    const cs_workspace &ws = *c.ws;
+    if (stage == 0) {
+        // tables, per-warp queues, per-warp candidate staging, cuts
+        const size_t sm_fast = (sm + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
+                               (size_t)A * sizeof(uint32_t);
+        if (c.prefetch) cs_launch_chained(cs_sel_fast_kernel<true>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);
+        else cs_launch_chained(cs_sel_fast_kernel<false>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);
+    } else if (stage == 1) {
+        if (c.prefetch) cs_launch_chained(cs_sel_hist_kernel<true>, grid, SEL_THREADS, sm, c.s, c.a, ws);
+        else cs_launch_chained(cs_sel_hist_kernel<false>, grid, SEL_THREADS, sm, c.s, c.a, ws);
+    } else if (stage == 2) {
+        // large indexes: the collect pass prefilters by age limits (one look-up per entry instead of the full key)
+        const uint32_t n_cls = c.a.ntok ? ctx->p.block_tokens : 1u;
+        size_t sm_collect = sm;
+        if (c.a.n >= CS_AGE_LIMIT_MIN_BLOCKS && (size_t)A * n_cls <= AGE_LIM_MAX) {
+            c.a.use_age_limits = 1;
+            sm_collect += (size_t)A * n_cls * sizeof(uint32_t);
+        }
+        if (c.prefetch) cs_launch_chained(cs_sel_collect_kernel<true>, grid, SEL_THREADS, sm_collect, c.s, c.a, ws);
+        else cs_launch_chained(cs_sel_collect_kernel<false>, grid, SEL_THREADS, sm_collect, c.s, c.a, ws);
+    } else if (stage == 3) {
+        cs_launch_chained(cs_sel_sample_kernel, SAMPLE_CTAS, 512, 0, c.s, c.a, ws, c.ids_out, c.n_out);
+    } else if (stage == 4) {
+        cs_launch_chained(cs_sel_place_kernel, grid_c, 256, 0, c.s, ws, c.a.max_blocks, c.a.region_cap_max, c.a.kind);
+    } else {
+        cs_launch_chained(cs_sel_finish_kernel, CS_BUCKETS, FINISH_THREADS, 0, c.s, ws, c.a.k, c.a.max_blocks, c.a.region_cap_max, c.a.kind,
+                          c.a.hint_slot, c.ids_out);
+    }
+    return cs_check_launch(ctx);
+}
+
+// One select: the single-launch cluster kernel where it applies, else the chain.
 static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier,
                              uint32_t k, uint32_t *ids_out, uint32_t *n_out, cudaStream_t s)
 {
-    const cs_workspace &ws = job == 0 ? ctx->ws : ctx->ws_job[job - 1];
-    SelArgs a;
-    cs_fill_sel_args(ctx, idx, now, ctx->fsurv_override ? ctx->fsurv_override : ctx->ws.fsurv, a);
-    a.tier = tier;
-    a.k = k;
-    a.hint_slot = ctx->no_speculation ? 3u : (prefetch ? 2u : tier);
-    a.kind = prefetch ? 2u : tier;
-    cs_fill_sel_bins(ctx, a, prefetch);
+    SelectChain c;
+    prepare_chain(ctx, job, idx, now, prefetch, tier, k, ids_out, n_out, s, c);
     if (ctx->select_path != CS_SELECT_MULTI && idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) {
-        const int rc1 = cs_launch_select_cluster(ctx, &a, &ws, prefetch, ids_out, n_out, s);
+        const int rc1 = cs_launch_select_cluster(ctx, &c.a, c.ws, prefetch, ids_out, n_out, s);
         if (rc1 != CS_ENOTIMPL) return rc1;          // no usable cluster on this device: fall through
     }
-    const uint32_t grid = cs_scan_grid(ctx, idx->n_blocks, SEL_THREADS * GRP);
-    const uint32_t grid_c = cs_scan_grid(ctx, idx->n_blocks, 1024);
-    const size_t sm = cs_table_smem(ctx);
-    int rc;
-    const size_t sm_fast = (sm + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
-                           (size_t)ctx->p.n_agents * sizeof(uint32_t);   // tables, per-warp queues, per-warp candidate staging, age cuts
-    if ((rc = scan_opt_in(ctx)) != CS_OK) return rc;
-    if (prefetch) cs_launch_chained(cs_sel_fast_kernel<true>, grid, SEL_THREADS, sm_fast, s, a, ws);
-    else cs_launch_chained(cs_sel_fast_kernel<false>, grid, SEL_THREADS, sm_fast, s, a, ws);
-    if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    if (prefetch) cs_launch_chained(cs_sel_hist_kernel<true>, grid, SEL_THREADS, sm, s, a, ws);
-    else cs_launch_chained(cs_sel_hist_kernel<false>, grid, SEL_THREADS, sm, s, a, ws);
-    if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    // large indexes: the collect pass prefilters by age limits (one look-up per entry instead of the full key)
-    const uint32_t n_cls = idx->n_tokens ? ctx->p.block_tokens : 1u;
-    size_t sm_collect = sm;
-    if (idx->n_blocks >= CS_AGE_LIMIT_MIN_BLOCKS && (size_t)ctx->p.n_agents * n_cls <= AGE_LIM_MAX) {
-        a.use_age_limits = 1;
-        sm_collect += (size_t)ctx->p.n_agents * n_cls * sizeof(uint32_t);
-        const int rc_opt = scan_opt_in(ctx);
-        if (rc_opt != CS_OK) return rc_opt;
-    }
-    if (prefetch) cs_launch_chained(cs_sel_collect_kernel<true>, grid, SEL_THREADS, sm_collect, s, a, ws);
-    else cs_launch_chained(cs_sel_collect_kernel<false>, grid, SEL_THREADS, sm_collect, s, a, ws);
-    if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_sample_kernel, SAMPLE_CTAS, 512, 0, s, a, ws, ids_out, n_out);
-    if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_place_kernel, grid_c, 256, 0, s, ws, a.max_blocks, a.region_cap_max, a.kind);
-    if ((rc = cs_check_launch(ctx)) != CS_OK) return rc;
-    cs_launch_chained(cs_sel_finish_kernel, CS_BUCKETS, 256, 0, s, ws, k, a.max_blocks, a.region_cap_max, a.kind, a.hint_slot, ids_out);
-    return cs_check_launch(ctx);
+    int rc = scan_opt_in(ctx);
+    for (int stage = 0; stage < SELECT_STAGES && rc == CS_OK; ++stage) rc = launch_stage(ctx, c, stage);
+    return rc;
 }
 
 int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier, uint32_t k,
@@ -1021,20 +1078,29 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
         const int rc = cs_launch_select_clusters(ctx, n_jobs, a, pf, j_ids, j_cnt, s);
         if (rc != CS_ENOTIMPL) return rc;
     }
-    const bool side_by_side = ctx->concurrent_selects && n_jobs > 1;
-    cudaError_t e = cudaSuccess;
-    if (side_by_side) e = cudaEventRecord(ctx->ev_sel_fork, s);
     int rc = CS_OK;
-    for (int i = 0; i < n_jobs && rc == CS_OK && e == cudaSuccess; ++i) {
-        const int q = jobs[i];
-        cudaStream_t sq = (side_by_side && i > 0) ? ctx->sel_stream[i - 1] : s;
-        if (side_by_side && i > 0) e = cudaStreamWaitEvent(sq, ctx->ev_sel_fork, 0);
-        if (e != cudaSuccess) break;
-        rc = launch_select_job(ctx, side_by_side ? i : 0, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], sq);
-        if (rc == CS_OK && side_by_side && i > 0) {
-            e = cudaEventRecord(ctx->ev_sel_join[i - 1], sq);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev_sel_join[i - 1], 0);
+    if (!ctx->concurrent_selects || n_jobs == 1) {
+        for (int i = 0; i < n_jobs && rc == CS_OK; ++i) {
+            const int q = jobs[i];
+            rc = launch_select_job(ctx, 0, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], s);
         }
+        return rc;
+    }
+    // The chains' launches are issued in turn: issued one chain after the other, the second one started 20 us (six
+    // launches) after the first and both ended that much later.
+    if ((rc = scan_opt_in(ctx)) != CS_OK) return rc;
+    SelectChain chain[3];
+    cudaError_t e = cudaEventRecord(ctx->ev_sel_fork, s);
+    for (int i = 0; i < n_jobs && e == cudaSuccess; ++i) {
+        const int q = jobs[i];
+        prepare_chain(ctx, i, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], i ? ctx->sel_stream[i - 1] : s, chain[i]);
+        if (i) e = cudaStreamWaitEvent(ctx->sel_stream[i - 1], ctx->ev_sel_fork, 0);
+    }
+    for (int stage = 0; stage < SELECT_STAGES && e == cudaSuccess; ++stage)
+        for (int i = 0; i < n_jobs && rc == CS_OK; ++i) rc = launch_stage(ctx, chain[i], stage);
+    for (int i = 1; i < n_jobs && e == cudaSuccess; ++i) {
+        e = cudaEventRecord(ctx->ev_sel_join[i - 1], ctx->sel_stream[i - 1]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ctx->ev_sel_join[i - 1], 0);
     }
     if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
     return rc;

@@ -27,7 +27,7 @@ static_assert(2 * CS_HIST_BINS * 4 <= 48 * 1024, "histograms");
 
 __host__ __device__ inline size_t csel_table_bytes(uint32_t A, uint32_t gtab_len)
 {
-    return (((size_t)(A + gtab_len) * 4 + (size_t)A * 2) + 15) / 16 * 16;
+    return (((size_t)(A + gtab_len + 1) * 4 + (size_t)A * 2) + 15) / 16 * 16;
 }
 // Candidates a CTA holds at once: no more than the index has entries.
 static uint32_t csel_cap(uint32_t n)
@@ -169,6 +169,10 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
     order_carve((unsigned char *)(tot + CS_HIST_BINS), cap, O);
     Tables T;
     load_tables_static(a, ws, (float *)dsm, T);
+    // the table covers every age before saturation: one entry more stands for all the others
+    T.anchor += 2;
+    const bool whole_table = a.gtab_len == a.age_sat;
+    if (tid == 0) T.gtab[a.gtab_len] = T.g_sat;
     for (uint32_t i = tid; i < CS_HIST_BINS / 4; i += CSEL_THREADS) ((uint4 *)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < OM_WORDS) O.misc[tid] = 0;
     CS_STAMP(ws, CS_PS_SCAN_SETUP + PS, stamp);
@@ -189,18 +193,22 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
         }
     };
     load_pass(0u);
+    const uint32_t t0 = n_units * CSEL_UNIT, ctid = rank * CSEL_THREADS + tid;     // the ragged tail: one entry per thread
+    bool tail = ctid < a.n - t0;
+    const uint32_t tail_id = t0 + ctid;
+    uint32_t tail_pr = 0, tail_se = 0, tl_ag = 0, tl_dp = 0, tl_rf = 0, tl_fl = 0, tl_la = 0, tl_tk = a.block_tokens;
+    if (tail) {
+        tl_ag = __ldg(a.agent + tail_id);
+        tl_dp = __ldg(a.depth + tail_id);
+        tl_rf = __ldg(a.ref + tail_id);
+        tl_fl = __ldg(a.flags + tail_id);
+        tl_la = __ldg(a.la + tail_id);
+        if (a.ntok) tl_tk = __ldg(a.ntok + tail_id);
+    }
     load_tables_dynamic(a, ws, T, PF && a.anchor);
     const bool enabled = !PF || prefetch_enabled(ws, a.A);
-    const uint32_t t0 = n_units * CSEL_UNIT, ctid = rank * CSEL_THREADS + tid;     // the ragged tail: one entry per thread
-    bool tail = enabled && ctid < a.n - t0;
-    uint32_t tail_pr = 0, tail_se = 0;
-    const uint32_t tail_id = t0 + ctid;
     __syncthreads();
-    if (tail) {
-        const uint32_t tok = a.ntok ? a.ntok[tail_id] : a.block_tokens;
-        tail = entry_key<PF>(a, T, &ws.sc->status, a.agent[tail_id], a.depth[tail_id], a.ref[tail_id], a.flags[tail_id], a.la[tail_id],
-                             tok, tail_pr, tail_se);
-    }
+    tail = tail && enabled && entry_key<PF>(a, T, &ws.sc->status, tl_ag, tl_dp, tl_rf, tl_fl, tl_la, tl_tk, tail_pr, tail_se);
     uint32_t pr[4 * CSEL_UNITS], em = 0;                          // primary keys; bit 4 q + r: entry r of unit q is eligible
     uint32_t b0 = 0xFFFFFFFFu, n_out = 0, c = 0;
     // candidates: in shared memory when one CTA is all there is and they fit, else in L2, numbered by the first CTA
@@ -221,19 +229,35 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
                     if (u0 + q * n_warps + gw >= n_units) break;
                     const uint32_t fmask = PF ? 0x0F0F0F0Fu : 0x07070707u;
                     const uint32_t fpat = PF ? 0x05050505u : (0x01010101u * (CS_FLAG_VALID | (a.tier << 2)));
-                    const uint32_t ok = nibble_of_flags(zero_bytes(((Q[q].fl & fmask) ^ fpat) | Q[q].rf));
+                    uint32_t ok = nibble_of_flags(zero_bytes(((Q[q].fl & fmask) ^ fpat) | Q[q].rf));
+                    if (!__any_sync(0xFFFFFFFFu, ok != 0u)) continue;
+                    // the four keys side by side, without a branch: an entry that is not eligible gets one nobody looks at
 #pragma unroll
                     for (int r = 0; r < 4; ++r) {
-                        if (!((ok >> r) & 1u)) continue;
                         const uint32_t ag = ((r < 2 ? Q[q].ag.x : Q[q].ag.y) >> ((r & 1) * 16)) & 0xFFFFu;
-                        const uint32_t dp = ((r < 2 ? Q[q].dp.x : Q[q].dp.y) >> ((r & 1) * 16)) & 0xFFFFu;
-                        const uint32_t tok = a.ntok ? (Q[q].tk >> (8 * r)) & 0xFFu : a.block_tokens;
-                        uint32_t p, se;
-                        if (entry_key_rest<PF>(a, T, &ws.sc->status, ag, dp, (Q[q].fl >> (8 * r)) & 0xFFu, u4_word(Q[q].la, r), tok, p, se)) {
-                            pr[4 * q + r] = p;
-                            em |= 1u << (4 * q + r);
-                            if (phase == 0) atomicAdd(&hist[bin_of<PF>(a, p)], 1u);
+                        const uint32_t agc = ag < a.A ? ag : 0u;
+                        if (ag >= a.A && ((ok >> r) & 1u)) {
+                            atomicOr(&ws.sc->status, CS_ST_BAD_AGENT);
+                            ok &= ~(1u << r);
                         }
+                        if (PF && a.anchor) {
+                            const uint32_t dp = ((r < 2 ? Q[q].dp.x : Q[q].dp.y) >> ((r & 1) * 16)) & 0xFFFFu;
+                            ok &= ~((dp < T.anchor[agc] ? 0u : 1u) << r);
+                        }
+                        const uint32_t tok = a.ntok ? (Q[q].tk >> (8 * r)) & 0xFFu : a.block_tokens, la = u4_word(Q[q].la, r);
+                        const uint32_t age = max(a.now, la) - la;
+                        float g;
+                        if (whole_table) g = T.gtab[min(age, a.gtab_len)];             // (its last entry is the saturated factor)
+                        else g = recency_of_age(a, T, age);
+                        const uint32_t bits = __float_as_uint(__fmul_rn(__fmul_rn(T.fsurv[agc], g), (float)tok));
+                        if (PF) pr[4 * q + r] = (agc == T.a_star ? 0u : 0x80000000u) | (~bits & 0x7FFFFFFFu);
+                        else pr[4 * q + r] = a.prefer_copy ? ((bits << 1) | ((Q[q].fl >> (8 * r + 3)) & 1u ^ 1u)) : bits;
+                    }
+                    em |= ok << (4 * q);
+                    if (phase == 0) {
+#pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            if ((ok >> r) & 1u) atomicAdd(&hist[bin_of<PF>(a, pr[4 * q + r])], 1u);
                     }
                 }
             }

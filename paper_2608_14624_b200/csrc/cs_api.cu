@@ -145,6 +145,8 @@ struct ModelParts { ModelPart part[MODEL_PARTS]; };
 __global__ void __launch_bounds__(EXPORT_THREADS) cs_export_kernel(const __grid_constant__ ModelParts parts)
 {
     const ModelPart p = parts.part[blockIdx.y];
+    cs_wait_for_predecessor();
+    cs_release_successor();
     const size_t tid = blockIdx.x * (size_t)EXPORT_THREADS + threadIdx.x, nth = gridDim.x * (size_t)EXPORT_THREADS;
     size_t done = 0;
     if (!(((uintptr_t)p.dst) & 15u)) {                      // (the tables themselves are 256-byte aligned)
@@ -483,7 +485,7 @@ int cs_get_model(cs_ctx *ctx, uint32_t *C_out, float *P_out, uint16_t *amax_out,
     if (e == cudaSuccess && n) {
         size_t ctas = (most / 16 + EXPORT_THREADS - 1) / EXPORT_THREADS;
         ctas = ctas < 1 ? 1 : (ctas > (size_t)ctx->sm_count ? (size_t)ctx->sm_count : ctas);
-        cs_export_kernel<<<dim3((unsigned)ctas, n), EXPORT_THREADS, 0, s>>>(copy);
+        cs_launch_chained(cs_export_kernel, dim3((unsigned)ctas, n), EXPORT_THREADS, 0, s, copy);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }

@@ -701,6 +701,8 @@ cs_survival_kernel(cs_workspace ws, uint32_t A, uint32_t W, const uint16_t *__re
     __shared__ uint32_t s_front[2 * PULL_MAX_WORDS];
     const uint32_t tid = threadIdx.x;
     uint32_t row[KW];
+    cs_wait_for_predecessor();
+    cs_release_successor();
 #pragma unroll
     for (int w = 0; w < KW; ++w) row[w] = ((uint32_t)w < W && tid < A) ? cs_ld_cg_pinned(ws.adjT + (size_t)w * A + tid) : 0u;
     for (uint32_t i = tid; i < 2 * PULL_MAX_WORDS; i += blockDim.x) s_front[i] = 0;
@@ -983,8 +985,11 @@ int cs_launch_survival(cs_ctx *ctx, const uint16_t *sources, uint32_t n_sources,
 {
     const cs_params &p = ctx->p;
     const dim3 block(32u * ctx->W);
-    if (ctx->W == 1) cs_survival_kernel<1><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
-    else if (ctx->W <= 8) cs_survival_kernel<8><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
-    else cs_survival_kernel<32><<<1, block, 0, s>>>(ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
+    const auto launch = [&](auto kernel) {
+        cs_launch_chained(kernel, 1, block, 0, s, ctx->ws, p.n_agents, ctx->W, sources, n_sources, p.e_max, p.delta);
+    };
+    if (ctx->W == 1) launch(cs_survival_kernel<1>);
+    else if (ctx->W <= 8) launch(cs_survival_kernel<8>);
+    else launch(cs_survival_kernel<32>);
     return cs_check_launch(ctx);
 }

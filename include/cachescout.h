@@ -418,8 +418,9 @@ int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream
 int cs_debug_phase_stamps(cs_ctx *ctx, uint64_t *out);
 
 /* Width of the mover (0 keeps the default): for transfers that cross the host link and for
- * device-to-device moves.  Unit: warp pipelines on the bulk path (each keeps up to two loads and two
- * stores of 16 KiB in flight; defaults 8 offload / 24 prefetch / 2 per SM device-to-device), CTAs of
+ * device-to-device moves.  Unit: warp pipelines on the bulk path (each keeps about 32 KiB of loads and 16 KiB of
+ * stores in flight, in pieces of at most 16 KiB; defaults 8 - 32 offload / 24 prefetch / 32 - 64 both ways, by the
+ * size of a chunk; 1.7 or, for short moves and small chunks, 4 per SM device-to-device), CTAs of
  * 256 threads on the load/store path.  Narrow host-link transfers disturb other kernels less. */
 int cs_set_mover_ctas(cs_ctx *ctx, uint32_t host_link_ctas, uint32_t d2d_ctas);
 

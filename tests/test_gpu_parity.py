@@ -286,6 +286,45 @@ def pinned_zeros(nbytes):
 PATHS = [cs.CS_MOVER_BULK, cs.CS_MOVER_LDST]
 
 
+@pytest.mark.parametrize("chunk", [16, 1008, 2048, 2064, 4096, 4112, 8192, 8208, 16384, 16400, 49_152])
+@pytest.mark.parametrize("gpu_layout,host_layout", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_mover_piece_sizes(chunk, gpu_layout, host_layout):
+    """Chunks on both sides of every slot size of the rings, layouts that merge a block into one run and those that do not;
+    one block, a few, and more items than a pipeline looks up at once; a sentinel and a bad slot among them."""
+    L = 3
+    for n in (1, 7, 300 if chunk <= 4112 else 60):
+        G = n + 9
+        rng = synth.rng_for(synth.CONFIGS["tiny"], chunk + n)
+        c, _ = make_ctx(synth.CONFIGS["tiny"], 64)
+        mk = lambda buf, layout: cs.KVPool(buf, G, layout, L, n_kv_heads=1, head_dim=chunk, block_tokens=1, elem_bytes=1)
+        gpu_np, host_np = (rng.integers(0, 256, G * L * 2 * chunk, dtype=np.uint8) for _ in range(2))
+        host_t = pinned_zeros(G * L * 2 * chunk)
+        host_t.copy_(torch.from_numpy(host_np))
+        gpu, host = mk(dev(gpu_np), gpu_layout), mk(host_t, host_layout)
+        g, h = rng.permutation(G).astype(np.uint32)[:n], rng.permutation(G).astype(np.uint32)[:n]
+        n_o = (n + 1) // 2
+        off_src, off_dst, pre_src, pre_dst = g[:n_o].copy(), h[:n_o].copy(), h[n_o:].copy(), g[n_o:].copy()
+        if n > 5:
+            off_src[1] = orc.ID_NONE
+            pre_dst[0] = G + 3
+        c.exchange_blocks(gpu, host, dev(off_src), dev(off_dst), dev(pre_src) if n > 1 else None, dev(pre_dst) if n > 1 else None)
+        torch.cuda.synchronize()
+        want_g, want_h = gpu_np.copy(), host_np.copy()
+        orc.move_blocks(gpu_np, gpu_layout, G, want_h, host_layout, G, L, chunk, off_src, off_dst)
+        keep = pre_dst < G
+        orc.move_blocks(host_np, host_layout, G, want_g, gpu_layout, G, L, chunk, pre_src[keep], pre_dst[keep])
+        assert np.array_equal(host_t.numpy(), want_h) and np.array_equal(gpu.buf.cpu().numpy(), want_g)
+        assert c.get_status() == (cs.CS_ST_BAD_SLOT if n > 5 else 0)
+        s2, d2 = rng.permutation(G).astype(np.uint32)[:n], rng.permutation(n).astype(np.uint32)
+        stage = cs.KVPool(torch.zeros(n * L * 2 * chunk, dtype=torch.uint8, device=DEV), n, host_layout, L, n_kv_heads=1, head_dim=chunk,
+                          block_tokens=1, elem_bytes=1)
+        c.compact_blocks(gpu, stage, dev(s2), dev(d2))
+        want_s = np.zeros(n * L * 2 * chunk, np.uint8)
+        orc.move_blocks(want_g, gpu_layout, G, want_s, host_layout, n, L, chunk, s2, d2)
+        assert np.array_equal(stage.buf.cpu().numpy(), want_s)
+        assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("path", PATHS)
 @pytest.mark.parametrize("gpu_layout", [synth.LAYER_MAJOR, synth.BLOCK_MAJOR])
 @pytest.mark.parametrize("host_layout", [synth.BLOCK_MAJOR, synth.LAYER_MAJOR])

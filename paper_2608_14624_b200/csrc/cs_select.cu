@@ -172,21 +172,23 @@ __device__ __forceinline__ uint32_t la_cut(const SelArgs &a, const Tables &T, ui
 {
     const uint32_t Tp = (uint32_t)(bound >> 32), Ts = (uint32_t)bound;
     const uint32_t flip = (PF && agent != T.a_star) ? 0x80000000u : 0u;
-    // smallest possible primary key at an age (a copy on the other tier would make it that; the exact test tells)
+    const float f = T.fsurv[agent], tb = (float)a.block_tokens;
+    // smallest possible primary key at an age (a copy on the other tier would make it that; the exact test tells).  The
+    // table covers every age before saturation (gtab_len = age_sat) and ends with the saturated factor.
     auto primary = [&](uint32_t age) {
-        const uint32_t bits = __float_as_uint(score_from_age(a, T, agent, age, a.block_tokens));
+        const uint32_t bits = __float_as_uint(__fmul_rn(__fmul_rn(f, T.gtab[age]), tb));
         return PF ? (flip | (~bits & 0x7FFFFFFFu)) : (a.prefer_copy ? bits << 1 : bits);
     };
     // victims: primary falls with age: n_le = first age with primary <= Tp, n_lt = first with primary < Tp (age_sat + 1: none);
-    // prefetch: it rises: n_le = first age with primary > Tp, n_lt = first with primary >= Tp
-    uint32_t lo0 = 0, hi0 = a.age_sat + 1, lo1 = 0, hi1 = a.age_sat + 1;
-    while (lo0 < hi0 || lo1 < hi1) {
-        const uint32_t m0 = lo0 + ((hi0 - lo0) >> 1), m1 = lo1 + ((hi1 - lo1) >> 1);
-        const uint32_t p0 = primary(m0 < a.age_sat ? m0 : a.age_sat), p1 = primary(m1 < a.age_sat ? m1 : a.age_sat);
-        if (lo0 < hi0) { if (PF ? p0 > Tp : p0 <= Tp) hi0 = m0; else lo0 = m0 + 1; }
-        if (lo1 < hi1) { if (PF ? p1 >= Tp : p1 < Tp) hi1 = m1; else lo1 = m1 + 1; }
+    // prefetch: it rises: n_le = first age with primary > Tp, n_lt = first with primary >= Tp.  Both found in step, without a
+    // branch: the binary search over 2,263 ages is the longest chain between the scan's first load and its first compare.
+    uint32_t n_le = 0, n_lt = 0;
+    for (uint32_t step = CS_GTAB_MAX; step > 0; step >>= 1) {
+        const uint32_t a0 = n_le + step - 1u, a1 = n_lt + step - 1u;
+        const uint32_t p0 = primary(min(a0, a.age_sat)), p1 = primary(min(a1, a.age_sat));
+        n_le += (a0 <= a.age_sat && (PF ? p0 <= Tp : p0 > Tp)) ? step : 0u;
+        n_lt += (a1 <= a.age_sat && (PF ? p1 < Tp : p1 >= Tp)) ? step : 0u;
     }
-    const uint32_t n_le = lo0, n_lt = lo1;
     if (!PF) {
         if (n_le > a.age_sat) return 0u;                                   // no age qualifies
         // la <= now - n_lt for the ages below T's score; at T's score (n_le <= age < n_lt) also la <= Ts.  Age 0 stands for
@@ -215,11 +217,12 @@ __global__ void __launch_bounds__(SEL_THREADS, 2) cs_sel_fast_kernel(SelArgs a, 
     cs_release_successor();
     // Before waiting for the predecessor grid: what depends only on the context's constants.
     Tables T;
-    const size_t table_words = ((size_t)(a.A + a.gtab_len) * 4 + (size_t)a.A * 2 + 15) / 16 * 4;
+    const size_t table_words = ((size_t)(a.A + a.gtab_len + 1) * 4 + (size_t)a.A * 2 + 15) / 16 * 4;
     uint32_t *queues = (uint32_t *)smem + table_words;
     uint32_t *s_cut = queues + (size_t)(SEL_THREADS / 32) * (FQ_CAP + STAGE_CAP * 3) + 4;     // after queues and staging
     load_tables_static(a, ws, smem, T);
-    if (threadIdx.x == 0) s_above = 0;
+    T.anchor += 2;                                  // (one entry more than the table: the saturated factor, for the cuts)
+    if (threadIdx.x == 0) { s_above = 0; T.gtab[a.gtab_len] = T.g_sat; }
     CS_STAMP(ws, CS_PS_SCAN_SETUP + PS, blockIdx.x == 0 && threadIdx.x == 0);
     cs_wait_for_predecessor();
     CS_STAMP(ws, CS_PS_SCAN_WAITED + PS, blockIdx.x == 0 && threadIdx.x == 0);
@@ -1063,7 +1066,7 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage)
     const cs_workspace &ws = *c.ws;
     if (stage == 0) {
         // tables, per-warp queues, per-warp candidate staging, cuts
-        const size_t sm_fast = (sm + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
+        const size_t sm_fast = (sm + 4 + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
                                (size_t)A * sizeof(uint32_t);
         if (c.prefetch) cs_launch_chained(cs_sel_fast_kernel<true>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);
         else cs_launch_chained(cs_sel_fast_kernel<false>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);

@@ -238,6 +238,7 @@ int cs_destroy(cs_ctx *ctx)
     if (!ctx) return CS_EINVAL;
     if (ctx->ev_fork) cudaEventDestroy(ctx->ev_fork);
     if (ctx->ev_join) cudaEventDestroy(ctx->ev_join);
+    cs_drop_select_graphs(ctx);
     if (ctx->ev_sel_fork) cudaEventDestroy(ctx->ev_sel_fork);
     for (int j = 0; j < 2; ++j) {
         if (ctx->ev_sel_join[j]) cudaEventDestroy(ctx->ev_sel_join[j]);

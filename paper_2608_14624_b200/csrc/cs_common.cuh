@@ -135,6 +135,15 @@ struct cs_workspace {
                           // 0.8 us on separate sectors; separate 128-byte lines are no faster and cost the readers more)
 };
 
+// Six-launch selects side by side as one graph: node[job][launch] gets its arguments anew on every call.
+#define CS_SELECT_STAGES 6
+struct cs_select_graph {
+    cudaGraph_t graph;
+    cudaGraphExec_t exec;
+    cudaGraphNode_t node[3][CS_SELECT_STAGES];
+    uint32_t asked, refused;       // calls that wanted it (up to 2); 1: it could not be built
+};
+
 struct cs_ctx {
     cs_params p;
     cs_workspace ws;
@@ -159,6 +168,7 @@ struct cs_ctx {
     cudaStream_t sel_stream[2];          // the second and third select of a step run here, beside the first
     cudaEvent_t ev_sel_fork, ev_sel_join[2];
     int concurrent_selects;              // the per-select scratch regions are full size
+    cs_select_graph sel_graph[8];        // selects side by side, by the lists wanted (bit q: select q)
     // copy-engine path of the mover (cs_set_mover_staging): caller-owned device ring split into four sub-buffers
     // (two per direction, double-buffered), two streams of the context for the two DMA directions, and the events
     // that order packing / copying / scattering
@@ -191,6 +201,7 @@ int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int p
 int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uint32_t k_victims, uint32_t k_prefetch,
                           uint32_t *gpu_victims, uint32_t *n_gpu, uint32_t *host_victims, uint32_t *n_host,
                           uint32_t *prefetch_ids, uint32_t *n_prefetch, cudaStream_t s);
+void cs_drop_select_graphs(cs_ctx *ctx);
 int cs_launch_select_clusters(cs_ctx *ctx, int n_jobs, const void *sel_args, const uint32_t *prefetch,
                               uint32_t *const *ids_out, uint32_t *const *n_out, cudaStream_t s);
 int cs_launch_select_cluster(cs_ctx *ctx, const void *sel_args, const cs_workspace *ws, int prefetch, uint32_t *ids_out,

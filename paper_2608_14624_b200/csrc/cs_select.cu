@@ -29,6 +29,10 @@
 // depend on the order in which atomics were served.
 #include "cs_common.cuh"
 
+#include <algorithm>
+#include <initializer_list>
+#include <tuple>
+
 #include "cs_select_common.cuh"
 
 // ---------------------------------------------------------------------------------------------
@@ -1036,13 +1040,48 @@ static int scan_opt_in(cs_ctx *ctx)
 }
 
 // One select through the grid-wide kernels, on the scratch of one job: the arguments, and its six launches one by one, so
-// that several selects' launches can be issued in turn.
-#define SELECT_STAGES 6
+// that the launches of several selects can be issued in turn or become the nodes of a graph.
+#define SELECT_STAGES CS_SELECT_STAGES
 struct SelectChain {
     SelArgs a;
     const cs_workspace *ws;
     uint32_t prefetch, *ids_out, *n_out;
     cudaStream_t s;
+};
+
+// Where a stage goes: launched on the chain's stream, or the node of (job, stage) in a graph of selects side by side --
+// added behind the node of the stage before it, or given new arguments.
+struct StageSink {
+    cs_select_graph *g;            // NULL: launched
+    int job, stage;
+    template <class... KArgs, class... Args>
+    cudaError_t put(cudaStream_t s, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) const
+    {
+        if (!g) {
+            cs_launch_chained(kernel, grid, block, smem, s, args...);
+            return cudaGetLastError();
+        }
+        std::tuple<KArgs...> held((KArgs)args...);
+        return std::apply([&](auto &...arg) { return put_node((void *)kernel, grid, block, smem, {(void *)&arg...}); }, held);
+    }
+    cudaError_t put_node(void *kernel, dim3 grid, dim3 block, size_t smem, std::initializer_list<void *> args) const
+    {
+        void *params[16];
+        std::copy(args.begin(), args.end(), params);
+        cudaGraphNodeParams np = {};
+        np.type = cudaGraphNodeTypeKernel;
+        np.kernel.func = kernel;
+        np.kernel.gridDim = grid;
+        np.kernel.blockDim = block;
+        np.kernel.sharedMemBytes = (unsigned)smem;
+        np.kernel.kernelParams = params;
+        if (g->exec) return cudaGraphExecNodeSetParams(g->exec, g->node[job][stage], &np);
+        cudaGraphEdgeData edge = {};
+        edge.type = cudaGraphDependencyTypeProgrammatic;
+        edge.from_port = cudaGraphKernelNodePortProgrammatic;
+        return cudaGraphAddNode_v2(&g->node[job][stage], g->graph, stage ? &g->node[job][stage - 1] : nullptr, stage ? &edge : nullptr,
+                                   stage ? 1 : 0, &np);
+    }
 };
 
 static void prepare_chain(const cs_ctx *ctx, int job, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier, uint32_t k,
@@ -1061,20 +1100,22 @@ static void prepare_chain(const cs_ctx *ctx, int job, const cs_block_index *idx,
     cs_fill_sel_bins(ctx, c.a, prefetch);
 }
 
-static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage)
+static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage, cs_select_graph *graph = nullptr, int job = 0)
 {
     const uint32_t grid = cs_scan_grid(ctx, c.a.n, SEL_THREADS * GRP), grid_c = cs_scan_grid(ctx, c.a.n, 1024), A = ctx->p.n_agents;
     const size_t sm = cs_table_smem(ctx);
     const cs_workspace &ws = *c.ws;
+    const StageSink to = {graph, job, stage};
+    cudaError_t e = cudaSuccess;
     if (stage == 0) {
         // tables, per-warp queues, per-warp candidate staging, cuts
         const size_t sm_fast = (sm + 4 + 15) / 16 * 16 + (size_t)(SEL_THREADS / 32) * (FQ_CAP * sizeof(uint32_t) + STAGE_CAP * 12) + 32 +
                                (size_t)A * sizeof(uint32_t);
-        if (c.prefetch) cs_launch_chained(cs_sel_fast_kernel<true>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);
-        else cs_launch_chained(cs_sel_fast_kernel<false>, grid, SEL_THREADS, sm_fast, c.s, c.a, ws);
+        if (c.prefetch) e = to.put(c.s, cs_sel_fast_kernel<true>, grid, SEL_THREADS, sm_fast, c.a, ws);
+        else e = to.put(c.s, cs_sel_fast_kernel<false>, grid, SEL_THREADS, sm_fast, c.a, ws);
     } else if (stage == 1) {
-        if (c.prefetch) cs_launch_chained(cs_sel_hist_kernel<true>, grid, SEL_THREADS, sm, c.s, c.a, ws);
-        else cs_launch_chained(cs_sel_hist_kernel<false>, grid, SEL_THREADS, sm, c.s, c.a, ws);
+        if (c.prefetch) e = to.put(c.s, cs_sel_hist_kernel<true>, grid, SEL_THREADS, sm, c.a, ws);
+        else e = to.put(c.s, cs_sel_hist_kernel<false>, grid, SEL_THREADS, sm, c.a, ws);
     } else if (stage == 2) {
         // large indexes: the collect pass prefilters by age limits (one look-up per entry instead of the full key)
         const uint32_t n_cls = c.a.ntok ? ctx->p.block_tokens : 1u;
@@ -1083,17 +1124,19 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage)
             c.a.use_age_limits = 1;
             sm_collect += (size_t)A * n_cls * sizeof(uint32_t);
         }
-        if (c.prefetch) cs_launch_chained(cs_sel_collect_kernel<true>, grid, SEL_THREADS, sm_collect, c.s, c.a, ws);
-        else cs_launch_chained(cs_sel_collect_kernel<false>, grid, SEL_THREADS, sm_collect, c.s, c.a, ws);
+        if (c.prefetch) e = to.put(c.s, cs_sel_collect_kernel<true>, grid, SEL_THREADS, sm_collect, c.a, ws);
+        else e = to.put(c.s, cs_sel_collect_kernel<false>, grid, SEL_THREADS, sm_collect, c.a, ws);
     } else if (stage == 3) {
-        cs_launch_chained(cs_sel_sample_kernel, SAMPLE_CTAS, 512, 0, c.s, c.a, ws, c.ids_out, c.n_out);
+        e = to.put(c.s, cs_sel_sample_kernel, SAMPLE_CTAS, 512, 0, c.a, ws, c.ids_out, c.n_out);
     } else if (stage == 4) {
-        cs_launch_chained(cs_sel_place_kernel, grid_c, 256, 0, c.s, ws, c.a.max_blocks, c.a.region_cap_max, c.a.kind);
+        e = to.put(c.s, cs_sel_place_kernel, grid_c, 256, 0, ws, c.a.max_blocks, c.a.region_cap_max, c.a.kind);
     } else {
-        cs_launch_chained(cs_sel_finish_kernel, CS_BUCKETS, FINISH_THREADS, 0, c.s, ws, c.a.k, c.a.max_blocks, c.a.region_cap_max, c.a.kind,
+        e = to.put(c.s, cs_sel_finish_kernel, CS_BUCKETS, FINISH_THREADS, 0, ws, c.a.k, c.a.max_blocks, c.a.region_cap_max, c.a.kind,
                           c.a.hint_slot, c.ids_out);
     }
-    return cs_check_launch(ctx);
+    ctx->n_launches++;
+    if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
+    return CS_OK;
 }
 
 // One select: the single-launch cluster kernel where it applies, else the chain.
@@ -1117,11 +1160,76 @@ int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int p
     return launch_select_job(ctx, 0, idx, now, prefetch, tier, k, ids_out, n_out, s);
 }
 
+// The chains of selects side by side as one graph launch: true when it was launched or failed (*rc tells), false when it has
+// to be done launch by launch.  A launch costs the host 2.5 us, so that the 12 or 18 of a step (33 and 50 us) took longer than
+// their kernels (34 us for two lists of 1,000,000 entries); a node's new arguments take 0.2 us and the graph's launch 2 us.
+// A single select stays six launches: its kernels take longer than issuing them (29 and 16 us), and its first launch
+// overlaps the work before it on the stream, which a graph's does not.  Every argument is set anew on every call.
+//
+// The graph of a mix of lists is built (150 to 220 us) when a context is asked for that mix a second time: one that is asked
+// once, or never has large indexes, does not pay for it.
+static void drop_select_graph(cs_select_graph &g)
+{
+    if (g.exec) (void)cudaGraphExecDestroy(g.exec);
+    if (g.graph) (void)cudaGraphDestroy(g.graph);
+    g.exec = nullptr;
+    g.graph = nullptr;
+}
+
+void cs_drop_select_graphs(cs_ctx *ctx)
+{
+    for (cs_select_graph &g : ctx->sel_graph) drop_select_graph(g);
+}
+
+static bool build_select_graph(cs_ctx *ctx, cs_select_graph &g, int n_jobs, SelectChain *chain)
+{
+    // (another thread may be capturing a stream of its own, which is nothing that these calls disturb)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    const uint64_t launches = ctx->n_launches;
+    bool ok = cudaGraphCreate(&g.graph, 0) == cudaSuccess;
+    for (int i = 0; i < n_jobs; ++i)
+        for (int stage = 0; stage < SELECT_STAGES && ok; ++stage) ok = launch_stage(ctx, chain[i], stage, &g, i) == CS_OK;
+    ok = ok && cudaGraphInstantiate(&g.exec, g.graph, 0) == cudaSuccess;
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    ctx->n_launches = launches;
+    if (!ok) {                                       // (no room for it: the launches stay single)
+        (void)cudaGetLastError();
+        drop_select_graph(g);
+    }
+    return ok;
+}
+
+static bool graph_of_selects(cs_ctx *ctx, uint32_t mask, int n_jobs, SelectChain *chain, cudaStream_t s, int *rc)
+{
+    cs_select_graph &g = ctx->sel_graph[mask];
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (st != cudaStreamCaptureStatusNone) return false;
+    if (!g.exec) {
+        if (g.asked < 2) ++g.asked;
+        if (g.asked != 2 || g.refused) return false;
+        g.refused = !build_select_graph(ctx, g, n_jobs, chain);
+        if (g.refused) return false;
+    }
+    *rc = CS_OK;
+    for (int i = 0; i < n_jobs && *rc == CS_OK; ++i)
+        for (int stage = 0; stage < SELECT_STAGES && *rc == CS_OK; ++stage) *rc = launch_stage(ctx, chain[i], stage, &g, i);
+    if (*rc == CS_OK) {
+        const cudaError_t e = cudaGraphLaunch(g.exec, s);
+        if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; *rc = CS_ECUDA; }
+    }
+    return true;
+}
+
 // The selects of a step side by side.  Select q (0 GPU-tier victims, 1 host-tier victims, 2 prefetch candidates)
 // is skipped when its count pointer is NULL.  Where the single-launch select applies they are the clusters of ONE
-// launch; otherwise every select is a chain of grid-wide kernels, the first on the caller's stream and the others
-// on the context's two extra streams, forked from and joined back into the caller's stream with events (each has
-// its own select state, histogram and candidate / sort regions).  Indexes beyond CS_CONCURRENT_MAX_BLOCKS entries
+// launch; otherwise every select is a chain of grid-wide kernels (each has its own select state, histogram and candidate /
+// sort regions), the chains side by side in one graph or, on the first call and while the caller's stream is being captured, the first on that
+// stream and the others on the context's two extra streams, forked from and joined back into it with events.  Indexes beyond CS_CONCURRENT_MAX_BLOCKS entries
 // have no private regions of that size: their selects run one after the other.
 int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uint32_t k_victims, uint32_t k_prefetch,
                           uint32_t *gpu_victims, uint32_t *n_gpu, uint32_t *host_victims, uint32_t *n_host,
@@ -1161,16 +1269,19 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
         }
         return rc;
     }
-    // The chains' launches are issued in turn: issued one chain after the other, the second one started 20 us (six
-    // launches) after the first and both ended that much later.
     if ((rc = scan_opt_in(ctx)) != CS_OK) return rc;
     SelectChain chain[3];
-    cudaError_t e = cudaEventRecord(ctx->ev_sel_fork, s);
-    for (int i = 0; i < n_jobs && e == cudaSuccess; ++i) {
+    for (int i = 0; i < n_jobs; ++i) {
         const int q = jobs[i];
         prepare_chain(ctx, i, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], i ? ctx->sel_stream[i - 1] : s, chain[i]);
-        if (i) e = cudaStreamWaitEvent(ctx->sel_stream[i - 1], ctx->ev_sel_fork, 0);
     }
+    uint32_t mask = 0;
+    for (int i = 0; i < n_jobs; ++i) mask |= 1u << jobs[i];
+    if (graph_of_selects(ctx, mask, n_jobs, chain, s, &rc)) return rc;
+    // Launched one by one: in turn, because issued one chain after the other the second one started 20 us (six launches) after
+    // the first and both ended that much later.
+    cudaError_t e = cudaEventRecord(ctx->ev_sel_fork, s);
+    for (int i = 1; i < n_jobs && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(ctx->sel_stream[i - 1], ctx->ev_sel_fork, 0);
     for (int stage = 0; stage < SELECT_STAGES && e == cudaSuccess; ++stage)
         for (int i = 0; i < n_jobs && rc == CS_OK; ++i) rc = launch_stage(ctx, chain[i], stage);
     for (int i = 1; i < n_jobs && e == cudaSuccess; ++i) {

@@ -955,6 +955,46 @@ def test_select_step_side_by_side_is_stable_over_many_calls():
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("wanted", [(0, 1), (0, 2), (1, 2), (0, 1, 2)])
+def test_select_step_graph_takes_new_arguments(wanted):
+    """Large selects side by side, for every two or three of the lists: indexes of different sizes, other list lengths and
+    other buffers on every call, on the null stream, a stream and inside a stream capture.  Each list must equal, bit for
+    bit, the one that the same select gives alone."""
+    cfg = synth.CONFIGS["meta1m"]
+    c, _ = warm_state(cfg, 800, 400_000, r_min=0.02)
+    alone, _ = warm_state(cfg, 800, 400_000, r_min=0.02)
+    indexes = [cs.DeviceIndex.from_host(synth.make_block_index(cfg, n=n, tier="random"), DEV) for n in (262_145, 400_000, 300_011)]
+    side = torch.cuda.Stream()
+    empty = lambda m: torch.full((m,), 7, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    for rep in range(9):
+        d, now, k = indexes[rep % 3], 100_000 + 5 * rep, (1, 700, 9_000, 40)[rep % 4]
+        bufs = [(empty(max(k, 4)), empty(4)) if q in wanted else (None, None) for q in range(3)]
+        torch.cuda.synchronize()
+        call = lambda: c.select_step(d, now, k, k, *bufs[0], *bufs[1], *bufs[2])
+        n0 = c.launch_count()
+        if rep % 3 == 0:
+            call()
+        elif rep % 3 == 1:
+            with torch.cuda.stream(side):
+                call()
+        else:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                call()
+            g.replay()
+        assert c.launch_count() - n0 == 6 * len(wanted)
+        torch.cuda.synchronize()
+        for q in wanted:
+            ids, cnt = empty(max(k, 4)), empty(4)
+            if q == 2:
+                alone.select_prefetch(d, now, k, ids, cnt)
+            else:
+                alone.select_victims(d, now, q, k, ids, cnt)
+            assert int(cnt[0]) == int(bufs[q][1][0]) and torch.equal(ids, bufs[q][0]), (rep, q)
+    assert c.get_status() == 0
+
+
 # ---- randomised small configurations ------------------------------------------------------------------------
 @pytest.mark.parametrize("case", range(48))
 def test_random_small_configurations(case):

@@ -58,6 +58,9 @@ size_t cs_layout_workspace(const cs_params *p, uint32_t gtab_len, void *base, cs
     TAKE(P, float, A * A);
     TAKE(amax, uint16_t, A);
     TAKE(adjT, uint32_t, A * W);
+    TAKE(qsum, unsigned long long, A);
+    TAKE(cta_base, unsigned long long, (A + 7) / 8);
+    TAKE(cta_hc, double, (A + 7) / 8);
     TAKE(hops, uint16_t, A);
     TAKE(fsurv, float, A);
     TAKE(hops_tmp, uint16_t, A);

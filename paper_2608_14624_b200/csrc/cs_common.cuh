@@ -78,6 +78,7 @@ struct cs_scalars {
     float R;                // Eq. 2
     uint32_t gate;          // Eq. 11: R >= r_min
     uint32_t n_transitions; // sum of all counts
+    uint32_t refresh_ticket;       // CTAs of a refresh of many agents that are done; 0 between calls
     uint32_t gtab_monotone; // the recency table covers every unsaturated age and never increases with age
     uint32_t status_read;   // cs_get_status(): the value swapped out of `status`
     uint32_t val_le, val_elig, val_ticket;   // cs_validate_selection(): keys at or below the last one, eligible entries, ticket
@@ -116,6 +117,9 @@ struct cs_workspace {
     uint16_t *amax;       // [A]
     uint32_t *adjT;       // [W][A] transpose of the Eq. 7 adjacency, W = ceil(A/32): bit b of word w of column v = an edge from
                           // agent 32 w + b to agent v (word by word, so that one thread per agent reads it coalesced)
+    unsigned long long *qsum;      // [A] a refresh of many agents: column sums of Eq. 2 in the making, 0 between calls
+    unsigned long long *cta_base;  // and what its CTAs leave for the last one (RfShared::base, hc)
+    double *cta_hc;
     uint16_t *hops;       // [A]
     float *fsurv;         // [A] p~ + delta for the cached source
     uint16_t *hops_tmp;   // [A] same, for cs_score_blocks() with explicit sources

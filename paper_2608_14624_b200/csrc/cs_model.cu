@@ -310,19 +310,17 @@ __device__ T cs_block_sum(T v, T *s_red)
 // ---------------------------------------------------------------------------------------------
 // The refresh of everything derived from the counts: Eq. 3 in canonical fp32 (one rounding per operation, no FMA), every
 // row's arg-max, adjacency bits (Eq. 7) and entropy term, then Eq. 2 / Eq. 11 over all rows and the cached search of
-// Eq. 7 / 8.  One thread-block cluster, one warp per row.
+// Eq. 7 / 8.
 //
 // A refresh is a chain of dependent steps on a few hundred kilobytes, so what counts is the number of trips to L2 and of
 // barriers between its first load and its last store -- and, once a row has a warp of its own, the instructions an SM has to
 // issue for its rows (about a thousand per row: 32 rows per CTA were slower than 16).  Every warp fetches its row, the row's
 // sum and -- redundantly per CTA -- the batch of events at once, and what has to meet (column sums of Eq. 2, the transposed
-// adjacency matrix for the search, entropies, arg-max) does so through distributed shared memory:
+// adjacency matrix for the search, entropies, arg-max) does so in one of them:
 //   * up to 32 agents: one CTA;
-//   * up to 256 (KW = 8): 8 or 16 rows per CTA, every CTA adds up its rows' share of all columns and adds it to the first CTA's;
-//   * more (KW = 32): a column's sum and its row of the transposed matrix belong to one CTA of the cluster, which the others
-//     reach with atomics (only entries that have a count, or an edge); that CTA passes the sums on to the first one and the
-//     matrix rows to global memory, from where the first CTA fetches them.
-// The first CTA then runs the search on some of its warps and the sums of Eq. 2 on others.
+//   * up to 256: one thread-block cluster, 8 or 16 rows per CTA, meeting in the first CTA's shared memory;
+//   * more: the whole GPU, 8 rows per CTA, meeting in global memory (cs_refresh_wide_kernel).
+// That CTA then runs the search on some of its warps and the sums of Eq. 2 on others.
 //
 // Rows are sparse: entries with a zero count all have the same P = eps / n_i, so one logarithm stands for all of them, the
 // entries with a count are compacted (one per lane), and their share of the column sums is one number per row with the
@@ -334,95 +332,55 @@ __device__ T cs_block_sum(T v, T *s_red)
 // global atomics and, above 256 agents, a search that pushed from global memory:
 //   agents / events      4/1   12/5   12/256   30/8   64/64   128/64   256/64   256/256   400/64   1,024/64
 //   before               7.7   8.4    14.8     8.7    12.3    11.9     10.9     21.9      35.8     93.4
-//   now                  4.6   4.8    7.5      6.0    6.8     7.2      9.2      11.1      17.2     35.2
+//   now                  4.0   4.4    6.9      5.4    6.4     6.7      8.5      10.3      13.9     17.8
 // ---------------------------------------------------------------------------------------------
-#define RF_OWN_COLS 128u                                  // KW = 32: columns a CTA owns in a cluster of 8 (64 in one of 16)
+#define RW_ROWS 8u                                        // rows per CTA of the kernel for many agents
+#define RW_COLS 256u                                      // columns of a row per warp
 template <int KW> struct RfShape {                        // KW: words of an adjacency row the kernel is compiled for
     static constexpr uint32_t COLS = KW * 32u;
-    static constexpr uint32_t ROWS = KW == 8 ? 16u : 32u;                            // most rows a CTA works on at a time, one per warp
-    static constexpr uint32_t CTAS = KW == 1 ? 1u : 16u;                             // most CTAs of the cluster
+    static constexpr uint32_t WARPS = KW == 8 ? 16u : 32u;                           // most warps of a CTA
+    static constexpr uint32_t CTAS = KW == 1 ? 1u : (KW == 8 ? 16u : 4u);                    // most partial sums: CTAs, or warps of the last one
     static constexpr int CHUNK = KW < 8 ? KW : 8;                                    // words of a row in registers at a time
-    static constexpr uint32_t T_COLS = KW == 32 ? RF_OWN_COLS : COLS;                // columns of the transposed matrix kept here
 };
 template <int KW> struct RfShared {
-    unsigned long long q[RfShape<KW>::COLS];                        // column sums: this CTA's, in the first one everybody's
+    unsigned long long q[RfShape<KW>::COLS];                        // column sums: this CTA's, in the end everybody's
     unsigned long long base[RfShape<KW>::CTAS];                     // what every column gets from a CTA's zero-count entries
     double hc[RfShape<KW>::CTAS];                                   // sum over a CTA's rows of n_i * (row entropy)
     double row_hc[32];
     unsigned long long row_base[32];
     double red[32];
-    unsigned long long own_q[KW == 32 ? RF_OWN_COLS : 1];
     __align__(16) uint32_t ev_chain[OBS_FUSED_MAX];                 // the batch: chain of event e (read as 16-byte words),
     uint16_t ev_agent[OBS_FUSED_MAX];                               // its agent (CS_AGENT_NONE: skipped),
     uint16_t ev_prev[OBS_FUSED_MAX];                                // and the agent it follows when that is a counted transition
-    uint32_t adj[KW == 32 ? 1 : RfShape<KW>::COLS];                 // bit i: this CTA's row i has an edge to the column
-    uint32_t adjT[KW][RfShape<KW>::T_COLS];                         // transposed matrix, word by word
-    uint32_t nz_v[RfShape<KW>::ROWS][32];                           // per warp: entries of its row that have a count, gathered
-    uint16_t nz_j[RfShape<KW>::ROWS][32];                           // so that every lane works on one
-    uint16_t amax[RfShape<KW>::COLS];
+    uint32_t adj[RfShape<KW>::COLS];                                // bit i: this CTA's row i has an edge to the column
+    uint32_t adjT[KW == 32 ? 1 : KW][KW == 32 ? 1 : RfShape<KW>::COLS];              // transposed matrix, word by word
+    uint32_t nz_v[RfShape<KW>::WARPS][32];                          // per warp: entries of its row that have a count, gathered
+    uint16_t nz_j[RfShape<KW>::WARPS][32];                          // so that every lane works on one
+    uint16_t amax[KW == 32 ? 1 : RfShape<KW>::COLS];
+    float best_v[KW == 32 ? 32 : 1];                                // KW = 32: what the four warps of a row found
+    uint32_t best_i[KW == 32 ? 32 : 1];
     uint32_t front[2 * PULL_MAX_WORDS];
     int last_live;
+    bool last_cta;
     uint8_t succ[OBS_FUSED_MAX];                                    // 1: a later live event of the batch has the same chain
 };
+static_assert(CS_MAX_AGENTS <= 4u * RW_COLS && CS_MAX_AGENTS <= 128u * RW_ROWS, "four warps per row, four warps of CTA sums");
 static_assert(sizeof(RfShared<8>) <= 48 * 1024 && sizeof(RfShared<32>) <= 48 * 1024, "the default shared-memory limit");
 static_assert(offsetof(RfShared<1>, ev_chain) % 16 == 0 && offsetof(RfShared<8>, ev_chain) % 16 == 0 &&
               offsetof(RfShared<32>, ev_chain) % 16 == 0, "read as 16-byte words");
 
 __device__ __forceinline__ double cs_xlogx(double x) { return x * log(x); }
 
-// blockDim.x / 32 rows at a time per CTA: 8, 16 or 32, all of them (KW = 1), 8 or 16 (KW = 8), 32 (KW = 32).
-template <int KW>
-__global__ void __launch_bounds__(RfShape<KW>::ROWS * 32u)
-cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
-                  uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
-                  const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
-                  const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
+// A small batch of events is applied by the refresh, by every CTA to its own rows: each CTA finds every event's predecessor (in
+// the batch, else the chain's current agent) as cs_observe_kernel does.  What is shared -- cur[], the last agent, the totals and
+// the counters -- is written by rf_finish(), in the one CTA that runs it, after every CTA has read it.
+template <class Shared>
+__device__ __forceinline__ void rf_read_batch(Shared &sm, const cs_workspace &ws, uint32_t A, uint32_t n_chains,
+                                              const uint32_t *__restrict__ ev_chain_in, const uint16_t *__restrict__ ev_agent_in,
+                                              const uint8_t *__restrict__ ev_flags, uint32_t n_events, bool first, bool count_skipped,
+                                              uint32_t &n_new, uint32_t &n_skipped)
 {
-    constexpr uint32_t COLS = RfShape<KW>::COLS, T_COLS = RfShape<KW>::T_COLS, ADJ = KW == 32 ? 1u : COLS, OWN = KW == 32 ? RF_OWN_COLS : 1u;
-    constexpr int CHUNK = RfShape<KW>::CHUNK;
-    __shared__ RfShared<KW> sm;
-    cg::cluster_group cluster = cg::this_cluster();
-    const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_threads = blockDim.x, rows = n_threads >> 5;
-    const uint32_t own = KW == 32 ? COLS / CL : 1u;           // columns per CTA
-    CS_STAMP(ws, CS_PS_REFRESH_ENTRY, blockIdx.x == 0 && tid == 0);
-    if (KW == 32) {
-        for (uint32_t x = tid; x < KW * T_COLS; x += n_threads) (&sm.adjT[0][0])[x] = 0;
-        if (tid < OWN) sm.own_q[tid] = 0;
-    } else if (tid < COLS) {
-        sm.q[tid] = 0;
-        sm.adj[tid % ADJ] = 0;
-#pragma unroll
-        for (int w = 0; w < KW; ++w) sm.adjT[w][tid % T_COLS] = 0;         // (bits past the last row)
-    }
-    if (tid == 0) sm.last_live = -1;
-    if (tid < OBS_FUSED_MAX) sm.succ[tid] = 0;
-    if (tid < 2 * PULL_MAX_WORDS) sm.front[tid] = 0;
-    if (KW > 1) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");             // waited for below
-    cs_wait_for_predecessor();
-    CS_STAMP(ws, CS_PS_REFRESH_WAITED, blockIdx.x == 0 && tid == 0);
-    cs_release_successor();
-
-    // ---- everything that depends on nothing, in one trip ---------------------------------------------------------
-    if (n_events_dev) n_events = min(n_events, cs_ld_cg_pinned(n_events_dev));
-    uint32_t c[CHUNK], n_i = 0;
-    auto load_chunk = [&](uint32_t row, uint32_t col0) {
-#pragma unroll
-        for (int k = 0; k < CHUNK; ++k) {
-            const uint32_t j = col0 + lane + 32u * k;
-            c[k] = 0;
-            if (row < A && j < A) c[k] = cs_ld_cg_pinned(ws.C + row * A + j);
-        }
-        if (col0 == 0) n_i = cs_ld_cg_pinned(ws.rowsum + (row < A ? row : 0u));
-    };
-    load_chunk(rank * rows + warp, 0u);
-    uint32_t n_total = cs_ld_cg_pinned(&ws.sc->n_transitions);
-    uint32_t la = cs_ld_cg_pinned(&ws.sc->last_agent);
-
-    // ---- a small batch of events is applied here, by every CTA to its own rows: each CTA finds every event's predecessor
-    // (in the batch, else the chain's current agent) as cs_observe_kernel does.  What is shared -- cur[], the last agent,
-    // the totals and the counters -- is written by the first CTA behind the cluster barrier, after every CTA has read it.
-    uint32_t n_new = 0, n_skipped = 0;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (n_events) {
         uint32_t ch = OBS_NO_CHAIN, a = CS_AGENT_NONE, before = CS_AGENT_NONE;
         if (tid < n_events) {
@@ -432,7 +390,7 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
             uint32_t bad = 0;
             if (!warm && a >= A) bad |= CS_ST_BAD_AGENT;
             if (!warm && ch >= n_chains) bad |= CS_ST_BAD_CHAIN;
-            if (bad && rank == 0) atomicOr(&ws.sc->status, bad);
+            if (bad && first) atomicOr(&ws.sc->status, bad);
             if (warm || bad) { a = CS_AGENT_NONE; ch = OBS_NO_CHAIN; }
             else before = cs_ld_cg_pinned(ws.cur + ch);        // in flight during the search below
         }
@@ -465,172 +423,20 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
         }
         if (tid < OBS_FUSED_MAX) sm.ev_prev[tid] = (uint16_t)(counted ? before : CS_AGENT_NONE);
         n_new = (uint32_t)__syncthreads_count(counted);
-        if (rank == 0) n_skipped = (uint32_t)__syncthreads_count(tid < n_events && !live);
+        if (count_skipped) n_skipped = (uint32_t)__syncthreads_count(tid < n_events && !live);
     } else {
         __syncthreads();
     }
-    n_total += n_new;
-    if (KW > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");                // every CTA has started and cleared its sums
+}
 
-    auto add_edge = [&](uint32_t i, uint32_t j) {
-        if (KW == 32) atomicOr(cluster.map_shared_rank(&sm.adjT[0][0], j / own) + (i >> 5) * T_COLS + j % own, 1u << (i & 31u));
-        else atomicOr(&sm.adj[j % ADJ], 1u << warp);                                       // (KW < 32: one row per warp)
-    };
-    // ---- this warp's rows (more than one only where the cluster holds fewer than A of them) -------------------------
-    double row_hc = 0.0;
-    unsigned long long row_base = 0;
-    const double inv_total = n_total ? 1.0 / (double)n_total : 0.0;
-    for (uint32_t i = rank * rows + warp; i < A; i += CL * rows) {
-        if (i >= CL * rows) load_chunk(i, 0u);
-        uint32_t n_add = 0;
-        if (n_new)
-            for (uint32_t e0 = 0; e0 < n_events; e0 += 32u)
-                n_add += __popc(__ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i));
-        n_i += n_add;
-        const bool write = every_row || n_add;
-        const double pi_fix = (double)n_i * inv_total * 1152921504606846976.0;      // pi_i * 2^60
-        const float den = __fadd_rn((float)n_i, __fmul_rn((float)A, eps));
-        const float p0 = __fdiv_rn(__fadd_rn(0.0f, eps), den);              // every entry with a zero count
-        const bool p0_edge = p0 >= tau;
-        const long long base_fix = __double2ll_rn(pi_fix * (double)p0);
-        float bestv = -1.0f;
-        uint32_t besti = 0xFFFFFFFFu, n_nz = 0, n_list = 0;
-        double h = 0.0;
-        uint32_t *lv = sm.nz_v[warp];
-        uint16_t *lj = sm.nz_j[warp];
-        // up to 32 entries that have a count, one per lane; in the lane behind them, the last time, those that have none
-        auto take = [&](uint32_t n, bool last) {
-            __syncwarp();
-            const bool mine = lane < n;
-            const uint32_t v = mine ? lv[lane] : 0u, j = mine ? lj[lane] : 0u;
-            const float p = mine ? __fdiv_rn(__fadd_rn((float)v, eps), den) : p0;
-            const double pd = (double)p, t = cs_xlogx(pd);
-            if (mine) {
-                if (write) {
-                    ws.P[(size_t)i * A + j] = p;
-                    ws.C[(size_t)i * A + j] = v;
-                }
-                if (p > bestv) { bestv = p; besti = j; }                       // strict: the lowest j among equals stays
-                if (p >= tau) add_edge(i, j);
-                if (n_i) {
-                    unsigned long long *q = KW == 32 ? cluster.map_shared_rank(sm.own_q, j / own) + j % own : &sm.q[j];
-                    atomicAdd(q, (unsigned long long)(__double2ll_rn(pi_fix * pd) - base_fix));
-                }
-                h += t;
-            } else if (last && lane == n) {
-                h += (double)(A - n_nz) * t;
-            }
-            __syncwarp();
-        };
-        for (uint32_t col0 = 0; col0 < A; col0 += 32u * CHUNK) {
-            if (col0) load_chunk(i, col0);
-            if (n_add) {
-                for (uint32_t e0 = 0; e0 < n_events; e0 += 32u) {
-                    uint32_t hits = __ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i);
-                    for (; hits; hits &= hits - 1u) {
-                        const uint32_t j = sm.ev_agent[e0 + __ffs(hits) - 1] - col0;
-#pragma unroll
-                        for (int k = 0; k < CHUNK; ++k)
-                            if (j == lane + 32u * k) ++c[k];
-                    }
-                }
-            }
-            // the entries that have a count go to the list, a word of 32 columns at a time; the rest is uniform
-            uint32_t words = 0;
-#pragma unroll
-            for (int k = 0; k < CHUNK; ++k) {
-                if (col0 + 32u * k >= A) break;
-                const uint32_t j = col0 + lane + 32u * k;
-                if (__any_sync(0xFFFFFFFFu, c[k] != 0u)) words |= 1u << k;
-                if (write && j < A) ws.P[(size_t)i * A + j] = p0;
-                if (p0_edge && j < A && c[k] == 0u) add_edge(i, j);
-            }
-            __syncwarp();                                                      // (an entry's P is written again by another lane)
-#pragma unroll 1
-            for (; words; words &= words - 1u) {
-                const uint32_t k = __ffs(words) - 1u;
-                uint32_t v = c[0];
-#pragma unroll
-                for (int u = 1; u < CHUNK; ++u) v = k == (uint32_t)u ? c[u] : v;
-                const uint32_t b = __ballot_sync(0xFFFFFFFFu, v != 0u), n_b = __popc(b);
-                if (n_list + n_b > 32u) { take(n_list, false); n_list = 0; }
-                if (v) {
-                    const uint32_t at = n_list + __popc(b & ((1u << lane) - 1u));
-                    lv[at] = v;
-                    lj[at] = (uint16_t)(col0 + lane + 32u * k);
-                }
-                n_list += n_b;
-                n_nz += n_b;
-            }
-        }
-#pragma unroll 1
-        do {                                                                   // (twice when the list is full: the last lane has to be free)
-            take(n_list, n_list < 32u);
-            n_list = n_list == 32u ? 0u : 33u;
-        } while (n_list != 33u);
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-            const float v = __shfl_xor_sync(0xFFFFFFFFu, bestv, d);
-            const uint32_t x = __shfl_xor_sync(0xFFFFFFFFu, besti, d);
-            if (v > bestv || (v == bestv && x < besti)) { bestv = v; besti = x; }
-            h += __shfl_xor_sync(0xFFFFFFFFu, h, d);
-        }
-        const uint32_t am = bestv > p0 ? besti : 0u;          // no entry above the zero-count ones: all are equal, the lowest wins
-        if (lane == 0) {
-            if (write) ws.amax[i] = (uint16_t)am;
-            if (n_add) ws.rowsum[i] = n_i;
-            cluster.map_shared_rank(sm.amax, 0)[i] = (uint16_t)am;
-        }
-        row_hc += (double)n_i * h;
-        row_base += n_i ? (unsigned long long)base_fix : 0ull;
-    }
-    if (lane == 0) { sm.row_hc[warp] = row_hc; sm.row_base[warp] = row_base; }
-    __syncthreads();
-    CS_STAMP(ws, CS_PS_REFRESH_ROWS_DONE, blockIdx.x == 0 && tid == 0);
-
-    // ---- everything meets in the first CTA -----------------------------------------------------------------------------
-    RfShared<KW> *first = cluster.map_shared_rank(&sm, 0);
-    if (KW != 32 && tid < A) {
-        const uint32_t bits = sm.adj[tid % ADJ];
-        if (KW == 8 && rank && sm.q[tid % COLS]) atomicAdd(&first->q[tid % COLS], sm.q[tid % COLS]);
-        // this CTA's rows are 32, 16 or 8 bits of a word
-        if (rows == 32u) first->adjT[0][tid % T_COLS] = bits;
-        else if (rows == 16u) ((uint16_t *)&first->adjT[rank / 2u % KW][tid % T_COLS])[rank & 1u] = (uint16_t)bits;
-        else ((uint8_t *)&first->adjT[rank / 4u % KW][tid % T_COLS])[rank & 3u] = (uint8_t)bits;
-    }
-    if (warp == rows - 1u) {
-        double s = lane < rows ? sm.row_hc[lane] : 0.0;
-        unsigned long long b = lane < rows ? sm.row_base[lane] : 0ull;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-            s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
-            b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
-        }
-        if (lane == 0) { first->hc[rank] = s; first->base[rank] = b; }
-    }
-    if (KW > 1) cluster.sync();
-    else __syncthreads();
-    if (KW == 32) {
-        // owned columns are complete: sums to the first CTA, rows of the transposed matrix to global memory
-        for (uint32_t x = tid; x < own * W; x += n_threads) {
-            const uint32_t w = x / own, jc = x - w * own, j = rank * own + jc;
-            if (j < A) ws.adjT[(size_t)w * A + j] = (&sm.adjT[0][0])[w * T_COLS + jc];
-        }
-        if (tid < own) first->q[(rank * own + tid) % COLS] = sm.own_q[tid % OWN];
-        cluster.sync();
-    }
-    if (rank != 0) return;
-    CS_STAMP(ws, CS_PS_REFRESH_LAST_CTA, tid == 0);
-    uint32_t row[KW];                                         // thread v: the predecessors of agent v
-#pragma unroll
-    for (int w = 0; w < KW; ++w) {
-        row[w] = 0;
-        if ((uint32_t)w < W && tid < A) {
-            row[w] = KW == 32 ? cs_ld_cg_pinned(ws.adjT + (size_t)w * A + tid) : sm.adjT[w][tid % T_COLS];
-            if (KW != 32) ws.adjT[(size_t)w * A + tid] = row[w];          // for searches from explicit sources
-        }
-    }
-
+// What the one CTA does that has everything: the batch's effect on the shared state, the sums of Eq. 2 and the search.  row:
+// thread v's words of the transposed adjacency matrix; base[] and hc[] have n_parts numbers each.
+template <int KW>
+__device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &ws, const uint32_t (&row)[KW], uint32_t A, uint32_t W,
+                                          uint32_t n_parts, uint32_t n_events, uint32_t n_new, uint32_t n_skipped, uint32_t n_total,
+                                          uint32_t la, float r_min, uint32_t e_max, float delta, uint32_t all_chains, uint32_t n_chains)
+{
+    const uint32_t tid = threadIdx.x, lane = tid & 31, n_threads = blockDim.x;
     if (n_events) {
         // the batch's effect on what all CTAs share
         const uint32_t a = tid < n_events ? sm.ev_agent[tid] : CS_AGENT_NONE;
@@ -660,8 +466,8 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
         const uint32_t j = tid - sum0;
         double Hm = 0.0;
         if (n_total && j < A) {
-            unsigned long long qf = sm.q[j % COLS];
-            for (uint32_t r = 0; r < CL; ++r) qf += sm.base[r];
+            unsigned long long qf = sm.q[j % RfShape<KW>::COLS];
+            for (uint32_t r = 0; r < n_parts; ++r) qf += sm.base[r];
             const double q = (double)qf * (1.0 / 1152921504606846976.0);
             if (q > 0.0) Hm = -cs_xlogx(q);
         }
@@ -669,16 +475,22 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
         for (int d = 16; d > 0; d >>= 1) Hm += __shfl_xor_sync(0xFFFFFFFFu, Hm, d);
         if (lane == 0) sm.red[j >> 5] = Hm;
         asm volatile("bar.sync 2, %0;" ::"r"(W * 32u) : "memory");
+        if (KW == 32 && j < 32u) {                             // (32 additions one after the other would be a microsecond)
+            double v = j < W ? sm.red[j] : 0.0;
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+            if (j == 0) sm.red[0] = v;
+        }
         if (j == 0) {
             double Hc = 0.0, Hs = 0.0;
-            for (uint32_t r = 0; r < CL; ++r) Hc -= sm.hc[r];
-            for (uint32_t w = 0; w < W; ++w) Hs += sm.red[w];
+            for (uint32_t r = 0; r < n_parts; ++r) Hc -= sm.hc[r];
+            for (uint32_t w = 0; w < (KW == 32 ? 1u : W); ++w) Hs += sm.red[w];
             double R = 0.0;
             if (n_total && Hs > 0.0) R = 1.0 - Hc / (double)n_total / Hs;
             const float Rf = (float)R;
             ws.sc->R = Rf;
             ws.sc->gate = (Rf >= r_min) ? 1u : 0u;
-            ws.sc->a_star = la < A ? (uint32_t)sm.amax[la] : 0xFFFFFFFFu;    // Eq. 10, for the prefetch ranking
+            ws.sc->a_star = la < A ? (uint32_t)(KW == 32 ? cs_ld_cg_pinned(ws.amax + la) : sm.amax[KW == 32 ? 0u : la]) : 0xFFFFFFFFu;    // Eq. 10, for the prefetch ranking
         }
         CS_STAMP(ws, CS_PS_REFRESH_SUMS_DONE, j == 0);
     }
@@ -690,6 +502,379 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
         cs_bfs_pull<KW>(row, A, W, sm.front, ws.hops, ws.fsurv, e_max, delta);
     }
     CS_STAMP(ws, CS_PS_REFRESH_END, tid == 0);
+}
+
+// blockDim.x / 32 rows per CTA, a warp each: 8, 16 or 32 in the one CTA (KW = 1), 8 or 16 in each of up to 16 (KW = 8).
+template <int KW>
+__global__ void __launch_bounds__(RfShape<KW>::WARPS * 32u)
+cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
+                  uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
+                  const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
+                  const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
+{
+    constexpr uint32_t COLS = RfShape<KW>::COLS;
+    constexpr int CHUNK = RfShape<KW>::CHUNK;
+    static_assert(CHUNK == KW, "a row is one chunk");
+    __shared__ RfShared<KW> sm;
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_threads = blockDim.x, rows = n_threads >> 5;
+    CS_STAMP(ws, CS_PS_REFRESH_ENTRY, blockIdx.x == 0 && tid == 0);
+    if (tid < COLS) {
+        sm.q[tid] = 0;
+        sm.adj[tid] = 0;
+#pragma unroll
+        for (int w = 0; w < KW; ++w) sm.adjT[w][tid] = 0;                  // (bits past the last row)
+    }
+    if (tid == 0) sm.last_live = -1;
+    if (tid < OBS_FUSED_MAX) sm.succ[tid] = 0;
+    if (tid < 2 * PULL_MAX_WORDS) sm.front[tid] = 0;
+    if (KW > 1) asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");             // waited for below
+    cs_wait_for_predecessor();
+    CS_STAMP(ws, CS_PS_REFRESH_WAITED, blockIdx.x == 0 && tid == 0);
+    cs_release_successor();
+
+    // ---- everything that depends on nothing, in one trip ---------------------------------------------------------
+    if (n_events_dev) n_events = min(n_events, cs_ld_cg_pinned(n_events_dev));
+    const uint32_t i = rank * rows + warp;                     // this warp's row
+    uint32_t c[CHUNK];
+#pragma unroll
+    for (int k = 0; k < CHUNK; ++k) {
+        const uint32_t j = lane + 32u * k;
+        c[k] = 0;
+        if (i < A && j < A) c[k] = cs_ld_cg_pinned(ws.C + i * A + j);
+    }
+    uint32_t n_i = cs_ld_cg_pinned(ws.rowsum + (i < A ? i : 0u));
+    uint32_t n_total = cs_ld_cg_pinned(&ws.sc->n_transitions);
+    const uint32_t la = cs_ld_cg_pinned(&ws.sc->last_agent);
+    uint32_t n_new = 0, n_skipped = 0;
+    rf_read_batch(sm, ws, A, n_chains, ev_chain_in, ev_agent_in, ev_flags, n_events, rank == 0, rank == 0, n_new, n_skipped);
+    n_total += n_new;
+    if (KW > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");                // every CTA has started and cleared its sums
+
+    double row_hc = 0.0;
+    unsigned long long row_base = 0;
+    const double inv_total = n_total ? 1.0 / (double)n_total : 0.0;
+    if (i < A) {                                               // (whole warps)
+        uint32_t n_add = 0;
+        if (n_new)
+            for (uint32_t e0 = 0; e0 < n_events; e0 += 32u) {
+                uint32_t hits = __ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i);
+                n_add += __popc(hits);
+                for (; hits; hits &= hits - 1u) {
+                    const uint32_t j = sm.ev_agent[e0 + __ffs(hits) - 1];
+#pragma unroll
+                    for (int k = 0; k < CHUNK; ++k)
+                        if (j == lane + 32u * k) ++c[k];
+                }
+            }
+        n_i += n_add;
+        const bool write = every_row || n_add;
+        const double pi_fix = (double)n_i * inv_total * 1152921504606846976.0;      // pi_i * 2^60
+        const float den = __fadd_rn((float)n_i, __fmul_rn((float)A, eps));
+        const float p0 = __fdiv_rn(__fadd_rn(0.0f, eps), den);              // every entry with a zero count
+        const bool p0_edge = p0 >= tau;
+        const long long base_fix = __double2ll_rn(pi_fix * (double)p0);
+        float bestv = -1.0f;
+        uint32_t besti = 0xFFFFFFFFu, n_nz = 0, n_list = 0;
+        double h = 0.0;
+        uint32_t *lv = sm.nz_v[warp];
+        uint16_t *lj = sm.nz_j[warp];
+        // up to 32 entries that have a count, one per lane; in the lane behind them, the last time, those that have none
+        auto take = [&](uint32_t n, bool last) {
+            __syncwarp();
+            const bool mine = lane < n;
+            const uint32_t v = mine ? lv[lane] : 0u, j = mine ? lj[lane] : 0u;
+            const float p = mine ? __fdiv_rn(__fadd_rn((float)v, eps), den) : p0;
+            const double pd = (double)p, t = cs_xlogx(pd);
+            if (mine) {
+                if (write) {
+                    ws.P[(size_t)i * A + j] = p;
+                    ws.C[(size_t)i * A + j] = v;
+                }
+                if (p > bestv) { bestv = p; besti = j; }                       // strict: the lowest j among equals stays
+                if (p >= tau) atomicOr(&sm.adj[j], 1u << warp);
+                if (n_i) atomicAdd(&sm.q[j], (unsigned long long)(__double2ll_rn(pi_fix * pd) - base_fix));
+                h += t;
+            } else if (last && lane == n) {
+                h += (double)(A - n_nz) * t;
+            }
+            __syncwarp();
+        };
+        // the entries that have a count go to the list, a word of 32 columns at a time; the rest is uniform
+        uint32_t words = 0;
+#pragma unroll
+        for (int k = 0; k < CHUNK; ++k) {
+            if (32u * k >= A) break;
+            const uint32_t j = lane + 32u * k;
+            if (__any_sync(0xFFFFFFFFu, c[k] != 0u)) words |= 1u << k;
+            if (write && j < A) ws.P[(size_t)i * A + j] = p0;
+            if (p0_edge && j < A && c[k] == 0u) atomicOr(&sm.adj[j], 1u << warp);
+        }
+        __syncwarp();                                                          // (an entry's P is written again by another lane)
+#pragma unroll 1
+        for (; words; words &= words - 1u) {
+            const uint32_t k = __ffs(words) - 1u;
+            uint32_t v = c[0];
+#pragma unroll
+            for (int u = 1; u < CHUNK; ++u) v = k == (uint32_t)u ? c[u] : v;
+            const uint32_t b = __ballot_sync(0xFFFFFFFFu, v != 0u), n_b = __popc(b);
+            if (n_list + n_b > 32u) { take(n_list, false); n_list = 0; }
+            if (v) {
+                const uint32_t at = n_list + __popc(b & ((1u << lane) - 1u));
+                lv[at] = v;
+                lj[at] = (uint16_t)(lane + 32u * k);
+            }
+            n_list += n_b;
+            n_nz += n_b;
+        }
+#pragma unroll 1
+        do {                                                                   // (twice when the list is full: the last lane has to be free)
+            take(n_list, n_list < 32u);
+            n_list = n_list == 32u ? 0u : 33u;
+        } while (n_list != 33u);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const float v = __shfl_xor_sync(0xFFFFFFFFu, bestv, d);
+            const uint32_t x = __shfl_xor_sync(0xFFFFFFFFu, besti, d);
+            if (v > bestv || (v == bestv && x < besti)) { bestv = v; besti = x; }
+            h += __shfl_xor_sync(0xFFFFFFFFu, h, d);
+        }
+        const uint32_t am = bestv > p0 ? besti : 0u;          // no entry above the zero-count ones: all are equal, the lowest wins
+        if (lane == 0) {
+            if (write) ws.amax[i] = (uint16_t)am;
+            if (n_add) ws.rowsum[i] = n_i;
+            cluster.map_shared_rank(sm.amax, 0)[i] = (uint16_t)am;
+        }
+        row_hc = (double)n_i * h;
+        row_base = n_i ? (unsigned long long)base_fix : 0ull;
+    }
+    if (lane == 0) { sm.row_hc[warp] = row_hc; sm.row_base[warp] = row_base; }
+    __syncthreads();
+    CS_STAMP(ws, CS_PS_REFRESH_ROWS_DONE, blockIdx.x == 0 && tid == 0);
+
+    // ---- everything meets in the first CTA -----------------------------------------------------------------------------
+    RfShared<KW> *first = cluster.map_shared_rank(&sm, 0);
+    if (tid < A) {
+        const uint32_t bits = sm.adj[tid];
+        if (KW == 8 && rank && sm.q[tid]) atomicAdd(&first->q[tid], sm.q[tid]);
+        // this CTA's rows are 32, 16 or 8 bits of a word
+        if (rows == 32u) first->adjT[0][tid] = bits;
+        else if (rows == 16u) ((uint16_t *)&first->adjT[rank / 2u % KW][tid])[rank & 1u] = (uint16_t)bits;
+        else ((uint8_t *)&first->adjT[rank / 4u % KW][tid])[rank & 3u] = (uint8_t)bits;
+    }
+    if (warp == rows - 1u) {
+        double s = lane < rows ? sm.row_hc[lane] : 0.0;
+        unsigned long long b = lane < rows ? sm.row_base[lane] : 0ull;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+            b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
+        }
+        if (lane == 0) { first->hc[rank] = s; first->base[rank] = b; }
+    }
+    if (KW > 1) cluster.sync();
+    else __syncthreads();
+    if (rank != 0) return;
+    CS_STAMP(ws, CS_PS_REFRESH_LAST_CTA, tid == 0);
+    uint32_t row[KW];                                         // thread v: the predecessors of agent v
+#pragma unroll
+    for (int w = 0; w < KW; ++w) {
+        row[w] = 0;
+        if ((uint32_t)w < W && tid < A) {
+            row[w] = sm.adjT[w][tid];
+            ws.adjT[(size_t)w * A + tid] = row[w];            // for searches from explicit sources
+        }
+    }
+
+    rf_finish<KW>(sm, ws, row, A, W, CL, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, all_chains, n_chains);
+}
+
+// The same for many agents (KW = 32): bound by the scan of the rows -- a megabyte and more of counts -- so they are spread over the
+// whole GPU, 8 rows per CTA, a row's 256-column quarters by a warp each.  Column sums meet in global memory (atomics, only of
+// columns some row of the CTA has a count in); 8 rows are one byte of every word of the transposed matrix, which their CTA stores
+// whole (words of rows past the last one stay zero, as the workspace is made).  The CTA that is done last does the rest.
+// A cluster of 16 CTAs with 32 or 64 rows each took 17.1 us for 400 agents, 28.8 for 600 and 35.3 for 1,024, most of it for
+// issuing four chunks per row; this takes 13.9, 15.6 and 17.8: 5.8 the rows, 2.7 the meeting, 4 the sums, up to 4.5 the search.
+// (For 256 agents or fewer the meeting in global memory costs more than it gives: 13.3 us instead of 8.5.)
+__global__ void __launch_bounds__(1024)
+cs_refresh_wide_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
+                       uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
+                       const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
+                       const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
+{
+    constexpr int CHUNK = RfShape<32>::CHUNK;
+    static_assert(CHUNK * 32u == RW_COLS, "a warp's columns are one chunk");
+    __shared__ RfShared<32> sm;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    CS_STAMP(ws, CS_PS_REFRESH_ENTRY, blockIdx.x == 0 && tid == 0);
+    sm.q[tid] = 0;
+    sm.adj[tid] = 0;
+    if (tid == 0) sm.last_live = -1;
+    if (tid < OBS_FUSED_MAX) sm.succ[tid] = 0;
+    if (tid < 2 * PULL_MAX_WORDS) sm.front[tid] = 0;
+    cs_wait_for_predecessor();
+    CS_STAMP(ws, CS_PS_REFRESH_WAITED, blockIdx.x == 0 && tid == 0);
+    cs_release_successor();
+
+    if (n_events_dev) n_events = min(n_events, cs_ld_cg_pinned(n_events_dev));
+    const uint32_t r = warp >> 2, i = blockIdx.x * RW_ROWS + r, col0 = (warp & 3u) * RW_COLS;
+    const uint32_t n_cols = i < A && col0 < A ? min(A - col0, RW_COLS) : 0u;
+    uint32_t c[CHUNK];
+#pragma unroll
+    for (int k = 0; k < CHUNK; ++k) {
+        const uint32_t j = lane + 32u * k;
+        c[k] = 0;
+        if (j < n_cols) c[k] = cs_ld_cg_pinned(ws.C + (size_t)i * A + col0 + j);
+    }
+    uint32_t n_i = cs_ld_cg_pinned(ws.rowsum + (i < A ? i : 0u));
+    uint32_t n_total = cs_ld_cg_pinned(&ws.sc->n_transitions);
+    const uint32_t la = cs_ld_cg_pinned(&ws.sc->last_agent);
+    uint32_t n_new = 0, n_skipped = 0;
+    rf_read_batch(sm, ws, A, n_chains, ev_chain_in, ev_agent_in, ev_flags, n_events, blockIdx.x == 0, true, n_new, n_skipped);
+    n_total += n_new;
+    const double inv_total = n_total ? 1.0 / (double)n_total : 0.0;
+
+    float bestv = -1.0f;
+    uint32_t besti = 0xFFFFFFFFu, n_add = 0;
+    double h = 0.0;
+    long long base_fix = 0;
+    float p0 = 0.0f;
+    if (n_cols) {                                              // (whole warps)
+        if (n_new)
+            for (uint32_t e0 = 0; e0 < n_events; e0 += 32u) {
+                uint32_t hits = __ballot_sync(0xFFFFFFFFu, e0 + lane < n_events && sm.ev_prev[e0 + lane] == i);
+                n_add += __popc(hits);
+                for (; hits; hits &= hits - 1u) {
+                    const uint32_t j = sm.ev_agent[e0 + __ffs(hits) - 1] - col0;
+#pragma unroll
+                    for (int k = 0; k < CHUNK; ++k)
+                        if (j == lane + 32u * k) ++c[k];
+                }
+            }
+        n_i += n_add;
+        const bool write = every_row || n_add;
+        const double pi_fix = (double)n_i * inv_total * 1152921504606846976.0;      // pi_i * 2^60
+        const float den = __fadd_rn((float)n_i, __fmul_rn((float)A, eps));
+        p0 = __fdiv_rn(__fadd_rn(0.0f, eps), den);                                  // every entry with a zero count
+        const bool p0_edge = p0 >= tau;
+        base_fix = __double2ll_rn(pi_fix * (double)p0);
+        uint32_t n_nz = 0, n_list = 0, words = 0;
+        uint32_t *lv = sm.nz_v[warp];
+        uint16_t *lj = sm.nz_j[warp];
+        auto take = [&](uint32_t n, bool last) {               // (as in cs_refresh_kernel)
+            __syncwarp();
+            const bool mine = lane < n;
+            const uint32_t v = mine ? lv[lane] : 0u, j = mine ? lj[lane] : 0u;
+            const float p = mine ? __fdiv_rn(__fadd_rn((float)v, eps), den) : p0;
+            const double pd = (double)p, t = cs_xlogx(pd);
+            if (mine) {
+                if (write) {
+                    ws.P[(size_t)i * A + j] = p;
+                    ws.C[(size_t)i * A + j] = v;
+                }
+                if (p > bestv) { bestv = p; besti = j; }                       // strict: the lowest j among equals stays
+                if (p >= tau) atomicOr(&sm.adj[j], 1u << r);
+                if (n_i) atomicAdd(&sm.q[j], (unsigned long long)(__double2ll_rn(pi_fix * pd) - base_fix));
+                h += t;
+            } else if (last && lane == n) {
+                h += (double)(n_cols - n_nz) * t;
+            }
+            __syncwarp();
+        };
+#pragma unroll
+        for (int k = 0; k < CHUNK; ++k) {
+            const uint32_t j = lane + 32u * k;
+            if (__any_sync(0xFFFFFFFFu, c[k] != 0u)) words |= 1u << k;
+            if (write && j < n_cols) ws.P[(size_t)i * A + col0 + j] = p0;
+            if (p0_edge && j < n_cols && c[k] == 0u) atomicOr(&sm.adj[col0 + j], 1u << r);
+        }
+        __syncwarp();                                                          // (an entry's P is written again by another lane)
+#pragma unroll 1
+        for (; words; words &= words - 1u) {
+            const uint32_t k = __ffs(words) - 1u;
+            uint32_t v = c[0];
+#pragma unroll
+            for (int u = 1; u < CHUNK; ++u) v = k == (uint32_t)u ? c[u] : v;
+            const uint32_t b = __ballot_sync(0xFFFFFFFFu, v != 0u), n_b = __popc(b);
+            if (n_list + n_b > 32u) { take(n_list, false); n_list = 0; }
+            if (v) {
+                const uint32_t at = n_list + __popc(b & ((1u << lane) - 1u));
+                lv[at] = v;
+                lj[at] = (uint16_t)(col0 + lane + 32u * k);
+            }
+            n_list += n_b;
+            n_nz += n_b;
+        }
+#pragma unroll 1
+        do {                                                                   // (twice when the list is full: the last lane has to be free)
+            take(n_list, n_list < 32u);
+            n_list = n_list == 32u ? 0u : 33u;
+        } while (n_list != 33u);
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            const float v = __shfl_xor_sync(0xFFFFFFFFu, bestv, d);
+            const uint32_t x = __shfl_xor_sync(0xFFFFFFFFu, besti, d);
+            if (v > bestv || (v == bestv && x < besti)) { bestv = v; besti = x; }
+            h += __shfl_xor_sync(0xFFFFFFFFu, h, d);
+        }
+    }
+    if (lane == 0) {
+        sm.best_v[warp] = bestv;
+        sm.best_i[warp] = besti;
+        sm.row_hc[warp] = (double)n_i * h;
+        sm.row_base[warp] = (warp & 3u) == 0 && n_i ? (unsigned long long)base_fix : 0ull;
+    }
+    __syncthreads();
+    CS_STAMP(ws, CS_PS_REFRESH_ROWS_DONE, blockIdx.x == 0 && tid == 0);
+    if ((warp & 3u) == 0 && lane == 0 && n_cols) {             // the row's arg-max, from its four quarters in order
+        for (uint32_t u = 1; u < 4u; ++u)
+            if (sm.best_v[warp + u] > bestv) { bestv = sm.best_v[warp + u]; besti = sm.best_i[warp + u]; }
+        if (every_row || n_add) ws.amax[i] = (uint16_t)(bestv > p0 ? besti : 0u);   // (all entries equal: the lowest wins)
+        if (n_add) ws.rowsum[i] = n_i;
+    }
+    if (tid < A) {
+        if (sm.q[tid]) atomicAdd(ws.qsum + tid, sm.q[tid]);
+        ((uint8_t *)(ws.adjT + (size_t)(blockIdx.x / 4u) * A + tid))[blockIdx.x & 3u] = (uint8_t)sm.adj[tid];
+    }
+    if (warp == 31u) {
+        double s = sm.row_hc[lane];
+        unsigned long long b = sm.row_base[lane];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+            b += __shfl_xor_sync(0xFFFFFFFFu, b, d);
+        }
+        if (lane == 0) { ws.cta_hc[blockIdx.x] = s; ws.cta_base[blockIdx.x] = b; }
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) sm.last_cta = atomicAdd(&ws.sc->refresh_ticket, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!sm.last_cta) return;
+    __threadfence();
+    CS_STAMP(ws, CS_PS_REFRESH_LAST_CTA, tid == 0);
+    const unsigned long long q = tid < A ? cs_ld_cg_pinned(ws.qsum + tid) : 0ull;
+    unsigned long long base = tid < gridDim.x ? cs_ld_cg_pinned(ws.cta_base + tid) : 0ull;
+    double hc = tid < gridDim.x ? __longlong_as_double((long long)cs_ld_cg_pinned((const unsigned long long *)ws.cta_hc + tid)) : 0.0;
+    uint32_t row[32];                                         // thread v: the predecessors of agent v
+#pragma unroll
+    for (int w = 0; w < 32; ++w) row[w] = ((uint32_t)w < W && tid < A) ? cs_ld_cg_pinned(ws.adjT + (size_t)w * A + tid) : 0u;
+    if (warp < 4u) {                                          // (at most 128 CTAs; one number per warp is left to add up)
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) {
+            hc += __shfl_xor_sync(0xFFFFFFFFu, hc, d);
+            base += __shfl_xor_sync(0xFFFFFFFFu, base, d);
+        }
+        if (lane == 0) { sm.hc[warp] = hc; sm.base[warp] = base; }
+    }
+    if (tid < A) {
+        sm.q[tid] = q;
+        ws.qsum[tid] = 0;
+    }
+    if (tid == 0) ws.sc->refresh_ticket = 0;
+    __syncthreads();
+    rf_finish<32>(sm, ws, row, A, W, 4u, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, all_chains, n_chains);
 }
 
 // BFS + Eq. 8 from explicit sources into the temporary tables (cs_score_blocks with sources): one thread per agent.
@@ -934,10 +1119,8 @@ static int obs_cluster_limit(int device)
 }
 static int refresh_cluster_limit(int device)
 {
-    static ClusterLimit l8, l32;                              // both kernels need their opt-in to clusters beyond 8
-    const int a = l8.get(device, cs_refresh_kernel<8>, RfShape<8>::CTAS, RfShape<8>::ROWS * 32);
-    const int b = l32.get(device, cs_refresh_kernel<32>, RfShape<32>::CTAS, RfShape<32>::ROWS * 32);
-    return a < b ? a : b;
+    static ClusterLimit limit;
+    return limit.get(device, cs_refresh_kernel<8>, RfShape<8>::CTAS, RfShape<8>::WARPS * 32);
 }
 
 int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent, const uint8_t *evflags,
@@ -961,22 +1144,22 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
     const uint32_t n_fused = fused ? n_events : 0u;
     const uint32_t *n_fused_dev = fused ? ctx->step_n_events_dev : nullptr;
     const uint32_t every_row = n_fused ? 0u : 1u;            // a row keeps its P when no event of a small batch starts at it
-    const auto launch = [&](auto kernel, uint32_t cl, uint32_t rows) {
-        cs_launch_chained_clusters(kernel, cl, cl, rows * 32u, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min, p.e_max,
-                                   p.delta, all_chains, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
+    const auto launch = [&](auto kernel, uint32_t ctas, uint32_t cluster, uint32_t warps) {
+        cs_launch_chained_clusters(kernel, ctas, cluster, warps * 32u, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min,
+                                   p.e_max, p.delta, all_chains, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
     };
     const uint32_t most = (uint32_t)refresh_cluster_limit(ctx->device);
     if (p.n_agents <= 32) {
         // one CTA of as many warps as there are rows, at least one thread per event of a small batch
-        launch(cs_refresh_kernel<1>, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));
-    } else if (p.n_agents <= RfShape<8>::COLS && p.n_agents <= RfShape<8>::ROWS * most) {
+        launch(cs_refresh_kernel<1>, 1u, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));
+    } else if (p.n_agents <= RfShape<8>::COLS && p.n_agents <= RfShape<8>::WARPS * most) {
         // few rows per CTA (64 agents: 8.8 us with 32, 7.4 with 16, 6.8 with 8), as far as the cluster goes
-        const uint32_t rows = p.n_agents <= 8u * most ? 8u : RfShape<8>::ROWS;
+        const uint32_t rows = p.n_agents <= 8u * most ? 8u : RfShape<8>::WARPS;
         uint32_t cl = 2;
         while (cl * rows < p.n_agents) cl <<= 1;
-        launch(cs_refresh_kernel<8>, cl, rows);
+        launch(cs_refresh_kernel<8>, cl, cl, rows);
     } else {
-        launch(cs_refresh_kernel<32>, most >= 16u ? 16u : 8u, 32u);
+        launch(cs_refresh_wide_kernel, (p.n_agents + RW_ROWS - 1u) / RW_ROWS, 0u, 32u);
     }
     return cs_check_launch(ctx);
 }

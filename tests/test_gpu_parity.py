@@ -709,8 +709,8 @@ def test_small_batches_ride_with_the_refresh(A, chains, all_sources):
 @pytest.mark.parametrize("A", [1, 2, 31, 32, 33, 64, 65, 129, 255, 256, 257, 511, 513, 1024])
 @pytest.mark.parametrize("tau,eps", [(0.05, 0.01), (0.001, 0.5)])
 def test_refresh_shapes(A, tau, eps):
-    """The learner refresh at the edges of its forms (one CTA up to 32 agents, clusters of several sizes up to 256, columns
-    owned by CTAs above, more than one row per warp above 512), with batches that touch one row, many rows and none, rows
+    """The learner refresh at the edges of its forms (one CTA up to 32 agents, clusters of several sizes up to 256, the
+    whole GPU above, a row by two to four warps), with batches that touch one row, many rows and none, rows
     with more counts than a warp has lanes, cold rows whose every entry is an edge (a small tau), and a state imported in
     between."""
     cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=5)

@@ -203,6 +203,25 @@ def test_select_ordering_routes(n, ks, ties):
     assert run_selects(c, o, idx, 100_000, ks, tiers=(0,) if n > 100_000 else (0, 1)) == 0
 
 
+@pytest.mark.parametrize("eligible,k", [(1, 1), (255, 255), (257, 20), (1024, 1024), (1025, 1), (2047, 2047), (2048, 700), (2048, 2048),
+                                        (2049, 3000), (2049, 1300)])
+@pytest.mark.parametrize("tied", [False, True])
+def test_few_candidates_of_the_launch_chain(eligible, k, tied):
+    """Where the multi-launch select changes from ranking all candidates against each other (at most 2,048) to a sample and buckets,
+    and around the steps of the ranking, with distinct keys and with all entries of an agent tied down to the id."""
+    cfg = synth.CONFIGS["llama8b"]
+    n = 20_000
+    c, o = warm_state(cfg, 1000, n, r_min=0.02)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    idx.flags[:] = 0
+    idx.flags[synth.rng_for(cfg, 31).permutation(n)[:eligible]] = synth.FLAG_VALID
+    idx.ref_count[:] = 0
+    if tied:
+        idx.last_access[:] = 90_000
+    for now in (100_000, 100_003):
+        assert run_selects(c, o, idx, now, (k,), tiers=(0,)) == 0
+
+
 def test_select_gate_closed_and_cold_start():
     cfg = synth.CONFIGS["tiny"]
     idx = synth.make_block_index(cfg, n=2560)

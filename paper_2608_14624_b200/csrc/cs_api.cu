@@ -289,13 +289,15 @@ int cs_score_blocks(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const 
     if (idx->n_blocks && (!scores_out || !aligned16(scores_out))) return CS_EINVAL;
     if (sources && !aligned16(sources)) return CS_EINVAL;
     const float *fsurv = ctx->fsurv_override ? ctx->fsurv_override : ctx->ws.fsurv;
+    if (sources && cs_score_searches(ctx, idx->n_blocks))
+        return cs_launch_score(ctx, idx, now, fsurv, sources, n_sources, scores_out, (cudaStream_t)stream);
     if (sources) {
         rc = cs_launch_survival(ctx, sources, n_sources, (cudaStream_t)stream);
         if (rc != CS_OK) return rc;
         fsurv = ctx->ws.fsurv_tmp;
     }
     if (idx->n_blocks == 0) return CS_OK;
-    return cs_launch_score(ctx, idx, now, fsurv, scores_out, (cudaStream_t)stream);
+    return cs_launch_score(ctx, idx, now, fsurv, nullptr, 0, scores_out, (cudaStream_t)stream);
 }
 
 static int select_common(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier,

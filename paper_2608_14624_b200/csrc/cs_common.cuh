@@ -198,8 +198,9 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
 int cs_launch_import(cs_ctx *ctx, const uint32_t *C_in, const uint16_t *cur_in, uint32_t last_agent, cudaStream_t s);
 int cs_launch_survival(cs_ctx *ctx, const uint16_t *sources, uint32_t n_sources, cudaStream_t s);
 int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_out, float *fsurv_out, cudaStream_t s);
-int cs_launch_score(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const float *fsurv,
-                    float *scores_out, cudaStream_t s);
+bool cs_score_searches(const cs_ctx *ctx, uint32_t n_blocks);     // a score of so many entries can search from sources itself
+int cs_launch_score(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const float *fsurv, const uint16_t *sources,
+                    uint32_t n_sources, float *scores_out, cudaStream_t s);
 int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier,
                      uint32_t k, uint32_t *ids_out, uint32_t *n_out, cudaStream_t s);
 int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uint32_t k_victims, uint32_t k_prefetch,
@@ -240,6 +241,14 @@ static inline int cs_check_launch(cs_ctx *ctx)
 }
 
 #ifdef __CUDACC__
+// Eq. 8 with the floor of Eq. 9 added: p~ + delta of an agent so many hops away.
+__device__ __forceinline__ float cs_survival_of(uint32_t hops, uint32_t e_max, float delta)
+{
+    const uint32_t m = hops < e_max ? hops : e_max;                        // CS_HOP_NONE > e_max by construction
+    const double ptilde = 1.0 - (double)m / (double)e_max;
+    return (float)(ptilde + (double)delta);
+}
+
 // Programmatic dependent launch.  The chains of small kernels (observe -> normalise; histogram -> collect ->
 // bucket -> scatter -> rank) are bound by launch latency, so each kernel of a chain is launched with the
 // programmatic-serialisation attribute: its launch overlaps the tail of its predecessor, and its first

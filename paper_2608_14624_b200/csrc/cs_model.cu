@@ -284,10 +284,8 @@ __device__ __forceinline__ void cs_bfs_pull(const uint32_t (&row)[KW], uint32_t 
         }
     }
     if (v < A) {
-        const uint32_t m = my_hops < e_max ? my_hops : e_max;             // CS_HOP_NONE > e_max by construction
-        const double ptilde = 1.0 - (double)m / (double)e_max;
         hops[v] = (uint16_t)my_hops;
-        fsurv[v] = (float)(ptilde + (double)delta);
+        fsurv[v] = cs_survival_of(my_hops, e_max, delta);
     }
 }
 

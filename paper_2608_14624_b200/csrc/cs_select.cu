@@ -83,7 +83,16 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_score_kernel(SelArgs a, cs_wor
 
 #define SCORE_SMALL_THREADS 256u
 #define SCORE_SMALL_MAX (1u << 17)
-__global__ void __launch_bounds__(SCORE_SMALL_THREADS) cs_score_small_kernel(SelArgs a, cs_workspace ws, float *__restrict__ out)
+// SEARCH (at most 32 agents): the search of Eq. 7 / 8 from the sources as well, by every warp for itself -- lane v holds agent v's
+// predecessors and in the end its survival factor -- so that it needs no launch of its own.  80,000 entries, 12 agents, three sources:
+// 9.6 us per call in two launches, which is what the host takes to issue them, 7.2 in one.  (More agents: the search wants a CTA.)
+struct ScoreSources {
+    const uint16_t *list;
+    uint32_t n, e_max;
+};
+template <bool SEARCH>
+__global__ void __launch_bounds__(SCORE_SMALL_THREADS)
+cs_score_small_kernel(SelArgs a, cs_workspace ws, float *__restrict__ out, ScoreSources src)
 {
     Tables T;
     T.gtab = ws.gtab;
@@ -91,11 +100,30 @@ __global__ void __launch_bounds__(SCORE_SMALL_THREADS) cs_score_small_kernel(Sel
     T.fsurv = const_cast<float *>(a.fsurv);
     cs_wait_for_predecessor();
     cs_release_successor();
+    float f_mine = 0.0f;
+    if (SEARCH) {
+        const uint32_t v = threadIdx.x & 31u, row = v < a.A ? cs_ld_cg_pinned(ws.adjT + v) : 0u;
+        uint32_t mine = 0;
+        for (uint32_t i = v; i < src.n; i += 32u) {
+            const uint32_t ag = src.list[i];
+            if (ag < a.A) mine |= 1u << ag;
+            else atomicOr(&ws.sc->status, CS_ST_BAD_SOURCE);
+        }
+        uint32_t front = __reduce_or_sync(0xFFFFFFFFu, mine), seen = front, hops = (front >> v) & 1u ? 0u : CS_HOP_NONE;
+        for (uint32_t level = 1; front; ++level) {            // (every level adds an agent to `seen`, or is the last)
+            const bool fresh = (row & front) != 0u && !((seen >> v) & 1u);
+            front = __ballot_sync(0xFFFFFFFFu, fresh);
+            seen |= front;
+            if (fresh) hops = level;
+        }
+        f_mine = cs_survival_of(hops, src.e_max, a.delta);
+    }
     const uint32_t lane = threadIdx.x & 31, gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t n_quads = (a.n + 3u) / 4u;                 // (the arrays' last quad may be short)
     resolve_now(a);
-    for (uint32_t q = gw * 32u + lane; q < n_quads; q += n_warps * 32u) {
-        const uint32_t i0 = 4u * q;
+    for (uint32_t q0 = gw * 32u; q0 < n_quads; q0 += n_warps * 32u) {       // (whole warps: the factors come by shuffle)
+        const bool any = q0 + lane < n_quads;
+        const uint32_t q = any ? q0 + lane : n_quads - 1u, i0 = 4u * q;
         const bool whole = i0 + 4u <= a.n;
         uint32_t la[4], ag[4], tk[4];
         if (whole) {
@@ -119,7 +147,8 @@ __global__ void __launch_bounds__(SCORE_SMALL_THREADS) cs_score_small_kernel(Sel
 #pragma unroll
         for (int r = 0; r < 4; ++r) {                         // the eight look-ups travel together
             const uint32_t age = max(a.now, la[r]) - la[r];
-            f[r] = __ldcg(T.fsurv + (ag[r] < a.A ? ag[r] : 0u));
+            if (SEARCH) f[r] = __shfl_sync(0xFFFFFFFFu, f_mine, (int)(ag[r] & 31u));
+            else f[r] = __ldcg(T.fsurv + (ag[r] < a.A ? ag[r] : 0u));
             g[r] = __ldg(T.gtab + (age < a.gtab_len ? age : 0u));
             if (age >= a.gtab_len) g[r] = age >= a.age_sat ? T.g_sat : cs_recency(a.lambda, a.delta, age);
         }
@@ -129,8 +158,8 @@ __global__ void __launch_bounds__(SCORE_SMALL_THREADS) cs_score_small_kernel(Sel
             if (ag[r] >= a.A) { s[r] = 0.0f; atomicOr(&ws.sc->status, CS_ST_BAD_AGENT); }
         }
         if (whole) {
-            __stcs((float4 *)out + q, make_float4(s[0], s[1], s[2], s[3]));
-        } else {
+            if (any) __stcs((float4 *)out + q, make_float4(s[0], s[1], s[2], s[3]));
+        } else if (any) {
 #pragma unroll
             for (int r = 0; r < 4; ++r)
                 if (i0 + r < a.n) out[i0 + r] = s[r];
@@ -1025,15 +1054,20 @@ size_t cs_table_smem(const cs_ctx *ctx)
     return (size_t)(ctx->p.n_agents + ctx->gtab_len) * sizeof(float) + (size_t)ctx->p.n_agents * sizeof(uint16_t) + 16;
 }
 
-int cs_launch_score(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const float *fsurv, float *scores_out,
-                    cudaStream_t s)
+bool cs_score_searches(const cs_ctx *ctx, uint32_t n_blocks) { return ctx->p.n_agents <= 32u && n_blocks && n_blocks <= SCORE_SMALL_MAX; }
+
+int cs_launch_score(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const float *fsurv, const uint16_t *sources, uint32_t n_sources,
+                    float *scores_out, cudaStream_t s)
 {
+    const uint32_t grid_small = cs_scan_grid(ctx, idx->n_blocks, SCORE_SMALL_THREADS * 4u, 8u);
+    const ScoreSources src = {sources, n_sources, ctx->p.e_max};
     SelArgs a;
     cs_fill_sel_args(ctx, idx, now, fsurv, a);
     a.anchor = nullptr;
-    if (idx->n_blocks <= SCORE_SMALL_MAX)
-        cs_launch_chained(cs_score_small_kernel, cs_scan_grid(ctx, idx->n_blocks, SCORE_SMALL_THREADS * 4u, 8u), SCORE_SMALL_THREADS, 0, s, a,
-                          ctx->ws, scores_out);
+    if (sources)
+        cs_launch_chained(cs_score_small_kernel<true>, grid_small, SCORE_SMALL_THREADS, 0, s, a, ctx->ws, scores_out, src);
+    else if (idx->n_blocks <= SCORE_SMALL_MAX)
+        cs_launch_chained(cs_score_small_kernel<false>, grid_small, SCORE_SMALL_THREADS, 0, s, a, ctx->ws, scores_out, src);
     else
         cs_launch_chained(cs_score_kernel, cs_scan_grid(ctx, idx->n_blocks, SEL_THREADS * GRP), SEL_THREADS, cs_table_smem(ctx), s, a,
                           ctx->ws, scores_out);

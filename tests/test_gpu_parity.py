@@ -117,6 +117,28 @@ def test_score_parity(name, n, with_tokens):
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("A", [1, 2, 31, 32, 33])
+@pytest.mark.parametrize("n", [1, 3, 127, 4097, 131_071, 131_072, 131_073])
+def test_score_from_sources_searches_where_it_scores(A, n):
+    """Explicit sources on both sides of the lines up to which the score launch does the search itself (32 agents, 131,072
+    entries): no source, one, all of them and more than a warp has lanes; a bad one is reported and left out."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=5, transitions=("sparse", 1))
+    c, o = make_ctx(cfg, n, tau=0.3)
+    chain, agent = np.arange(600, dtype=np.uint32) % 3, (np.arange(600) // 3 % A).astype(np.uint16)      # a ring of the agents
+    c.observe_invocations(dev(chain), dev(agent), None)
+    o.observe(chain, agent)
+    idx = synth.make_block_index(cfg, n=n)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    for src in ([0], [A - 1, 0], list(range(A)), [A // 2] * 40):
+        s = c.score_blocks(d, 100_000, sources=dev(np.array(src, np.uint16))).cpu().numpy()
+        o.survival(np.unique(np.array(src, np.uint16)))
+        assert np.array_equal(s, o.scores(idx, 100_000)[1]), src
+    assert c.get_status() == 0
+    s = c.score_blocks(d, 100_000, sources=dev(np.array([A // 2, A, 0xFFFF], np.uint16))).cpu().numpy()
+    o.survival(np.array([A // 2], np.uint16))
+    assert np.array_equal(s, o.scores(idx, 100_000)[1]) and c.get_status() == cs.CS_ST_BAD_SOURCE
+
+
 def test_score_slow_decay_uses_direct_path():
     """A decay rate so small that the recency table does not cover all unsaturated ages."""
     cfg = synth.CONFIGS["tiny"]

@@ -12,12 +12,14 @@
  *  - "dev" pointers are caller-owned device memory, "pinned" pointers caller-owned
  *    page-locked host memory that the device can address (cudaHostAlloc /
  *    cudaHostRegister; with unified addressing the host pointer is used as is).  The
- *    library never allocates or frees device or pinned memory; it owns only the small
+ *    library itself never allocates or frees device or pinned memory; it owns only the small
  *    host-side cs_ctx, with a few CUDA events and two streams of its own (made by cs_create,
  *    released by cs_destroy; cs_step and cs_select_step fork onto them and join back, so callers
  *    see everything ordered on the streams they pass), one graph for each mix of lists that
  *    cs_select_step() is asked for twice over a large index, and five more streams and their events
- *    once cs_set_mover_staging() has been called.  All scratch lives in the workspace the
+ *    once cs_set_mover_staging() has been called.  The driver keeps the nodes of such a graph in device
+ *    memory of its own; where it refuses, for lack of memory or anything else, the selects are launched
+ *    one by one instead, with the same results.  All scratch lives in the workspace the
  *    caller hands to cs_create() (and, for the copy-engine transfers, in the ring handed to
  *    cs_set_mover_staging()).
  *  - Block-index arrays, score / id output arrays and pool bases must be 16-byte aligned (the

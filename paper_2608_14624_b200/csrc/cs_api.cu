@@ -217,7 +217,8 @@ int cs_create(const cs_params *p, void *dev_workspace, size_t bytes, cs_stream_t
     ctx->host_link_ctas = 0;
     ctx->d2d_ctas = 0;
     // fork / join events of cs_step() and the two extra streams (with their events) on which the second and third
-    // select of a step run: host objects, created here so that the calls themselves create nothing
+    // select of a step run: host objects, created here so that the calls themselves create none (but the graph of a mix of
+    // lists, on the second cs_select_step() over a large index that asks for it)
     e = cudaEventCreateWithFlags(&ctx->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_sel_fork, cudaEventDisableTiming);

@@ -145,7 +145,7 @@ struct cs_select_graph {
     cudaGraph_t graph;
     cudaGraphExec_t exec;
     cudaGraphNode_t node[3][CS_SELECT_STAGES];
-    uint32_t asked, refused;       // calls that wanted it (up to 2); 1: it could not be built
+    uint32_t asked, refused;       // calls that wanted it before it was there (up to 2); 1: it could not be built or launched
 };
 
 struct cs_ctx {

@@ -1218,14 +1218,16 @@ int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int p
     return launch_select_job(ctx, 0, idx, now, prefetch, tier, k, ids_out, n_out, s);
 }
 
-// The chains of selects side by side as one graph launch: true when it was launched or failed (*rc tells), false when it has
-// to be done launch by launch.  A launch costs the host 2.5 us, so that the 12 or 18 of a step (33 and 50 us) took longer than
+// The chains of selects side by side as one graph launch: true when it was launched, false when it has to be done launch by launch.
+// A launch costs the host 2.5 us, so that the 12 or 18 of a step (33 and 50 us) took longer than
 // their kernels (34 us for two lists of 1,000,000 entries); a node's new arguments take 0.2 us and the graph's launch 2 us.
 // A single select stays six launches: its kernels take longer than issuing them (29 and 16 us), and its first launch
 // overlaps the work before it on the stream, which a graph's does not.  Every argument is set anew on every call.
 //
 // The graph of a mix of lists is built (150 to 220 us) when a context is asked for that mix a second time: one that is asked
-// once, or never has large indexes, does not pay for it.
+// once, or never has large indexes, does not pay for it.  The driver keeps a graph's nodes in device memory, so on a GPU that its
+// user has filled any of these calls may be refused.  None of them has then enqueued anything: the launches stay single, in that call
+// and from then on, and the call reports no error of its own.
 static void drop_select_graph(cs_select_graph &g)
 {
     if (g.exec) (void)cudaGraphExecDestroy(g.exec);
@@ -1244,43 +1246,40 @@ static bool build_select_graph(cs_ctx *ctx, cs_select_graph &g, int n_jobs, Sele
     // (another thread may be capturing a stream of its own, which is nothing that these calls disturb)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-    const uint64_t launches = ctx->n_launches;
     bool ok = cudaGraphCreate(&g.graph, 0) == cudaSuccess;
+    if (!ok) g.graph = nullptr;
     for (int i = 0; i < n_jobs; ++i)
         for (int stage = 0; stage < SELECT_STAGES && ok; ++stage) ok = launch_stage(ctx, chain[i], stage, &g, i) == CS_OK;
-    ok = ok && cudaGraphInstantiate(&g.exec, g.graph, 0) == cudaSuccess;
+    if (ok && cudaGraphInstantiate(&g.exec, g.graph, 0) != cudaSuccess) { ok = false; g.exec = nullptr; }
     (void)cudaThreadExchangeStreamCaptureMode(&mode);
-    ctx->n_launches = launches;
-    if (!ok) {                                       // (no room for it: the launches stay single)
-        (void)cudaGetLastError();
-        drop_select_graph(g);
-    }
+    if (!ok) drop_select_graph(g);
     return ok;
 }
 
-static bool graph_of_selects(cs_ctx *ctx, uint32_t mask, int n_jobs, SelectChain *chain, cudaStream_t s, int *rc)
+static bool graph_of_selects(cs_ctx *ctx, uint32_t mask, int n_jobs, SelectChain *chain, cudaStream_t s)
 {
     cs_select_graph &g = ctx->sel_graph[mask];
+    if (g.refused) return false;
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
     if (st != cudaStreamCaptureStatusNone) return false;
-    if (!g.exec) {
-        if (g.asked < 2) ++g.asked;
-        if (g.asked != 2 || g.refused) return false;
-        g.refused = !build_select_graph(ctx, g, n_jobs, chain);
-        if (g.refused) return false;
-    }
-    *rc = CS_OK;
-    for (int i = 0; i < n_jobs && *rc == CS_OK; ++i)
-        for (int stage = 0; stage < SELECT_STAGES && *rc == CS_OK; ++stage) *rc = launch_stage(ctx, chain[i], stage, &g, i);
-    if (*rc == CS_OK) {
-        const cudaError_t e = cudaGraphLaunch(g.exec, s);
-        if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; *rc = CS_ECUDA; }
-    }
-    return true;
+    if (!g.exec && ++g.asked < 2) return false;
+    const uint64_t launches = ctx->n_launches;
+    const int last_error = ctx->last_cuda_error;
+    bool ok = g.exec || build_select_graph(ctx, g, n_jobs, chain);
+    ctx->n_launches = launches;                      // (adding the nodes launched nothing)
+    for (int i = 0; i < n_jobs; ++i)
+        for (int stage = 0; stage < SELECT_STAGES && ok; ++stage) ok = launch_stage(ctx, chain[i], stage, &g, i) == CS_OK;
+    if (ok && cudaGraphLaunch(g.exec, s) == cudaSuccess) return true;
+    // (a graph that has run stays until the context goes: earlier launches of it may still be running)
+    g.refused = 1;
+    ctx->n_launches = launches;
+    ctx->last_cuda_error = last_error;
+    (void)cudaGetLastError();
+    return false;
 }
 
 // The selects of a step side by side.  Select q (0 GPU-tier victims, 1 host-tier victims, 2 prefetch candidates)
@@ -1335,7 +1334,7 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
     }
     uint32_t mask = 0;
     for (int i = 0; i < n_jobs; ++i) mask |= 1u << jobs[i];
-    if (graph_of_selects(ctx, mask, n_jobs, chain, s, &rc)) return rc;
+    if (graph_of_selects(ctx, mask, n_jobs, chain, s)) return CS_OK;
     // Launched one by one: in turn, because issued one chain after the other the second one started 20 us (six launches) after
     // the first and both ended that much later.
     cudaError_t e = cudaEventRecord(ctx->ev_sel_fork, s);

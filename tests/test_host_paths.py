@@ -1,0 +1,90 @@
+"""The library's host code without a GPU: its sources linked against a CUDA runtime that counts calls and fails the ones it is told
+to (tests/fake_cudart.cpp).  Covers what a working GPU does not show: which route a call takes when the driver refuses something."""
+import ctypes as C
+import os
+import subprocess
+from concurrent.futures import ThreadPoolExecutor
+
+import pytest
+
+from paper_2608_14624_b200 import binding as cs
+from paper_2608_14624_b200 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OUT_OF_MEMORY = 2
+DEVICE_MEMORY, HOST_MEMORY = 2, 1            # cudaMemoryType
+WORKSPACE, BUF = 1 << 40, 1 << 41            # addresses nobody follows
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The library over the counting runtime, as the binding's own library for this module."""
+    out = tmp_path_factory.mktemp("host_paths")
+    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcicc", "-O0", "-Xptxas", "-O0",
+             "-I", os.path.join(build.ROOT, "include")]
+    nvcc = os.environ.get("NVCC", "nvcc")
+
+    def compile_one(src):
+        obj = str(out / (os.path.basename(src) + ".o"))
+        subprocess.run([nvcc, *flags, "-c", "-o", obj, src], check=True, capture_output=True)
+        return obj
+
+    with ThreadPoolExecutor(8) as pool:
+        objs = list(pool.map(compile_one, build.sources() + [os.path.join(HERE, "fake_cudart.cpp")]))
+    so = str(out / "libcachescout_host.so")
+    subprocess.run([nvcc, "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", so, *objs], check=True, capture_output=True)
+    saved = cs._lib, cs.LIB_PATH
+    cs._lib, cs.LIB_PATH = None, so
+    L = cs.lib()
+    L.fake_calls.argtypes, L.fake_fail.argtypes = [C.c_char_p], [C.c_char_p, C.c_int, C.c_int, C.c_int]
+    yield L
+    cs._lib, cs.LIB_PATH = saved
+
+
+@pytest.fixture
+def rt(fake):
+    fake.fake_reset()
+    return fake
+
+
+def calls(rt, name):
+    return rt.fake_calls(name.encode())
+
+
+def make_ctx(rt, **kw):
+    p, ctx = cs.make_params(**kw), C.c_void_p()
+    assert rt.cs_create(C.byref(p), WORKSPACE, cs.cs_workspace_bytes(p), None, C.byref(ctx)) == cs.CS_OK
+    return ctx.value
+
+
+def index(n):
+    return cs.cs_block_index(n, BUF, BUF, BUF, BUF, BUF, None, None)
+
+
+@pytest.mark.parametrize("call,skip", [("cudaGraphCreate", 0), ("cudaGraphAddNode", 0), ("cudaGraphAddNode", 7), ("cudaGraphInstantiate", 0),
+                                       ("cudaGraphExecNodeSetParams", 0), ("cudaGraphExecNodeSetParams", 11), ("cudaGraphLaunch", 0),
+                                       ("cudaGraphLaunch", 2), ("cudaThreadExchangeStreamCaptureMode", 0), ("cudaStreamIsCapturing", 1)])
+def test_selects_are_launched_one_by_one_when_their_graph_fails(rt, call, skip):
+    """Two lists of a large index, five times.  Whatever the driver refuses of their graph, at whichever call: the call succeeds by
+    single launches, no error is left behind, and a graph that failed is not tried again."""
+    ctx = make_ctx(rt, n_agents=12, n_chains=4, max_blocks=400_000)
+    idx = index(300_000)
+    rt.fake_fail(call.encode(), skip, 1, OUT_OF_MEMORY)
+    by_graph = []
+    for _ in range(5):
+        launched, graphs, n0 = calls(rt, "cs_sel_"), calls(rt, "cudaGraphLaunch"), cs.cs_launch_count(ctx)
+        cs.cs_select_step(ctx, idx, 5, 100, 100, BUF, BUF, None, None, BUF, BUF, stream=0)
+        assert cs.cs_launch_count(ctx) - n0 == 12
+        single = calls(rt, "cs_sel_") - launched
+        assert single in (0, 12)
+        assert single == 12 or calls(rt, "cudaGraphLaunch") == graphs + 1
+        by_graph.append(single == 0)
+        assert rt.cs_last_cuda_error(ctx) == 0 and rt.cudaGetLastError() == 0
+    if call == "cudaStreamIsCapturing":
+        assert by_graph == [False, False, True, True, True]          # (not the graph's fault: the next call builds it)
+    elif (call, skip) == ("cudaGraphLaunch", 2):
+        assert by_graph == [False, True, True, False, False]
+    else:
+        assert not any(by_graph)
+    cs.cs_destroy(ctx)
+    assert calls(rt, "cudaGraphCreate") - (call == "cudaGraphCreate") == calls(rt, "cudaGraphDestroy")

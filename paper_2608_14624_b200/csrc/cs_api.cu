@@ -143,6 +143,8 @@ bool cs_device_can_address(const void *ptr)
 // gap of 2 us behind it), 2.1 us like this.
 #define MODEL_PARTS 8
 #define EXPORT_THREADS 256
+// Only into memory of the context's own GPU: another GPU's may be out of a kernel's reach, and everything else (odd addresses, host
+// memory) is left to cudaMemcpyAsync as well.
 struct ModelPart { void *dst; const void *src; size_t bytes; };
 struct ModelParts { ModelPart part[MODEL_PARTS]; };
 __global__ void __launch_bounds__(EXPORT_THREADS) cs_export_kernel(const __grid_constant__ ModelParts parts)
@@ -157,6 +159,13 @@ __global__ void __launch_bounds__(EXPORT_THREADS) cs_export_kernel(const __grid_
         done = p.bytes / 16 * 8;
     }
     for (size_t i = done + tid; i < p.bytes / 2; i += nth) ((uint16_t *)p.dst)[i] = __ldcg((const unsigned short *)p.src + i);
+}
+
+static bool export_kernel_reaches(const cs_ctx *ctx, const void *dst)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+    return at.type == cudaMemoryTypeDevice && at.device == ctx->device && !(((uintptr_t)dst) & 1u);
 }
 
 // cs_get_status(): read and clear in one atomic step, so that a bit another stream sets in between is kept.
@@ -482,10 +491,10 @@ int cs_get_model(cs_ctx *ctx, uint32_t *C_out, float *P_out, uint16_t *amax_out,
     int n = 0;
     for (int i = 0; i < MODEL_PARTS && e == cudaSuccess; ++i) {
         if (!parts[i].dst) continue;
-        if (cs_device_can_address(parts[i].dst) && !(((uintptr_t)parts[i].dst) & 1u)) {
+        if (export_kernel_reaches(ctx, parts[i].dst)) {
             copy.part[n++] = parts[i];
             if (parts[i].bytes > most) most = parts[i].bytes;
-        } else {                                            // memory the kernel cannot write: the runtime's verdict
+        } else {
             e = cudaMemcpyAsync(parts[i].dst, parts[i].src, parts[i].bytes, cudaMemcpyDeviceToDevice, s);
         }
     }

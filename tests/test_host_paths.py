@@ -88,3 +88,17 @@ def test_selects_are_launched_one_by_one_when_their_graph_fails(rt, call, skip):
         assert not any(by_graph)
     cs.cs_destroy(ctx)
     assert calls(rt, "cudaGraphCreate") - (call == "cudaGraphCreate") == calls(rt, "cudaGraphDestroy")
+
+
+@pytest.mark.parametrize("device,kind,odd,by_kernel", [(0, DEVICE_MEMORY, 0, 8), (1, DEVICE_MEMORY, 0, 0), (0, HOST_MEMORY, 0, 0),
+                                                       (0, 0, 0, 0), (0, DEVICE_MEMORY, 1, 0)])
+def test_model_is_exported_by_a_kernel_to_its_own_gpu_only(rt, device, kind, odd, by_kernel):
+    """The export kernel stores to memory of the context's GPU; another GPU's memory, host memory, memory unknown to the runtime and odd
+    addresses are copied by the runtime, one copy per table."""
+    ctx = make_ctx(rt, n_agents=12, n_chains=4)
+    rt.fake_pointers(device, kind)
+    copies = calls(rt, "cudaMemcpyAsync")
+    cs.cs_get_model(ctx, *[BUF + 4096 * i + odd for i in range(8)], stream=0)
+    assert calls(rt, "cs_export_kernel") == (1 if by_kernel else 0)
+    assert calls(rt, "cudaMemcpyAsync") - copies == 8 - by_kernel
+    cs.cs_destroy(ctx)

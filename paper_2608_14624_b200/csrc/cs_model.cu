@@ -1097,25 +1097,25 @@ int cs_launch_init(cs_ctx *ctx, cudaStream_t s)
     return cs_launch_observe(ctx, nullptr, nullptr, nullptr, 0, s);
 }
 
-// Largest cluster (a power of two) a kernel can run as on a device; asked once per process and device, with that device
-// current.
+// Largest cluster (a power of two) a kernel can run as on a device, 0 when the driver would not say that any fits; asked once per
+// process and device, with that device current.
 struct ClusterLimit {
     std::mutex mu;
     int known[64];                                            // 0: not asked yet
-    template <class Kernel> int get(int device, Kernel kernel, int most, int threads)
+    template <class Kernel> uint32_t get(int device, Kernel kernel, int most, int threads)
     {
-        if (device < 0 || device >= 64) return 1;
+        if (device < 0 || device >= 64) return 0;
         std::lock_guard<std::mutex> lock(mu);
         if (!known[device]) known[device] = cs_probe_cluster(kernel, most, threads, 0, 1);
-        return known[device];
+        return known[device] > 0 ? (uint32_t)known[device] : 0u;
     }
 };
-static int obs_cluster_limit(int device)
+static uint32_t obs_cluster_limit(int device)
 {
     static ClusterLimit limit;
     return limit.get(device, cs_observe_kernel, OBS_MAX_CLUSTER, OBS_THREADS);
 }
-static int refresh_cluster_limit(int device)
+static uint32_t refresh_cluster_limit(int device)
 {
     static ClusterLimit limit;
     return limit.get(device, cs_refresh_kernel<8>, RfShape<8>::CTAS, RfShape<8>::WARPS * 32);
@@ -1128,10 +1128,9 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
     const bool fused = n_events <= OBS_FUSED_MAX;             // small batches ride along with the refresh
     if (n_events && !fused) {
         // one event per thread and round: no more CTAs than the batch fills
-        const int most = obs_cluster_limit(ctx->device);
-        if (most < 1) { ctx->last_cuda_error = (int)cudaErrorInvalidClusterSize; return CS_ECUDA; }
+        const uint32_t most = obs_cluster_limit(ctx->device);
         uint32_t cl = 1;
-        while ((int)cl < most && cl * OBS_THREADS < n_events) cl <<= 1;
+        while (cl < most && cl * OBS_THREADS < n_events) cl <<= 1;
         cs_launch_chained_clusters(cs_observe_kernel, cl, cl, OBS_THREADS, 0, s, ctx->ws, p.n_agents, p.n_chains, chain, agent,
                                    evflags, n_events, ctx->step_n_events_dev);
         int rc = cs_check_launch(ctx);
@@ -1146,7 +1145,7 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
         cs_launch_chained_clusters(kernel, ctas, cluster, warps * 32u, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min,
                                    p.e_max, p.delta, all_chains, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
     };
-    const uint32_t most = (uint32_t)refresh_cluster_limit(ctx->device);
+    const uint32_t most = refresh_cluster_limit(ctx->device);
     if (p.n_agents <= 32) {
         // one CTA of as many warps as there are rows, at least one thread per event of a small batch
         launch(cs_refresh_kernel<1>, 1u, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));

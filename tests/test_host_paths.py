@@ -2,6 +2,7 @@
 to (tests/fake_cudart.cpp).  Covers what a working GPU does not show: which route a call takes when the driver refuses something."""
 import ctypes as C
 import os
+import shutil
 import subprocess
 from concurrent.futures import ThreadPoolExecutor
 
@@ -17,8 +18,8 @@ WORKSPACE, BUF = 1 << 40, 1 << 41            # addresses nobody follows
 
 
 @pytest.fixture(scope="module")
-def fake(tmp_path_factory):
-    """The library over the counting runtime, as the binding's own library for this module."""
+def host_library(tmp_path_factory):
+    """The library's sources linked against the counting runtime; returns the path."""
     out = tmp_path_factory.mktemp("host_paths")
     flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcicc", "-O0", "-Xptxas", "-O0",
              "-I", os.path.join(build.ROOT, "include")]
@@ -33,18 +34,19 @@ def fake(tmp_path_factory):
         objs = list(pool.map(compile_one, build.sources() + [os.path.join(HERE, "fake_cudart.cpp")]))
     so = str(out / "libcachescout_host.so")
     subprocess.run([nvcc, "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", so, *objs], check=True, capture_output=True)
+    return so
+
+
+@pytest.fixture
+def rt(host_library, tmp_path):
+    """A fresh copy of that library (what it has learnt about a device is kept per process), as the binding's own for one test."""
+    so = str(shutil.copy(host_library, tmp_path))
     saved = cs._lib, cs.LIB_PATH
     cs._lib, cs.LIB_PATH = None, so
     L = cs.lib()
     L.fake_calls.argtypes, L.fake_fail.argtypes = [C.c_char_p], [C.c_char_p, C.c_int, C.c_int, C.c_int]
     yield L
     cs._lib, cs.LIB_PATH = saved
-
-
-@pytest.fixture
-def rt(fake):
-    fake.fake_reset()
-    return fake
 
 
 def calls(rt, name):
@@ -101,4 +103,24 @@ def test_model_is_exported_by_a_kernel_to_its_own_gpu_only(rt, device, kind, odd
     cs.cs_get_model(ctx, *[BUF + 4096 * i + odd for i in range(8)], stream=0)
     assert calls(rt, "cs_export_kernel") == (1 if by_kernel else 0)
     assert calls(rt, "cudaMemcpyAsync") - copies == 8 - by_kernel
+    cs.cs_destroy(ctx)
+
+
+@pytest.mark.parametrize("call,code", [("cudaOccupancyMaxActiveClusters", OUT_OF_MEMORY), ("cudaFuncSetAttribute", OUT_OF_MEMORY), (None, 0)])
+@pytest.mark.parametrize("A,kernel", [(12, "cs_refresh_kernelILi1"), (64, "cs_refresh_wide_kernel"), (256, "cs_refresh_wide_kernel"),
+                                      (300, "cs_refresh_wide_kernel")])
+def test_the_learner_runs_where_no_cluster_size_can_be_found(rt, call, code, A, kernel):
+    """When the driver does not say that any cluster fits (an error, or none), the refresh takes a kernel that needs none and a long
+    batch one CTA; every call succeeds and leaves no error."""
+    if call:
+        rt.fake_fail(call.encode(), 0, -1, code)
+    else:
+        rt.fake_clusters(0)
+    ctx = make_ctx(rt, n_agents=A, n_chains=4)
+    for n in (3, 2000):
+        before = calls(rt, kernel)
+        cs.cs_observe_invocations(ctx, BUF, BUF, None, n, stream=0)
+        assert calls(rt, kernel) == before + 1
+    assert calls(rt, "cs_observe_kernel") == 1 and calls(rt, "cs_refresh_kernelILi8") == 0
+    assert rt.cs_last_cuda_error(ctx) == 0 and rt.cudaGetLastError() == 0
     cs.cs_destroy(ctx)

@@ -46,7 +46,10 @@ struct OrderSmem {
     uint32_t *misc;               // [OM_WORDS]
     uint32_t cap;
 };
+// OM_BELOW and OM_FILL (one word per part) are order_few()'s own: it clears them on entry with no barrier before that, while slower
+// warps may still be reading any other word (OM_TOTAL in particular, on the way from a cut of the candidates).
 enum { OM_B0 = 0, OM_CTOT, OM_LIST, OM_GLOBAL, OM_GLOBAL2, OM_OVERFLOW, OM_BELOW, OM_IN, OM_TOTAL, OM_FILL = 16, OM_LO_ID = 24, OM_WORDS = 48 };
+static_assert(OM_TOTAL != OM_BELOW && (OM_TOTAL < OM_FILL || OM_TOTAL >= OM_FILL + (int)OR_PARTS), "read while order_few() clears its words");
 
 // Where the candidates are and where they may be moved to; all of it private to the select.
 struct OrderBufs {
@@ -126,7 +129,7 @@ __device__ __noinline__ void order_few(const OrderSmem &O, const u64 *src_km, co
             }
         }
     }
-    if (tid < OM_WORDS - OM_BELOW) O.misc[OM_BELOW + tid] = 0;
+    if (tid <= OR_PARTS) O.misc[tid < OR_PARTS ? OM_FILL + tid : OM_BELOW] = 0;
     __syncthreads();
     if ((unsigned long long)c * c <= 32768ull * CL) {
         // few: every CTA places an equal share of the keys, each counted against all of them
@@ -210,7 +213,7 @@ __device__ __noinline__ void order_few(const OrderSmem &O, const u64 *src_km, co
             __syncthreads();                                           // the sample misjudged: take the rest as well
             hi_km = ~0ull;
             hi_id = 0xFFFFFFFFu;
-            if (tid < OM_WORDS - OM_BELOW) O.misc[OM_BELOW + tid] = 0;
+            if (tid <= OR_PARTS) O.misc[tid < OR_PARTS ? OM_FILL + tid : OM_BELOW] = 0;
             __syncthreads();
             continue;
         }

@@ -225,6 +225,29 @@ def test_select_ordering_routes(n, ks, ties):
     assert run_selects(c, o, idx, 100_000, ks, tiers=(0,) if n > 100_000 else (0, 1)) == 0
 
 
+@pytest.mark.parametrize("n", [20_000, 60_000, 200_001])
+def test_short_lists_out_of_many_tied_candidates_over_and_over(n):
+    """Lists of a few ids out of more candidates than a CTA holds: the candidates are cut at a sample and what is left is ordered
+    right behind the cut, by warps that need not wait for one another.  A thousand selects of each length must all give the oracle's list."""
+    cfg = synth.CONFIGS["llama8b"]
+    c, o = warm_state(cfg, 1000, n, r_min=0.02)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    idx.agent[:], idx.n_tokens[:] = 3, 16                    # one score: the threshold bin holds every eligible entry
+    idx.last_access[:] = 10_000 + synth.rng_for(cfg, 61).integers(0, 60_000, n)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    s32 = o.scores(idx, 100_000)[1]
+    for k in (1, 16, 40):
+        want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+        outs = torch.full((1000, max(4, (k + 3) // 4 * 4)), 7, dtype=torch.int32, device=DEV)
+        cnt = torch.zeros(1, dtype=torch.int32, device=DEV)
+        for row in outs:
+            c.select_victims(d, 100_000, 0, k, row, cnt)
+        got = outs[:, :k].cpu().numpy().view(np.uint32)
+        assert int(cnt.item()) == n_want == k and (got == want[:k]).all(), (k, np.flatnonzero((got != want[:k]).any(axis=1))[:5])
+        assert c.counters()["candidates"][0] > 4096
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("eligible,k", [(1, 1), (255, 255), (257, 20), (1024, 1024), (1025, 1), (2047, 2047), (2048, 700), (2048, 2048),
                                         (2049, 3000), (2049, 1300)])
 @pytest.mark.parametrize("tied", [False, True])

@@ -128,8 +128,9 @@ struct cs_workspace {
     uint32_t *hist;       // [CS_HIST_BINS]
     unsigned long long *cand_km;    // [max_blocks] (primary<<32 | secondary) of each candidate
     uint32_t *cand_id;    // [max_blocks]
-    uint32_t *cand_bkt;   // [max_blocks]
-    uint32_t *cand_slot;  // [max_blocks]
+    uint32_t *cand_bkt;   // [max_blocks] cluster select, ordering through global memory: bucket of each candidate; launch chain: places of
+                          // the keys of buckets that outgrow the tile, every bucket at its offset in the order
+    uint32_t *cand_slot;  // [max_blocks] cluster select: slot in that bucket
     unsigned long long *sort_km;    // [max_blocks] candidates grouped by bucket
     uint32_t *sort_id;    // [max_blocks]
     unsigned long long *spl_km;     // [CS_SAMPLE] the ranked sample; the splitters of the general route

@@ -882,11 +882,15 @@ __device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u6
     return more < all - st.bound ? st.bound + more : all;
 }
 
-// Bucket b of CTA b: ranked by counting while it is small, sorted in the tile (bitonic, O(m log^2 m)) when it is large.
+// Bucket b of CTA b: ranked by counting while it is small, sorted in the tile (bitonic, O(m log^2 m)) when it is larger, and through a
+// list of its keys' places, sorted in global memory, when the tile does not hold it.  The list lies where the bucket's ids lie in the
+// whole order -- [off, off + m) of an array of one word per entry -- so that no two buckets share a word.  Long lists come here as a
+// matter of course: the keys between two samples are exponentially spread, so the largest of several hundred buckets is four to six times
+// the mean one (432,000 candidates, k = 150,000: one or two buckets of 2,300 keys; 1,730,000, k = 600,000: 9,000).
 #define FINISH_THREADS 512u
 #define FINISH_COUNT_MAX 512u
 static_assert(FINISH_THREADS == CS_BUCKETS, "one bucket size per thread");
-__global__ void __launch_bounds__(FINISH_THREADS)
+__global__ void __launch_bounds__(FINISH_THREADS, 3)
 cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t region_max, uint32_t kind, uint32_t hint_slot,
                      uint32_t *__restrict__ ids_out)
 {
@@ -931,47 +935,53 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
         ids_out[pos] = id;
         if (pos == n_out - 1 && hint_slot < 3) ws.sc->sel_T[hint_slot] = next_bound(*ws.sel, k, km);
     };
-    if (m > P.cap || rest) {
+    const bool outgrown = m > P.cap || rest, fits = m <= RANK_TILE;
+    uint32_t *const list = ws.cand_bkt + off;                 // [m] places of the keys when the tile does not hold them
+    if (outgrown) {
         // the region was too small: the bucket's keys once more, out of all candidates
         u64 lo_km, hi_km;
         uint32_t lo_id, hi_id;
         bucket_start(P, ws.spl_km, ws.spl_id, b, lo_km, lo_id);
         bucket_start(P, ws.spl_km, ws.spl_id, b + 1u, hi_km, hi_id);
         if (b == P.nb - 1u && P.J < P.S && !rest) { hi_km = ws.spl_km[P.J - 1]; hi_id = ws.spl_id[P.J - 1]; }
-        const bool fits = m <= RANK_TILE;
-        for (uint32_t i = tid; i < c; i += FINISH_THREADS) {
-            const u64 km = __ldcg(ws.cand_km + i);
-            const uint32_t id = __ldcg(ws.cand_id + i);
-            if (less96(km, id, lo_km, lo_id) || !less96(km, id, hi_km, hi_id)) continue;
-            if (fits) {
-                const uint32_t at = atomicAdd(&s_n, 1u);
-                t_km[at] = km;
-                t_id[at] = id;
-            } else {                                          // nor does the tile hold them: each against all candidates
-                uint32_t r = 0;
-                for (uint32_t q = 0; q < c; ++q) {
-                    const u64 qk = __ldcg(ws.cand_km + q);
-                    const uint32_t qi = __ldcg(ws.cand_id + q);
-                    if (!less96(qk, qi, lo_km, lo_id)) count_less(r, qk, qi, km, id);
-                }
-                emit(r, km, id);
+        for (uint32_t i0 = tid; i0 < c; i0 += 4u * FINISH_THREADS) {
+            u64 km[4];
+            uint32_t id[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * FINISH_THREADS;
+                km[u] = __ldcg(ws.cand_km + (i < c ? i : 0u));
+                id[u] = __ldcg(ws.cand_id + (i < c ? i : 0u));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * FINISH_THREADS;
+                if (i >= c || less96(km[u], id[u], lo_km, lo_id) || !less96(km[u], id[u], hi_km, hi_id)) continue;
+                const uint32_t at = atomicAdd(&s_n, 1u);      // (m of them: the bucket's counter has counted the same keys)
+                if (at >= m) continue;
+                if (fits) { t_km[at] = km[u]; t_id[at] = id[u]; }
+                else list[at] = i;
             }
         }
-        if (!fits) return;
         __syncthreads();
-    } else if (m <= RANK_TILE) {
+        m = min(m, s_n);
+    } else if (fits) {
         for (uint32_t i = tid; i < m; i += FINISH_THREADS) {
             t_km[i] = __ldcg(src_km + i);
             t_id[i] = __ldcg(src_id + i);
         }
         __syncthreads();
-    } else {                                                  // larger than the tile: ranked straight from global memory
-        for (uint32_t i = tid; i < m; i += FINISH_THREADS) {
-            const u64 km = __ldcg(src_km + i);
-            const uint32_t id = __ldcg(src_id + i);
-            uint32_t r = 0;
-            for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(src_km + q), __ldcg(src_id + q), km, id);
-            emit(r, km, id);
+    } else {
+        for (uint32_t i = tid; i < m; i += FINISH_THREADS) list[i] = i;
+        __syncthreads();
+    }
+    if (!fits) {
+        const u64 *k_km = outgrown ? ws.cand_km : src_km;
+        const uint32_t *k_id = outgrown ? ws.cand_id : src_id;
+        sort_places(list, m, k_km, k_id);
+        for (uint32_t i = tid; i < m && off + i < n_out; i += FINISH_THREADS) {
+            const uint32_t at = __ldcg(list + i);
+            emit(i, __ldcg(k_km + at), __ldcg(k_id + at));
         }
         return;
     }

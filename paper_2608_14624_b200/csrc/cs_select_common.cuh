@@ -450,6 +450,43 @@ __device__ __forceinline__ void rank_keys(const u64 *km, const uint32_t *id, uin
     }
 }
 
+// Sorts a list of places of keys, ascending by the keys.  Whole CTA.  Bitonic, with the first step of every merge between mirror images,
+// so that every comparator moves the smaller key to the lower place: places past the end then never take part, and any length will do.
+static __device__ __noinline__ void sort_places(uint32_t *list, uint32_t m, const u64 *__restrict__ km, const uint32_t *__restrict__ id)
+{
+    constexpr int ITEMS = 4;                                  // comparators per thread whose loads travel together
+    uint32_t P = 2;
+    while (P < m) P <<= 1;                                    // (at most 2^31: a list is no longer than an index)
+    for (uint32_t half = 1; half < m; half <<= 1)
+        for (uint32_t step = half, mirror = 1; step > 0; step >>= 1, mirror = 0) {
+            for (uint32_t t0 = threadIdx.x; t0 < P / 2; t0 += ITEMS * blockDim.x) {
+                uint32_t lo[ITEMS], hi[ITEMS], a[ITEMS], b[ITEMS], ia[ITEMS], ib[ITEMS];
+                u64 ka[ITEMS], kb[ITEMS];
+                bool in[ITEMS];
+#pragma unroll
+                for (int u = 0; u < ITEMS; ++u) {
+                    const uint32_t t = t0 + u * blockDim.x, x = t & (step - 1u);
+                    lo[u] = 2u * t - x;
+                    hi[u] = mirror ? lo[u] + 2u * (step - x) - 1u : lo[u] + step;
+                    in[u] = t < P / 2 && hi[u] < m;
+                    a[u] = in[u] ? __ldcg(list + lo[u]) : 0u;
+                    b[u] = in[u] ? __ldcg(list + hi[u]) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < ITEMS; ++u) {
+                    ka[u] = __ldcg(km + a[u]);
+                    kb[u] = __ldcg(km + b[u]);
+                    ia[u] = __ldcg(id + a[u]);
+                    ib[u] = __ldcg(id + b[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < ITEMS; ++u)
+                    if (in[u] && less96(kb[u], ib[u], ka[u], ia[u])) { list[lo[u]] = b[u]; list[hi[u]] = a[u]; }
+            }
+            __syncthreads();
+        }
+}
+
 __device__ __forceinline__ bool key_less(unsigned long long km_a, uint32_t id_a, unsigned long long km_b,
                                          uint32_t id_b)
 {

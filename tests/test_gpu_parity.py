@@ -907,6 +907,57 @@ def test_bucket_regions_and_their_fallback(max_keys):
         assert cn["region_overflows"] == [0, 0, 0]
 
 
+@pytest.mark.parametrize("k", [300_000, 399_000])
+def test_buckets_beyond_the_tile(k):
+    """Lists so long that ordinary buckets outgrow the 2,048-key tile and their regions: 400,000 eligible entries per tier, by the chain (one
+    call, a second one with the remembered key, and both lists side by side, each on scratch of its own)."""
+    cfg = synth.CONFIGS["meta1m"]
+    n = 800_000
+    c, o = warm_state(cfg, 3000, n, r_min=0.02)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    idx.flags[:], idx.ref_count[:], idx.depth[:] = synth.FLAG_VALID, 0, 0
+    idx.flags[n // 2:] |= synth.FLAG_TIER_HOST
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    s64, s32 = o.scores(idx, 100_000)
+    want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+    want_p, n_want_p = o.select_prefetch(idx, 100_000, k, s32)
+    assert n_want == n_want_p == k
+    for rep in range(3):
+        ids, cnt, p_ids, p_cnt = (torch.full((m,), 7, dtype=torch.int32, device=DEV) for m in (k, 1, k, 1))
+        if rep < 2:
+            c.select_victims(d, 100_000, 0, k, ids, cnt)
+            c.select_prefetch(d, 100_000, k, p_ids, p_cnt)
+        else:
+            c.select_step(d, 100_000, k, k, ids, cnt, None, None, p_ids, p_cnt)
+        assert H.assert_list_matches(ids.cpu().numpy().view(np.uint32), int(cnt.item()), want, n_want, s64) == 0
+        assert H.assert_list_matches(p_ids.cpu().numpy().view(np.uint32), int(p_cnt.item()), want_p, n_want_p, s64) == 0
+    cn = c.counters()
+    assert cn["region_overflows"][0] > 0 and cn["region_overflows"][2] > 0 and c.get_status() == 0
+
+
+@pytest.mark.parametrize("k,seen_are_old", [(1000, False), (5000, True), (524_288, False)])
+def test_samples_that_mislead(k, seen_are_old):
+    """Candidates are sampled at even distances.  524,288 entries, all eligible, all of one score, of which the sample sees every 512th:
+    as the oldest of all (the cut then lies below the list's end and the last bucket takes the rest) and as the youngest (everything
+    else falls into one bucket); 523,000 keys in one bucket are ordered all the same."""
+    n, step = 524_288, 512
+    p = cs.make_params(n_agents=2, max_blocks=n)
+    c, o = cs.CacheScout(p, DEV), orc.Oracle(H.oracle_params(p))
+    idx = synth.make_block_index(synth.shrink(synth.CONFIGS["tiny"], n_agents=2), n=n)
+    rng = synth.rng_for(synth.CONFIGS["tiny"], 77)
+    idx.flags[:], idx.ref_count[:], idx.agent[:], idx.n_tokens[:] = synth.FLAG_VALID, 0, 0, p.block_tokens
+    idx.last_access[:] = rng.integers(2_000, 60_000, n)
+    idx.last_access[::step] = rng.integers(0, 1_000, n // step) if seen_are_old else rng.integers(80_000, 90_000, n // step)
+    s64, s32 = o.scores(idx, 100_000)
+    assert len(np.unique(s32)) == 1
+    want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    for _ in range(2):
+        ids, cnt = c.select_victims(d, 100_000, 0, k)
+        assert H.assert_list_matches(ids.cpu().numpy().view(np.uint32)[:k], int(cnt.item()), want, n_want, s64) == 0
+    assert (c.counters()["region_overflows"][0] > 0) != seen_are_old and c.get_status() == 0
+
+
 # ---- hop table from every live session's current agent ----------------------------------------------------
 @pytest.mark.parametrize("name,n_inv", [("tiny", 60), ("llama8b", 400), ("meta1m", 3000)])
 def test_survival_from_all_chains(name, n_inv):

@@ -137,7 +137,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
             bitonic_sort_fast(km_s, id_s, P, whole_cta());
             for (uint32_t i = tid; i < m; i += CSEL_THREADS)
                 if (beg + i < n_out) ids_out[beg + i] = id_s[i];
-        } else {                                     // a large bucket: ranked straight from global memory
+        } else if (m <= OR_ALL) {                    // a large bucket: ranked straight from global memory
             for (uint32_t i = tid; i < m; i += CSEL_THREADS) {
                 const u64 km = __ldcg(&ws.sort_km[beg + i]);
                 const uint32_t id = __ldcg(&ws.sort_id[beg + i]);
@@ -145,6 +145,12 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
                 for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(&ws.sort_km[beg + q]), __ldcg(&ws.sort_id[beg + q]), km, id);
                 if (beg + r < n_out) ids_out[beg + r] = id;
             }
+        } else {                                     // beyond that counting, which grows with the square, would take milliseconds to seconds
+            uint32_t *list = ws.cand_bkt + beg;      // (the candidates' buckets are no longer wanted; nobody else's part of the array)
+            for (uint32_t i = tid; i < m; i += CSEL_THREADS) list[i] = i;
+            __syncthreads();
+            sort_places(list, m, ws.sort_km + beg, ws.sort_id + beg);
+            for (uint32_t i = tid; i < m && beg + i < n_out; i += CSEL_THREADS) ids_out[beg + i] = __ldcg(&ws.sort_id[beg + __ldcg(list + i)]);
         }
     }
 }

@@ -297,7 +297,9 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
         const uint32_t beg = (uint32_t)((unsigned long long)rank * c / CL), end = (uint32_t)((unsigned long long)(rank + 1u) * c / CL);
         const bool fill = J >= 96u;                                 // enough samples below the cut to split the output evenly
         const uint32_t nb = J < OR_BUCKETS ? J : OR_BUCKETS;
-        const uint32_t cap = B.dst_cap / nb;
+        // (no more than a warp can rank by counting: the workspace may have been made for a far larger index than this one, and a sample
+        // that misleads may put nearly all candidates into one bucket)
+        const uint32_t cap = min(B.dst_cap / nb, OR_ALL);
         // ---- what lies below the cut: into buckets, or into dst for another round ----------------------------------------
         for (uint32_t i0 = beg; i0 < end; i0 += 4u * OR_THREADS) {
             u64 km[4];

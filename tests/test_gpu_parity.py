@@ -248,6 +248,30 @@ def test_short_lists_out_of_many_tied_candidates_over_and_over(n):
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("k,seen_are_old", [(1000, False), (20_000, False), (20_000, True), (262_144, False)])
+@pytest.mark.parametrize("max_blocks", [262_144, 40_000_000])
+def test_samples_that_mislead_a_cluster(max_blocks, k, seen_are_old):
+    """The samples of the single-launch select lie at even distances as well.  262,144 entries of one score, all eligible, of which a sample
+    sees only every 64th, as the youngest or the oldest of all; with a workspace of the index's size and with one whose bucket regions would
+    hold everything."""
+    n = 262_144
+    p = cs.make_params(n_agents=2, max_blocks=max_blocks)
+    c, o = cs.CacheScout(p, DEV), orc.Oracle(H.oracle_params(p))
+    idx = synth.make_block_index(synth.shrink(synth.CONFIGS["tiny"], n_agents=2), n=n)
+    rng = synth.rng_for(synth.CONFIGS["tiny"], 79)
+    idx.flags[:], idx.ref_count[:], idx.agent[:], idx.n_tokens[:] = synth.FLAG_VALID, 0, 0, p.block_tokens
+    idx.last_access[:] = rng.integers(5_000, 60_000, n)
+    idx.last_access[::64] = rng.integers(0, 4_000, n // 64) if seen_are_old else rng.integers(80_000, 90_000, n // 64)
+    s64, s32 = o.scores(idx, 100_000)
+    assert len(np.unique(s32)) == 1
+    want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    for _ in range(2):
+        ids, cnt = c.select_victims(d, 100_000, 0, k)
+        assert H.assert_list_matches(ids.cpu().numpy().view(np.uint32)[:k], int(cnt.item()), want, n_want, s64) == 0
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("eligible,k", [(1, 1), (255, 255), (257, 20), (1024, 1024), (1025, 1), (2047, 2047), (2048, 700), (2048, 2048),
                                         (2049, 3000), (2049, 1300)])
 @pytest.mark.parametrize("tied", [False, True])

@@ -67,35 +67,39 @@ __device__ __forceinline__ uint2 fetch_slots(const MoverArgs &a, unsigned long l
     return make_uint2(a.src_slots ? __ldg(a.src_slots + i) : i, a.dst_slots ? __ldg(a.dst_slots + i) : i);
 }
 
-// Resolves work item w to a source / destination address and a byte count; false = skip.
-__device__ __forceinline__ bool resolve_piece(const MoverArgs &a, unsigned long long w, uint32_t per_block, uint2 slots,
-                                              const char *&sp, char *&dp, uint32_t &bytes, bool report)
+// Resolves work item w to a source / destination address and a byte count; `bytes` is 0 when there is nothing to copy.  Returns what the
+// work counters are owed for it -- one piece per block does the block's bookkeeping, so 0 for all others -- to be handed to book_block()
+// when the piece's turn has come.
+enum { BOOK_NOTHING = 0, BOOK_MOVED, BOOK_SKIPPED, BOOK_BAD_SLOT };
+__device__ __forceinline__ uint32_t resolve_piece(const MoverArgs &a, unsigned long long w, uint32_t per_block, uint2 slots,
+                                                  const char *&sp, char *&dp, uint32_t &bytes)
 {
     const uint32_t i = (uint32_t)(w / per_block);
     const uint32_t r = (uint32_t)(w - (unsigned long long)i * per_block);
     const uint32_t lp = r / a.pieces, piece = r - lp * a.pieces;
     uint32_t s = slots.x, d = slots.y;
-    const bool first = report && r == 0;                // one piece per block does the block's bookkeeping
-    if (s == CS_ID_NONE || d == CS_ID_NONE) {
-        if (first) atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, 1ull);
-        return false;
-    }
+    bytes = 0;
+    if (s == CS_ID_NONE || d == CS_ID_NONE) return r ? BOOK_NOTHING : BOOK_SKIPPED;
     s -= a.src_first;                                   // ids below first_id wrap and fail the range check
     d -= a.dst_first;
-    if (s >= a.src_total || d >= a.dst_total) {
-        if (first) { atomicOr(a.status, CS_ST_BAD_SLOT); atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, 1ull); }
-        return false;
-    }
-    if (first) {
-        atomicAdd((unsigned long long *)&a.cnt->blocks_moved[a.kind], 1ull);
-        atomicAdd((unsigned long long *)&a.cnt->bytes_moved[a.kind], a.block_bytes);
-    }
+    if (s >= a.src_total || d >= a.dst_total) return r ? BOOK_NOTHING : BOOK_BAD_SLOT;
     const unsigned long long in_chunk = (unsigned long long)piece * a.piece_bytes;
     sp = a.src + chunk_offset(a.src_layout, a.n_chunks, a.src_total, lp, s, a.chunk) + in_chunk;
     dp = a.dst + chunk_offset(a.dst_layout, a.n_chunks, a.dst_total, lp, d, a.chunk) + in_chunk;
     const unsigned long long left = a.chunk - in_chunk;
     bytes = (uint32_t)(left < a.piece_bytes ? left : a.piece_bytes);
-    return true;
+    return r ? BOOK_NOTHING : BOOK_MOVED;
+}
+
+__device__ __forceinline__ void book_block(const MoverArgs &a, uint32_t what)
+{
+    if (what == BOOK_MOVED) {
+        atomicAdd((unsigned long long *)&a.cnt->blocks_moved[a.kind], 1ull);
+        atomicAdd((unsigned long long *)&a.cnt->bytes_moved[a.kind], a.block_bytes);
+    } else {
+        if (what == BOOK_BAD_SLOT) atomicOr(a.status, CS_ST_BAD_SLOT);
+        atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, 1ull);
+    }
 }
 
 __device__ __forceinline__ uint32_t mover_count(const MoverArgs &a)
@@ -117,7 +121,9 @@ __global__ void __launch_bounds__(MV_THREADS) cs_mover_kernel(MoverArgs a)
         const char *sp0;
         char *dp0;
         uint32_t bytes;
-        if (!resolve_piece(a, w, per_block, fetch_slots(a, w, per_block), sp0, dp0, bytes, threadIdx.x == 0)) continue;
+        const uint32_t what = resolve_piece(a, w, per_block, fetch_slots(a, w, per_block), sp0, dp0, bytes);
+        if (what && threadIdx.x == 0) book_block(a, what);
+        if (!bytes) continue;
         const uint4 *sp = (const uint4 *)sp0;
         uint4 *dp = (uint4 *)dp0;
         const uint32_t nvec = bytes >> 4;
@@ -210,15 +216,16 @@ __device__ __forceinline__ void bulk_store(void *dst, uint32_t src_smem, uint32_
 // cost as much time as moving 2 KiB); lane 0 issues the copies.  Iteration `it` first stores item it - LAG, whose load was
 // issued LAG iterations ago, and then issues the load of item `it` into the ring slot whose previous store has finished
 // reading shared memory.  `fetch(it)` looks an item's list entries up, a batch of 32 ahead of
-// `item(it, slots, sp, dp, bytes)`, which resolves it; false = nothing to copy.
+// `item(it, slots, sp, dp, bytes)`, which resolves it and returns what is to be booked: `book(it, what)` is called once the item's load
+// has been issued (or it was found to have none), never for the items behind a wait that ran out.
 template <int STAGES> struct PipeShared {
     unsigned long long bar[STAGES];
     char *dst[STAGES];                // destination of the item loaded into each ring slot
     uint32_t bytes[STAGES];           // 0: nothing in flight there
 };
-template <int STAGES, class Fetch, class Item>
+template <int STAGES, class Fetch, class Item, class Book>
 __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared<STAGES> &ps, unsigned long long n_items, uint32_t *status,
-                                              Fetch fetch, Item item)
+                                              Fetch fetch, Item item, Book book)
 {
     constexpr uint32_t PIECE = TM_RING / STAGES;
     constexpr int LAG = STAGES - (STAGES + 2) / 3;    // two thirds of the slots load, one third store
@@ -228,15 +235,15 @@ __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared
     uint32_t phase_bits = 0;          // parity to wait for, one bit per ring slot
     bool failed = false;
     char *sp = nullptr, *dp = nullptr;
-    uint32_t bytes = 0;
+    uint32_t bytes = 0, what = 0;
     uint2 next = make_uint2(CS_ID_NONE, CS_ID_NONE);
     if (lane < n_items) next = fetch(lane);
     int st_load = 0, st_store = 0;    // ring slots of items it and it - LAG
     for (unsigned long long it = 0; it < n_items + LAG; ++it) {
         if ((it & 31u) == 0 && it < n_items) {                // resolve the next 32 items
             const char *s = nullptr;
-            bytes = 0;
-            if (it + lane < n_items && !item(it + lane, next, s, dp, bytes)) bytes = 0;
+            bytes = what = 0;
+            if (it + lane < n_items) what = item(it + lane, next, s, dp, bytes);
             sp = const_cast<char *>(s);
             if (it + 32u + lane < n_items) next = fetch(it + 32u + lane);
         }
@@ -276,6 +283,7 @@ __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared
         st_load = st_load + 1 == STAGES ? 0 : st_load + 1;
         if (it >= (unsigned long long)LAG) st_store = st_store + 1 == STAGES ? 0 : st_store + 1;
         if (__shfl_sync(ALL, failed ? 1 : 0, 0)) break;
+        if (what && (int)lane == from && it < n_items) book(it, what);
     }
     if (lane == 0) {
         if (failed) {
@@ -327,8 +335,9 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 1) cs_mover_bulk_kernel(MoverAr
     bulk_pipeline<STAGES>(my_ring, pipes[threadIdx.x >> 5], items_of_pipe(total, first, n_pipes), a.status,
                           [&](unsigned long long it) { return fetch_slots(a, first + it * n_pipes, per_block); },
                           [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes) {
-                              return resolve_piece(a, first + it * n_pipes, per_block, slots, sp, dp, bytes, true);
-                          });
+                              return resolve_piece(a, first + it * n_pipes, per_block, slots, sp, dp, bytes);
+                          },
+                          [&](unsigned long long, uint32_t what) { book_block(a, what); });
 }
 
 // Two transfers in opposite directions over the host link in one launch.  Every pipeline takes its
@@ -361,8 +370,12 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 1) cs_exchange_bulk_kernel(Move
                           },
                           [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes) {
                               unsigned long long w;
-                              return offloads(it, w) ? resolve_piece(off, w, per_block, slots, sp, dp, bytes, true)
-                                                     : resolve_piece(pre, w, per_block, slots, sp, dp, bytes, true);
+                              return offloads(it, w) ? resolve_piece(off, w, per_block, slots, sp, dp, bytes)
+                                                     : resolve_piece(pre, w, per_block, slots, sp, dp, bytes);
+                          },
+                          [&](unsigned long long it, uint32_t what) {
+                              unsigned long long w;
+                              book_block(offloads(it, w) ? off : pre, what);
                           });
 }
 

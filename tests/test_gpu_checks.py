@@ -264,3 +264,35 @@ def test_phase_stamps_need_the_profiling_build():
     with pytest.raises(cs.CacheScoutError) as e:
         c.phase_stamps()
     assert e.value.code == cs.CS_ENOTIMPL
+
+
+@pytest.mark.parametrize("width", [1, 2, 0])
+@pytest.mark.parametrize("path", [cs.CS_MOVER_BULK, cs.CS_MOVER_LDST])
+def test_every_list_entry_is_booked_once(width, path):
+    """Moved, skipped and bad entries where a pipeline walks many batches of 32 pieces (one or two pipelines for hundreds of pieces, blocks
+    that start anywhere in a batch): one booking per entry, in either direction and in the two-way transfer."""
+    L, chunk, G, n = 3, 2064, 150, 131                       # 6 runs of 2 pieces per block
+    rng = synth.rng_for(synth.CONFIGS["tiny"], 83)
+    c = cs.CacheScout(cs.make_params(4), DEV)
+    c.set_mover_path(path)
+    c.set_mover_ctas(width, width)
+    mk = lambda buf, layout: cs.KVPool(buf, G, layout, L, n_kv_heads=1, head_dim=chunk, block_tokens=1, elem_bytes=1)
+    gpu, gpu2 = (mk(torch.zeros(G * L * 2 * chunk, dtype=torch.uint8, device=DEV), layout) for layout in (0, 1))
+    host = mk(torch.zeros(G * L * 2 * chunk, dtype=torch.uint8).pin_memory(), 1)
+    a, b = rng.permutation(G).astype(np.uint32)[:n], rng.permutation(G).astype(np.uint32)[:n]
+    a[[0, 31, 32, 77]] = orc.ID_NONE
+    b[[5, 77, 130]] = G + 1
+    moved, bad = n - 6, 2                                    # (entry 77 is skipped for its sentinel)
+    for call, direction in ((lambda: c.compact_blocks(gpu, gpu2, dev(a), dev(b)), 0), (lambda: c.offload_blocks(gpu, host, dev(a), dev(b)), 1),
+                            (lambda: c.prefetch_blocks(host, gpu, dev(a), dev(b)), 2)):
+        c.counters(reset=True)
+        call()
+        cn = c.counters()
+        assert cn["blocks_moved"] == [moved if q == direction else 0 for q in range(3)]
+        assert cn["bytes_moved"][direction] == moved * L * 2 * chunk and cn["blocks_skipped"] == n - moved
+        assert c.get_status() == (cs.CS_ST_BAD_SLOT if bad else 0)
+    if path == cs.CS_MOVER_BULK:
+        c.counters(reset=True)
+        c.exchange_blocks(gpu, host, dev(a[:50].copy()), dev(b[:50].copy()), dev(b[50:].copy()), dev(a[50:].copy()))
+        cn = c.counters()
+        assert cn["blocks_moved"] == [0, 46, 79] and cn["blocks_skipped"] == 6 and c.get_status() == cs.CS_ST_BAD_SLOT

@@ -58,7 +58,8 @@ __device__ __forceinline__ void load_quad(const SelArgs &a, uint32_t q, Quad &Q)
 }
 
 // Ordering through global memory, for candidates the cluster's buckets cannot hold: a 1,024-key sample is sorted, every
-// candidate finds its bucket, the needed buckets are grouped and each is sorted in a shared-memory tile.
+// candidate finds its bucket, the needed buckets are grouped and each is sorted in shared memory (a padded bucket has room there: more
+// candidates than O.cap come here, and O.cap is then OR_ALL, a power of two).
 __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const OrderSmem &O, uint32_t c, uint32_t n_out,
                                                 uint32_t *__restrict__ ids_out)
 {
@@ -126,26 +127,19 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
     for (uint32_t b = rank; b <= b_last; b += CL) {
         const uint32_t beg = s_off[b], m = s_off[b + 1] - beg;
         __syncthreads();
-        if (m <= 2u * CSEL_THREADS) {
+        if (m <= O.cap) {
             uint32_t P = 64;
             while (P < m) P <<= 1;
             for (uint32_t i = tid; i < P; i += CSEL_THREADS) {
-                km_s[i] = i < m ? __ldcg(&ws.sort_km[beg + i]) : ~0ull;
-                id_s[i] = i < m ? __ldcg(&ws.sort_id[beg + i]) : 0xFFFFFFFFu;
+                O.all_km[i] = i < m ? __ldcg(&ws.sort_km[beg + i]) : ~0ull;
+                O.all_id[i] = i < m ? __ldcg(&ws.sort_id[beg + i]) : 0xFFFFFFFFu;
             }
             __syncthreads();
-            bitonic_sort_fast(km_s, id_s, P, whole_cta());
+            if (P <= 2u * CSEL_THREADS) bitonic_sort_fast(O.all_km, O.all_id, P, whole_cta());
+            else sort_tile(O.all_km, O.all_id, P);
             for (uint32_t i = tid; i < m; i += CSEL_THREADS)
-                if (beg + i < n_out) ids_out[beg + i] = id_s[i];
-        } else if (m <= OR_ALL) {                    // a large bucket: ranked straight from global memory
-            for (uint32_t i = tid; i < m; i += CSEL_THREADS) {
-                const u64 km = __ldcg(&ws.sort_km[beg + i]);
-                const uint32_t id = __ldcg(&ws.sort_id[beg + i]);
-                uint32_t r = 0;
-                for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(&ws.sort_km[beg + q]), __ldcg(&ws.sort_id[beg + q]), km, id);
-                if (beg + r < n_out) ids_out[beg + r] = id;
-            }
-        } else {                                     // beyond that counting, which grows with the square, would take milliseconds to seconds
+                if (beg + i < n_out) ids_out[beg + i] = O.all_id[i];
+        } else {                                     // more than shared memory holds
             uint32_t *list = ws.cand_bkt + beg;      // (the candidates' buckets are no longer wanted; nobody else's part of the array)
             for (uint32_t i = tid; i < m; i += CSEL_THREADS) list[i] = i;
             __syncthreads();

@@ -552,3 +552,35 @@ __device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32
     if (act) { km[2 * t] = k0; km[2 * t + 1] = k1; id[2 * t] = i0; id[2 * t + 1] = i1; }
     part_sync(cp);
 }
+
+// ---------------------------------------------------------------------------------------------
+// Sorts the first m keys of a shared-memory tile ascending (bitonic; m is padded to a power of two, which the tile has to hold,
+// with keys that sort last).  Whole CTA.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void sort_tile(unsigned long long *t_km, uint32_t *t_id, uint32_t m)
+{
+    uint32_t P = 64;
+    while (P < m) P <<= 1;
+    for (uint32_t i = m + threadIdx.x; i < P; i += blockDim.x) { t_km[i] = ~0ull; t_id[i] = 0xFFFFFFFFu; }
+    __syncthreads();
+    if (P <= 2 * blockDim.x) {
+        bitonic_sort_fast(t_km, t_id, P, whole_cta());
+        return;
+    }
+    for (uint32_t size = 2; size <= P; size <<= 1) {
+        for (uint32_t stride = size >> 1; stride > 0; stride >>= 1) {
+            for (uint32_t t = threadIdx.x; t < P / 2; t += blockDim.x) {
+                const uint32_t lo = 2 * t - (t & (stride - 1));
+                const uint32_t hi = lo + stride;
+                const bool up = (lo & size) == 0;
+                const unsigned long long ka = t_km[lo], kb = t_km[hi];
+                const uint32_t ia = t_id[lo], ib = t_id[hi];
+                if (key_less(kb, ib, ka, ia) == up) {
+                    t_km[lo] = kb; t_id[lo] = ib;
+                    t_km[hi] = ka; t_id[hi] = ia;
+                }
+            }
+            __syncthreads();
+        }
+    }
+}

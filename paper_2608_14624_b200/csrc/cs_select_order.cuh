@@ -12,7 +12,9 @@
 //               inside it and counts within the parts;
 //   more        the whole cluster ranks a sample of 512 or 1,024.  Where the output is a small part of the candidates, what
 //               lies beyond it is dropped and the rest is looked at afresh; else the keys go to up to 256 buckets, one
-//               range each, whose keys are counted by the warps of one CTA, 32 at a time.
+//               range each, whose keys are counted by the warps of one CTA, 32 at a time;
+//   long lists  (more than 28,672 ids) are not ordered here: a bucket of m keys takes m^2 comparisons, and 256 buckets are all there
+//               are.  The caller's sample sort does them (OR_LONG).
 //
 // What CTAs hand each other goes through L2, in runs: distributed shared memory moves scattered 8-byte words at about one
 // per four cycles and SM (handing the ranked sample of 1,024 to 16 CTAs that way took 8.6 us with the ranking, 6.4 us through L2;
@@ -31,6 +33,9 @@ namespace cg = cooperative_groups;
 #define OR_WARPS (OR_THREADS / 32u)
 #define OR_ALL 4096u              // candidates a CTA holds at once
 #define OR_BUCKETS 256u
+// Longest list whose buckets are counted: 112 keys per bucket on average.  Per select of 262,144 entries, counted / sorted (us):
+// k = 24,577 77 / 96, 32,768 108 / 103, 65,536 1,044 / 144, all 112,700 446 / 229.
+#define OR_LONG (112u * OR_BUCKETS)
 #define OR_SAMPLE CS_SAMPLE       // largest sample
 #define OR_SMALL_SAMPLE 128u
 #define OR_PART 256u              // keys of a part of a CTA's range (few candidates)
@@ -243,7 +248,8 @@ __device__ __noinline__ void order_few(const OrderSmem &O, const u64 *src_km, co
 
 // What order_candidates reports.
 struct OrderResult {
-    bool done;                // false: the buckets overflowed or a sample misled (nothing was stored); the candidates are in src
+    bool done;                // false: the list is too long, the buckets overflowed or a sample misled (nothing was stored); the candidates
+                              // are in src
 };
 
 // c > 0 candidates in B.src, n_out > 0.  Every CTA of the cluster calls, after a cluster barrier; the candidates' writes are
@@ -262,7 +268,7 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
             order_few(O, B.src_km, B.src_id, c, n_out, ids_out);
             return OrderResult{true};
         }
-        if (round == 6) return OrderResult{false};           // (every round drops most of the candidates)
+        if (n_out > OR_LONG || round == 6) return OrderResult{false};        // (every round drops most of the candidates)
         // ---- a sample, ranked by the cluster; CL lanes share a key ------------------------------------------------------
         const uint32_t S = c <= 12288u ? OR_SAMPLE / 2 : OR_SAMPLE;
         for (uint32_t s = tid; s < S; s += OR_THREADS) {
@@ -297,9 +303,9 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
         const uint32_t beg = (uint32_t)((unsigned long long)rank * c / CL), end = (uint32_t)((unsigned long long)(rank + 1u) * c / CL);
         const bool fill = J >= 96u;                                 // enough samples below the cut to split the output evenly
         const uint32_t nb = J < OR_BUCKETS ? J : OR_BUCKETS;
-        // (no more than a warp can rank by counting: the workspace may have been made for a far larger index than this one, and a sample
-        // that misleads may put nearly all candidates into one bucket)
-        const uint32_t cap = min(B.dst_cap / nb, OR_ALL);
+        // (no more than a CTA holds: the workspace may have been made for a far larger index than this one, and a sample that misleads
+        // may put nearly all candidates into one bucket)
+        const uint32_t cap = min(B.dst_cap / nb, O.cap);
         // ---- what lies below the cut: into buckets, or into dst for another round ----------------------------------------
         for (uint32_t i0 = beg; i0 < end; i0 += 4u * OR_THREADS) {
             u64 km[4];
@@ -372,46 +378,31 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
         cluster.barrier_arrive();                                   // (the leader's flag has been read; waited for at the end)
         __syncthreads();
         const uint32_t per = nb > rank ? (nb - rank + CL - 1u) / CL : 0u;      // this CTA's buckets
-        bool ok = !O.misc[OM_TOTAL] && total >= n_out;
-        uint32_t need = 0;
-        if (ok) {
-            // keys into shared memory, a warp per bucket in turn; buckets beyond the output are left out
-            for (uint32_t lb = 0; lb < per; ++lb) {
-                const uint32_t g = lb * CL + rank, m = O.cnt[g];
-                if (O.off[g] >= n_out) break;                       // (offsets grow with the bucket)
-                if ((lb & (OR_WARPS - 1u)) == warp && need + m <= O.cap)
+        const bool ok = !O.misc[OM_TOTAL] && total >= n_out;
+        // as many buckets at a time as shared memory holds (one always fits), up to the end of the output (offsets grow with the bucket)
+        for (uint32_t first = 0; ok && first < per && O.off[first * CL + rank] < n_out;) {
+            uint32_t need = 0, last = first;
+            for (; last < per; ++last) {                            // keys into shared memory, a warp per bucket in turn
+                const uint32_t g = last * CL + rank, m = O.cnt[g];
+                if (O.off[g] >= n_out || need + m > O.cap) break;
+                if ((last & (OR_WARPS - 1u)) == warp)
                     for (uint32_t i = lane; i < m; i += 32u) {
                         O.all_km[need + i] = __ldcg(B.dst_km + (size_t)g * cap + i);
                         O.all_id[need + i] = __ldcg(B.dst_id + (size_t)g * cap + i);
                     }
                 need += m;
             }
-        }
-        __syncthreads();
-        if (ok && need <= O.cap) {
+            __syncthreads();
             uint32_t item = 0, at = 0;
-            for (uint32_t lb = 0; lb < per; ++lb) {
+            for (uint32_t lb = first; lb < last; ++lb) {
                 const uint32_t g = lb * CL + rank, m = O.cnt[g];
-                if (O.off[g] >= n_out) break;
                 for (uint32_t k0 = 0; k0 < m; k0 += 32u, ++item)    // items of 32 keys, dealt to the warps in turn
                     if ((item & (OR_WARPS - 1u)) == warp)
                         rank_item(O.all_km + at, O.all_id + at, m, k0, O.off[g], n_out, ids_out);
                 at += m;
             }
-        } else if (ok) {                                            // more than shared memory holds: straight from L2
-            for (uint32_t lb = warp; lb < per; lb += OR_WARPS) {
-                const uint32_t g = lb * CL + rank, m = O.cnt[g];
-                if (O.off[g] >= n_out) break;
-                const u64 *k_km = B.dst_km + (size_t)g * cap;
-                const uint32_t *k_id = B.dst_id + (size_t)g * cap;
-                for (uint32_t k = lane; k < m; k += 32u) {
-                    const u64 km = __ldcg(k_km + k);
-                    const uint32_t id = __ldcg(k_id + k);
-                    uint32_t r = 0;
-                    for (uint32_t q = 0; q < m; ++q) count_less(r, __ldcg(k_km + q), __ldcg(k_id + q), km, id);
-                    if (O.off[g] + r < n_out) ids_out[O.off[g] + r] = id;
-                }
-            }
+            first = last;
+            __syncthreads();                                        // (before the next buckets take their place)
         }
         cluster.barrier_wait();
         return OrderResult{ok};

@@ -272,6 +272,51 @@ def test_samples_that_mislead_a_cluster(max_blocks, k, seen_are_old):
     assert c.get_status() == 0
 
 
+def test_buckets_of_one_cta_beyond_its_shared_memory():
+    """The single-launch select with six buckets of 3,500 keys, all of them the first CTA's (every 16th bucket): it holds 4,096 keys at a
+    time.  Of 131,072 candidates the sample sees every 32nd of the first 32,768, whose keys mark where the buckets lie; a workspace large
+    enough for regions of that size."""
+    n, k = 131_072, 20_000
+    p = cs.make_params(n_agents=2, max_blocks=1_000_000)
+    c, o = cs.CacheScout(p, DEV), orc.Oracle(H.oracle_params(p))
+    idx = synth.make_block_index(synth.shrink(synth.CONFIGS["tiny"], n_agents=2), n=n)
+    rng = synth.rng_for(synth.CONFIGS["tiny"], 80)
+    idx.flags[:], idx.ref_count[:], idx.agent[:], idx.n_tokens[:] = synth.FLAG_VALID, 0, 0, p.block_tokens
+    marks = np.arange(0, 32_768, 32)
+    others = np.setdiff1d(np.arange(n), marks)
+    idx.last_access[others] = rng.integers(50_000, 60_000, len(others))
+    idx.last_access[marks] = 1_000 + 10 * rng.permutation(len(marks))
+    for q, bucket in enumerate(range(0, 96, 16)):
+        ids = others[q * 20_000:q * 20_000 + 3_500]
+        idx.last_access[ids] = 1_000 + 10 * bucket + rng.integers(1, 10, len(ids))
+    s64, s32 = o.scores(idx, 100_000)
+    assert len(np.unique(s32)) == 1
+    want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    for _ in range(3):
+        ids, cnt = c.select_victims(d, 100_000, 0, k)
+        assert H.assert_list_matches(ids.cpu().numpy().view(np.uint32)[:k], int(cnt.item()), want, n_want, s64) == 0
+    assert c.get_status() == 0
+
+
+@pytest.mark.parametrize("k", [28_671, 28_672, 28_673, 60_000, 110_000])
+def test_long_lists_of_the_single_launch(k):
+    """Around the longest list whose buckets are counted, and far beyond it; all three lists of a step side by side."""
+    cfg = synth.CONFIGS["llama8b"]
+    n = 262_144
+    c, o = warm_state(cfg, 1000, n, r_min=0.02)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    s64, s32 = o.scores(idx, 100_000)
+    want = [o.select_victims(idx, 100_000, 0, k, s32), o.select_victims(idx, 100_000, 1, k, s32), o.select_prefetch(idx, 100_000, k, s32)]
+    bufs = [torch.full((m,), 7, dtype=torch.int32, device=DEV) for _ in range(3) for m in (k + 3 & ~3, 1)]
+    c.select_step(d, 100_000, k, k, *bufs)
+    ids, cnt = c.select_victims(d, 100_000, 0, k)
+    for got, got_n, (w, wn) in ((bufs[0], bufs[1], want[0]), (bufs[2], bufs[3], want[1]), (bufs[4], bufs[5], want[2]), (ids, cnt, want[0])):
+        assert H.assert_list_matches(got.cpu().numpy().view(np.uint32)[:k], int(got_n.item()), w, wn, s64) == 0
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("eligible,k", [(1, 1), (255, 255), (257, 20), (1024, 1024), (1025, 1), (2047, 2047), (2048, 700), (2048, 2048),
                                         (2049, 3000), (2049, 1300)])
 @pytest.mark.parametrize("tied", [False, True])

@@ -1028,6 +1028,25 @@ def test_samples_that_mislead(k, seen_are_old):
 
 
 # ---- hop table from every live session's current agent ----------------------------------------------------
+@pytest.mark.parametrize("A", [12, 200, 700])
+@pytest.mark.parametrize("chains", [1, 7, 8, 9, 8197, 100_003])
+def test_sources_of_many_chains(A, chains):
+    """Every chain's current agent as a source of the search, with chain counts around the eight that are read at once and the rounds
+    they are read in; few agents, so that most chains bring one that another has brought, and chains that have none."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=chains)
+    c, o = make_ctx(cfg, 64, tau=0.02)
+    c.set_survival_sources(cs.CS_SOURCES_ALL_CHAINS)
+    rng = synth.rng_for(cfg, 91)
+    for size, agents in ((3, A // 2), (chains + 300, A // 2), (200, A)):      # (the last batch rides with the refresh)
+        chain = rng.permutation(chains + size)[:size].astype(np.uint32) % chains
+        agent = rng.integers(0, agents, size).astype(np.uint16)
+        c.observe_invocations(dev(chain), dev(agent), None)
+        o.observe(chain, agent)
+        o.survival(sources=np.unique(o.cur[o.cur != orc.AGENT_NONE]))
+        H.compare_model(c, o)
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("name,n_inv", [("tiny", 60), ("llama8b", 400), ("meta1m", 3000)])
 def test_survival_from_all_chains(name, n_inv):
     """CS_SOURCES_ALL_CHAINS: the cached BFS starts at the current agent of every chain; the oracle runs its

@@ -78,11 +78,13 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
         }
         __syncthreads();
         bitonic_sort_fast(km_s, id_s, CS_SAMPLE, whole_cta());
+        // buckets of about 384 keys, which a CTA sorts in little more time than 128, but a bucket for every CTA at least
+        const uint32_t n_spl = min(CS_MAX_SPLITTERS, max(c / 384u, CL));
         for (uint32_t j = tid; j <= CS_MAX_SPLITTERS; j += CSEL_THREADS) {
             if (j < CS_MAX_SPLITTERS) {
-                const uint32_t q = (uint32_t)(((unsigned long long)(j + 1) * CS_SAMPLE) / (CS_MAX_SPLITTERS + 1));
-                ws.spl_km[j] = km_s[q];
-                ws.spl_id[j] = id_s[q];
+                const uint32_t q = (j + 1u) * CS_SAMPLE / (n_spl + 1u);
+                ws.spl_km[j] = j < n_spl ? km_s[q] : ~0ull;      // (behind every key: the buckets beyond stay empty)
+                ws.spl_id[j] = j < n_spl ? id_s[q] : 0xFFFFFFFFu;
             }
             CS_BCOUNT(ws, j) = 0;
         }

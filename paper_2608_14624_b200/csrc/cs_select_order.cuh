@@ -13,7 +13,7 @@
 //   more        the whole cluster ranks a sample of 512 or 1,024.  Where the output is a small part of the candidates, what
 //               lies beyond it is dropped and the rest is looked at afresh; else the keys go to up to 256 buckets, one
 //               range each, whose keys are counted by the warps of one CTA, 32 at a time;
-//   long lists  (more than 28,672 ids) are not ordered here: a bucket of m keys takes m^2 comparisons, and 256 buckets are all there
+//   long lists  (more than 30,720 ids) are not ordered here: a bucket of m keys takes m^2 comparisons, and 256 buckets are all there
 //               are.  The caller's sample sort does them (OR_LONG).
 //
 // What CTAs hand each other goes through L2, in runs: distributed shared memory moves scattered 8-byte words at about one
@@ -33,9 +33,10 @@ namespace cg = cooperative_groups;
 #define OR_WARPS (OR_THREADS / 32u)
 #define OR_ALL 4096u              // candidates a CTA holds at once
 #define OR_BUCKETS 256u
-// Longest list whose buckets are counted: 112 keys per bucket on average.  Per select of 262,144 entries, counted / sorted (us):
-// k = 24,577 77 / 96, 32,768 108 / 103, 65,536 1,044 / 144, all 112,700 446 / 229.
-#define OR_LONG (112u * OR_BUCKETS)
+// Longest list whose buckets are counted: 120 keys per bucket on average.  Per select of 262,144 entries, counted / sorted (us):
+// k = 28,672 80 - 93 / 89, 32,768 103 - 108 / 94, 65,536 878 - 1,095 / 143 - 160, all 112,700 415 - 432 / 221 - 228 (the lower figures with
+// every entry of one age).
+#define OR_LONG (120u * OR_BUCKETS)
 #define OR_SAMPLE CS_SAMPLE       // largest sample
 #define OR_SMALL_SAMPLE 128u
 #define OR_PART 256u              // keys of a part of a CTA's range (few candidates)

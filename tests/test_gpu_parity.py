@@ -299,7 +299,7 @@ def test_buckets_of_one_cta_beyond_its_shared_memory():
     assert c.get_status() == 0
 
 
-@pytest.mark.parametrize("k", [28_671, 28_672, 28_673, 60_000, 110_000])
+@pytest.mark.parametrize("k", [30_719, 30_720, 30_721, 60_000, 110_000])
 def test_long_lists_of_the_single_launch(k):
     """Around the longest list whose buckets are counted, and far beyond it; all three lists of a step side by side."""
     cfg = synth.CONFIGS["llama8b"]

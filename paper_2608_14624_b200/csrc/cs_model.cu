@@ -451,22 +451,27 @@ __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &
     if (all_chains) {
         // sources: the current agent of every chain that has one (all live sessions)
         __syncthreads();
-        // (eight chains to a load; an agent that another chain has brought costs a look, not an atomic)
+        // (many chains: eight to a load; an agent that another chain has brought costs a look, not an atomic)
         auto source = [&](uint32_t a) {
             if (a < A && !((*(volatile uint32_t *)&sm.front[a >> 5] >> (a & 31)) & 1u)) atomicOr(&sm.front[a >> 5], 1u << (a & 31));
         };
-        const uint32_t n8 = n_chains / 8u;
-        for (uint32_t x0 = tid; x0 < n8; x0 += 4u * n_threads) {
-            uint4 v[4];                                       // (a round's loads travel together)
+        if (n_chains <= 4u * n_threads) {
+            for (uint32_t x = tid; x < n_chains; x += n_threads) source(__ldcg(&ws.cur[x]));
+        } else {
+            const uint32_t n8 = n_chains / 8u;
+            for (uint32_t x0 = tid; x0 < n8; x0 += 4u * n_threads) {
+                uint4 v[4];                                   // (a round's loads travel together)
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) v[u] = cs_ld_cg_pinned((const uint4 *)ws.cur + min(x0 + u * n_threads, n8 - 1u));
+                for (uint32_t u = 0; u < 4; ++u) v[u] = cs_ld_cg_pinned((const uint4 *)ws.cur + min(x0 + u * n_threads, n8 - 1u));
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {                // (the last one again where there is no other)
-                source(v[u].x & 0xFFFFu); source(v[u].x >> 16); source(v[u].y & 0xFFFFu); source(v[u].y >> 16);
-                source(v[u].z & 0xFFFFu); source(v[u].z >> 16); source(v[u].w & 0xFFFFu); source(v[u].w >> 16);
+                for (uint32_t u = 0; u < 4; ++u) {
+                    if (x0 + u * n_threads >= n8) break;
+                    source(v[u].x & 0xFFFFu); source(v[u].x >> 16); source(v[u].y & 0xFFFFu); source(v[u].y >> 16);
+                    source(v[u].z & 0xFFFFu); source(v[u].z >> 16); source(v[u].w & 0xFFFFu); source(v[u].w >> 16);
+                }
             }
+            if (tid < (n_chains & 7u)) source(__ldcg(&ws.cur[(n_chains & ~7u) + tid]));
         }
-        if (tid < (n_chains & 7u)) source(__ldcg(&ws.cur[(n_chains & ~7u) + tid]));
         __syncthreads();
     }
     // The search by the first W warps; the sums of Eq. 2 by the warps behind them, side by side, where the CTA has enough of

@@ -1029,10 +1029,10 @@ def test_samples_that_mislead(k, seen_are_old):
 
 # ---- hop table from every live session's current agent ----------------------------------------------------
 @pytest.mark.parametrize("A", [12, 200, 700])
-@pytest.mark.parametrize("chains", [1, 7, 8, 9, 8197, 100_003])
+@pytest.mark.parametrize("chains", [1, 9, 1023, 1025, 4099, 8197, 100_003])
 def test_sources_of_many_chains(A, chains):
-    """Every chain's current agent as a source of the search, with chain counts around the eight that are read at once and the rounds
-    they are read in; few agents, so that most chains bring one that another has brought, and chains that have none."""
+    """Every chain's current agent as a source of the search, with chain counts around the lines from which they are read eight at a time
+    and the rounds they are read in; few agents, so that most chains bring one that another has brought, and chains that have none."""
     cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, n_chains=chains)
     c, o = make_ctx(cfg, 64, tau=0.02)
     c.set_survival_sources(cs.CS_SOURCES_ALL_CHAINS)

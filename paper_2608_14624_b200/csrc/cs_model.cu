@@ -930,12 +930,13 @@ cs_survival_kernel(cs_workspace ws, uint32_t A, uint32_t W, const uint16_t *__re
 // for its targets in shared memory, [agent][target], and its columns of the new V go to every CTA of the cluster through
 // distributed shared memory); inside a CTA a warp owns 64 columns (two per lane, 16 accumulators) and a slice of the
 // agents summed over, so that 16 warps stay busy however few the columns; the slices' partial sums meet in shared memory.
-// P comes from global memory; a CTA's columns stay in its L1 for the later steps.  The last step needs column a only: one
-// dot product per target, one warp each.
+// P comes from global memory (a CTA on its own finds its columns in its L1 in the later steps; a cluster barrier makes L1 forget
+// them).  The last step needs column a only: one dot product per target, one warp each.
 //
 // Bound by the fp64 pipe for many agents (2 A^3 (K - 2) operations), by latency for few.  256 agents, K = 4: 62.7 us with
 // one CTA per 8 targets that walked the matrix column by column (32 CTAs, one serial chain of 256 loads per step),
-// 13.7 us per call like this (128 CTAs).
+// 13.7 us per call like this (128 CTAs).  Few agents, one CTA, K = 32, with cluster barriers / with its own: 4 agents 42 / 17 us,
+// 12 44 / 25, 64 85 / 42.
 // ---------------------------------------------------------------------------------------------
 #define XS_TARGETS 8u
 #define XS_THREADS 512u
@@ -973,21 +974,27 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
             const uint32_t j = e / XS_TARGETS, m = e % XS_TARGETS;
             v_all[e] = j == base + m ? 0.0 : (double)P[(size_t)a0 * A + j];
         }
-        cluster.sync();                                            // (also: every CTA has started before its memory is written)
-        const uint32_t col_warps = (n_cols + 63u) / 64u, slices = XS_WARPS / col_warps;
+        // what does not change from step to step: this warp's columns and its slice of the agents summed over (no slice
+        // of fewer than eight agents, because the slices' sums are added up one after the other: 64 agents, K = 32 41.5 us, with four 50.8)
+        const uint32_t col_warps = (n_cols + 63u) / 64u, slices = min(XS_WARPS / col_warps, max(2u, (A + 7u) / 8u));
         const uint32_t cw = warp % col_warps, sl = warp / col_warps;
+        const uint32_t j0 = col0 + cw * 64u + lane, j1 = j0 + 32u, mine = col1 > col0 ? col1 - col0 : 0u;
+        const float *const p0 = P + (j0 < col1 ? j0 : 0u), *const p1 = P + (j1 < col1 ? j1 : 0u);    // (columns past the end: unused)
+        const uint32_t i_beg = sl * A / slices, i_end = (sl + 1u) * A / slices;
+        // (a CTA on its own keeps to its own barrier: a cluster's makes its L1 forget the matrix)
+        const auto everywhere = [&] { if (CL > 1) cluster.sync(); else __syncthreads(); };
+        everywhere();                                              // (also: every CTA has started before its memory is written)
         uint32_t cur = 0;
         for (uint32_t t = 1; t + 1 < K; ++t) {
             const double *v = v_all + (size_t)cur * A * XS_TARGETS;
+            double *const nxt = v_all + (size_t)(cur ^ 1u) * A * XS_TARGETS;
+            cur ^= 1u;
             if (sl < slices) {
-                const uint32_t j0 = col0 + cw * 64u + lane, j1 = j0 + 32u;
-                const float *p0 = P + (j0 < col1 ? j0 : 0u), *p1 = P + (j1 < col1 ? j1 : 0u);    // (columns past the end: unused)
-                const uint32_t i_end = (uint32_t)((unsigned long long)(sl + 1u) * A / slices);
                 double acc0[XS_TARGETS], acc1[XS_TARGETS];
 #pragma unroll
                 for (uint32_t m = 0; m < XS_TARGETS; ++m) acc0[m] = acc1[m] = 0.0;
 #pragma unroll 8
-                for (uint32_t i = (uint32_t)((unsigned long long)sl * A / slices); i < i_end; ++i) {
+                for (uint32_t i = i_beg; i < i_end; ++i) {
                     const double x0 = (double)__ldg(p0 + (size_t)i * A), x1 = (double)__ldg(p1 + (size_t)i * A);
                     const double2 *vi = (const double2 *)(v + (size_t)i * XS_TARGETS);
 #pragma unroll
@@ -1004,17 +1011,18 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
                 for (uint32_t m = 0; m < XS_TARGETS; ++m) { o[m * XS_PART_ROW] = acc0[m]; o[m * XS_PART_ROW + 32u] = acc1[m]; }
             }
             __syncthreads();
-            double *nxt = v_all + (size_t)(cur ^ 1u) * A * XS_TARGETS;
-            for (uint32_t e = tid; e < (col1 > col0 ? col1 - col0 : 0u) * XS_TARGETS; e += XS_THREADS) {
+            for (uint32_t e = tid; e < mine * XS_TARGETS; e += XS_THREADS) {
                 const uint32_t jc = e / XS_TARGETS, m = e % XS_TARGETS, j = col0 + jc;
                 const double *q = part + (size_t)(jc / 64u) * XS_TARGETS * XS_PART_ROW + m * XS_PART_ROW + jc % 64u;
                 double sum = 0.0;
                 for (uint32_t u = 0; u < slices; ++u) sum += q[(size_t)u * col_warps * XS_TARGETS * XS_PART_ROW];
                 if (j == base + m) { s_hit[m] += sum; sum = 0.0; }   // (one thread per target)
-                for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)j * XS_TARGETS + m] = sum;
+                if (CL > 1)
+                    for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)j * XS_TARGETS + m] = sum;
+                else
+                    nxt[(size_t)j * XS_TARGETS + m] = sum;
             }
-            cluster.sync();                                        // the new V is complete everywhere; `part` is free again
-            cur ^= 1u;
+            everywhere();                                          // the new V is complete everywhere; `part` is free again
         }
         if (K > 1 && warp < XS_TARGETS && base + warp < A && owner(base + warp)) {
             const double *v = v_all + (size_t)cur * A * XS_TARGETS + warp;

@@ -740,7 +740,7 @@ def test_exact_survival_parity_and_select(name, K):
 
 
 @pytest.mark.parametrize("A,Ks", [(1, (0, 1, 3)), (2, (2, 5)), (9, (3, 6)), (64, (4,)), (65, (2, 4)), (130, (3, 4)), (296, (4,)), (700, (4,)),
-                                  (1024, (3,))])
+                                  (1024, (3,)), (4, (1, 2, 3, 33)), (7, (5,)), (8, (4, 32)), (12, (32,)), (57, (3, 9)), (593, (5,))])
 def test_exact_survival_table_shapes(A, Ks):
     """Agent counts on both sides of the target groups (8), the column tiles (64) and every cluster size, with the step
     counts that take no product (0, 1, 2) and several; both outputs.  Bound: the oracle multiplies K entries of the fp64

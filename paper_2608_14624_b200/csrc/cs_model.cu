@@ -117,6 +117,8 @@ cs_observe_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, const uint32_t
     if (n_events_dev) n_events = min(n_events, *n_events_dev);   // device-resident count (graph replay)
     const uint32_t rounds = (n_events + CL * OBS_THREADS - 1) / (CL * OBS_THREADS);
     const uint32_t share = rounds ? (n_events + rounds * CL - 1) / (rounds * CL) : 0u;      // events per CTA and round
+    // (a CTA on its own needs no cluster barriers, and with one round nothing it looks up in cur[] changes before it does)
+    const auto everywhere = [&] { if (CL > 1) cluster.sync(); else __syncthreads(); };
     const bool local = A <= OBS_SMEM_AGENTS;
     if (local) {
         for (uint32_t i = tid; i < A * A; i += OBS_THREADS) s_C[i] = 0;
@@ -137,6 +139,8 @@ cs_observe_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, const uint32_t
             if (warm || bad) { c = OBS_NO_CHAIN; a = CS_AGENT_NONE; ++n_skipped; }
         }
         const bool live = a != CS_AGENT_NONE;
+        uint32_t carried = CS_AGENT_NONE;                        // in flight during the searches below
+        if (live && rounds == 1u) carried = cs_ld_cg_pinned(ws.cur + c);
         s_chain[tid] = c;
         sh.agent[tid] = (uint16_t)a;
         for (uint32_t i = tid; i < OBS_HASH; i += OBS_THREADS) { sh.h_chain[i] = OBS_NO_CHAIN; h_warps[i] = 0; }
@@ -185,14 +189,14 @@ cs_observe_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, const uint32_t
         }
         const bool last_in_cta = last_in_warp && (wm >> warp) == 1u;
         if (last_in_cta) sh.h_last[slot] = (uint16_t)a;
-        cluster.sync();                                          // every table of the cluster is complete
+        everywhere();                                            // every table of the cluster is complete
         if (need_far) {
             for (int r = (int)rank - 1; r >= 0 && prev == CS_AGENT_NONE; --r) {
                 const ObsShare *o = cluster.map_shared_rank(&sh, r);
                 const uint32_t s = obs_find(o->h_chain, c);
                 if (s < OBS_HASH) prev = o->h_last[s];
             }
-            if (prev == CS_AGENT_NONE) prev = __ldcg(&ws.cur[c]);
+            if (prev == CS_AGENT_NONE) prev = rounds == 1u ? carried : (uint32_t)__ldcg(&ws.cur[c]);
         }
         bool writes_cur = last_in_cta;
         for (uint32_t r = rank + 1; r < CL && writes_cur; ++r)
@@ -213,7 +217,7 @@ cs_observe_kernel(cs_workspace ws, uint32_t A, uint32_t n_chains, const uint32_t
                 atomicAdd(&ws.rowsum[prev], 1u);
             }
         }
-        cluster.sync();                                          // every read of cur[] and of the tables precedes the writes below
+        everywhere();                                            // every read of cur[] and of the tables precedes the writes below
         if (writes_cur) ws.cur[c] = (uint16_t)a;
         if (newest != CS_AGENT_NONE) ws.sc->last_agent = newest;
     }
@@ -1156,7 +1160,7 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
         const uint32_t most = obs_cluster_limit(ctx->device);
         uint32_t cl = 1;
         while (cl < most && cl * OBS_THREADS < n_events) cl <<= 1;
-        cs_launch_chained_clusters(cs_observe_kernel, cl, cl, OBS_THREADS, 0, s, ctx->ws, p.n_agents, p.n_chains, chain, agent,
+        cs_launch_chained_clusters(cs_observe_kernel, cl, cl > 1u ? cl : 0u, OBS_THREADS, 0, s, ctx->ws, p.n_agents, p.n_chains, chain, agent,
                                    evflags, n_events, ctx->step_n_events_dev);
         int rc = cs_check_launch(ctx);
         if (rc != CS_OK) return rc;

@@ -67,39 +67,37 @@ __device__ __forceinline__ uint2 fetch_slots(const MoverArgs &a, unsigned long l
     return make_uint2(a.src_slots ? __ldg(a.src_slots + i) : i, a.dst_slots ? __ldg(a.dst_slots + i) : i);
 }
 
-// Resolves work item w to a source / destination address and a byte count; `bytes` is 0 when there is nothing to copy.  Returns what the
-// work counters are owed for it -- one piece per block does the block's bookkeeping, so 0 for all others -- to be handed to book_block()
-// when the piece's turn has come.
-enum : uint32_t { BOOK_NOTHING = 0, BOOK_MOVED, BOOK_SKIPPED, BOOK_BAD_SLOT, BOOK_SECOND = 4 /* of the two transfers of a launch */ };
-__device__ __forceinline__ uint32_t resolve_piece(const MoverArgs &a, unsigned long long w, uint32_t per_block, uint2 slots,
-                                                  const char *&sp, char *&dp, uint32_t &bytes)
+// Resolves work item w to a source / destination address and a byte count; false = skip.  One piece per block does the block's
+// bookkeeping: book = 1 adds it to the work counters, -1 takes it back (a bad slot stays reported: the list does hold it), 0 leaves them.
+__device__ __forceinline__ bool resolve_piece(const MoverArgs &a, unsigned long long w, uint32_t per_block, uint2 slots,
+                                              const char *&sp, char *&dp, uint32_t &bytes, int book)
 {
     const uint32_t i = (uint32_t)(w / per_block);
     const uint32_t r = (uint32_t)(w - (unsigned long long)i * per_block);
     const uint32_t lp = r / a.pieces, piece = r - lp * a.pieces;
     uint32_t s = slots.x, d = slots.y;
-    bytes = 0;
-    if (s == CS_ID_NONE || d == CS_ID_NONE) return r ? BOOK_NOTHING : BOOK_SKIPPED;
+    const bool first = book != 0 && r == 0;
+    const unsigned long long one = (unsigned long long)(long long)book;
+    if (s == CS_ID_NONE || d == CS_ID_NONE) {
+        if (first) atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, one);
+        return false;
+    }
     s -= a.src_first;                                   // ids below first_id wrap and fail the range check
     d -= a.dst_first;
-    if (s >= a.src_total || d >= a.dst_total) return r ? BOOK_NOTHING : BOOK_BAD_SLOT;
+    if (s >= a.src_total || d >= a.dst_total) {
+        if (first) { atomicOr(a.status, CS_ST_BAD_SLOT); atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, one); }
+        return false;
+    }
+    if (first) {
+        atomicAdd((unsigned long long *)&a.cnt->blocks_moved[a.kind], one);
+        atomicAdd((unsigned long long *)&a.cnt->bytes_moved[a.kind], one * a.block_bytes);
+    }
     const unsigned long long in_chunk = (unsigned long long)piece * a.piece_bytes;
     sp = a.src + chunk_offset(a.src_layout, a.n_chunks, a.src_total, lp, s, a.chunk) + in_chunk;
     dp = a.dst + chunk_offset(a.dst_layout, a.n_chunks, a.dst_total, lp, d, a.chunk) + in_chunk;
     const unsigned long long left = a.chunk - in_chunk;
     bytes = (uint32_t)(left < a.piece_bytes ? left : a.piece_bytes);
-    return r ? BOOK_NOTHING : BOOK_MOVED;
-}
-
-__device__ __forceinline__ void book_block(const MoverArgs &a, uint32_t what)
-{
-    if (what == BOOK_MOVED) {
-        atomicAdd((unsigned long long *)&a.cnt->blocks_moved[a.kind], 1ull);
-        atomicAdd((unsigned long long *)&a.cnt->bytes_moved[a.kind], a.block_bytes);
-    } else {
-        if (what == BOOK_BAD_SLOT) atomicOr(a.status, CS_ST_BAD_SLOT);
-        atomicAdd((unsigned long long *)&a.cnt->blocks_skipped, 1ull);
-    }
+    return true;
 }
 
 __device__ __forceinline__ uint32_t mover_count(const MoverArgs &a)
@@ -121,9 +119,7 @@ __global__ void __launch_bounds__(MV_THREADS) cs_mover_kernel(MoverArgs a)
         const char *sp0;
         char *dp0;
         uint32_t bytes;
-        const uint32_t what = resolve_piece(a, w, per_block, fetch_slots(a, w, per_block), sp0, dp0, bytes);
-        if (what && threadIdx.x == 0) book_block(a, what);
-        if (!bytes) continue;
+        if (!resolve_piece(a, w, per_block, fetch_slots(a, w, per_block), sp0, dp0, bytes, threadIdx.x == 0 ? 1 : 0)) continue;
         const uint4 *sp = (const uint4 *)sp0;
         uint4 *dp = (uint4 *)dp0;
         const uint32_t nvec = bytes >> 4;
@@ -216,17 +212,16 @@ __device__ __forceinline__ void bulk_store(void *dst, uint32_t src_smem, uint32_
 // cost as much time as moving 2 KiB); lane 0 issues the copies.  Iteration `it` first stores item it - LAG, whose load was
 // issued LAG iterations ago, and then issues the load of item `it` into the ring slot whose previous store has finished
 // reading shared memory.  `fetch(it)` looks an item's list entries up, a batch of 32 ahead of
-// `item(it, slots, sp, dp, bytes)`, which resolves it and returns what is to be booked: `book(what)` is called for every item whose load
-// has been issued (or that was found to have none), never for the items behind a wait that ran out -- by the item's lane, when the next
-// batch is due or the pipeline ends: bookings between the copies, one lane at a time, took a tenth of the time of 4 KiB pieces.
+// `item(it, slots, sp, dp, bytes, book)`, which resolves it; false = nothing to copy.  The work counters are booked with the batch; when a
+// wait runs out, what the batch holds from the item on whose load was never issued is taken back.
 template <int STAGES> struct PipeShared {
     unsigned long long bar[STAGES];
     char *dst[STAGES];                // destination of the item loaded into each ring slot
     uint32_t bytes[STAGES];           // 0: nothing in flight there
 };
-template <int STAGES, class Fetch, class Item, class Book>
+template <int STAGES, class Fetch, class Item>
 __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared<STAGES> &ps, unsigned long long n_items, uint32_t *status,
-                                              Fetch fetch, Item item, Book book)
+                                              Fetch fetch, Item item)
 {
     constexpr uint32_t PIECE = TM_RING / STAGES;
     constexpr int LAG = STAGES - (STAGES + 2) / 3;    // two thirds of the slots load, one third store
@@ -236,18 +231,16 @@ __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared
     uint32_t phase_bits = 0;          // parity to wait for, one bit per ring slot
     bool failed = false;
     char *sp = nullptr, *dp = nullptr;
-    uint32_t bytes = 0, what = 0;
-    unsigned long long turn = 0;      // the item that this lane has resolved, and `what` is owed for it
+    uint32_t bytes = 0;
     uint2 next = make_uint2(CS_ID_NONE, CS_ID_NONE);
     if (lane < n_items) next = fetch(lane);
     int st_load = 0, st_store = 0;    // ring slots of items it and it - LAG
-    for (unsigned long long it = 0; it < n_items + LAG; ++it) {
-        if ((it & 31u) == 0 && it < n_items) {                // resolve the next 32 items (those before have all had their turn)
+    unsigned long long it = 0;
+    for (; it < n_items + LAG; ++it) {
+        if ((it & 31u) == 0 && it < n_items) {                // resolve the next 32 items
             const char *s = nullptr;
-            if (what) book(what);
-            bytes = what = 0;
-            turn = it + lane;
-            if (turn < n_items) what = item(turn, next, s, dp, bytes);
+            bytes = 0;
+            if (it + lane < n_items && !item(it + lane, next, s, dp, bytes, 1)) bytes = 0;
             sp = const_cast<char *>(s);
             if (it + 32u + lane < n_items) next = fetch(it + 32u + lane);
         }
@@ -286,12 +279,13 @@ __device__ __forceinline__ void bulk_pipeline(unsigned char *my_ring, PipeShared
         }
         st_load = st_load + 1 == STAGES ? 0 : st_load + 1;
         if (it >= (unsigned long long)LAG) st_store = st_store + 1 == STAGES ? 0 : st_store + 1;
-        if (__shfl_sync(ALL, failed ? 1 : 0, 0)) {
-            if (turn >= it) what = 0;                         // (the load of item `it` was not issued)
-            break;
-        }
+        if (__shfl_sync(ALL, failed ? 1 : 0, 0)) break;
     }
-    if (what) book(what);
+    if (it < n_items) {                                       // a wait ran out before the load of item `it` was issued
+        const unsigned long long mine = (it & ~31ull) + lane;
+        const char *s;
+        if (mine >= it && mine < n_items) (void)item(mine, fetch(mine), s, dp, bytes, -1);
+    }
     if (lane == 0) {
         if (failed) {
             // give the loads still in flight a bounded chance to land before shared memory is released
@@ -341,10 +335,9 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 1) cs_mover_bulk_kernel(MoverAr
     const unsigned long long n_pipes = a.n_pipes;
     bulk_pipeline<STAGES>(my_ring, pipes[threadIdx.x >> 5], items_of_pipe(total, first, n_pipes), a.status,
                           [&](unsigned long long it) { return fetch_slots(a, first + it * n_pipes, per_block); },
-                          [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes) {
-                              return resolve_piece(a, first + it * n_pipes, per_block, slots, sp, dp, bytes);
-                          },
-                          [&](uint32_t what) { book_block(a, what); });
+                          [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes, int book) {
+                              return resolve_piece(a, first + it * n_pipes, per_block, slots, sp, dp, bytes, book);
+                          });
 }
 
 // Two transfers in opposite directions over the host link in one launch.  Every pipeline takes its
@@ -375,13 +368,11 @@ __global__ void __launch_bounds__(TM_WARPS * 32, 1) cs_exchange_bulk_kernel(Move
                               unsigned long long w;
                               return offloads(it, w) ? fetch_slots(off, w, per_block) : fetch_slots(pre, w, per_block);
                           },
-                          [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes) {
+                          [&](unsigned long long it, uint2 slots, const char *&sp, char *&dp, uint32_t &bytes, int book) {
                               unsigned long long w;
-                              if (offloads(it, w)) return resolve_piece(off, w, per_block, slots, sp, dp, bytes);
-                              const uint32_t what = resolve_piece(pre, w, per_block, slots, sp, dp, bytes);
-                              return what ? what | BOOK_SECOND : 0u;
-                          },
-                          [&](uint32_t what) { book_block(what & BOOK_SECOND ? pre : off, what & ~BOOK_SECOND); });
+                              return offloads(it, w) ? resolve_piece(off, w, per_block, slots, sp, dp, bytes, book)
+                                                     : resolve_piece(pre, w, per_block, slots, sp, dp, bytes, book);
+                          });
 }
 
 // ---------------------------------------------------------------------------------------------

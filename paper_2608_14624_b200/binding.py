@@ -385,7 +385,7 @@ def cs_debug_phase_stamps(ctx):
 
 
 def cs_set_select_bucket_regions(ctx, max_keys: int):
-    _chk(lib().cs_set_select_bucket_regions(ctx, int(max_keys)), "cs_set_select_bucket_regions", "cs_debug_phase_stamps")
+    _chk(lib().cs_set_select_bucket_regions(ctx, int(max_keys)), "cs_set_select_bucket_regions")
 
 
 def cs_set_select_path(ctx, path: int):

@@ -34,7 +34,7 @@ struct cs_nvtx_range {
 #define CS_MOVE_PREFETCH 2
 #define CS_MOVE_STAGE 3            // pack / scatter launch of the copy-engine path: inside the device, deliberately narrow
 
-#define CS_HIST_BINS 4096u        // first radix digit of the select: top 12 bits of the primary key
+#define CS_HIST_BINS 4096u        // bins of the select's histogram: the range that scores can have, divided evenly
 #define CS_MAX_SPLITTERS 255u     // bucket sort of the candidates: up to 256 buckets
 #define CS_SAMPLE 1024u           // candidates sampled to choose the splitters
 #define CS_BUCKETS 512u           // buckets of the grid-wide ordering
@@ -250,8 +250,8 @@ __device__ __forceinline__ float cs_survival_of(uint32_t hops, uint32_t e_max, f
     return (float)(ptilde + (double)delta);
 }
 
-// Programmatic dependent launch.  The chains of small kernels (observe -> normalise; histogram -> collect ->
-// bucket -> scatter -> rank) are bound by launch latency, so each kernel of a chain is launched with the
+// Programmatic dependent launch.  The chains of small kernels (observe -> refresh; scan -> histogram ->
+// collect -> sample -> place -> finish) are bound by launch latency, so each kernel of a chain is launched with the
 // programmatic-serialisation attribute: its launch overlaps the tail of its predecessor, and its first
 // instruction waits until the predecessor grid has completed and its writes are visible.  A kernel launched
 // without the attribute executes the wait as a no-op.

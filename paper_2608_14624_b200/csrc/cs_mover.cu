@@ -421,8 +421,8 @@ static void fill_mover_args(cs_ctx *ctx, MoverArgs &a, const cs_kv_pool *src, co
 //    split).  8 out, 24 in, 32 both ways; more for small pieces, whose issue takes longer than their flight (4 KiB pieces out:
 //    8 pipelines 51.0 GB/s, 24 52.4; 2 KiB: 8 45.5, 32 52.4; 1 KiB both ways: 32 76.6, 64 79.0).
 //  inside the device: much in flight, but no more than the memory takes.  Long moves: 1.7 pipelines per SM, two per CTA
-//    (256 blocks of 2 MiB: 220 pipelines 169.7 us, 252 166.2, 296 177, 328 198; four per CTA need 280 for the same 166, and
-//    longer to start).  Short ones, where starting and draining decide, and small pieces: four per SM, one per CTA (16 blocks
+//    (256 blocks of 2 MiB: 148 pipelines 207 us, 200 182, 220 to 268 178, 296 179, 328 197; four per CTA need 280 for the same,
+//    and longer to start).  Short ones, where starting and draining decide, and small pieces: four per SM, one per CTA (16 blocks
 //    of 2 MiB: 9.5 us against 12.7 with 296 in CTAs of four; 64 blocks: 47.5 against 45.2, so the line lies between; 400 blocks
 //    of 64 chunks of 4 KiB: 252 pipelines 42.4 us, 592 37.9).
 #define D2D_SHORT_BYTES (48ull << 20)

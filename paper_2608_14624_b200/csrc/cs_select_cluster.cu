@@ -77,7 +77,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
             id_s[i] = __ldcg(&ws.cand_id[pos]);
         }
         __syncthreads();
-        bitonic_sort_fast(km_s, id_s, CS_SAMPLE, whole_cta());
+        bitonic_sort_fast(km_s, id_s, CS_SAMPLE);
         // buckets of about 384 keys, which a CTA sorts in little more time than 128, but a bucket for every CTA at least
         const uint32_t n_spl = min(CS_MAX_SPLITTERS, max(c / 384u, CL));
         for (uint32_t j = tid; j <= CS_MAX_SPLITTERS; j += CSEL_THREADS) {
@@ -111,7 +111,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
     // offsets (every CTA computes the same prefix sum), then scatter the needed buckets into bucket order
     const uint32_t mine = tid <= CS_MAX_SPLITTERS ? __ldcg(&CS_BCOUNT(ws, tid)) : 0u;
     uint32_t total;
-    const uint32_t excl = sel_block_scan(mine, O.part, total, whole_cta());
+    const uint32_t excl = sel_block_scan(mine, O.part, total);
     if (tid <= CS_MAX_SPLITTERS) s_off[tid] = excl;
     if (tid == CS_MAX_SPLITTERS) s_off[CS_MAX_SPLITTERS + 1] = excl + mine;
     if (mine && excl <= n_out - 1 && n_out - 1 < excl + mine) O.misc[OM_IN] = tid;     // last needed bucket (n_out > 0 here)
@@ -137,7 +137,7 @@ __device__ __noinline__ void csel_order_general(const cs_workspace &ws, const Or
                 O.all_id[i] = i < m ? __ldcg(&ws.sort_id[beg + i]) : 0xFFFFFFFFu;
             }
             __syncthreads();
-            if (P <= 2u * CSEL_THREADS) bitonic_sort_fast(O.all_km, O.all_id, P, whole_cta());
+            if (P <= 2u * CSEL_THREADS) bitonic_sort_fast(O.all_km, O.all_id, P);
             else sort_tile(O.all_km, O.all_id, P);
             for (uint32_t i = tid; i < m; i += CSEL_THREADS)
                 if (beg + i < n_out) ids_out[beg + i] = O.all_id[i];
@@ -201,7 +201,7 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
     uint32_t tail_pr = 0, tail_se = 0, tl_ag = 0, tl_dp = 0, tl_rf = 0, tl_fl = 0, tl_la = 0, tl_tk = a.block_tokens;
     if (tail) {
         tl_ag = __ldg(a.agent + tail_id);
-        tl_dp = __ldg(a.depth + tail_id);
+        if (PF && a.anchor) tl_dp = __ldg(a.depth + tail_id);    // (a caller without workspace vouches for no depth array)
         tl_rf = __ldg(a.ref + tail_id);
         tl_fl = __ldg(a.flags + tail_id);
         tl_la = __ldg(a.la + tail_id);
@@ -318,7 +318,7 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
             sum += v.x + v.y + v.z + v.w;
         }
         uint32_t n_elig;
-        const uint32_t before = sel_block_scan(sum, O.part, n_elig, whole_cta());
+        const uint32_t before = sel_block_scan(sum, O.part, n_elig);
         n_out = n_elig < a.k ? n_elig : a.k;
         if (a.k && n_elig >= a.k && before < a.k && a.k <= before + sum) {
             uint32_t run = before;
@@ -355,8 +355,7 @@ __device__ __forceinline__ void csel_body(SelArgs a, const cs_workspace &ws, uin
         __threadfence();
         cluster.sync();
         OrderBufs B = order_bufs(ws, a.max_blocks);
-        const OrderResult res = order_candidates(O, B, c, n_out, ids_out);
-        if (!res.done) {
+        if (!order_candidates(O, B, c, n_out, ids_out)) {
             order_restore(B, ws.cand_km, ws.cand_id, c);
             csel_order_general(ws, O, c, n_out, ids_out);
         }
@@ -434,7 +433,7 @@ static int csel_cluster_size(uint32_t n, uint32_t k, int max_cl)
 
 // A cluster launch; chained to the kernel before it (programmatic dependent launch) unless that kernel writes the recency
 // table, which the kernels read ahead of the dependency wait (the static-scratch entry point, the only one with no workspace).
-static cudaError_t csel_config(cs_ctx *ctx, cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int cl, int n_jobs, size_t smem,
+static void csel_config(cs_ctx *ctx, cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int cl, int n_jobs, size_t smem,
                                cudaStream_t s)
 {
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -449,7 +448,6 @@ static cudaError_t csel_config(cs_ctx *ctx, cudaLaunchConfig_t &cfg, cudaLaunchA
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = ctx->ws_bytes ? 2 : 1;
-    return cudaSuccess;
 }
 
 template <bool PF>

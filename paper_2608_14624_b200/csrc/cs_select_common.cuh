@@ -35,16 +35,6 @@ void cs_fill_sel_bins(const cs_ctx *ctx, SelArgs &a, int prefetch);
 uint32_t cs_scan_grid(const cs_ctx *ctx, uint32_t n, uint32_t per_cta, uint32_t ctas_per_sm = 2);
 size_t cs_table_smem(const cs_ctx *ctx);
 
-// A group of whole warps of a CTA that synchronises on a barrier of its own, so that two halves of a CTA can work on
-// different things at the same time: t = index of the calling thread within the group, n = its threads,
-// bar = hardware barrier (0 = the one of __syncthreads(), for the whole CTA).
-struct CtaPart { uint32_t t, n, bar; };
-__device__ __forceinline__ CtaPart whole_cta() { return CtaPart{threadIdx.x, blockDim.x, 0u}; }
-__device__ __forceinline__ void part_sync(const CtaPart &p)
-{
-    asm volatile("bar.sync %0, %1;" ::"r"(p.bar), "r"(p.n) : "memory");
-}
-
 // How many candidates the next large select of a kind should find at or below the key it is given: enough that an index
 // which loses its k best entries between calls, or whose survival table shifts, still has k of them; few enough that
 // collecting and ordering them costs little.
@@ -383,20 +373,20 @@ __device__ __forceinline__ bool last_cta_done(uint32_t *ticket, bool *s_flag)
     return last;
 }
 
-// Exclusive prefix sum of one value per thread over a group of warps (warp shuffles, three barriers); also returns
-// the total.  s_part: at least 64 words.
-__device__ __forceinline__ uint32_t sel_block_scan(uint32_t v, uint32_t *s_part, uint32_t &total, const CtaPart &cp)
+// Exclusive prefix sum of one value per thread over the CTA (warp shuffles, three barriers); also returns the total.
+// s_part: at least 64 words.
+__device__ __forceinline__ uint32_t sel_block_scan(uint32_t v, uint32_t *s_part, uint32_t &total)
 {
-    const uint32_t lane = cp.t & 31, warp = cp.t >> 5, n_warps = cp.n >> 5;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     uint32_t incl = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, d);
         if (lane >= d) incl += t;
     }
-    part_sync(cp);
+    __syncthreads();
     if (lane == 31) s_part[warp] = incl;
-    part_sync(cp);
+    __syncthreads();
     if (warp == 0) {
         uint32_t w = lane < n_warps ? s_part[lane] : 0;
 #pragma unroll
@@ -406,7 +396,7 @@ __device__ __forceinline__ uint32_t sel_block_scan(uint32_t v, uint32_t *s_part,
         }
         s_part[32 + lane] = w;                         // inclusive warp totals
     }
-    part_sync(cp);
+    __syncthreads();
     total = s_part[32 + n_warps - 1];
     const uint32_t before = warp ? s_part[32 + warp - 1] : 0;
     return before + incl - v;
@@ -496,10 +486,10 @@ __device__ __forceinline__ bool key_less(unsigned long long km_a, uint32_t id_a,
 
 
 // ---------------------------------------------------------------------------------------------
-// Bitonic sort of P keys (power of two, 64 <= P <= 2 * threads of the group) held in shared memory,
+// Bitonic sort of P keys (power of two, 64 <= P <= 2 * threads of the CTA) held in shared memory,
 // ascending by (km, id).  Each thread keeps two neighbouring elements in registers; compare-
 // exchange steps whose partner lies in the same warp (element distance <= 32) use shuffles and
-// no barrier, only the longer distances go through shared memory.  Called by every thread of the group.
+// no barrier, only the longer distances go through shared memory.  Called by every thread.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void cx_keep(unsigned long long &k, uint32_t &i, unsigned long long pk, uint32_t pi,
                                         bool keep_min)
@@ -508,9 +498,9 @@ __device__ __forceinline__ void cx_keep(unsigned long long &k, uint32_t &i, unsi
     if (partner_less == keep_min) { k = pk; i = pi; }
 }
 
-__device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32_t *id, uint32_t P, const CtaPart &cp)
+__device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32_t *id, uint32_t P)
 {
-    const uint32_t t = cp.t;
+    const uint32_t t = threadIdx.x;
     const bool act = t < P / 2;                           // whole warps, because P >= 64
     unsigned long long k0 = 0, k1 = 0;
     uint32_t i0 = 0, i1 = 0;
@@ -520,7 +510,7 @@ __device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32
         uint32_t stride = size >> 1;
         if (stride >= 64) {                               // partners in other warps: through shared memory
             if (act) { km[2 * t] = k0; km[2 * t + 1] = k1; id[2 * t] = i0; id[2 * t + 1] = i1; }
-            part_sync(cp);
+            __syncthreads();
             for (; stride >= 64; stride >>= 1) {
                 if (act) {
                     const uint32_t lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
@@ -529,7 +519,7 @@ __device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32
                     const uint32_t ia = id[lo], ib = id[hi];
                     if (key_less(kb, ib, ka, ia) == up2) { km[lo] = kb; id[lo] = ib; km[hi] = ka; id[hi] = ia; }
                 }
-                part_sync(cp);
+                __syncthreads();
             }
             if (act) { k0 = km[2 * t]; k1 = km[2 * t + 1]; i0 = id[2 * t]; i1 = id[2 * t + 1]; }
         }
@@ -548,9 +538,9 @@ __device__ __forceinline__ void bitonic_sort_fast(unsigned long long *km, uint32
             }
         }
     }
-    part_sync(cp);
+    __syncthreads();
     if (act) { km[2 * t] = k0; km[2 * t + 1] = k1; id[2 * t] = i0; id[2 * t + 1] = i1; }
-    part_sync(cp);
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -564,7 +554,7 @@ __device__ __forceinline__ void sort_tile(unsigned long long *t_km, uint32_t *t_
     for (uint32_t i = m + threadIdx.x; i < P; i += blockDim.x) { t_km[i] = ~0ull; t_id[i] = 0xFFFFFFFFu; }
     __syncthreads();
     if (P <= 2 * blockDim.x) {
-        bitonic_sort_fast(t_km, t_id, P, whole_cta());
+        bitonic_sort_fast(t_km, t_id, P);
         return;
     }
     for (uint32_t size = 2; size <= P; size <<= 1) {

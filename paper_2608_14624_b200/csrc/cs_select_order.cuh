@@ -54,7 +54,7 @@ struct OrderSmem {
 };
 // OM_BELOW and OM_FILL (one word per part) are order_few()'s own: it clears them on entry with no barrier before that, while slower
 // warps may still be reading any other word (OM_TOTAL in particular, on the way from a cut of the candidates).
-enum { OM_B0 = 0, OM_CTOT, OM_LIST, OM_GLOBAL, OM_GLOBAL2, OM_OVERFLOW, OM_BELOW, OM_IN, OM_TOTAL, OM_FILL = 16, OM_LO_ID = 24, OM_WORDS = 48 };
+enum { OM_B0 = 0, OM_CTOT, OM_LIST, OM_GLOBAL, OM_GLOBAL2, OM_OVERFLOW, OM_BELOW, OM_IN, OM_TOTAL, OM_FILL = 16, OM_WORDS = OM_FILL + (int)OR_PARTS };
 static_assert(OM_TOTAL != OM_BELOW && (OM_TOTAL < OM_FILL || OM_TOTAL >= OM_FILL + (int)OR_PARTS), "read while order_few() clears its words");
 
 // Where the candidates are and where they may be moved to; all of it private to the select.
@@ -247,15 +247,9 @@ __device__ __noinline__ void order_few(const OrderSmem &O, const u64 *src_km, co
     }
 }
 
-// What order_candidates reports.
-struct OrderResult {
-    bool done;                // false: the list is too long, the buckets overflowed or a sample misled (nothing was stored); the candidates
-                              // are in src
-};
-
 // c > 0 candidates in B.src, n_out > 0.  Every CTA of the cluster calls, after a cluster barrier; the candidates' writes are
-// visible.
-__device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBufs &B, uint32_t &c, uint32_t n_out,
+// visible.  False: the list is too long, the buckets overflowed or a sample misled; nothing was stored, the candidates are in B.src.
+__device__ __noinline__ bool order_candidates(const OrderSmem &O, OrderBufs &B, uint32_t &c, uint32_t n_out,
                                                      uint32_t *__restrict__ ids_out)
 {
     cg::cluster_group cluster = cg::this_cluster();
@@ -267,9 +261,9 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
     for (uint32_t round = 0;; ++round) {
         if (c <= OR_ALL && c <= O.cap) {
             order_few(O, B.src_km, B.src_id, c, n_out, ids_out);
-            return OrderResult{true};
+            return true;
         }
-        if (n_out > OR_LONG || round == 6) return OrderResult{false};        // (every round drops most of the candidates)
+        if (n_out > OR_LONG || round == 6) return false;        // (every round drops most of the candidates)
         // ---- a sample, ranked by the cluster; CL lanes share a key ------------------------------------------------------
         const uint32_t S = c <= 12288u ? OR_SAMPLE / 2 : OR_SAMPLE;
         for (uint32_t s = tid; s < S; s += OR_THREADS) {
@@ -364,7 +358,7 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
             __syncthreads();
             const uint32_t total = O.misc[OM_TOTAL];
             cluster.barrier_wait();                                 // (the leader may go on, or leave)
-            if (total < n_out || total >= c) return OrderResult{false};      // the sample misjudged
+            if (total < n_out || total >= c) return false;      // the sample misjudged
             u64 *a_km = B.src_km; B.src_km = B.dst_km; B.dst_km = a_km;
             uint32_t *a_id = B.src_id; B.src_id = B.dst_id; B.dst_id = a_id;
             c = total;
@@ -374,7 +368,7 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
         const uint32_t mine = tid < nb ? cs_ld_cg_pinned(B.bcount + (size_t)tid * CS_BCOUNT_STRIDE) : 0u;
         if (tid == 0) O.misc[OM_TOTAL] = lead[OM_OVERFLOW];
         uint32_t total;
-        const uint32_t excl = sel_block_scan(mine, O.part, total, whole_cta());
+        const uint32_t excl = sel_block_scan(mine, O.part, total);
         if (tid < nb) { O.off[tid] = excl; O.cnt[tid] = mine; }
         cluster.barrier_arrive();                                   // (the leader's flag has been read; waited for at the end)
         __syncthreads();
@@ -406,7 +400,7 @@ __device__ __noinline__ OrderResult order_candidates(const OrderSmem &O, OrderBu
             __syncthreads();                                        // (before the next buckets take their place)
         }
         cluster.barrier_wait();
-        return OrderResult{ok};
+        return ok;
     }
 }
 

@@ -956,11 +956,12 @@ def test_select_large_index_uses_age_limits(with_tokens, prefer):
 
 @pytest.mark.parametrize("max_keys", [0, 1, 40, 100_000])
 def test_bucket_regions_and_their_fallback(max_keys):
-    """With few candidates the sample sort's buckets live in fixed regions of the sort arrays that the bucket launch
-    fills directly; a bucket that outgrows its region sends the call down the general route (buckets grouped by a
-    launch of its own).  Capping the region (1 and 40 keys against buckets of ~64) forces that route on every call;
-    the lists must not change.  Three clocks in a row, so that both the first call (full histogram and collect passes)
-    and the calls that reuse the remembered threshold are covered; the cluster path is unaffected by the setting."""
+    """The buckets of the launch chain live in fixed regions of the sort arrays that the place launch fills; a bucket that
+    outgrows its region is gathered again out of all candidates by the CTA that ranks it.  Capping the region (1 and 40 keys
+    against buckets of a few dozen) forces that on every call, with buckets that fit the CTA's tile (larger ones:
+    test_buckets_beyond_the_tile); the lists must not change.  Three clocks in a row, so that both the first call (full
+    histogram and collect passes) and the calls that reuse the remembered key are covered; the cluster path is unaffected
+    by the setting."""
     cfg = synth.CONFIGS["meta1m"]
     n = 400_000
     c, o = warm_state(cfg, 3000, n, r_min=0.02)
@@ -969,7 +970,7 @@ def test_bucket_regions_and_their_fallback(max_keys):
     for now in (100_000, 100_001, 100_007):
         assert run_selects(c, o, idx, now, (9_000, 700)) == 0
     cn = c.counters()
-    assert all(x > 0 for x in cn["region_selects"])          # 8 c <= 400,000 for k = 700, and mostly for k = 9,000
+    assert all(x > 0 for x in cn["region_selects"])          # (more than 2,048 candidates: buckets)
     if max_keys in (1, 40):
         assert all(x > 0 for x in cn["region_overflows"])
     else:

@@ -430,6 +430,34 @@ __device__ __forceinline__ void rf_read_batch(Shared &sm, const cs_workspace &ws
     }
 }
 
+// The current agent of every chain that has one, as bits of front[] (zero before; whole CTA).  Many chains: eight to a load, four loads
+// together, and an agent that another chain has brought costs a look, not an atomic.  Out of line: the refresh waits for its
+// instructions, and this code in its middle took 0.75 us from every refresh that never enters it.
+__device__ __noinline__ void rf_sources_of_chains(uint32_t *front, const uint16_t *cur, uint32_t A, uint32_t n_chains)
+{
+    const uint32_t tid = threadIdx.x, n_threads = blockDim.x;
+    auto source = [&](uint32_t a) {
+        if (a < A && !((*(volatile uint32_t *)&front[a >> 5] >> (a & 31)) & 1u)) atomicOr(&front[a >> 5], 1u << (a & 31));
+    };
+    if (n_chains <= 4u * n_threads) {
+        for (uint32_t x = tid; x < n_chains; x += n_threads) source(__ldcg(&cur[x]));
+        return;
+    }
+    const uint32_t n8 = n_chains / 8u;
+    for (uint32_t x0 = tid; x0 < n8; x0 += 4u * n_threads) {
+        uint4 v[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) v[u] = cs_ld_cg_pinned((const uint4 *)cur + min(x0 + u * n_threads, n8 - 1u));
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            if (x0 + u * n_threads >= n8) break;
+            source(v[u].x & 0xFFFFu); source(v[u].x >> 16); source(v[u].y & 0xFFFFu); source(v[u].y >> 16);
+            source(v[u].z & 0xFFFFu); source(v[u].z >> 16); source(v[u].w & 0xFFFFu); source(v[u].w >> 16);
+        }
+    }
+    if (tid < (n_chains & 7u)) source(__ldcg(&cur[(n_chains & ~7u) + tid]));
+}
+
 // What the one CTA does that has everything: the batch's effect on the shared state, the sums of Eq. 2 and the search.  row:
 // thread v's words of the transposed adjacency matrix; base[] and hc[] have n_parts numbers each.
 template <int KW>
@@ -454,27 +482,7 @@ __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &
     if (all_chains) {
         // sources: the current agent of every chain that has one (all live sessions)
         __syncthreads();
-        // (many chains: eight to a load; an agent that another chain has brought costs a look, not an atomic)
-        auto source = [&](uint32_t a) {
-            if (a < A && !((*(volatile uint32_t *)&sm.front[a >> 5] >> (a & 31)) & 1u)) atomicOr(&sm.front[a >> 5], 1u << (a & 31));
-        };
-        if (n_chains <= 4u * n_threads) {
-            for (uint32_t x = tid; x < n_chains; x += n_threads) source(__ldcg(&ws.cur[x]));
-        } else {
-            const uint32_t n8 = n_chains / 8u;
-            for (uint32_t x0 = tid; x0 < n8; x0 += 4u * n_threads) {
-                uint4 v[4];                                   // (a round's loads travel together)
-#pragma unroll
-                for (uint32_t u = 0; u < 4; ++u) v[u] = cs_ld_cg_pinned((const uint4 *)ws.cur + min(x0 + u * n_threads, n8 - 1u));
-#pragma unroll
-                for (uint32_t u = 0; u < 4; ++u) {
-                    if (x0 + u * n_threads >= n8) break;
-                    source(v[u].x & 0xFFFFu); source(v[u].x >> 16); source(v[u].y & 0xFFFFu); source(v[u].y >> 16);
-                    source(v[u].z & 0xFFFFu); source(v[u].z >> 16); source(v[u].w & 0xFFFFu); source(v[u].w >> 16);
-                }
-            }
-            if (tid < (n_chains & 7u)) source(__ldcg(&ws.cur[(n_chains & ~7u) + tid]));
-        }
+        rf_sources_of_chains(sm.front, ws.cur, A, n_chains);
         __syncthreads();
     }
     // The search by the first W warps; the sums of Eq. 2 by the warps behind them, side by side, where the CTA has enough of
@@ -951,6 +959,7 @@ static size_t xs_smem_bytes(uint32_t A)
     return (2 * (size_t)A * XS_TARGETS + XS_WARPS * XS_TARGETS * XS_PART_ROW) * sizeof(double);
 }
 
+template <bool ONE>          // one CTA does all columns of its targets; else a cluster shares them
 __global__ void __launch_bounds__(XS_THREADS, 1)
 cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t K, uint32_t n_cols, float delta,
                          float *__restrict__ psurv_out, float *__restrict__ fsurv_out)
@@ -977,15 +986,12 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
             const uint32_t j = e / XS_TARGETS, m = e % XS_TARGETS;
             v_all[e] = j == base + m ? 0.0 : (double)P[(size_t)a0 * A + j];
         }
-        // what does not change from step to step: this warp's columns and its slice of the agents summed over (no slice
-        // of fewer than eight agents, because the slices' sums are added up one after the other: 64 agents, K = 32 41.5 us, with four 50.8)
+        // (no slice of fewer than eight agents, because the slices' sums are added up one after the other: 64 agents, K = 32 41.5 us, with
+        // four 50.8)
         const uint32_t col_warps = (n_cols + 63u) / 64u, slices = min(XS_WARPS / col_warps, max(2u, (A + 7u) / 8u));
         const uint32_t cw = warp % col_warps, sl = warp / col_warps;
-        const uint32_t j0 = col0 + cw * 64u + lane, j1 = j0 + 32u, mine = col1 > col0 ? col1 - col0 : 0u;
-        const float *const p0 = P + (j0 < col1 ? j0 : 0u), *const p1 = P + (j1 < col1 ? j1 : 0u);    // (columns past the end: unused)
-        const uint32_t i_beg = sl * A / slices, i_end = (sl + 1u) * A / slices;
         // (a CTA on its own keeps to its own barrier: a cluster's makes its L1 forget the matrix)
-        const auto everywhere = [&] { if (CL > 1) cluster.sync(); else __syncthreads(); };
+        const auto everywhere = [&] { if (ONE) __syncthreads(); else cluster.sync(); };
         everywhere();                                              // (also: every CTA has started before its memory is written)
         uint32_t cur = 0;
         for (uint32_t t = 1; t + 1 < K; ++t) {
@@ -993,11 +999,13 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
             double *const nxt = v_all + (size_t)(cur ^ 1u) * A * XS_TARGETS;
             cur ^= 1u;
             if (sl < slices) {
+                const uint32_t j0 = col0 + cw * 64u + lane, j1 = j0 + 32u, i_end = (sl + 1u) * A / slices;
+                const float *p0 = P + (j0 < col1 ? j0 : 0u), *p1 = P + (j1 < col1 ? j1 : 0u);    // (columns past the end: unused)
                 double acc0[XS_TARGETS], acc1[XS_TARGETS];
 #pragma unroll
                 for (uint32_t m = 0; m < XS_TARGETS; ++m) acc0[m] = acc1[m] = 0.0;
 #pragma unroll 8
-                for (uint32_t i = i_beg; i < i_end; ++i) {
+                for (uint32_t i = sl * A / slices; i < i_end; ++i) {
                     const double x0 = (double)__ldg(p0 + (size_t)i * A), x1 = (double)__ldg(p1 + (size_t)i * A);
                     const double2 *vi = (const double2 *)(v + (size_t)i * XS_TARGETS);
 #pragma unroll
@@ -1014,16 +1022,16 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
                 for (uint32_t m = 0; m < XS_TARGETS; ++m) { o[m * XS_PART_ROW] = acc0[m]; o[m * XS_PART_ROW + 32u] = acc1[m]; }
             }
             __syncthreads();
-            for (uint32_t e = tid; e < mine * XS_TARGETS; e += XS_THREADS) {
+            for (uint32_t e = tid; e < (col1 > col0 ? col1 - col0 : 0u) * XS_TARGETS; e += XS_THREADS) {
                 const uint32_t jc = e / XS_TARGETS, m = e % XS_TARGETS, j = col0 + jc;
                 const double *q = part + (size_t)(jc / 64u) * XS_TARGETS * XS_PART_ROW + m * XS_PART_ROW + jc % 64u;
                 double sum = 0.0;
                 for (uint32_t u = 0; u < slices; ++u) sum += q[(size_t)u * col_warps * XS_TARGETS * XS_PART_ROW];
                 if (j == base + m) { s_hit[m] += sum; sum = 0.0; }   // (one thread per target)
-                if (CL > 1)
-                    for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)j * XS_TARGETS + m] = sum;
-                else
+                if (ONE)
                     nxt[(size_t)j * XS_TARGETS + m] = sum;
+                else
+                    for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)j * XS_TARGETS + m] = sum;
             }
             everywhere();                                          // the new V is complete everywhere; `part` is free again
         }
@@ -1052,8 +1060,9 @@ int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_
         std::lock_guard<std::mutex> lock(mu);
         if (ctx->device < 0 || ctx->device >= 64) return CS_EINVAL;
         if (!opted[ctx->device]) {
-            const cudaError_t e = cudaFuncSetAttribute(cs_exact_survival_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)xs_smem_bytes(CS_MAX_AGENTS));
+            const int most = (int)xs_smem_bytes(CS_MAX_AGENTS);
+            cudaError_t e = cudaFuncSetAttribute(cs_exact_survival_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(cs_exact_survival_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
             opted[ctx->device] = true;
         }
@@ -1063,8 +1072,8 @@ int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_
     uint32_t cl = 1;
     while (cl < XS_MAX_CLUSTER && p.n_agents > 64u * cl && 2u * cl * n_clusters <= (uint32_t)ctx->sm_count) cl *= 2;
     const uint32_t n_cols = (p.n_agents + cl - 1) / cl;
-    cs_launch_chained_clusters(cs_exact_survival_kernel, n_clusters * cl, cl, XS_THREADS, xs_smem_bytes(p.n_agents), s, ctx->ws,
-                               p.n_agents, a0, K, n_cols, p.delta, psurv_out, fsurv_out);
+    cs_launch_chained_clusters(cl == 1u ? cs_exact_survival_kernel<true> : cs_exact_survival_kernel<false>, n_clusters * cl, cl > 1u ? cl : 0u,
+                               XS_THREADS, xs_smem_bytes(p.n_agents), s, ctx->ws, p.n_agents, a0, K, n_cols, p.delta, psurv_out, fsurv_out);
     return cs_check_launch(ctx);
 }
 

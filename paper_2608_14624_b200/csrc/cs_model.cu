@@ -431,9 +431,9 @@ __device__ __forceinline__ void rf_read_batch(Shared &sm, const cs_workspace &ws
 }
 
 // The current agent of every chain that has one, as bits of front[] (zero before; whole CTA).  Many chains: eight to a load, four loads
-// together, and an agent that another chain has brought costs a look, not an atomic.  Out of line: the refresh waits for its
-// instructions, and this code in its middle took 0.75 us from every refresh that never enters it.
-__device__ __noinline__ void rf_sources_of_chains(uint32_t *front, const uint16_t *cur, uint32_t A, uint32_t n_chains)
+// together, and an agent that another chain has brought costs a look, not an atomic.  Only in kernels of their own (ALL): the refresh
+// waits for its instructions, and this code in its middle took 0.75 us from every refresh of few agents that never entered it.
+__device__ __forceinline__ void rf_sources_of_chains(uint32_t *front, const uint16_t *cur, uint32_t A, uint32_t n_chains)
 {
     const uint32_t tid = threadIdx.x, n_threads = blockDim.x;
     auto source = [&](uint32_t a) {
@@ -460,10 +460,10 @@ __device__ __noinline__ void rf_sources_of_chains(uint32_t *front, const uint16_
 
 // What the one CTA does that has everything: the batch's effect on the shared state, the sums of Eq. 2 and the search.  row:
 // thread v's words of the transposed adjacency matrix; base[] and hc[] have n_parts numbers each.
-template <int KW>
+template <int KW, bool ALL>
 __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &ws, const uint32_t (&row)[KW], uint32_t A, uint32_t W,
                                           uint32_t n_parts, uint32_t n_events, uint32_t n_new, uint32_t n_skipped, uint32_t n_total,
-                                          uint32_t la, float r_min, uint32_t e_max, float delta, uint32_t all_chains, uint32_t n_chains)
+                                          uint32_t la, float r_min, uint32_t e_max, float delta, uint32_t n_chains)
 {
     const uint32_t tid = threadIdx.x, lane = tid & 31, n_threads = blockDim.x;
     if (n_events) {
@@ -479,7 +479,7 @@ __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &
             if (n_new) atomicAdd((unsigned long long *)&ws.cnt->transitions_counted, (unsigned long long)n_new);
         }
     }
-    if (all_chains) {
+    if (ALL) {
         // sources: the current agent of every chain that has one (all live sessions)
         __syncthreads();
         rf_sources_of_chains(sm.front, ws.cur, A, n_chains);
@@ -521,7 +521,7 @@ __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &
         CS_STAMP(ws, CS_PS_REFRESH_SUMS_DONE, j == 0);
     }
     if (tid < 32u * W) {
-        if (!all_chains) {
+        if (!ALL) {
             if (tid == 0 && la < A) sm.front[la >> 5] = 1u << (la & 31);
             asm volatile("bar.sync 1, %0;" ::"r"(W * 32u) : "memory");
         }
@@ -531,10 +531,10 @@ __device__ __forceinline__ void rf_finish(RfShared<KW> &sm, const cs_workspace &
 }
 
 // blockDim.x / 32 rows per CTA, a warp each: 8, 16 or 32 in the one CTA (KW = 1), 8 or 16 in each of up to 16 (KW = 8).
-template <int KW>
+template <int KW, bool ALL>
 __global__ void __launch_bounds__(RfShape<KW>::WARPS * 32u)
 cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
-                  uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
+                  uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
                   const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
                   const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
 {
@@ -713,7 +713,7 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
         }
     }
 
-    rf_finish<KW>(sm, ws, row, A, W, CL, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, all_chains, n_chains);
+    rf_finish<KW, ALL>(sm, ws, row, A, W, CL, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, n_chains);
 }
 
 // The same for many agents (KW = 32): bound by the scan of the rows -- a megabyte and more of counts -- so they are spread over the
@@ -723,9 +723,10 @@ cs_refresh_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau,
 // A cluster of 16 CTAs with 32 or 64 rows each took 17.1 us for 400 agents, 28.8 for 600 and 35.3 for 1,024, most of it for
 // issuing four chunks per row; this takes 13.9, 15.6 and 17.8: 5.8 the rows, 2.7 the meeting, 4 the sums, up to 4.5 the search.
 // (For 256 agents or fewer the meeting in global memory costs more than it gives: 13.3 us instead of 8.5.)
+template <bool ALL>
 __global__ void __launch_bounds__(1024)
 cs_refresh_wide_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float tau, float r_min, uint32_t e_max, float delta,
-                       uint32_t all_chains, uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
+                       uint32_t n_chains, const uint32_t *__restrict__ ev_chain_in,
                        const uint16_t *__restrict__ ev_agent_in, const uint8_t *__restrict__ ev_flags, uint32_t n_events,
                        const uint32_t *__restrict__ n_events_dev, uint32_t every_row)
 {
@@ -900,7 +901,7 @@ cs_refresh_wide_kernel(cs_workspace ws, uint32_t A, uint32_t W, float eps, float
     }
     if (tid == 0) ws.sc->refresh_ticket = 0;
     __syncthreads();
-    rf_finish<32>(sm, ws, row, A, W, 4u, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, all_chains, n_chains);
+    rf_finish<32, ALL>(sm, ws, row, A, W, 4u, n_events, n_new, n_skipped, n_total, la, r_min, e_max, delta, n_chains);
 }
 
 // BFS + Eq. 8 from explicit sources into the temporary tables (cs_score_blocks with sources): one thread per agent.
@@ -1154,8 +1155,10 @@ static uint32_t obs_cluster_limit(int device)
 }
 static uint32_t refresh_cluster_limit(int device)
 {
-    static ClusterLimit limit;
-    return limit.get(device, cs_refresh_kernel<8>, RfShape<8>::CTAS, RfShape<8>::WARPS * 32);
+    static ClusterLimit limit[2];
+    const uint32_t last = limit[0].get(device, cs_refresh_kernel<8, false>, RfShape<8>::CTAS, RfShape<8>::WARPS * 32);
+    const uint32_t all = limit[1].get(device, cs_refresh_kernel<8, true>, RfShape<8>::CTAS, RfShape<8>::WARPS * 32);
+    return last < all ? last : all;
 }
 
 int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent, const uint8_t *evflags,
@@ -1173,27 +1176,27 @@ int cs_launch_observe(cs_ctx *ctx, const uint32_t *chain, const uint16_t *agent,
         int rc = cs_check_launch(ctx);
         if (rc != CS_OK) return rc;
     }
-    const uint32_t all_chains = ctx->source_mode == CS_SOURCES_ALL_CHAINS ? 1u : 0u;
+    const bool all = ctx->source_mode == CS_SOURCES_ALL_CHAINS;
     if (!fused) chain = nullptr, agent = nullptr, evflags = nullptr;
     const uint32_t n_fused = fused ? n_events : 0u;
     const uint32_t *n_fused_dev = fused ? ctx->step_n_events_dev : nullptr;
     const uint32_t every_row = n_fused ? 0u : 1u;            // a row keeps its P when no event of a small batch starts at it
     const auto launch = [&](auto kernel, uint32_t ctas, uint32_t cluster, uint32_t warps) {
         cs_launch_chained_clusters(kernel, ctas, cluster, warps * 32u, 0, s, ctx->ws, p.n_agents, ctx->W, p.eps, p.tau, p.r_min,
-                                   p.e_max, p.delta, all_chains, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
+                                   p.e_max, p.delta, p.n_chains, chain, agent, evflags, n_fused, n_fused_dev, every_row);
     };
     const uint32_t most = refresh_cluster_limit(ctx->device);
     if (p.n_agents <= 32) {
         // one CTA of as many warps as there are rows, at least one thread per event of a small batch
-        launch(cs_refresh_kernel<1>, 1u, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));
+        launch(all ? cs_refresh_kernel<1, true> : cs_refresh_kernel<1, false>, 1u, 1u, p.n_agents <= 8 ? 8u : (p.n_agents <= 16 ? 16u : 32u));
     } else if (p.n_agents <= RfShape<8>::COLS && p.n_agents <= RfShape<8>::WARPS * most) {
         // few rows per CTA (64 agents: 8.8 us with 32, 7.4 with 16, 6.8 with 8), as far as the cluster goes
         const uint32_t rows = p.n_agents <= 8u * most ? 8u : RfShape<8>::WARPS;
         uint32_t cl = 2;
         while (cl * rows < p.n_agents) cl <<= 1;
-        launch(cs_refresh_kernel<8>, cl, cl, rows);
+        launch(all ? cs_refresh_kernel<8, true> : cs_refresh_kernel<8, false>, cl, cl, rows);
     } else {
-        launch(cs_refresh_wide_kernel, (p.n_agents + RW_ROWS - 1u) / RW_ROWS, 0u, 32u);
+        launch(all ? cs_refresh_wide_kernel<true> : cs_refresh_wide_kernel<false>, (p.n_agents + RW_ROWS - 1u) / RW_ROWS, 0u, 32u);
     }
     return cs_check_launch(ctx);
 }

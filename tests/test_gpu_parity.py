@@ -272,6 +272,37 @@ def test_samples_that_mislead_a_cluster(max_blocks, k, seen_are_old):
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("k", [4096, 3900, 1500, 100])
+@pytest.mark.parametrize("kind", ["young", "old", "gap", "wide_gap"])
+def test_few_candidates_with_a_long_part(kind, k):
+    """4,096 candidates in a cluster, which samples every 32nd: a gap between two samples longer than a part's 256 places (300 keys, and 2,500),
+    and samples that see only the youngest or only the oldest entries."""
+    n = 4096
+    p = cs.make_params(n_agents=2, max_blocks=n)
+    c, o = cs.CacheScout(p, DEV), orc.Oracle(H.oracle_params(p))
+    idx = synth.make_block_index(synth.shrink(synth.CONFIGS["tiny"], n_agents=2), n=n)
+    rng = synth.rng_for(synth.CONFIGS["tiny"], 81)
+    idx.flags[:], idx.ref_count[:], idx.agent[:], idx.n_tokens[:] = synth.FLAG_VALID, 0, 0, p.block_tokens
+    seen = np.arange(0, n, 32)
+    others = np.setdiff1d(np.arange(n), seen)
+    idx.last_access[:] = rng.integers(5_000, 60_000, n)
+    if kind == "young":
+        idx.last_access[seen] = rng.integers(80_000, 90_000, len(seen))
+    elif kind == "old":
+        idx.last_access[seen] = rng.integers(0, 4_000, len(seen))
+    else:
+        idx.last_access[seen] = np.linspace(5_000, 60_000, len(seen)).astype(np.uint32)
+        idx.last_access[rng.permutation(others)[:300 if kind == "gap" else 2500]] = idx.last_access[seen[40]] + 1
+    s64, s32 = o.scores(idx, 100_000)
+    assert len(np.unique(s32)) == 1
+    want, n_want = o.select_victims(idx, 100_000, 0, k, s32)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    for _ in range(3):
+        ids, cnt = c.select_victims(d, 100_000, 0, k)
+        assert H.assert_list_matches(ids.cpu().numpy().view(np.uint32)[:k], int(cnt.item()), want, n_want, s64) == 0
+    assert c.get_status() == 0
+
+
 def test_buckets_of_one_cta_beyond_its_shared_memory():
     """The single-launch select with six buckets of 3,500 keys, all of them the first CTA's (every 16th bucket): it holds 4,096 keys at a
     time.  Of 131,072 candidates the sample sees every 32nd of the first 32,768, whose keys mark where the buckets lie; a workspace large

@@ -254,7 +254,7 @@ __device__ __noinline__ void order_few(const OrderSmem &O, const u64 *src_km, co
         } else {
             // A part too long for its place: gaps between samples are exponentially spread, so of 4,000 candidates one list in thirty has
             // a gap of 256 keys or more, and a sample that misleads has nearly all of them in one.  All candidates are here: sorted,
-            // every key is at its place in the list.  (Counting each of the range's keys against all of them took 800 us, this 40.)
+            // every key is at its place in the list.  (Counting each of the range's keys against all of them took 800 us, this 55.)
             sort_keys(all_km, all_id, c);
             for (uint32_t i = base + tid; i < base + m && i < n_out; i += OR_THREADS) ids_out[i] = all_id[i];
         }

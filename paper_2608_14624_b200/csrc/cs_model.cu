@@ -947,7 +947,7 @@ cs_survival_kernel(cs_workspace ws, uint32_t A, uint32_t W, const uint16_t *__re
 //
 // Bound by the fp64 pipe for many agents (2 A^3 (K - 2) operations), by latency for few.  256 agents, K = 4: 62.7 us with
 // one CTA per 8 targets that walked the matrix column by column (32 CTAs, one serial chain of 256 loads per step),
-// 13.7 us per call like this (128 CTAs).  Few agents, one CTA, K = 32, with cluster barriers / with its own: 4 agents 42 / 17 us,
+// 13.4 us per call like this (128 CTAs).  Few agents, one CTA, K = 32, with cluster barriers / with its own: 4 agents 42 / 17 us,
 // 12 44 / 25, 64 85 / 42.
 // ---------------------------------------------------------------------------------------------
 #define XS_TARGETS 8u

@@ -59,7 +59,7 @@ typedef struct CUstream_st *cs_stream_t;   /* the same type as cudaStream_t */
 #define CS_ST_BAD_CHAIN 2u      /* an event named a chain >= n_chains */
 #define CS_ST_BAD_SLOT 4u       /* a mover list entry named a slot >= n_slots */
 #define CS_ST_BAD_SOURCE 8u     /* a BFS source >= n_agents */
-#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer is incomplete */
+#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer is incomplete, or the select's lists are empty */
 #define CS_ST_LIST_CONFLICT 32u /* cs_validate_*_lists(): a slot is written twice, or written and read, by one transfer */
 #define CS_ST_BAD_SELECTION 64u /* cs_validate_selection(): a list is not the ordered k best eligible entries */
 
@@ -352,7 +352,8 @@ int cs_import_state(cs_ctx *ctx, const uint32_t *C_in, const uint16_t *cur_in, u
  * Returns CS_EDEVICE_STATUS when the word was non-zero. */
 int cs_get_status(cs_ctx *ctx, uint32_t *device_status, cs_stream_t stream);
 
-/* Number of kernels this context has launched so far (host counter); the copy made by cs_get_model() is not counted. */
+/* Number of kernels this context has launched so far (host counter); the copy made by cs_get_model() is not counted.
+ * A select of an index above 262,144 entries counts as six whichever way it goes. */
 int cs_launch_count(cs_ctx *ctx, uint64_t *n_launches);
 
 /* Work counters kept in the workspace by the kernels themselves (the paper reports only hit rate and
@@ -371,7 +372,7 @@ typedef struct cs_counters {
     uint64_t blocks_moved[3];       /* blocks copied, per direction */
     uint64_t bytes_moved[3];        /* their bytes (block_bytes each) */
     uint64_t blocks_skipped;        /* mover list entries skipped: CS_ID_NONE or slot out of range */
-    uint64_t region_selects[3];     /* multi-launch selects whose sample-sort buckets were filled in place (cs_set_select_bucket_regions) */
+    uint64_t region_selects[3];     /* multi-launch and whole-GPU selects whose buckets were filled in place (cs_set_select_bucket_regions) */
     uint64_t region_overflows[3];   /* of those: a bucket outgrew its region and was gathered again out of all candidates */
 } cs_counters;
 
@@ -461,16 +462,17 @@ int cs_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t n_steps, float *psurv_o
  * of the hop-distance table of Eq. 8; NULL restores the default.  Host-side switch, no launch. */
 int cs_use_survival_table(cs_ctx *ctx, const float *fsurv);
 
-/* Implementation of the two select calls: CS_SELECT_AUTO (= the single-launch cluster kernel up
- * to 262,144 index entries, the multi-launch path above), CS_SELECT_CLUSTER, CS_SELECT_MULTI
- * (fast pass / histogram / collect / sample / place / finish as six grid-wide launches).  Both give the
- * same lists. */
+/* Implementation of the two select calls: CS_SELECT_AUTO (= the single-launch cluster kernel for small
+ * indexes, one launch on the whole GPU for all lists of large ones from a list's second call on, the
+ * multi-launch path for the largest and for longer lists than 100,000 ids), CS_SELECT_CLUSTER (AUTO, with
+ * the cluster kernel up to 262,144 entries), CS_SELECT_MULTI (fast pass / histogram / collect / sample /
+ * place / finish as six grid-wide launches).  All give the same lists. */
 #define CS_SELECT_AUTO 0u
 #define CS_SELECT_CLUSTER 1u
 #define CS_SELECT_MULTI 2u
 int cs_set_select_path(cs_ctx *ctx, uint32_t path);
 
-/* The multi-launch select remembers a key somewhat above the one each kind of call (GPU victims, host victims,
+/* The multi-launch and the whole-GPU select remember a key somewhat above the one each kind of call (GPU victims, host victims,
  * prefetch) ended with, and the next call of that kind collects the entries at or below it in one scan; when the list
  * lies within them the index is read once instead of three times.  The result never depends on it.  enabled = 0
  * turns the speculation off. */

@@ -52,6 +52,7 @@ size_t cs_layout_workspace(const cs_params *p, uint32_t gtab_len, void *base, cs
     TAKE(sc, cs_scalars, 1);
     TAKE(cnt, cs_counters, 1);
     TAKE(sel, cs_sel_state, 1);
+    TAKE(grid, cs_grid_state, 1);
     TAKE(C, uint32_t, A * A);
     TAKE(rowsum, uint32_t, A);
     TAKE(cur, uint16_t, p->n_chains);

@@ -23,7 +23,16 @@ struct cs_nvtx_range {
 #error "libcachescout is written for sm_100a (B200) only"
 #endif
 
-#define CS_SELECT_CLUSTER_MAX_BLOCKS (1u << 18)   // above this the index is scanned by the whole grid instead
+#define CS_SELECT_CLUSTER_MAX_BLOCKS (1u << 18)   // largest index of the single-launch cluster select
+
+// Index sizes and list lengths that take the one-launch select on the whole GPU (cs_select_grid.cu).
+#ifndef CS_SELECT_GRID_MIN_BLOCKS
+#define CS_SELECT_GRID_MIN_BLOCKS (1u << 17)
+#endif
+#define CS_SELECT_GRID_LONG_BLOCKS (1u << 16)      // with a list of CS_SELECT_GRID_LONG_LIST ids or more
+#define CS_SELECT_GRID_LONG_LIST 2048u
+#define CS_SELECT_GRID_MAX_BLOCKS (1u << 25)
+#define CS_SELECT_GRID_MAX_LIST 100000u
 
 #define CS_CONCURRENT_MAX_BLOCKS (1u << 22)        // up to this index size every select of a step has full-size scratch of its own
 
@@ -105,11 +114,31 @@ struct cs_sel_state {
     uint32_t spec;          // 1: the fast pass's candidates cover the k winners, the histogram and collect passes are skipped
 };
 
+// State of the one-launch select of large indexes (cs_select_grid.cu), one per context.  What a launch counts in lies twice, used by turns:
+// a launch clears the set of the next one.
+struct cs_grid_list {
+    uint32_t c_scan, c_collect, eligible, pad; // candidates of the scan and of the collect pass; eligible entries that the scan saw
+    unsigned long long ahead;                  // key below which about cs_ahead(k) candidates lie, ~0: there are fewer
+    uint32_t pad2[2];
+};
+struct cs_grid_state {
+    uint32_t epoch, broken, pad[30];           // the set in use; a wait has run out once: no launch counts on the words any more
+    uint32_t bar[2][8][32];                    // grid barriers, a line each
+    cs_grid_list list[2][4];
+    uint32_t count[2][3][CS_BUCKETS * CS_BCOUNT_STRIDE];       // keys per bucket
+    uint32_t rem_n[4];                         // by list: buckets of the next call of the kind, and where they start (from 1 on; [rem_n]: the end)
+    uint32_t rem_now[4];                       // the clock at which that was so,
+    unsigned long long rem_T[4];               // and the key remembered with it (cs_scalars.sel_T, unless another route has chosen one since)
+    unsigned long long rem_km[3][CS_BUCKETS + 8];
+    uint32_t rem_id[3][CS_BUCKETS + 8];
+};
+
 // Device pointers into the caller's workspace.
 struct cs_workspace {
     cs_scalars *sc;
     cs_counters *cnt;     // work counters (cs_get_counters)
     cs_sel_state *sel;    // this select's state (one per concurrent select)
+    cs_grid_state *grid;  // large indexes in one launch
     uint32_t *C;          // [A*A] transition counts
     uint32_t *rowsum;     // [A]
     uint16_t *cur;        // [n_chains]
@@ -173,6 +202,8 @@ struct cs_ctx {
     cudaStream_t sel_stream[2];          // the second and third select of a step run here, beside the first
     cudaEvent_t ev_sel_fork, ev_sel_join[2];
     int concurrent_selects;              // the per-select scratch regions are full size
+    uint32_t lists_asked;                // lists that a select has been asked for, one bit each
+    uint32_t grid_refused;               // 1: the driver would not launch the cooperative select; the launch chain does from then on
     cs_select_graph sel_graph[8];        // selects side by side, by the lists wanted (bit q: select q)
     // copy-engine path of the mover (cs_set_mover_staging): caller-owned device ring split into four sub-buffers
     // (two per direction, double-buffered), two streams of the context for the two DMA directions, and the events
@@ -207,6 +238,8 @@ int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int p
 int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uint32_t k_victims, uint32_t k_prefetch,
                           uint32_t *gpu_victims, uint32_t *n_gpu, uint32_t *host_victims, uint32_t *n_host,
                           uint32_t *prefetch_ids, uint32_t *n_prefetch, cudaStream_t s);
+int cs_launch_select_grid(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, const uint32_t k[3], uint32_t *const ids[3],
+                          uint32_t *const n_out[3], cudaStream_t s);
 void cs_drop_select_graphs(cs_ctx *ctx);
 int cs_launch_select_clusters(cs_ctx *ctx, int n_jobs, const void *sel_args, const uint32_t *prefetch,
                               uint32_t *const *ids_out, uint32_t *const *n_out, cudaStream_t s);

@@ -10,8 +10,8 @@
 //   victims : primary = score bits,                      secondary = last_access
 //   prefetch: primary = (not a*)<<31 | ~score bits[30:0], secondary = ~last_access
 //
-// This file holds the multi-launch path, used for indexes above 262,144 entries (smaller ones take
-// the single-launch cluster kernel of cs_select_cluster.cu).  Six launches, none of which waits
+// This file holds the choice of the way (select_route()) and the multi-launch path, used above 262,144 entries for a list's first call, for
+// the largest indexes and the longest lists (others take the single launch of cs_select_cluster.cu or cs_select_grid.cu).  Six launches, none of which waits
 // on another CTA outside its own cluster:
 //   0 fast pass : one scan against a key remembered from the last call of this kind; when the k
 //                 winners lie at or below it (the usual case) the candidates are complete and launches 1 and 2
@@ -33,7 +33,7 @@
 #include <initializer_list>
 #include <tuple>
 
-#include "cs_select_common.cuh"
+#include "cs_select_buckets.cuh"
 
 // ---------------------------------------------------------------------------------------------
 // ScoreBlock for every entry (cs_score_blocks).
@@ -167,8 +167,6 @@ cs_score_small_kernel(SelArgs a, cs_workspace ws, float *__restrict__ out, Score
     }
 }
 
-#define RANK_TILE 2048u                 // keys of the shared-memory tile a bucket is sorted in
-
 // ---------------------------------------------------------------------------------------------
 // 0 fast pass (remembered key)
 //
@@ -196,46 +194,6 @@ __device__ __forceinline__ uint32_t max_halves(const uint4 &a, const uint4 &b)
     const uint32_t m0 = __vmaxu2(__vmaxu2(a.x, a.y), __vmaxu2(a.z, a.w)), m1 = __vmaxu2(__vmaxu2(b.x, b.y), __vmaxu2(b.z, b.w));
     const uint32_t m = __vmaxu2(m0, m1);
     return max(m & 0xFFFFu, m >> 16);
-}
-
-// End of the half-line of last_access that an agent's blocks of the common size need for a key at or below T: victims
-// la <= cut, prefetch la >= cut.  (Entries on the line's side of it that fail after all are sorted out by the exact test.)
-template <bool PF>
-__device__ __forceinline__ uint32_t la_cut(const SelArgs &a, const Tables &T, uint32_t agent, u64 bound)
-{
-    const uint32_t Tp = (uint32_t)(bound >> 32), Ts = (uint32_t)bound;
-    const uint32_t flip = (PF && agent != T.a_star) ? 0x80000000u : 0u;
-    const float f = T.fsurv[agent], tb = (float)a.block_tokens;
-    // smallest possible primary key at an age (a copy on the other tier would make it that; the exact test tells).  The
-    // table covers every age before saturation (gtab_len = age_sat) and ends with the saturated factor.
-    auto primary = [&](uint32_t age) {
-        const uint32_t bits = __float_as_uint(__fmul_rn(__fmul_rn(f, T.gtab[age]), tb));
-        return PF ? (flip | (~bits & 0x7FFFFFFFu)) : (a.prefer_copy ? bits << 1 : bits);
-    };
-    // victims: primary falls with age: n_le = first age with primary <= Tp, n_lt = first with primary < Tp (age_sat + 1: none);
-    // prefetch: it rises: n_le = first age with primary > Tp, n_lt = first with primary >= Tp.  Both found in step, without a
-    // branch: the binary search over 2,263 ages is the longest chain between the scan's first load and its first compare.
-    uint32_t n_le = 0, n_lt = 0;
-    for (uint32_t step = CS_GTAB_MAX; step > 0; step >>= 1) {
-        const uint32_t a0 = n_le + step - 1u, a1 = n_lt + step - 1u;
-        const uint32_t p0 = primary(min(a0, a.age_sat)), p1 = primary(min(a1, a.age_sat));
-        n_le += (a0 <= a.age_sat && (PF ? p0 <= Tp : p0 > Tp)) ? step : 0u;
-        n_lt += (a1 <= a.age_sat && (PF ? p1 < Tp : p1 >= Tp)) ? step : 0u;
-    }
-    if (!PF) {
-        if (n_le > a.age_sat) return 0u;                                   // no age qualifies
-        // la <= now - n_lt for the ages below T's score; at T's score (n_le <= age < n_lt) also la <= Ts.  Age 0 stands for
-        // every last_access from now on.
-        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt : 0u));
-        const uint32_t at_score = min(n_le == 0 ? 0xFFFFFFFFu : (a.now >= n_le ? a.now - n_le : 0u), Ts);
-        return max(by_score, at_score);
-    } else {
-        if (n_le == 0) return 0xFFFFFFFFu;                                 // not even age 0
-        // la > now - n_lt for the ages above T's score; at T's score (n_lt <= age < n_le) also ~la <= Ts
-        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt + 1u : 0u));
-        const uint32_t at_score = max(n_le > a.age_sat ? 0u : (a.now >= n_le ? a.now - n_le + 1u : 0u), ~Ts);
-        return min(by_score, at_score);
-    }
 }
 
 template <bool PF>
@@ -654,70 +612,21 @@ __global__ void __launch_bounds__(SEL_THREADS) cs_sel_collect_kernel(SelArgs a, 
 }
 
 // ---------------------------------------------------------------------------------------------
-// 3 - 5 ordering the candidates
-//
-// The n_out smallest of c candidates, in order, by ranks of a sample: 1,024 candidates at even distances are ranked against
-// each other (counting smaller ones: 96-bit compares spread over 64 CTAs), and J of them cover the output with four
-// standard deviations to spare.  Everything beyond the J-th is dropped; the rest is split at the samples into nb buckets of a few dozen
-// keys, which are small enough to be ranked by counting as well.  Whole-GPU launches, because the work is comparisons:
-// one cluster of 16 SMs took 36 us for 35,000 candidates, k = 10,000 (8 us the sample, 14 us the buckets, 8 us the ranks).
-// A bucket has a fixed region of the sort arrays; one that outgrows it is gathered again from the candidates by its CTA.
-//
-// At most FEW_MAX candidates (short lists: the remembered key follows a list of a few hundred down to about a thousand) all go into the
-// sample: their ranks are their places, and the other two launches return at once.  Per select of 741,250 entries, k = 300: 22.1 us
-// with buckets, 18.7 so; three lists side by side 33.2 and 26.2.  The line: with 1,024 the three lists of k = 800 stay at 32.6 (30.5
-// with 2,048); 3,072 gives a list of 2,500 candidates nothing or costs it 2 us.  (Ranges of a sample in each of the 64 CTAs, as in a cluster,
-// for up to 8,192: as fast up to about 1,400 candidates, 1 to 2 us slower than the buckets beyond.)
+// 3 - 5 ordering the candidates (cs_select_buckets.cuh), a launch per step
 // ---------------------------------------------------------------------------------------------
 #define SAMPLE_CTAS 64u
-#define FEW_MAX 2048u             // a multiple of 1,024
-struct OrderPlan {
-    uint32_t S, J;            // samples; of those, how many cover the output
-    uint32_t gaps;            // gap g lies between samples g - 1 and g (the first from the smallest key, the last to the largest
-                              // key when no sample lies beyond the output)
-    uint32_t sub, join;       // buckets per gap, gaps per bucket; one of them is 1
-    uint32_t nb, cap;         // buckets, and keys a bucket's region holds
-};
-__device__ __forceinline__ OrderPlan order_plan(uint32_t c, uint32_t n_out, uint32_t max_blocks, uint32_t region_max)
+// The key the next call of this kind gets, from whoever places the list's last id.
+__device__ __forceinline__ void remember_key(const cs_workspace &ws, const cs_sel_state &st, uint32_t k, uint32_t hint_slot, uint32_t pos, u64 km)
 {
-    OrderPlan P;
-    P.S = c < CS_SAMPLE ? c : CS_SAMPLE;
-    const float e = (float)n_out * (float)P.S / (float)c;
-    const uint32_t want = (uint32_t)(e + 4.0f * sqrtf(e)) + 3u;
-    P.J = want < P.S ? want : P.S;
-    P.gaps = P.J + (P.J == P.S ? 1u : 0u);
-    P.sub = P.gaps <= CS_BUCKETS ? CS_BUCKETS / P.gaps : 1u;
-    P.join = (P.gaps + CS_BUCKETS - 1u) / CS_BUCKETS;
-    P.nb = P.join > 1u ? (P.gaps + P.join - 1u) / P.join : P.gaps * P.sub;
-    P.cap = max_blocks / P.nb;
-    if (region_max && P.cap > region_max) P.cap = region_max;
-    return P;
+    if (pos == st.n_out - 1u && hint_slot < 3u) ws.sc->sel_T[hint_slot] = next_bound(st, k, km, cs_ahead(k));
 }
-// Smallest key of bucket j.  A gap that is several buckets is divided evenly: locally the keys of a tie in score are spread
-// evenly over last_access, and the largest of a few hundred gaps is six times the mean one.
-__device__ __forceinline__ void bucket_start(const OrderPlan &P, const u64 *s_km, const uint32_t *s_id, uint32_t j, u64 &km, uint32_t &id)
-{
-    const uint32_t g = P.join > 1u ? j * P.join : j / P.sub, f = P.join > 1u ? 0u : j - g * P.sub;
-    km = g ? s_km[g - 1] : 0ull;
-    id = g ? s_id[g - 1] : 0u;
-    if (j >= P.nb) {
-        km = ~0ull;
-        id = 0xFFFFFFFFu;
-    } else if (f) {
-        const u64 step = ((g < P.J ? s_km[g] : ~0ull) - km) / P.sub;
-        if (step) id = 0u;                                    // (a gap inside a tie down to the id is not divided)
-        km += step * f;
-    }
-}
-
-__device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u64 kth);
 
 __global__ void __launch_bounds__(512) cs_sel_sample_kernel(SelArgs a, cs_workspace ws, uint32_t *__restrict__ ids_out,
                                                             uint32_t *__restrict__ n_out_dev)
 {
     __shared__ u64 s_km[FEW_MAX];
     __shared__ uint32_t s_id[FEW_MAX];
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x;
     cs_wait_for_predecessor();
     CS_STAMP(ws, CS_PS_SAMPLE_WAITED + (a.kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
     cs_release_successor();
@@ -729,46 +638,12 @@ __global__ void __launch_bounds__(512) cs_sel_sample_kernel(SelArgs a, cs_worksp
         if (tid == 0) *n_out_dev = n_out;
     }
     if (n_out == 0) return;
-    const bool few = c <= FEW_MAX;
-    const uint32_t S = few ? c : CS_SAMPLE, ahead = cs_ahead(a.k), padded = (S + 255u) & ~255u;
-    for (uint32_t s0 = 0; s0 < S; s0 += 1024u) {
-        u64 km[2];
-        uint32_t id[2];
-#pragma unroll
-        for (uint32_t u = 0; u < 2; ++u) {
-            const uint32_t s = s0 + tid + u * 512u, at = s < S ? (uint32_t)((u64)s * c / S) : 0u;
-            km[u] = cs_ld_cg_pinned(ws.cand_km + at);
-            id[u] = cs_ld_cg_pinned(ws.cand_id + at);
-        }
-#pragma unroll
-        for (uint32_t u = 0; u < 2; ++u) {
-            const uint32_t s = s0 + tid + u * 512u;
-            s_km[s] = s < S ? km[u] : ~0ull;
-            s_id[s] = s < S ? id[u] : 0xFFFFFFFFu;
-        }
-    }
-    if (blockIdx.x == 0 && tid == 0 && c <= ahead) ws.sel->ahead = ~0ull;
-    __syncthreads();
-    for (uint32_t s = blockIdx.x * 16u + warp; s < S; s += gridDim.x * 16u) {       // a warp per sample
-        const u64 my = s_km[s];
-        const uint32_t mine = s_id[s];
-        uint32_t r = 0;
-#pragma unroll 8
-        for (uint32_t q = lane; q < padded; q += 32u) count_less(r, s_km[q], s_id[q], my, mine);
-        r = __reduce_add_sync(0xFFFFFFFFu, r);
-        if (few) {
-            if (lane == 0 && r < n_out) ids_out[r] = mine;
-            if (lane == 0 && r == n_out - 1u && a.hint_slot < 3u) {       // the k-th key: it chooses the next call's
-                cs_sel_state now = *ws.sel;
-                now.ahead = ~0ull;
-                ws.sc->sel_T[a.hint_slot] = next_bound(now, a.k, my);
-            }
-        } else if (lane == 0) {
-            ws.spl_km[r] = my;
-            ws.spl_id[r] = mine;
-            if (c > ahead && r == (uint32_t)((u64)ahead * S / c)) ws.sel->ahead = my;
-        }
-    }
+    rank_sample(ws, c, n_out, cs_ahead(a.k), &ws.sel->ahead, s_km, s_id, blockIdx.x, gridDim.x, ids_out, [&](uint32_t pos, u64 km, uint32_t) {
+        if (pos != n_out - 1u) return;
+        cs_sel_state now = *ws.sel;
+        now.ahead = ~0ull;                                    // (another CTA may not have stored it yet)
+        remember_key(ws, now, a.k, a.hint_slot, pos, km);
+    });
     CS_STAMP(ws, CS_PS_SAMPLE_DONE + (a.kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
 }
 
@@ -776,88 +651,15 @@ __global__ void __launch_bounds__(256) cs_sel_place_kernel(cs_workspace ws, uint
 {
     __shared__ u64 s_km[CS_SAMPLE], b_km[CS_BUCKETS];         // the sample, and where the buckets start
     __shared__ uint32_t s_id[CS_SAMPLE], b_id[CS_BUCKETS];
-    constexpr int ITEMS = 4;                                  // candidates per thread and round
-    const uint32_t tid = threadIdx.x;
     cs_wait_for_predecessor();
-    CS_STAMP(ws, CS_PS_PLACE_WAITED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
+    CS_STAMP(ws, CS_PS_PLACE_WAITED + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
     (void)kind;
-    // Everything the first round needs is asked for at once -- the select's state, the ranked sample and the round's keys
-    // (addresses bounded by the capacity of the buffers; what lies beyond the live counts is ignored below).  Item u of a
-    // round lies a grid-wide sweep after item u - 1, so that few candidates spread over all CTAs.
-    const uint32_t sweep = gridDim.x * 256u, lane0 = blockIdx.x * 256u + tid;
     const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_out, n_elig, b0
-    u64 km[ITEMS], sk[4];
-    uint32_t id[ITEMS], si[4];
-#pragma unroll
-    for (int u = 0; u < ITEMS; ++u) {
-        const uint32_t i = u * sweep + lane0, ii = i < max_blocks ? i : 0u;
-        km[u] = cs_ld_cg_pinned(ws.cand_km + ii);
-        id[u] = cs_ld_cg_pinned(ws.cand_id + ii);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) { sk[u] = cs_ld_cg_pinned(ws.spl_km + tid + 256 * u); si[u] = cs_ld_cg_pinned(ws.spl_id + tid + 256 * u); }
-    const uint32_t c = st.x, n_out = st.y;
-    if (n_out == 0 || c <= FEW_MAX) return;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) { s_km[tid + 256 * u] = sk[u]; s_id[tid + 256 * u] = si[u]; }
-    const OrderPlan P = order_plan(c, n_out, max_blocks, region_max);
-    __syncthreads();
-    const u64 cut_km = s_km[P.J - 1];
-    const uint32_t cut_id = s_id[P.J - 1];
-    for (uint32_t j = tid; j < CS_BUCKETS; j += 256u) bucket_start(P, s_km, s_id, j, b_km[j], b_id[j]);
-    __syncthreads();
-    cs_release_successor();                                   // (the ranking CTAs, four per SM, not before these keys are here)
-    for (uint32_t base = 0; base < c; base += sweep * ITEMS) {
-        if (base != 0) {
-#pragma unroll
-            for (int u = 0; u < ITEMS; ++u) {
-                const uint32_t i = base + u * sweep + lane0, ii = i < c ? i : 0u;
-                km[u] = cs_ld_cg_pinned(ws.cand_km + ii);
-                id[u] = cs_ld_cg_pinned(ws.cand_id + ii);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < ITEMS; ++u) {
-            const uint32_t i = base + u * sweep + lane0;
-            // keys from the cut up are dropped when there are samples beyond it
-            if (i >= c || (P.J < P.S && !less96(km[u], id[u], cut_km, cut_id))) continue;
-            uint32_t b = 0;                                   // the last bucket that starts at or below the key
-#pragma unroll
-            for (uint32_t step = CS_BUCKETS / 2; step > 0; step >>= 1)
-                b += less96(km[u], id[u], b_km[b + step], b_id[b + step]) ? 0u : step;
-            const uint32_t slot = atomicAdd(&CS_BCOUNT(ws, b), 1u);
-            if (slot < P.cap) {
-                ws.sort_km[(size_t)b * P.cap + slot] = km[u];
-                ws.sort_id[(size_t)b * P.cap + slot] = id[u];
-            }
-        }
-    }
-    CS_STAMP(ws, CS_PS_PLACE_DONE + (kind == 2 ? 8 : 0), blockIdx.x == 0 && tid == 0);
+    // (the ranking CTAs, four per SM, not before these keys are here)
+    place_candidates(ws, st, max_blocks, region_max, s_km, s_id, b_km, b_id, blockIdx.x, gridDim.x, [] { cs_release_successor(); });
+    CS_STAMP(ws, CS_PS_PLACE_DONE + (kind == 2 ? 8 : 0), blockIdx.x == 0 && threadIdx.x == 0);
 }
 
-// The key the next call of this kind gets: the one it had while the candidates it gave were enough and not too many; where
-// they were too many, the key below which cs_ahead(k) of them lay; where they were few, as much beyond it as the
-// candidates above the list's last entry say that cs_ahead(k) would need.
-__device__ __forceinline__ u64 next_bound(const cs_sel_state &st, uint32_t k, u64 kth)
-{
-    const u64 none = ~0ull, all = ~0ull - 1ull;
-    if (st.n_elig <= k) return all;                           // everything eligible is wanted
-    const uint32_t ahead = cs_ahead(k);
-    if (st.ahead != none && (!st.spec || st.c > ahead + ahead / 4u)) return st.ahead < all ? st.ahead : all;
-    if (st.c >= 2ull * k + 1024ull || st.c >= st.n_elig || st.bound >= all || st.bound < kth) return st.bound < all ? st.bound : all;
-    const u64 gap = st.bound - kth, per = (ahead - st.c) / (st.c - k + 1u);
-    const u64 more = (gap < (1ull << 40) ? gap : (1ull << 40)) * (per < 8ull ? per : 8ull) + 64ull;
-    return more < all - st.bound ? st.bound + more : all;
-}
-
-// Bucket b of CTA b: ranked by counting while it is small, sorted in the tile (bitonic, O(m log^2 m)) when it is larger, and through a
-// list of its keys' places, sorted in global memory, when the tile does not hold it.  The list lies where the bucket's ids lie in the
-// whole order -- [off, off + m) of an array of one word per entry -- so that no two buckets share a word.  Long lists come here as a
-// matter of course: the keys between two samples are exponentially spread, so the largest of several hundred buckets is four to six times
-// the mean one (432,000 candidates, k = 150,000: one or two buckets of 2,300 keys; 1,730,000, k = 600,000: 9,000).
-#define FINISH_THREADS 512u
-#define FINISH_COUNT_MAX 512u
-static_assert(FINISH_THREADS == CS_BUCKETS, "one bucket size per thread");
 __global__ void __launch_bounds__(FINISH_THREADS, 3)
 cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t region_max, uint32_t kind, uint32_t hint_slot,
                      uint32_t *__restrict__ ids_out)
@@ -872,93 +674,12 @@ cs_sel_finish_kernel(cs_workspace ws, uint32_t k, uint32_t max_blocks, uint32_t 
     CS_STAMP(ws, CS_PS_FINISH_WAITED + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
     cs_release_successor();
     const uint4 st = cs_ld_cg_pinned((const uint4 *)&ws.sel->c);          // c, n_out, n_elig, b0
-    const uint32_t n_t = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid));
-    uint32_t m = cs_ld_cg_pinned(&CS_BCOUNT(ws, b));
-    const uint32_t c = st.x, n_out = st.y;
+    const uint32_t n_t = cs_ld_cg_pinned(&CS_BCOUNT(ws, tid)), m = cs_ld_cg_pinned(&CS_BCOUNT(ws, b)), c = st.x, n_out = st.y;
     if (n_out == 0 || c <= FEW_MAX) return;
     const OrderPlan P = order_plan(c, n_out, max_blocks, region_max);
     if (b >= P.nb) return;
-    const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, tid < b ? n_t : 0u);
-    if ((tid & 31) == 0 && before) atomicAdd(&s_off, before);
-    if (b == 0) {                                             // work counters, and whether any bucket outgrew its region
-        const uint32_t most = __reduce_max_sync(0xFFFFFFFFu, n_t);
-        if ((tid & 31) == 0) atomicMax(&s_max, most);
-    }
-    __syncthreads();
-    const uint32_t off = s_off;
-    if (b == 0 && tid == 0 && kind < 3) {
-        atomicAdd((unsigned long long *)&ws.cnt->region_selects[kind], 1ull);
-        if (s_max > P.cap) atomicAdd((unsigned long long *)&ws.cnt->region_overflows[kind], 1ull);
-    }
-    // (should the sample have misled, the last bucket takes everything from its start on)
-    const bool rest = b == P.nb - 1u && P.J < P.S && off + m < n_out;
-    if (rest) m = c - off;
-    if (off >= n_out || m == 0) return;
-    const u64 *src_km = ws.sort_km + (size_t)b * P.cap;
-    const uint32_t *src_id = ws.sort_id + (size_t)b * P.cap;
-    // one id of the list; whoever places the last one knows the k-th key and chooses the next call's
-    auto emit = [&](uint32_t r, u64 km, uint32_t id) {
-        const uint32_t pos = off + r;
-        if (pos >= n_out) return;
-        ids_out[pos] = id;
-        if (pos == n_out - 1 && hint_slot < 3) ws.sc->sel_T[hint_slot] = next_bound(*ws.sel, k, km);
-    };
-    const bool outgrown = m > P.cap || rest, fits = m <= RANK_TILE;
-    uint32_t *const list = ws.cand_bkt + off;                 // [m] places of the keys when the tile does not hold them
-    if (outgrown) {
-        // the region was too small: the bucket's keys once more, out of all candidates
-        u64 lo_km, hi_km;
-        uint32_t lo_id, hi_id;
-        bucket_start(P, ws.spl_km, ws.spl_id, b, lo_km, lo_id);
-        bucket_start(P, ws.spl_km, ws.spl_id, b + 1u, hi_km, hi_id);
-        if (b == P.nb - 1u && P.J < P.S && !rest) { hi_km = ws.spl_km[P.J - 1]; hi_id = ws.spl_id[P.J - 1]; }
-        for (uint32_t i0 = tid; i0 < c; i0 += 4u * FINISH_THREADS) {
-            u64 km[4];
-            uint32_t id[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t i = i0 + u * FINISH_THREADS;
-                km[u] = __ldcg(ws.cand_km + (i < c ? i : 0u));
-                id[u] = __ldcg(ws.cand_id + (i < c ? i : 0u));
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t i = i0 + u * FINISH_THREADS;
-                if (i >= c || less96(km[u], id[u], lo_km, lo_id) || !less96(km[u], id[u], hi_km, hi_id)) continue;
-                const uint32_t at = atomicAdd(&s_n, 1u);      // (m of them: the bucket's counter has counted the same keys)
-                if (at >= m) continue;
-                if (fits) { t_km[at] = km[u]; t_id[at] = id[u]; }
-                else list[at] = i;
-            }
-        }
-        __syncthreads();
-        m = min(m, s_n);
-    } else if (fits) {
-        for (uint32_t i = tid; i < m; i += FINISH_THREADS) {
-            t_km[i] = __ldcg(src_km + i);
-            t_id[i] = __ldcg(src_id + i);
-        }
-        __syncthreads();
-    } else {
-        for (uint32_t i = tid; i < m; i += FINISH_THREADS) list[i] = i;
-        __syncthreads();
-    }
-    if (!fits) {
-        const u64 *k_km = outgrown ? ws.cand_km : src_km;
-        const uint32_t *k_id = outgrown ? ws.cand_id : src_id;
-        sort_places(list, m, k_km, k_id);
-        for (uint32_t i = tid; i < m && off + i < n_out; i += FINISH_THREADS) {
-            const uint32_t at = __ldcg(list + i);
-            emit(i, __ldcg(k_km + at), __ldcg(k_id + at));
-        }
-        return;
-    }
-    if (m <= FINISH_COUNT_MAX) {
-        rank_keys(t_km, t_id, m, t_km, t_id, m, emit);
-    } else {
-        sort_tile(t_km, t_id, m);
-        for (uint32_t i = tid; i < m; i += FINISH_THREADS) emit(i, t_km[i], t_id[i]);
-    }
+    finish_bucket(ws, c, n_out, P, b, n_t, m, kind, t_km, t_id, &s_off, &s_max, &s_n, ids_out,
+                  [&](uint32_t pos, u64 km, uint32_t) { if (pos == n_out - 1u) remember_key(ws, *ws.sel, k, hint_slot, pos, km); });
     CS_STAMP(ws, CS_PS_FINISH_DONE + (kind == 2 ? 8 : 0), b == 0 && tid == 0);
 }
 
@@ -1175,17 +896,49 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage, cs_select_graph 
     return CS_OK;
 }
 
-// One select: the single-launch cluster kernel where it applies, else the chain.
-static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier,
+// The route of selects over n entries, the longest list k: a cluster per list, one launch on the whole GPU for all of them, or a launch chain
+// per list.  Both sides of the lines, us per call: three lists and the refresh before them, back to back in a graph (static index), and the
+// three lists alone where every list's entries have left the index before the next call (moving).
+//   cluster / whole GPU  static 80,000 entries, k = 256 19.0 / 18.2, 131,072 22.1 / 20, 262,000 27.4 / 18.2; 131,072, k = 4,000 41.0 / 24.6,
+//                        262,000, k = 16,000 69.3 / 35.9; moving 80,000, k = 256 27.6 / 37.0, 131,072, k = 4,000 45.1 / 46.1
+//   chain / whole GPU    static 300,000, k = 256 28.6 / 20.6, 1,000,000, k = 10,000 48.3 / 30.8, 4,000,000, k = 20,000 75.9 / 49; moving
+//                        44.9 / 32.0, 52.6 / 51.2, 85.9 / 71.7; a remembered key that does not hold, 4,000,000, k = 1,359 70 / 66; one list 1,000,000, k = 10,000 29.2 / 13.5, 32,000,000 73.7 / 70.4, 64,000,000
+//                        114.3 / 119.5; 300,000, k = 75,000 63.8 / 39.7, 1,000,000, k = 142,857 87 / 89
+// A list's first call finds nothing remembered and has four passes more: it takes the route that the list would have without this one
+// (1,000,000 entries, two lists: 114 us, 123 in one launch).
+enum { ROUTE_CLUSTER, ROUTE_GRID, ROUTE_CHAIN };
+static int select_route(cs_ctx *ctx, uint32_t n, uint32_t k, uint32_t lists)
+{
+    if (ctx->select_path == CS_SELECT_MULTI) return ROUTE_CHAIN;
+    const bool fits = n <= CS_SELECT_CLUSTER_MAX_BLOCKS, asked = (ctx->lists_asked & lists) == lists;
+    const bool grid = fits ? ctx->select_path != CS_SELECT_CLUSTER && (n > CS_SELECT_GRID_MIN_BLOCKS || (n > CS_SELECT_GRID_LONG_BLOCKS && k >= CS_SELECT_GRID_LONG_LIST))
+                           : n <= CS_SELECT_GRID_MAX_BLOCKS && k <= CS_SELECT_GRID_MAX_LIST;
+    if (grid) ctx->lists_asked |= lists;
+    if (grid && asked) return ROUTE_GRID;
+    return fits ? ROUTE_CLUSTER : ROUTE_CHAIN;
+}
+
+// One select.
+static int launch_select_job(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier,
                              uint32_t k, uint32_t *ids_out, uint32_t *n_out, cudaStream_t s)
 {
-    SelectChain c;
-    prepare_chain(ctx, job, idx, now, prefetch, tier, k, ids_out, n_out, s, c);
-    if (ctx->select_path != CS_SELECT_MULTI && idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) {
-        const int rc1 = cs_launch_select_cluster(ctx, &c.a, c.ws, prefetch, ids_out, n_out, s);
-        if (rc1 != CS_ENOTIMPL) return rc1;          // no usable cluster on this device: fall through
+    const uint32_t l = prefetch ? 2u : tier, ks[3] = {k, k, k};
+    int route = select_route(ctx, idx->n_blocks, k, 1u << l), rc = CS_ENOTIMPL;
+    if (route == ROUTE_GRID) {
+        uint32_t *ids[3] = {}, *cnt[3] = {};
+        ids[l] = ids_out;
+        cnt[l] = n_out;
+        rc = cs_launch_select_grid(ctx, idx, now, ks, ids, cnt, s);
+        if (rc != CS_ENOTIMPL) return rc;
+        if (idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) route = ROUTE_CLUSTER;
     }
-    int rc = scan_opt_in(ctx);
+    SelectChain c;
+    prepare_chain(ctx, 0, idx, now, prefetch, tier, k, ids_out, n_out, s, c);
+    if (route == ROUTE_CLUSTER) {
+        rc = cs_launch_select_cluster(ctx, &c.a, c.ws, prefetch, ids_out, n_out, s);
+        if (rc != CS_ENOTIMPL) return rc;            // no usable cluster on this device: fall through
+    }
+    rc = scan_opt_in(ctx);
     for (int stage = 0; stage < SELECT_STAGES && rc == CS_OK; ++stage) rc = launch_stage(ctx, c, stage);
     return rc;
 }
@@ -1193,7 +946,7 @@ static int launch_select_job(cs_ctx *ctx, int job, const cs_block_index *idx, ui
 int cs_launch_select(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, int prefetch, uint32_t tier, uint32_t k,
                      uint32_t *ids_out, uint32_t *n_out, cudaStream_t s)
 {
-    return launch_select_job(ctx, 0, idx, now, prefetch, tier, k, ids_out, n_out, s);
+    return launch_select_job(ctx, idx, now, prefetch, tier, k, ids_out, n_out, s);
 }
 
 // The chains of selects side by side as one graph launch: true when it was launched, false when it has to be done launch by launch.
@@ -1277,7 +1030,19 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
     for (int q = 0; q < 3; ++q)
         if (cnt[q]) jobs[n_jobs++] = q;
     if (n_jobs == 0) return CS_OK;
-    if (ctx->select_path != CS_SELECT_MULTI && idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS) {
+    uint32_t k_most = 0, lists = 0;
+    for (int i = 0; i < n_jobs; ++i) {
+        k_most = std::max(k_most, ks[jobs[i]]);
+        lists |= 1u << jobs[i];
+    }
+    const bool together = ctx->concurrent_selects || idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS;           // every list has scratch of its own
+    int route = together ? select_route(ctx, idx->n_blocks, k_most, lists) : ROUTE_CHAIN, rc = CS_OK;
+    if (route == ROUTE_GRID) {
+        rc = cs_launch_select_grid(ctx, idx, now, ks, ids, cnt, s);
+        if (rc != CS_ENOTIMPL) return rc;
+        route = idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS ? ROUTE_CLUSTER : ROUTE_CHAIN;
+    }
+    if (route == ROUTE_CLUSTER) {
         SelArgs a[3];
         uint32_t *j_ids[3], *j_cnt[3];
         uint32_t pf[3];
@@ -1293,14 +1058,14 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
             j_cnt[i] = cnt[q];
             pf[i] = q == 2 ? 1u : 0u;
         }
-        const int rc = cs_launch_select_clusters(ctx, n_jobs, a, pf, j_ids, j_cnt, s);
+        rc = cs_launch_select_clusters(ctx, n_jobs, a, pf, j_ids, j_cnt, s);
         if (rc != CS_ENOTIMPL) return rc;
     }
-    int rc = CS_OK;
+    rc = CS_OK;
     if (!ctx->concurrent_selects || n_jobs == 1) {
         for (int i = 0; i < n_jobs && rc == CS_OK; ++i) {
             const int q = jobs[i];
-            rc = launch_select_job(ctx, 0, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], s);
+            rc = launch_select_job(ctx, idx, now, q == 2, q == 0 ? 0u : 1u, ks[q], ids[q], cnt[q], s);
         }
         return rc;
     }

@@ -125,8 +125,8 @@ __device__ __forceinline__ float score_of(const SelArgs &a, const Tables &T, uin
 
 // Histogram bin of a primary key: the range of possible scores divided evenly over the bins (of both classes of a prefetch
 // list), clamped at its ends, which keeps the order whatever the survival table holds.
-template <bool PF>
-__device__ __forceinline__ uint32_t bin_of(const SelArgs &a, uint32_t pr)
+template <bool PF, class Bins>
+__device__ __forceinline__ uint32_t bin_of(const Bins &a, uint32_t pr)
 {
     const uint32_t v = PF ? pr & 0x7FFFFFFFu : pr;
     const uint32_t x = (v > a.bin_lo ? v - a.bin_lo : 0u) >> a.bin_shift;
@@ -136,8 +136,8 @@ __device__ __forceinline__ uint32_t bin_of(const SelArgs &a, uint32_t pr)
 }
 
 // "bin <= b0" as a limit on the primary key: candidate <=> primary < limit.
-template <bool PF>
-__device__ __forceinline__ u64 primary_limit(const SelArgs &a, uint32_t b0)
+template <bool PF, class Bins>
+__device__ __forceinline__ u64 primary_limit(const Bins &a, uint32_t b0)
 {
     constexpr uint32_t PER_CLASS = PF ? CS_HIST_BINS / 2 : CS_HIST_BINS;
     const uint32_t b = b0 % PER_CLASS;

@@ -1230,6 +1230,70 @@ def test_select_step_graph_takes_new_arguments(wanted):
     assert c.get_status() == 0
 
 
+# CTA and quad boundaries of 148 CTAs of 512 threads, four entries each, with the one to three entries behind the last whole quad; the shortest
+# indexes of the route with long lists and with short ones; more than three steps per thread.
+@pytest.mark.parametrize("n", [65_537, 131_073, 303_104, 303_107, 303_105 + 2048, 1_212_418])
+@pytest.mark.parametrize("kind", ["spread", "tied", "few", "bad", "bare"])
+def test_select_on_the_whole_gpu(n, kind):
+    """One launch for all lists of a large index.  Nine calls with lists of several lengths, a clock that goes on and back and an index whose
+    victims have been used again (remembered keys and buckets that hold, and that do not); ages tied down to the id; an index with few eligible
+    entries; agents out of range; no token counts or anchors, one list at a time.  Every list against the launch chain, bit for bit,
+    the last ones against the oracle."""
+    cfg = synth.CONFIGS["meta1m"]
+    c, o = warm_state(cfg, 800, n, r_min=0.02, prefer_other_copy=int(kind == "few"))
+    chain, _ = warm_state(cfg, 800, n, r_min=0.02, prefer_other_copy=int(kind == "few"))
+    chain.set_select_path(cs.CS_SELECT_MULTI)
+    idx = synth.make_block_index(cfg, n=n, tier="random", with_tokens=kind != "bare", with_anchor=kind != "bare")
+    rng = synth.rng_for(cfg, 97)
+    if kind == "tied":
+        idx.last_access[:] = 90_000 + rng.integers(0, 2, n)
+    elif kind == "few":
+        idx.ref_count[rng.permutation(n)[:n - 900]] = 1
+    elif kind == "bad":
+        idx.agent[rng.permutation(n)[:50]] = 0xFFFF
+        idx.agent[n - 1] = cfg.n_agents
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    la = d.last_access.view(torch.int32)
+    empty = lambda m: torch.full((m,), 7, dtype=torch.int32, device=DEV)
+    side = torch.cuda.Stream()
+    for rep in range(9):
+        now = 100_000 + (0, 1, 2, 500, 501, 3, 4, 5, 6)[rep]
+        kv, kp = ((2500, 2100), (1, 37), (2500, 2500))[rep // 3]
+        outs = []
+        for x in (c, chain):
+            b = [empty(max(k, 4)) if i % 2 == 0 else empty(4) for k in (kv, kv, kp) for i in range(2)]
+            if kind == "bare":
+                x.select_victims(d, now, 0, kv, b[0], b[1])
+                x.select_victims(d, now, 1, kv, b[2], b[3])
+                x.select_prefetch(d, now, kp, b[4], b[5])
+            elif rep == 7 and x is c:
+                torch.cuda.synchronize()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=side):
+                    x.select_step(d, now, kv, kp, *b)
+                g.replay()
+            else:
+                x.select_step(d, now, kv, kp, *b)
+            outs.append(b)
+        torch.cuda.synchronize()
+        for got, want in zip(*outs):
+            assert torch.equal(got, want), rep
+        if rep < 8 and kind != "bad":
+            la[outs[1][0][:kv].long().clamp_(min=0)] = now - 3
+    ca, cb = c.counters(), chain.counters()
+    assert ca["eligible"] == cb["eligible"] and ca["selected"] == cb["selected"]
+    status = cs.CS_ST_BAD_AGENT if kind == "bad" else 0
+    assert c.get_status() == chain.get_status() == status
+    idx.last_access[:] = d.last_access.cpu().numpy()
+    if kind == "bad":
+        idx.ref_count[idx.agent >= cfg.n_agents] = 1           # (in no list)
+        idx.agent[idx.agent >= cfg.n_agents] = 0
+    s64, s32 = o.scores(idx, now)
+    for got, got_n, k, (o_ids, o_n) in ((b[0], b[1], kv, o.select_victims(idx, now, 0, kv, s32)), (b[2], b[3], kv, o.select_victims(idx, now, 1, kv, s32)),
+                                        (b[4], b[5], kp, o.select_prefetch(idx, now, kp, s32))):
+        assert H.assert_list_matches(got.cpu().numpy().view(np.uint32)[:k], int(got_n[0].item()), o_ids, o_n, s64) == 0
+
+
 # ---- randomised small configurations ------------------------------------------------------------------------
 @pytest.mark.parametrize("case", range(48))
 def test_random_small_configurations(case):

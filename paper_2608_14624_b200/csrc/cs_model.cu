@@ -1052,6 +1052,214 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The same table with one product less.  A path's first visit to a splits its later ones off: with g_n = P^n[a0][a] and d_n = P^n[a][a],
+//     f_n = g_n - sum_{t < n} f_t d_{n-t}   is the probability that step n is the first at a, and p = f_1 + ... + f_K.
+// All of g and d come from the columns w_n = P^n[:, a], which are the same product for every start and with nothing removed:
+//     g_n = w_n[a0], d_n = w_n[a] for n <= K - 2;  g_{K-1} = r_1 w_{K-2}, g_K = r_2 w_{K-2}, d_{K-1} = P[a, :] w_{K-2},
+// r_1 and r_2 being rows a0 of P and P^2.  So w_{K-2} is enough, K - 3 products; r_2 is summed up from the tiles of P that the first of them brings.
+// The differences lose nothing that p has: every term of f_n is at most p, so what f_n is off by, before it goes on, is at most n roundings of p,
+// and it goes on as e_n = delta_n - sum e_t d_{n-t}, which the renewal equation sums to at most twice the deltas' sum.
+//
+// (Against extended precision, matrices of 4 to 256 agents, dense, sparse, nearly a chain, and of entries from 1e-9 to 1: both ways are within
+// 1.5e-15 of p, and after the rounding to fp32 the largest errors are the same to three digits, 6e-8.)
+//
+// Clusters as above, but a warp multiplies 16 rows by a slice of the agents with matrix instructions (m16n8k8; rows of the new w by the agents summed
+// over, times 8 targets), so that few slices are left to add up and the vectors are read from shared memory once for 16 rows.  Bound by the fp64 pipe
+// (64 rows, 256 agents, 8 targets: 2.1 us at 32 multiply-adds per clock and SM) and, as much again, by the exchange between two products.  us per call, products above /
+// here: K = 4 65 agents 8.3 / 7.3, 128 9.5 / 8.2, 256 13.5 / 10.9, 400 36.7 / 28.7; K = 6 13.2 / 10.2, 15.1 / 13.5, 22.0 / 19.7, 67.8 / 53.9.  Warps of 64
+// rows and short slices: 256 agents 11.9; two chains of instructions per warp 11.2.
+// Fewer steps than four have no product to save (r_2 costs what it saves with three: 400 agents 21.4 / 23.8), and one CTA's agents (64 at most) are
+// bound by the steps' latency (12 agents 4.4 / 4.5, six steps 5.9 / 7.0): they go as above.
+// ---------------------------------------------------------------------------------------------
+#define XS_ROWS 16u                      // rows of a warp's tile
+#define XS_DEEP 4u                       // instructions of eight agents whose part of the matrix is in flight
+#define XS_ROWS_PAD 18u                  // 16 rows of one target, padded: written and summed without bank conflicts
+#define XS_RENEWAL_STEPS 32u             // a lane per step in the end
+#define XS_SMEM_MOST (227u * 1024u - 256u)
+static size_t xs_renewal_smem(uint32_t A, uint32_t cl)
+{
+    return (2 * (size_t)A * XS_TARGETS + XS_WARPS * XS_TARGETS * XS_ROWS_PAD + (cl + 1u) * (size_t)A + XS_WARPS * 32u + 2u * XS_TARGETS * XS_RENEWAL_STEPS) * sizeof(double);
+}
+// c += a b: 16 x 8 by 8 x 8.  Lane l: a rows l/4 (a0, a2) and l/4 + 8 (a1, a3), columns l%4 (a0, a1) and l%4 + 4 (a2, a3); b rows l%4 and
+// l%4 + 4, column l/4; c rows l/4 (c0, c1) and l/4 + 8 (c2, c3), columns 2 (l%4) and 2 (l%4) + 1.
+__device__ __forceinline__ void mma_f64(double (&c)[4], double a0, double a1, double a2, double a3, double b0, double b1)
+{
+    asm("mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3]) : "d"(a0), "d"(a1), "d"(a2), "d"(a3), "d"(b0), "d"(b1));
+}
+// A probability of the matrix (0, or 2^-32 to 1) times 2^-896: a float's bits in a double's place, which costs no conversion.  The vectors that it is
+// multiplied with are kept times 2^896.  (A product of 64 rows, 256 agents and 8 targets 0.3 us less.)
+#define XS_UP 0x1p896
+#define XS_DOWN 0x1p-896
+__device__ __forceinline__ double scaled_down(float x)
+{
+    const uint32_t b = __float_as_uint(x);
+    return __hiloint2double((int)(b >> 3), (int)(b << 29));
+}
+__device__ __forceinline__ double warp_sum(double x)
+{
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, d);
+    return x;
+}
+
+__global__ void __launch_bounds__(XS_THREADS, 1)
+cs_renewal_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t K, uint32_t n_rows, float delta,
+                           float *__restrict__ psurv_out, float *__restrict__ fsurv_out)
+{
+    cg::cluster_group cluster = cg::this_cluster();
+    const uint32_t CL = cluster.num_blocks(), rank = cluster.block_rank();
+    const uint32_t row_warps = (n_rows + XS_ROWS - 1u) / XS_ROWS;            // (at most 16)
+    extern __shared__ __align__(16) double s_xs[];
+    double *const w_all = s_xs;                                    // [2][A][XS_TARGETS]
+    double *const part = w_all + 2 * (size_t)A * XS_TARGETS;       // [XS_WARPS][XS_TARGETS][XS_ROWS_PAD]
+    double *const r2_part = part + XS_WARPS * XS_TARGETS * XS_ROWS_PAD;      // [XS_WARPS][32]: r_2 over some of the CTA's rows,
+    double *const r2 = r2_part + XS_WARPS * 32u;                   // [CL][A]: over all of each CTA's
+    double *const r1 = r2 + (size_t)CL * A;                        // [A]
+    double *const s_g = r1 + A, *const s_d = s_g + XS_TARGETS * XS_RENEWAL_STEPS;      // [XS_TARGETS][XS_RENEWAL_STEPS]
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t base = (blockIdx.x / CL) * XS_TARGETS;          // this cluster's targets
+    const uint32_t row0 = min(rank * n_rows, A), row1 = min(row0 + n_rows, A);
+    const float *__restrict__ P = ws.P;
+    // this CTA holds the rows of the target that is this warp's
+    const uint32_t a = base + warp;
+    const bool mine = warp < XS_TARGETS && a < A && a >= row0 && a < row1;
+    cs_wait_for_predecessor();
+    cs_release_successor();
+    const uint32_t a0 = a0_arg == CS_AGENT_NONE ? ws.sc->last_agent : a0_arg;
+    double p = 0.0;
+    if (a0 < A) {
+        for (uint32_t e = tid; e < A * XS_TARGETS; e += XS_THREADS) {
+            const uint32_t j = e / XS_TARGETS, m = e % XS_TARGETS;
+            w_all[e] = base + m < A ? (double)P[(size_t)j * A + base + m] * XS_UP : 0.0;
+        }
+        for (uint32_t j = tid; j < A; j += XS_THREADS) r1[j] = (double)P[(size_t)a0 * A + j];
+        const uint32_t slices = XS_WARPS / row_warps, rw = warp % row_warps, sl = warp / row_warps;
+        const uint32_t groups = (A + 7u) / 8u, i_first = sl * groups / slices * 8u, i_end = sl < slices ? min((sl + 1u) * groups / slices * 8u, A) : i_first;
+        const uint32_t row = lane / 4u, depth = lane % 4u, j0 = row0 + rw * XS_ROWS + row;               // a lane's place in the operands
+        float next[XS_DEEP][4];                                    // of the matrix, on its way
+        const auto ask = [&](uint32_t i0) {
+#pragma unroll
+            for (uint32_t x = 0; x < XS_DEEP; ++x)
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; ++q) {
+                    const uint32_t i = i0 + 8u * x + depth + 4u * (q >> 1), j = j0 + 8u * (q & 1u);
+                    next[x][q] = i < i_end && j < row1 ? __ldg(P + (size_t)j * A + i) : 0.0f;
+                }
+        };
+        ask(i_first);
+        float own[8];                                              // the target's row of the matrix
+#pragma unroll
+        for (uint32_t h = 0; h < 8u; ++h) own[h] = mine && lane + 32u * h < A ? __ldg(P + (size_t)a * A + lane + 32u * h) : 0.0f;
+        cluster.sync();                                            // (also: every CTA has started before its memory is written)
+        uint32_t cur = 0;
+        const auto note = [&](uint32_t n) {                        // w_{n + 1} at a0 and at its own target
+            const double *w = w_all + (size_t)cur * A * XS_TARGETS;
+            if (tid < XS_TARGETS && base + tid < A) {
+                s_g[tid * XS_RENEWAL_STEPS + n] = w[(size_t)a0 * XS_TARGETS + tid] * XS_DOWN;
+                s_d[tid * XS_RENEWAL_STEPS + n] = w[(size_t)(base + tid) * XS_TARGETS + tid] * XS_DOWN;
+            }
+        };
+        for (uint32_t t = 0; t + 3u < K; ++t) {
+            const double *w = w_all + (size_t)cur * A * XS_TARGETS;
+            double *const nxt = w_all + (size_t)(cur ^ 1u) * A * XS_TARGETS;
+            note(t);
+            if (sl < slices) {
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+                for (uint32_t i0 = i_first; i0 < i_end; i0 += 8u * XS_DEEP) {
+                    float now[XS_DEEP][4];
+#pragma unroll
+                    for (uint32_t x = 0; x < XS_DEEP; ++x)
+#pragma unroll
+                        for (uint32_t q = 0; q < 4u; ++q) now[x][q] = next[x][q];
+                    if (i0 + 8u * XS_DEEP < i_end) ask(i0 + 8u * XS_DEEP);
+                    else if (t + 4u < K) ask(i_first);             // (the next product's)
+#pragma unroll
+                    for (uint32_t x = 0; x < XS_DEEP; ++x) {
+                        const uint32_t i = i0 + 8u * x + depth;
+                        if (i0 + 8u * x < i_end)                   // (past the end: times zero)
+                            mma_f64(acc, scaled_down(now[x][0]), scaled_down(now[x][1]), scaled_down(now[x][2]), scaled_down(now[x][3]),
+                                    w[(size_t)min(i, A - 1u) * XS_TARGETS + row], w[(size_t)min(i + 4u, A - 1u) * XS_TARGETS + row]);
+                    }
+                }
+                double *o = part + (size_t)warp * XS_TARGETS * XS_ROWS_PAD + row;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; ++q) o[(2u * depth + (q & 1u)) * XS_ROWS_PAD + 8u * (q >> 1)] = acc[q];
+            }
+            // r_2 over this CTA's rows, which the products above have brought to its L1: 32 agents per warp, what warps are over share the rows
+            const uint32_t chunks = (A + 31u) / 32u, sharers = max(1u, XS_WARPS / chunks), share = warp / chunks;
+            if (t == 0u && share < sharers)
+                for (uint32_t c = warp % chunks; c < chunks; c += XS_WARPS) {
+                    const uint32_t i = min(32u * c + lane, A - 1u), j_end = row0 + (row1 - row0) * (share + 1u) / sharers;
+                    double s0 = 0.0, s1 = 0.0;
+                    uint32_t j = row0 + (row1 - row0) * share / sharers;
+#pragma unroll 8
+                    for (; j + 1u < j_end; j += 2u) {
+                        s0 = fma(r1[j], scaled_down(__ldg(P + (size_t)j * A + i)), s0);
+                        s1 = fma(r1[j + 1u], scaled_down(__ldg(P + (size_t)(j + 1u) * A + i)), s1);
+                    }
+                    if (j < j_end) s0 = fma(r1[j], scaled_down(__ldg(P + (size_t)j * A + i)), s0);
+                    if (sharers > 1u) r2_part[32u * warp + lane] = s0 + s1;
+                    else if (32u * c + lane < A)
+                        for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(r2, r)[(size_t)rank * A + i] = s0 + s1;
+                }
+            __syncthreads();
+            for (uint32_t e = tid; e < (row1 - row0) * XS_TARGETS; e += XS_THREADS) {
+                const uint32_t jc = e / XS_TARGETS, m = e % XS_TARGETS;
+                const double *q = part + (size_t)(jc / XS_ROWS) * XS_TARGETS * XS_ROWS_PAD + m * XS_ROWS_PAD + jc % XS_ROWS;
+                double sum = 0.0;
+#pragma unroll 4
+                for (uint32_t u = 0; u < slices; ++u) sum += q[(size_t)u * row_warps * XS_TARGETS * XS_ROWS_PAD];
+                for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(nxt, r)[(size_t)(row0 + jc) * XS_TARGETS + m] = sum * XS_UP;
+            }
+            if (t == 0u && sharers > 1u)
+                for (uint32_t i = tid; i < A; i += XS_THREADS) {
+                    double sum = 0.0;
+                    for (uint32_t u = 0; u < sharers; ++u) sum += r2_part[32u * (u * chunks + i / 32u) + i % 32u];
+                    for (uint32_t r = 0; r < CL; ++r) cluster.map_shared_rank(r2, r)[(size_t)rank * A + i] = sum;
+                }
+            cluster.sync();                                        // the new w is complete everywhere; `part` is free again
+            cur ^= 1u;
+        }
+        note(K - 3u);
+        __syncthreads();
+        if (mine) {
+            const double *w = w_all + (size_t)cur * A * XS_TARGETS + warp;
+            double x1 = 0.0, x2 = 0.0, x3 = 0.0;
+#pragma unroll 1
+            for (uint32_t i0 = 0; i0 < A; i0 += 256u)
+#pragma unroll
+                for (uint32_t h = 0; h < 8u; ++h) {
+                    const uint32_t i = i0 + lane + 32u * h;
+                    if (i >= A) continue;
+                    const double y = w[(size_t)i * XS_TARGETS];
+                    double r = 0.0;
+                    for (uint32_t c = 0; c < CL; ++c) r += r2[(size_t)c * A + i];
+                    x1 = fma(r1[i], y * XS_DOWN, x1);
+                    x2 = fma(r, y, x2);                            // (r_2 is scaled down)
+                    x3 = fma(scaled_down(i0 ? __ldg(P + (size_t)a * A + i) : own[h]), y, x3);
+                }
+            x1 = warp_sum(x1);
+            x2 = warp_sum(x2);
+            x3 = warp_sum(x3);
+            // step lane + 1: its g, from which the steps before it are taken in turn, and its d
+            double f = lane + 2u < K ? s_g[warp * XS_RENEWAL_STEPS + lane] : x2, d = lane + 2u < K ? s_d[warp * XS_RENEWAL_STEPS + lane] : x3;
+            if (lane + 2u == K) f = x1;
+            for (uint32_t n = 0; n < K; ++n) {
+                const double f_n = __shfl_sync(0xFFFFFFFFu, f, n), d_n = __shfl_sync(0xFFFFFFFFu, d, (lane - n - 1u) & 31u);
+                p += f_n;
+                if (lane > n) f = fma(-f_n, d_n, f);
+            }
+        }
+    }
+    if (mine && lane == 0) {
+        if (psurv_out) psurv_out[a] = (float)p;
+        if (fsurv_out) fsurv_out[a] = (float)(p + (double)delta);
+    }
+}
+
 int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_out, float *fsurv_out, cudaStream_t s)
 {
     const cs_params &p = ctx->p;
@@ -1064,6 +1272,7 @@ int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_
             const int most = (int)xs_smem_bytes(CS_MAX_AGENTS);
             cudaError_t e = cudaFuncSetAttribute(cs_exact_survival_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(cs_exact_survival_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(cs_renewal_survival_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XS_SMEM_MOST);
             if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
             opted[ctx->device] = true;
         }
@@ -1073,6 +1282,12 @@ int cs_launch_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t K, float *psurv_
     uint32_t cl = 1;
     while (cl < XS_MAX_CLUSTER && p.n_agents > 64u * cl && 2u * cl * n_clusters <= (uint32_t)ctx->sm_count) cl *= 2;
     const uint32_t n_cols = (p.n_agents + cl - 1) / cl;
+    const size_t smem = xs_renewal_smem(p.n_agents, cl);
+    if (cl > 1u && n_cols <= XS_WARPS * XS_ROWS && K >= 4u && K <= XS_RENEWAL_STEPS && smem <= XS_SMEM_MOST) {
+        cs_launch_chained_clusters(cs_renewal_survival_kernel, n_clusters * cl, cl, XS_THREADS, smem, s, ctx->ws, p.n_agents, a0, K, n_cols, p.delta,
+                                   psurv_out, fsurv_out);
+        return cs_check_launch(ctx);
+    }
     cs_launch_chained_clusters(cl == 1u ? cs_exact_survival_kernel<true> : cs_exact_survival_kernel<false>, n_clusters * cl, cl > 1u ? cl : 0u,
                                XS_THREADS, xs_smem_bytes(p.n_agents), s, ctx->ws, p.n_agents, a0, K, n_cols, p.delta, psurv_out, fsurv_out);
     return cs_check_launch(ctx);

@@ -907,13 +907,19 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage, cs_select_graph 
 // A list's first call finds nothing remembered and has four passes more: it takes the route that the list would have without this one
 // (1,000,000 entries, two lists: 114 us, 123 in one launch).
 enum { ROUTE_CLUSTER, ROUTE_GRID, ROUTE_CHAIN };
-static int select_route(cs_ctx *ctx, uint32_t n, uint32_t k, uint32_t lists)
+static int select_route(cs_ctx *ctx, uint32_t n, uint32_t k, uint32_t lists, cudaStream_t s)
 {
     if (ctx->select_path == CS_SELECT_MULTI) return ROUTE_CHAIN;
     const bool fits = n <= CS_SELECT_CLUSTER_MAX_BLOCKS, asked = (ctx->lists_asked & lists) == lists;
     const bool grid = fits ? ctx->select_path != CS_SELECT_CLUSTER && (n > CS_SELECT_GRID_MIN_BLOCKS || (n > CS_SELECT_GRID_LONG_BLOCKS && k >= CS_SELECT_GRID_LONG_LIST))
                            : n <= CS_SELECT_GRID_MAX_BLOCKS && k <= CS_SELECT_GRID_MAX_LIST;
     if (grid) ctx->lists_asked |= lists;
+    if (grid && !asked) {
+        // (what is captured runs again: its later runs are not first calls)
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) (void)cudaGetLastError();
+        if (capture == cudaStreamCaptureStatusActive) return ROUTE_GRID;
+    }
     if (grid && asked) return ROUTE_GRID;
     return fits ? ROUTE_CLUSTER : ROUTE_CHAIN;
 }
@@ -923,7 +929,7 @@ static int launch_select_job(cs_ctx *ctx, const cs_block_index *idx, uint32_t no
                              uint32_t k, uint32_t *ids_out, uint32_t *n_out, cudaStream_t s)
 {
     const uint32_t l = prefetch ? 2u : tier, ks[3] = {k, k, k};
-    int route = select_route(ctx, idx->n_blocks, k, 1u << l), rc = CS_ENOTIMPL;
+    int route = select_route(ctx, idx->n_blocks, k, 1u << l, s), rc = CS_ENOTIMPL;
     if (route == ROUTE_GRID) {
         uint32_t *ids[3] = {}, *cnt[3] = {};
         ids[l] = ids_out;
@@ -1036,7 +1042,7 @@ int cs_launch_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
         lists |= 1u << jobs[i];
     }
     const bool together = ctx->concurrent_selects || idx->n_blocks <= CS_SELECT_CLUSTER_MAX_BLOCKS;           // every list has scratch of its own
-    int route = together ? select_route(ctx, idx->n_blocks, k_most, lists) : ROUTE_CHAIN, rc = CS_OK;
+    int route = together ? select_route(ctx, idx->n_blocks, k_most, lists, s) : ROUTE_CHAIN, rc = CS_OK;
     if (route == ROUTE_GRID) {
         rc = cs_launch_select_grid(ctx, idx, now, ks, ids, cnt, s);
         if (rc != CS_ENOTIMPL) return rc;

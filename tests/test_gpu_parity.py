@@ -787,6 +787,24 @@ def test_exact_survival_table_shapes(A, Ks):
         assert np.all(np.abs(fs.cpu().numpy().astype(np.float64) - (want + d64)) <= (3 * K + 2) * 2.0 ** -24 * (want + d64)), (A, K)
 
 
+@pytest.mark.parametrize("A,Ks", [(65, (4, 5, 31, 32, 33)), (66, (4,)), (127, (5,)), (128, (4,)), (129, (6,)), (257, (4, 7)), (304, (5,)), (511, (4,)),
+                                  (512, (4,)), (513, (4,))])
+@pytest.mark.parametrize("links", [1, 6])
+def test_exact_survival_by_first_visits(A, Ks, links):
+    """More agents than one CTA's, on both sides of the tiles (16 rows, 8 agents), of every cluster size and of the widest share of a CTA (256 rows),
+    with the fewest and the most steps that take this way and one more; a chain of agents that return rarely and one of few links, where most
+    targets cannot be reached.  The bound of the test above; the differences that first visits are add 2 K^2 roundings of fp64."""
+    cfg = synth.shrink(synth.CONFIGS["meta1m"], n_agents=A, transitions=("sparse", links))
+    c, o = warm_state(cfg, 3000, 64, r_min=0.0)
+    for K in Ks:
+        for a0 in (None, A - 1):
+            ps, _ = c.exact_survival(K, a0=a0) if a0 is not None else c.exact_survival(K)
+            want = o.exact_survival(K, a0)
+            got = ps.cpu().numpy().astype(np.float64)
+            assert np.all(np.abs(got - want) <= (3 * K + 1) * 2.0 ** -24 * want + 2 * K * K * 2.0 ** -53), (A, K)
+            assert np.all(got[want == 0] == 0)
+
+
 def test_select_with_other_tier_copy_preference():
     """cs_params.prefer_other_copy = 1: (score, has no copy, last_access, id), both select paths."""
     cfg = synth.CONFIGS["llama8b"]

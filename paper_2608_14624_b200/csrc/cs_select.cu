@@ -900,9 +900,9 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage, cs_select_graph 
 // per list.  Both sides of the lines, us per call: three lists and the refresh before them, back to back in a graph (static index), and the
 // three lists alone where every list's entries have left the index before the next call (moving).
 //   cluster / whole GPU  static 80,000 entries, k = 256 19.0 / 18.2, 131,072 22.1 / 20, 262,000 27.4 / 18.2; 131,072, k = 4,000 41.0 / 24.6,
-//                        262,000, k = 16,000 69.3 / 35.9; moving 80,000, k = 256 27.6 / 37.0, 131,072, k = 4,000 45.1 / 46.1
+//                        262,000, k = 16,000 69.3 / 35.9; moving 80,000, k = 256 27.6 / 37.0, 131,072, k = 4,000 45.1 / 50.3
 //   chain / whole GPU    static 300,000, k = 256 28.6 / 20.6, 1,000,000, k = 10,000 48.3 / 30.8, 4,000,000, k = 20,000 75.9 / 49; moving
-//                        44.9 / 32.0, 52.6 / 51.2, 85.9 / 71.7; a remembered key that does not hold, 4,000,000, k = 1,359 70 / 66; one list 1,000,000, k = 10,000 29.2 / 13.5, 32,000,000 73.7 / 70.4, 64,000,000
+//                        44.9 / 29.9, 52.6 / 33.8, 85.9 / 75.8; a remembered key that does not hold, 4,000,000, k = 1,359 70 / 66; one list 1,000,000, k = 10,000 29.2 / 13.5, 32,000,000 73.7 / 70.4, 64,000,000
 //                        114.3 / 119.5; 300,000, k = 75,000 63.8 / 39.7, 1,000,000, k = 142,857 87 / 89
 // A list's first call finds nothing remembered and has four passes more: it takes the route that the list would have without this one
 // (1,000,000 entries, two lists: 114 us, 123 in one launch).

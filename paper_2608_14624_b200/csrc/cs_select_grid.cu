@@ -8,7 +8,7 @@
 //              of eight keys.  Whoever places every step-th key stores it as a boundary for the next call: exact quantiles of this call's
 //              order, up to 2.25 lists from its beginning, because a list's entries are usually gone by then.
 //
-// The boundaries decide nothing but the sizes of the buckets.  Where they do not hold -- a bucket of many times the keys aimed at, too few
+// The boundaries decide nothing but the sizes of the buckets.  Where they do not hold -- a bucket of more than 1,024 keys, too few
 // keys below the last boundary, the first calls -- the candidates are ordered by a ranked sample instead (cs_select_buckets.cuh; two more
 // barriers), and where the remembered key does not, a histogram and a collect pass come first (two more).  Both are remembered as scores and
 // ages: their last_access moves on with the clock.
@@ -33,8 +33,8 @@
 #define SG_STEP 24u                    // keys of a bucket aimed at, as long as CS_BUCKETS buckets hold the list
 #define SG_BUCKET_WARP 96u             // largest bucket that one warp ranks, three keys per lane
 #define SG_KEYS 128u                   // keys that a warp holds at a time
-#define SG_BUCKET_MAX 256u             // largest bucket that is counted, or twelve times the mean: a cluster of 1,000 keys takes its CTAs longer than
-#define SG_SAMPLED_MAX 1024u           // the sample's two barriers (index that moves, 1,000,000 entries: 53 / 42 us).  With the sample's boundaries: this
+#define SG_BUCKET_MAX 1024u            // largest bucket that is counted.  (Index that moves, 1,000,000 entries, lists of 10,000 and 2,000: 256 keys 49 us,
+                                       // 512 49, this 39; three lists 57, 41, 41)
 #define SG_MAP 512u                    // parts of larger buckets per CTA
 #define SG_MIN_CTAS 48u                // (a warp for every bucket of three lists)
 #define SG_WAIT_LIMIT (1u << 23)       // polls of a grid barrier (seconds)
@@ -737,7 +737,7 @@ __device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_st
 #pragma unroll
     for (uint32_t l = 0; l < 3u; ++l) {                        // buckets for more than one warp, and those that no warp of a small grid has
         const bool shared = n[l] > SG_BUCKET_WARP || l * CS_BUCKETS + tid >= G * SG_WARPS;
-        parts[l] = shared && n[l] <= SG_SAMPLED_MAX ? (n[l] + SG_PART - 1u) / SG_PART : 0u;
+        parts[l] = shared && n[l] <= SG_BUCKET_MAX ? (n[l] + SG_PART - 1u) / SG_PART : 0u;
         at[3] += parts[l];
     }
     block_scan4(at, sum);                              // (orders the words above as well)
@@ -745,8 +745,7 @@ __device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_st
     for (uint32_t l = 0; l < 3u; ++l) {
         F.off[l][tid] = at[l];
         F.cnt[l][tid] = n[l];
-        const uint32_t most = sampled ? SG_SAMPLED_MAX : max(SG_BUCKET_MAX, list[l].nb ? 12u * list[l].n_out / list[l].nb : 0u);
-        if (n[l] > min(list[l].cap, min(most, SG_SAMPLED_MAX))) atomicMin(&list[l].bad_at, at[l]);
+        if (n[l] > min(list[l].cap, SG_BUCKET_MAX)) atomicMin(&list[l].bad_at, at[l]);
         // part x of the whole grid's belongs to CTA x % G
         for (uint32_t x = at[3] + (cta + G - at[3] % G) % G; x < at[3] + parts[l]; x += G)
             if (x / G < SG_MAP) F.map[x / G] = l << 30 | tid << 16 | (x - at[3]);

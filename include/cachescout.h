@@ -59,7 +59,7 @@ typedef struct CUstream_st *cs_stream_t;   /* the same type as cudaStream_t */
 #define CS_ST_BAD_CHAIN 2u      /* an event named a chain >= n_chains */
 #define CS_ST_BAD_SLOT 4u       /* a mover list entry named a slot >= n_slots */
 #define CS_ST_BAD_SOURCE 8u     /* a BFS source >= n_agents */
-#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer is incomplete, or the select's lists are empty */
+#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer or the list is incomplete */
 #define CS_ST_LIST_CONFLICT 32u /* cs_validate_*_lists(): a slot is written twice, or written and read, by one transfer */
 #define CS_ST_BAD_SELECTION 64u /* cs_validate_selection(): a list is not the ordered k best eligible entries */
 
@@ -450,10 +450,11 @@ int cs_set_survival_sources(cs_ctx *ctx, uint32_t mode, cs_stream_t stream);
 
 /* Eq. 6 for every agent a: p_surv(a; a0, K) = Pr(a is invoked within the next K dispatches | the
  * current agent is a0), computed exactly from the matrix of Eq. 3 by pushing the unit mass at a0
- * through K steps of the chain with state a removed.  a0 = CS_AGENT_NONE uses the current agent
+ * through K steps of the chain with state a removed (or, the same number, by first visits split off the
+ * matrix's powers).  a0 = CS_AGENT_NONE uses the current agent
  * (agent of the last observed event; all zeros while there is none).  n_steps = K <= 4096.
  * psurv_out: dev [n_agents] p_surv; fsurv_out: dev [n_agents] p_surv + delta, the first factor of
- * Eq. 9 (either may be NULL).  fp64 accumulation, fp32 results.  Cost n_agents^3 * K multiply-adds. */
+ * Eq. 9 (either may be NULL).  fp64 accumulation, fp32 results.  Cost up to n_agents^3 * (K - 2) multiply-adds. */
 int cs_exact_survival(cs_ctx *ctx, uint32_t a0, uint32_t n_steps, float *psurv_out, float *fsurv_out,
                       cs_stream_t stream);
 

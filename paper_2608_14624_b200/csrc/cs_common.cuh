@@ -26,9 +26,7 @@ struct cs_nvtx_range {
 #define CS_SELECT_CLUSTER_MAX_BLOCKS (1u << 18)   // largest index of the single-launch cluster select
 
 // Index sizes and list lengths that take the one-launch select on the whole GPU (cs_select_grid.cu).
-#ifndef CS_SELECT_GRID_MIN_BLOCKS
 #define CS_SELECT_GRID_MIN_BLOCKS (1u << 17)
-#endif
 #define CS_SELECT_GRID_LONG_BLOCKS (1u << 16)      // with a list of CS_SELECT_GRID_LONG_LIST ids or more
 #define CS_SELECT_GRID_LONG_LIST 2048u
 #define CS_SELECT_GRID_MAX_BLOCKS (1u << 25)

@@ -4,46 +4,6 @@
 #pragma once
 #include "cs_select_common.cuh"
 
-// End of the half-line of last_access that an agent's blocks of the common size need for a key at or below T: victims
-// la <= cut, prefetch la >= cut.  (Entries on the line's side of it that fail after all are sorted out by the exact test.)
-template <bool PF>
-__device__ __forceinline__ uint32_t la_cut(const SelArgs &a, const Tables &T, uint32_t agent, u64 bound)
-{
-    const uint32_t Tp = (uint32_t)(bound >> 32), Ts = (uint32_t)bound;
-    const uint32_t flip = (PF && agent != T.a_star) ? 0x80000000u : 0u;
-    const float f = T.fsurv[agent], tb = (float)a.block_tokens;
-    // smallest possible primary key at an age (a copy on the other tier would make it that; the exact test tells).  The
-    // table covers every age before saturation (gtab_len = age_sat) and ends with the saturated factor.
-    auto primary = [&](uint32_t age) {
-        const uint32_t bits = __float_as_uint(__fmul_rn(__fmul_rn(f, T.gtab[age]), tb));
-        return PF ? (flip | (~bits & 0x7FFFFFFFu)) : (a.prefer_copy ? bits << 1 : bits);
-    };
-    // victims: primary falls with age: n_le = first age with primary <= Tp, n_lt = first with primary < Tp (age_sat + 1: none);
-    // prefetch: it rises: n_le = first age with primary > Tp, n_lt = first with primary >= Tp.  Both found in step, without a
-    // branch: the binary search over 2,263 ages is the longest chain between the scan's first load and its first compare.
-    uint32_t n_le = 0, n_lt = 0;
-    for (uint32_t step = CS_GTAB_MAX; step > 0; step >>= 1) {
-        const uint32_t a0 = n_le + step - 1u, a1 = n_lt + step - 1u;
-        const uint32_t p0 = primary(min(a0, a.age_sat)), p1 = primary(min(a1, a.age_sat));
-        n_le += (a0 <= a.age_sat && (PF ? p0 <= Tp : p0 > Tp)) ? step : 0u;
-        n_lt += (a1 <= a.age_sat && (PF ? p1 < Tp : p1 >= Tp)) ? step : 0u;
-    }
-    if (!PF) {
-        if (n_le > a.age_sat) return 0u;                                   // no age qualifies
-        // la <= now - n_lt for the ages below T's score; at T's score (n_le <= age < n_lt) also la <= Ts.  Age 0 stands for
-        // every last_access from now on.
-        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt : 0u));
-        const uint32_t at_score = min(n_le == 0 ? 0xFFFFFFFFu : (a.now >= n_le ? a.now - n_le : 0u), Ts);
-        return max(by_score, at_score);
-    } else {
-        if (n_le == 0) return 0xFFFFFFFFu;                                 // not even age 0
-        // la > now - n_lt for the ages above T's score; at T's score (n_lt <= age < n_le) also ~la <= Ts
-        const uint32_t by_score = n_lt > a.age_sat ? 0u : (n_lt == 0 ? 0xFFFFFFFFu : (a.now >= n_lt ? a.now - n_lt + 1u : 0u));
-        const uint32_t at_score = max(n_le > a.age_sat ? 0u : (a.now >= n_le ? a.now - n_le + 1u : 0u), ~Ts);
-        return min(by_score, at_score);
-    }
-}
-
 // ---------------------------------------------------------------------------------------------
 // Ordering the candidates.
 //

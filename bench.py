@@ -14,8 +14,9 @@ step's selection.  value = KV bytes moved across the host link per second over t
     python bench.py --config llama70b         # the 70B-shaped configuration as the timed workload
     python bench.py --impl reference          # the CPU oracle on the host cores, same metric
 
-The default run times the Llama-3-8B-shaped step (the headline line) and then, as extra keys of the same
-JSON line, the 70B-shaped step, the mover sweep, the metadata-scale calls and the large-index regime.
+The default run times the Llama-3-8B-shaped step and then the 70B-shaped step, the mover sweep, the metadata-scale
+calls and the large-index regime.  Standard output gets ONE JSON line, the headline (headline()); the whole report, of which
+the line is a part, goes to standard error as another.
 """
 from __future__ import annotations
 
@@ -1512,6 +1513,22 @@ def job_value(world: int, bytes_per_step_per_rank: int, steps: int, job_ms: floa
 
 
 # ---- main ------------------------------------------------------------------------------------------------------
+# What the headline keeps of the report: whole, or the named entries of a section.  (The report is some 17 KB long; a reader that keeps the last
+# few KB of standard output would find no line that it can parse.)
+HEADLINE = {"metric": None, "value": None, "unit": None, "n_gpus": None, "steps": None, "warmup": None, "ms_per_step": None, "higher_is_better": None,
+            "scaling": None, "vs_baseline": None, "dtype": None, "data": None, "config": None, "gpu_launches": None, "clocks": None, "e2e": None,
+            "blocks_scored_selected_per_s": None, "blocks_moved_in_timed_steps": None,
+            "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic", "ms_per_launch"),
+            "roofline_hbm": ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_kind", "ms_per_launch"),
+            "select": ("ms_three_selects", "ms_observe", "n_out_last_step", "device_status")}
+
+
+def headline(report):
+    """The JSON line of standard output: the report without its sections beside the timed step."""
+    return {key: report[key] if kept is None else {k: report[key][k] for k in kept if k in report[key]}
+            for key, kept in HEADLINE.items() if key in report}
+
+
 def main():
     args = parse_args()
     if args.impl == "reference":
@@ -1577,7 +1594,8 @@ def main():
         out["exact_survival"] = exact_survival_section(torch, cs, synth, device)
         out["hbm_regime"] = hbm_regime_section(torch, cs, synth, device, hbm_peak)
     out["cpu_baseline"] = oracle_baseline(args.config, budget_s=10.0)     # the oracle, as it stands, on this machine's host cores
-    print(json.dumps(out))
+    print(json.dumps(out), file=sys.stderr)
+    print(json.dumps(headline(out)))
     if world > 1:
         dist.destroy_process_group()
 

@@ -58,3 +58,17 @@ def test_in_flight_slowdown_factor():
     assert bench.in_flight_factor(5.0, 12.0, 16.0) == pytest.approx(2.4)
     # nothing got done while the transfer ran
     assert bench.in_flight_factor(20.0, 30.0, 10.0) == float("inf")
+
+
+def test_the_headline_fits_a_reader_that_keeps_little():
+    """The line of standard output holds what its readers need and no section beside it, whatever the report holds."""
+    import json
+    import bench
+    report = {key: 1.0 if kept is None else {k: "x" * 150 for k in (*kept, "note")} for key, kept in bench.HEADLINE.items()}
+    report.update(config={"workload": "w" * 400}, e2e={"value": 2.0, "unit": "GB/s", "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2}, mover_sweep=["m" * 9000])
+    line = json.dumps(bench.headline(report))
+    assert len(line) < 5000 and "mover_sweep" not in line and "note" not in line
+    got = json.loads(line)
+    for key in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline", "dtype", "data",
+                "config", "e2e", "clocks", "gpu_launches", "roofline"):
+        assert key in got, key

@@ -59,7 +59,7 @@ typedef struct CUstream_st *cs_stream_t;   /* the same type as cudaStream_t */
 #define CS_ST_BAD_CHAIN 2u      /* an event named a chain >= n_chains */
 #define CS_ST_BAD_SLOT 4u       /* a mover list entry named a slot >= n_slots */
 #define CS_ST_BAD_SOURCE 8u     /* a BFS source >= n_agents */
-#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer or the list is incomplete */
+#define CS_ST_TIMEOUT 16u       /* a bounded wait inside a kernel ran out; the transfer is incomplete, the select's lists are empty */
 #define CS_ST_LIST_CONFLICT 32u /* cs_validate_*_lists(): a slot is written twice, or written and read, by one transfer */
 #define CS_ST_BAD_SELECTION 64u /* cs_validate_selection(): a list is not the ordered k best eligible entries */
 
@@ -411,6 +411,13 @@ int cs_validate_exchange_lists(cs_ctx *ctx, const cs_kv_pool *gpu, const cs_kv_p
  * sets CS_ST_TIMEOUT in the status word -- the path a stalled transfer would take -- and returns.  No data
  * is in flight, so nothing is left behind; the context stays usable. */
 int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream);
+
+/* Self-test of the bounded waits of the select on the whole GPU.  From the next call on, the waits at its grid barrier
+ * `barrier` (1: after the scan; 2, 3: after the histogram and the second scan of a list without a key that holds; 4, 5:
+ * between the steps of a ranked sample) give up at once; 0 (the default): none does.  A select that gives up leaves
+ * empty lists (count 0, every id CS_ID_NONE) and CS_ST_TIMEOUT, and the calls behind it find nothing of it; calls
+ * that do not come to that barrier are as ever. */
+int cs_selftest_select_wait(cs_ctx *ctx, uint32_t barrier);
 
 /* Phase stamps of the latest calls (profiling builds only: a library compiled with -DCS_PHASE_STAMPS makes its kernels
  * store the GPU's global nanosecond timer at phase boundaries -- refresh: entry, dependency wait over, rows done, last

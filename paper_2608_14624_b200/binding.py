@@ -34,7 +34,7 @@ EXPORTS = ("cs_workspace_bytes", "cs_create", "cs_destroy", "cs_observe_invocati
            "cs_last_cuda_error", "cs_strerror", "cs_version", "cs_select_victims_static", "cs_set_mover_path", "cs_set_select_path",
            "cs_exact_survival", "cs_use_survival_table", "cs_import_state", "cs_set_select_speculation", "cs_exchange_blocks", "cs_step", "cs_set_survival_sources", "cs_select_step",
            "cs_get_counters", "cs_validate_selection", "cs_validate_move_lists", "cs_validate_exchange_lists",
-           "cs_selftest_bounded_wait", "cs_set_device_clock", "cs_set_mover_staging", "cs_exchange_blocks_staged",
+           "cs_selftest_bounded_wait", "cs_selftest_select_wait", "cs_set_device_clock", "cs_set_mover_staging", "cs_exchange_blocks_staged",
            "cs_offload_blocks_staged", "cs_prefetch_blocks_staged", "cs_set_select_bucket_regions", "cs_debug_phase_stamps")
 
 
@@ -131,6 +131,7 @@ def lib():
         L.cs_validate_exchange_lists.argtypes = [vp, C.POINTER(cs_kv_pool), C.POINTER(cs_kv_pool), vp, vp, u32, vp, vp, vp,
                                                  u32, vp, vp]
         L.cs_selftest_bounded_wait.argtypes = [vp, u32, vp]
+        L.cs_selftest_select_wait.argtypes = [vp, u32]
         L.cs_set_device_clock.argtypes = [vp, vp]
         L.cs_set_mover_staging.argtypes = [vp, vp, C.c_size_t]
         L.cs_exchange_blocks_staged.argtypes = [vp, C.POINTER(cs_kv_pool), C.POINTER(cs_kv_pool), vp, vp, u32, vp, vp, u32, vp]
@@ -303,6 +304,10 @@ def cs_validate_exchange_lists(ctx, gpu: cs_kv_pool, host: cs_kv_pool, off_gpu_s
 
 def cs_selftest_bounded_wait(ctx, max_polls: int, stream=None):
     _chk(lib().cs_selftest_bounded_wait(ctx, max_polls, _stream(stream)), "cs_selftest_bounded_wait", ctx)
+
+
+def cs_selftest_select_wait(ctx, barrier: int):
+    _chk(lib().cs_selftest_select_wait(ctx, barrier), "cs_selftest_select_wait", ctx)
 
 
 def _host_ids(a):
@@ -628,6 +633,9 @@ class CacheScout:
 
     def selftest_bounded_wait(self, max_polls: int = 1000, stream=None):
         cs_selftest_bounded_wait(self.ctx, max_polls, stream)
+
+    def selftest_select_wait(self, barrier: int):
+        cs_selftest_select_wait(self.ctx, barrier)
 
     def exact_survival(self, n_steps: int, a0: int = CS_AGENT_NONE, stream=None):
         """Eq. 6 for every agent: returns (p_surv, p_surv + delta) as device tensors."""

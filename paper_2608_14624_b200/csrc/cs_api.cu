@@ -612,6 +612,13 @@ int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream
     return cs_launch_bounded_wait_selftest(ctx, max_polls, (cudaStream_t)stream);
 }
 
+int cs_selftest_select_wait(cs_ctx *ctx, uint32_t barrier)
+{
+    if (!ctx || barrier > 5u) return CS_EINVAL;
+    ctx->grid_give_up = barrier;
+    return CS_OK;
+}
+
 int cs_launch_count(cs_ctx *ctx, uint64_t *n)
 {
     if (!ctx || !n) return CS_EINVAL;

@@ -116,12 +116,12 @@ struct cs_sel_state {
 // a launch clears the set of the next one.
 struct cs_grid_list {
     uint32_t c_scan, c_collect, eligible, pad; // candidates of the scan and of the collect pass; eligible entries that the scan saw
-    unsigned long long ahead;                  // key below which about cs_ahead(k) candidates lie, ~0: there are fewer
+    unsigned long long ahead;                  // key below which about sg_ahead(k) candidates lie, ~0: there are fewer
     uint32_t pad2[2];
 };
 struct cs_grid_state {
-    uint32_t epoch, broken, pad[30];           // the set in use; a wait has run out once: no launch counts on the words any more
-    uint32_t bar[2][8][32];                    // grid barriers, a line each
+    uint32_t epoch, failed, pad[30];           // the set in use; CTAs that have left a launch because a wait ran out, 0 between launches
+    uint32_t bar[2][8][32];                    // grid barriers, a line each: CTAs that have come, and whether a wait for the others has run out
     cs_grid_list list[2][4];
     uint32_t count[2][3][CS_BUCKETS * CS_BCOUNT_STRIDE];       // keys per bucket
     uint32_t rem_n[4];                         // by list: buckets of the next call of the kind, and where they start (from 1 on; [rem_n]: the end)
@@ -202,6 +202,7 @@ struct cs_ctx {
     int concurrent_selects;              // the per-select scratch regions are full size
     uint32_t lists_asked;                // lists that a select has been asked for, one bit each
     uint32_t grid_refused;               // 1: the driver would not launch the cooperative select; the launch chain does from then on
+    uint32_t grid_give_up;               // cs_selftest_select_wait(): the grid barrier (1 ..) at which its waits give up at once, 0: none
     cs_select_graph sel_graph[8];        // selects side by side, by the lists wanted (bit q: select q)
     // copy-engine path of the mover (cs_set_mover_staging): caller-owned device ring split into four sub-buffers
     // (two per direction, double-buffered), two streams of the context for the two DMA directions, and the events

@@ -49,6 +49,7 @@ struct GridArgs {
     uint32_t k[3], bin_lo[3], bin_shift[3];
     uint32_t *ids[3], *n_out[3];
     uint32_t want, speculate;          // lists wanted, one bit each; 0: nothing is remembered
+    uint32_t give_up;                  // the barrier (1 ..) whose waits run out at once; 0: none
 };
 
 __host__ __device__ inline size_t sg_table_bytes(uint32_t A, uint32_t gtab_len)
@@ -110,7 +111,7 @@ struct CtaShared {
     StepShared step;
     ScanOrHist u;
     ListShared list[3];
-    uint32_t part[4 * 64], elig[3], bad[3], words[4], scalar[6];
+    uint32_t part[4 * 64], elig[3], bad[3], words[4], scalar[5];
     uint32_t ok;
 };
 extern __shared__ __align__(128) unsigned char sg_smem[];
@@ -128,27 +129,61 @@ struct Sg {                            // what the passes over the index share
 };
 
 // ---- grid barrier -----------------------------------------------------------------------------------------------------------------
-// Every CTA is resident (cooperative launch).  Words are used once per launch, in two sets by turns: CTA 0 clears the other set after the
-// first barrier, when nobody can be in the launch before any more.
+// Every CTA is resident (cooperative launch).  Words are used once per launch, in two sets by turns: the last CTA clears the other set after
+// the first barrier, when nobody can be in the launch before any more.
+//
+// All CTAs pass a barrier or none does: a wait that runs out marks the word unless everybody has come, in one step with that look at it, and
+// who comes late finds the mark.
+#define SG_GIVEN_UP 0x80000000u
 __device__ __noinline__ bool grid_barrier(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t which)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         uint32_t *word = g->bar[epoch][which], v = 0, polls = 0;
+        if (ga.give_up == which + 1u) atomicOr(word, SG_GIVEN_UP);
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
-            if (v >= gridDim.x || ++polls > SG_WAIT_LIMIT) break;
+            if (v >= gridDim.x) break;                         // (everybody, or the mark)
+            if (++polls > SG_WAIT_LIMIT) atomicCAS(word, v, v | SG_GIVEN_UP);
             if (polls > 4096u) __nanosleep(256);
         }
-        SH.ok = v >= gridDim.x ? 1u : 0u;
-        if (v < gridDim.x) {
-            g->broken = 1u;
-            atomicOr(&ga.ws[0].sc->status, CS_ST_TIMEOUT);
-        }
+        SH.ok = v & SG_GIVEN_UP ? 0u : 1u;
     }
     __syncthreads();
     return SH.ok != 0u;
+}
+
+// A wait has run out, and every CTA comes here once its own work up to that barrier is done.  The last one leaves empty lists, the status that says
+// why, and nothing that a later call would trip over: no counts in the histograms, nothing remembered, the words of the barriers as they were.
+__device__ __noinline__ void give_up(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, bool first)       // first: it was the launch's first barrier
+{
+    const uint32_t tid = threadIdx.x;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) SH.ok = atomicAdd(&g->failed, 1u) == gridDim.x - 1u ? 1u : 0u;
+    __syncthreads();
+    if (!SH.ok) return;
+    __threadfence();
+    for (uint32_t l = 0; l < 3u; ++l) {
+        if (!((ga.want >> l) & 1u)) continue;
+        for (uint32_t i = tid; i < ga.k[l]; i += SG_THREADS) ga.ids[l][i] = CS_ID_NONE;
+        for (uint32_t i = tid; i < CS_HIST_BINS; i += SG_THREADS) ga.ws[l].hist[i] = 0;
+        if (tid == 0) {
+            *ga.n_out[l] = 0;
+            g->rem_n[l] = 0;
+            ga.ws[0].sc->sel_T[l] = ~0ull;
+        }
+    }
+    if (first) {                                               // (its set of words is the next launch's again)
+        for (uint32_t l = 0; l < 3u; ++l) g->count[epoch][l][tid * CS_BCOUNT_STRIDE] = 0;
+        if (tid < 8u) g->bar[epoch][tid][0] = 0;
+        if (tid < 3u) { g->list[epoch][tid].c_scan = 0; g->list[epoch][tid].c_collect = 0; g->list[epoch][tid].eligible = 0; }
+    }
+    if (tid == 0) {
+        g->failed = 0;
+        atomicOr(&ga.ws[0].sc->status, CS_ST_TIMEOUT);
+    }
 }
 
 // Loads of the tables by shared-memory address.
@@ -840,8 +875,8 @@ __device__ __noinline__ void sample_for_next(const GridArgs &ga, cs_grid_state *
 }
 
 // Lists whose buckets do not hold: a ranked sample, buckets between the samples, keys counted within them.  Two more grid barriers.  The lists
-// share the CTAs up to there: one after the other, every list would take the trips of all its steps.
-__device__ __noinline__ void order_by_sample(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t lists)
+// share the CTAs up to there: one after the other, every list would take the trips of all its steps.  false: a wait ran out.
+__device__ __noinline__ bool order_by_sample(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t lists)
 {
     StepShared &S = SH.step;
     const uint32_t tid = threadIdx.x, cta = blockIdx.x, G = gridDim.x;
@@ -863,8 +898,8 @@ __device__ __noinline__ void order_by_sample(const GridArgs &ga, cs_grid_state *
         if (pos == L.n_out - 1u) remember_bound(ga, g, L, l, list_next_bound(L, ga.k[l], ~0ull, km));
     });
     if (my_cta == 0 && tid == 0 && ga.speculate) g->rem_n[l] = N.nb;
-    if (!many) return;
-    if (!grid_barrier(ga, g, epoch, 3u)) return;
+    if (!many) return true;
+    if (!grid_barrier(ga, g, epoch, 3u)) return false;
     if ((many >> l) & 1u) {
         PlaceShared &Q = S.place;
         place_candidates(ws, make_uint4(L.c, L.n_out, L.n_elig, 0u), ga.a.max_blocks, ga.a.region_cap_max, Q.s_km, Q.s_id, Q.b_km, Q.b_id, my_cta, my_G, [] {});
@@ -880,7 +915,7 @@ __device__ __noinline__ void order_by_sample(const GridArgs &ga, cs_grid_state *
             }
         }
     }
-    if (!grid_barrier(ga, g, epoch, 4u)) return;
+    if (!grid_barrier(ga, g, epoch, 4u)) return false;
     if (tid < 3u && (many >> tid) & 1u) {
         const OrderPlan P = order_plan(SH.list[tid].c, SH.list[tid].n_out, ga.a.max_blocks, ga.a.region_cap_max);
         SH.list[tid].nb = P.nb;
@@ -906,6 +941,7 @@ __device__ __noinline__ void order_by_sample(const GridArgs &ga, cs_grid_state *
                           });
         }
     }
+    return true;
 }
 
 // ---- the kernel -------------------------------------------------------------------------------------------------------------------------------
@@ -936,9 +972,9 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     for (uint32_t l = 0; l < 3u; ++l)
         if ((ga.want >> l) & 1u) { b_km[l] = cs_ld_cg_pinned(&g->rem_km[l][tid]); b_id[l] = cs_ld_cg_pinned(&g->rem_id[l][tid]); }
     // (one thread per word: 2,368 warps asking for one sector each wait for another)
-    const uint32_t *word = tid == 32u ? &g->epoch : (tid == 33u ? &g->broken : (tid == 34u ? &ws.sc->a_star : (tid == 35u ? &ws.sc->gate : (tid == 36u ? &ws.sc->last_agent : a.now_dev))));
+    const uint32_t *word = tid == 32u ? &g->epoch : (tid == 33u ? &ws.sc->a_star : (tid == 34u ? &ws.sc->gate : (tid == 35u ? &ws.sc->last_agent : a.now_dev)));
     uint32_t scalar = a.now;
-    if (tid >= 32u && tid < (a.now_dev ? 38u : 37u)) scalar = cs_ld_cg_pinned(word);
+    if (tid >= 32u && tid < (a.now_dev ? 37u : 36u)) scalar = cs_ld_cg_pinned(word);
 #pragma unroll
     for (uint32_t h = 0; h < 2u; ++h) {                        // (at most 1,024 agents, at least 512 threads)
         const uint32_t i = tid + h * n_threads;
@@ -954,7 +990,7 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         end_km = cs_ld_cg_pinned(&g->rem_km[tid][CS_BUCKETS]);
         end_id = cs_ld_cg_pinned(&g->rem_id[tid][CS_BUCKETS]);
     }
-    if (tid >= 32u && tid < 38u) SH.scalar[tid - 32u] = scalar;
+    if (tid >= 32u && tid < 37u) SH.scalar[tid - 32u] = scalar;
 #pragma unroll
     for (uint32_t h = 0; h < 2u; ++h)
         if (tid + h * n_threads < a.A) agent[tid + h * n_threads] = t[h];
@@ -979,10 +1015,10 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     Sg s = {g, 0u, 0u, 0u, (uint32_t)__cvta_generic_to_shared(agent), (uint32_t)__cvta_generic_to_shared(gtab), a.gtab_len == a.age_sat, depth};
     walk_start(ga, s);
     __syncthreads();
-    const uint32_t epoch = SH.scalar[0] & 1u, broken = SH.scalar[1];
+    const uint32_t epoch = SH.scalar[0] & 1u;
     s.epoch = epoch;
-    s.a_star = SH.scalar[2];
-    s.now = SH.scalar[5];
+    s.a_star = SH.scalar[1];
+    s.now = SH.scalar[4];
     // Blocks age as the clock goes on, and those that leave the index are replaced by those that reach their age: what is remembered stands for
     // scores and ages, so its last_access moves on with the clock.
 #pragma unroll
@@ -996,7 +1032,7 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         if (L.moves) L.bound = moved_key(L.bound, s.now - L.then, tid == 2u);
     }
     __syncthreads();
-    const uint32_t open = ga.want & (PF && SH.scalar[3] && SH.scalar[4] < a.A ? 7u : 3u);       // (the prefetch list is empty while the gate is closed)
+    const uint32_t open = ga.want & (PF && SH.scalar[2] && SH.scalar[3] < a.A ? 7u : 3u);       // (the prefetch list is empty while the gate is closed)
     uint32_t scanned = 0;
 #pragma unroll
     for (uint32_t l = 0; l < 3u; ++l)
@@ -1009,28 +1045,15 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     if (tid < 3u && SH.bad[tid]) SH.list[tid].nb = 0;
     __syncthreads();
     bool primed = true;                                        // tiles of a walk that nobody has begun are on their way
-    bool ok = !broken;
-    if (ok && scanned) {
+    if (scanned) {
         scan_index<TIERS, PF>(ga, s, scanned, 0u);
         primed = false;
         __syncthreads();
         if (tid < 3u && SH.elig[tid]) atomicAdd(&g->list[epoch][tid].eligible, SH.elig[tid]);
     }
-    ok = ok && grid_barrier(ga, g, epoch, 0u);
-    if (!ok) {
+    if (!grid_barrier(ga, g, epoch, 0u)) {
         walk_drain();
-        // a wait has run out, in this launch or an earlier one (whose words nobody counts on any more): empty lists, and the status says why
-        if (tid == 0) {
-            g->broken = 1u;
-            atomicOr(&ws.sc->status, CS_ST_TIMEOUT);
-        }
-        __syncthreads();
-        for (uint32_t l = 0; l < 3u; ++l) {
-            if (!((ga.want >> l) & 1u)) continue;
-            for (uint32_t i = cta * n_threads + tid; i < ga.k[l]; i += G * n_threads) ga.ids[l][i] = CS_ID_NONE;
-            if (cta == 0 && tid == 0) *ga.n_out[l] = 0;
-        }
-        return;
+        return give_up(ga, g, epoch, true);
     }
     cs_release_successor();
     if (cta == G - 1u) {                                       // the other set of words is the next launch's
@@ -1059,30 +1082,20 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
                 if (v) atomicAdd(&ga.ws[l].hist[i], v);
             }
         }
-        ok = grid_barrier(ga, g, epoch, 1u);
-        if (ok) {
-            uint32_t collect = 0;
+        if (!grid_barrier(ga, g, epoch, 1u)) return give_up(ga, g, epoch, false);
+        uint32_t collect = 0;
 #pragma unroll
-            for (uint32_t l = 0; l < 3u; ++l) {
-                if (!((missed >> l) & 1u)) continue;
-                if (PF && l == 2u) list_threshold<true>(ga, l);
-                else list_threshold<false>(ga, l);
-                if (ga.k[l]) collect |= 1u << l;
-            }
-            if (collect) {
-                walk_start(ga, s);
-                scan_index<TIERS, PF>(ga, s, collect, 1u);
-            }
+        for (uint32_t l = 0; l < 3u; ++l) {
+            if (!((missed >> l) & 1u)) continue;
+            if (PF && l == 2u) list_threshold<true>(ga, l);
+            else list_threshold<false>(ga, l);
+            if (ga.k[l]) collect |= 1u << l;
         }
-        ok = ok && grid_barrier(ga, g, epoch, 2u);
-        if (!ok) {
-            if (tid == 0) {
-                g->broken = 1u;
-                atomicOr(&ws.sc->status, CS_ST_TIMEOUT);
-            }
-            __syncthreads();
-            return;
+        if (collect) {
+            walk_start(ga, s);
+            scan_index<TIERS, PF>(ga, s, collect, 1u);
         }
+        if (!grid_barrier(ga, g, epoch, 2u)) return give_up(ga, g, epoch, false);
         if (cta == 0)                                          // ready for the next call
             for (uint32_t l = 0; l < 3u; ++l)
                 if ((missed >> l) & 1u)
@@ -1107,7 +1120,7 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
             if (bound || L.refresh) sample_for_next(ga, g, l, L.refresh != 0u, bound);
         }
     }
-    if (rest) order_by_sample(ga, g, epoch, rest);
+    if (rest && !order_by_sample(ga, g, epoch, rest)) give_up(ga, g, epoch, false);
 }
 
 // ---- host -----------------------------------------------------------------------------------------------------------------------------------
@@ -1167,6 +1180,7 @@ int cs_launch_select_grid(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
         ga.want |= 1u << l;
     }
     ga.speculate = ctx->no_speculation ? 0u : 1u;
+    ga.give_up = ctx->grid_give_up;
     const bool pf = (ga.want & 4u) != 0;
     const uint32_t G = std::min<uint32_t>(most, std::max<uint32_t>(SG_MIN_CTAS, idx->n_blocks / 512u));
     cudaLaunchConfig_t cfg = {};

@@ -55,6 +55,51 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable():
         c.selftest_bounded_wait(0)
 
 
+@pytest.mark.parametrize("barrier", [1, 2, 3, 4, 5])
+def test_a_select_that_gives_up_leaves_empty_lists_and_nothing_behind(barrier):
+    """The waits at one of the five grid barriers of the whole-GPU select run out, called and replayed from a graph: empty lists, also where
+    buffers held something else, and the status.  The calls behind it, on the same route and on the launch chain, whose histograms it shares,
+    give what a context gives that has never seen a wait run out."""
+    cfg, n, k, kp = synth.CONFIGS["meta1m"], 150_001, 2500, 2100
+    c, _, _ = warm(cfg, 800, n, r_min=0.02)
+    ref, _, _ = warm(cfg, 800, n, r_min=0.02)
+    ref.set_select_path(cs.CS_SELECT_MULTI)
+    d = cs.DeviceIndex.from_host(synth.make_block_index(cfg, n=n, tier="random"), DEV)
+    lists = lambda: [torch.full((m,), 7, dtype=torch.int32, device=DEV) for m in (k, 4, k, 4, kp, 4)]
+    want = lists()
+    ref.select_step(d, 100_000, k, kp, *want)
+    for _ in range(2):                                          # (the second call takes the whole GPU)
+        b = lists()
+        c.select_step(d, 100_000, k, kp, *b)
+        assert all(torch.equal(x, y) for x, y in zip(b, want))
+    c.set_select_speculation(False)                             # every list goes by all five barriers
+    c.selftest_select_wait(barrier)
+    b, side = lists(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        c.select_step(d, 100_000, k, kp, *b)
+    for call in (lambda: c.select_step(d, 100_000, k, kp, *b), g.replay, g.replay):
+        for x in b:
+            x.fill_(7)
+        call()
+        torch.cuda.synchronize()
+        for ids, cnt in zip(b[0::2], b[1::2]):
+            assert bool((ids == -1).all()) and int(cnt[0]) == 0
+    c.selftest_select_wait(0)
+    for path, speculate in ((cs.CS_SELECT_AUTO, False), (cs.CS_SELECT_MULTI, False), (cs.CS_SELECT_AUTO, True), (cs.CS_SELECT_AUTO, True),
+                            (cs.CS_SELECT_MULTI, True)):
+        c.set_select_path(path)
+        c.set_select_speculation(speculate)
+        b = lists()
+        c.select_step(d, 100_000, k, kp, *b)
+        assert all(torch.equal(x, y) for x, y in zip(b, want)), (path, speculate)
+    assert c.get_status() == cs.CS_ST_TIMEOUT
+    assert c.get_status() == 0 and ref.get_status() == 0
+    with pytest.raises(cs.CacheScoutError):
+        c.selftest_select_wait(6)
+
+
 @pytest.mark.parametrize("path", [cs.CS_SELECT_CLUSTER, cs.CS_SELECT_MULTI])
 def test_selection_checker_accepts_the_oracle_list_and_catches_every_kind_of_damage(path):
     cfg = synth.CONFIGS["llama8b"]

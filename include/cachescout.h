@@ -416,7 +416,8 @@ int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream
  * `barrier` (1: after the scan; 2, 3: after the histogram and the second scan of a list without a key that holds; 4, 5:
  * between the steps of a ranked sample) give up at once; 0 (the default): none does.  A select that gives up leaves
  * empty lists (count 0, every id CS_ID_NONE) and CS_ST_TIMEOUT, and the calls behind it find nothing of it; calls
- * that do not come to that barrier are as ever. */
+ * that do not come to that barrier are as ever.  6: two CTAs in three start only when the others have taken over their
+ * work, as they do for CTAs that other kernels keep off the GPU; the lists are the same. */
 int cs_selftest_select_wait(cs_ctx *ctx, uint32_t barrier);
 
 /* Phase stamps of the latest calls (profiling builds only: a library compiled with -DCS_PHASE_STAMPS makes its kernels

@@ -614,7 +614,7 @@ int cs_selftest_bounded_wait(cs_ctx *ctx, uint32_t max_polls, cs_stream_t stream
 
 int cs_selftest_select_wait(cs_ctx *ctx, uint32_t barrier)
 {
-    if (!ctx || barrier > 5u) return CS_EINVAL;
+    if (!ctx || barrier > 6u) return CS_EINVAL;
     ctx->grid_give_up = barrier;
     return CS_OK;
 }

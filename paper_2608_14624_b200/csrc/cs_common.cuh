@@ -114,14 +114,17 @@ struct cs_sel_state {
 
 // State of the one-launch select of large indexes (cs_select_grid.cu), one per context.  What a launch counts in lies twice, used by turns:
 // a launch clears the set of the next one.
+#define CS_GRID_MAX_CTAS 160u
 struct cs_grid_list {
     uint32_t c_scan, c_collect, eligible, pad; // candidates of the scan and of the collect pass; eligible entries that the scan saw
     unsigned long long ahead;                  // key below which about sg_ahead(k) candidates lie, ~0: there are fewer
     uint32_t pad2[2];
 };
 struct cs_grid_state {
-    uint32_t epoch, failed, pad[30];           // the set in use; CTAs that have left a launch because a wait ran out, 0 between launches
-    uint32_t bar[2][8][32];                    // grid barriers, a line each: CTAs that have come, and whether a wait for the others has run out
+    uint32_t failed, pad[31];                  // shares of a launch whose CTAs have left it because a wait ran out, 0 between launches
+    unsigned long long taken[CS_GRID_MAX_CTAS];        // by share: starts of its CTA (the launch's number, its parity the set in use), and, in the upper
+                                               // half, the complement of the last launch in which another CTA took the share over
+    uint32_t bar[2][8][32];                    // grid barriers, a line each: shares that are done, and whether a wait for the others has run out
     cs_grid_list list[2][4];
     uint32_t count[2][3][CS_BUCKETS * CS_BCOUNT_STRIDE];       // keys per bucket
     uint32_t rem_n[4];                         // by list: buckets of the next call of the kind, and where they start (from 1 on; [rem_n]: the end)
@@ -201,8 +204,8 @@ struct cs_ctx {
     cudaEvent_t ev_sel_fork, ev_sel_join[2];
     int concurrent_selects;              // the per-select scratch regions are full size
     uint32_t lists_asked;                // lists that a select has been asked for, one bit each
-    uint32_t grid_refused;               // 1: the driver would not launch the cooperative select; the launch chain does from then on
-    uint32_t grid_give_up;               // cs_selftest_select_wait(): the grid barrier (1 ..) at which its waits give up at once, 0: none
+    uint32_t grid_refused;               // 1: the driver would not launch the whole-GPU select; the launch chain does from then on
+    uint32_t grid_give_up;               // cs_selftest_select_wait(): the grid barrier (1 ..) at which its waits give up at once, 6: late CTAs, 0: neither
     cs_select_graph sel_graph[8];        // selects side by side, by the lists wanted (bit q: select q)
     // copy-engine path of the mover (cs_set_mover_staging): caller-owned device ring split into four sub-buffers
     // (two per direction, double-buffered), two streams of the context for the two DMA directions, and the events

@@ -1,4 +1,4 @@
-// Selects over a large index in ONE launch on the whole GPU: a cooperative kernel, one CTA per SM, that reads the index once for up to
+// Selects over a large index in ONE launch on the whole GPU: a kernel of one CTA per SM that reads the index once for up to
 // three lists (GPU-tier victims, host-tier victims, prefetch candidates), with grid barriers in place of kernel boundaries.  Same key,
 // same eligibility rules, same exact ordered output as the launch chain of cs_select.cu, whose six launches per list it replaces.
 //
@@ -36,8 +36,8 @@
 #define SG_BUCKET_MAX 1024u            // largest bucket that is counted.  (Index that moves, 1,000,000 entries, lists of 10,000 and 2,000: 256 keys 49 us,
                                        // 512 49, this 39; three lists 57, 41, 41)
 #define SG_MAP 512u                    // parts of larger buckets per CTA
-#define SG_MIN_CTAS 48u                // (a warp for every bucket of three lists)
 #define SG_WAIT_LIMIT (1u << 23)       // polls of a grid barrier (seconds)
+#define SG_PATIENCE 64u                // polls (about 50 us) between two looks for shares that nobody has begun
 static_assert(SG_THREADS == CS_BUCKETS, "one bucket per thread");
 
 // Candidates that a call should find (as cs_ahead(); a few thousand more cost less here than the shortest list's key that no longer holds).
@@ -49,7 +49,7 @@ struct GridArgs {
     uint32_t k[3], bin_lo[3], bin_shift[3];
     uint32_t *ids[3], *n_out[3];
     uint32_t want, speculate;          // lists wanted, one bit each; 0: nothing is remembered
-    uint32_t give_up;                  // the barrier (1 ..) whose waits run out at once; 0: none
+    uint32_t give_up;                  // the barrier (1 ..) whose waits run out at once; SG_LATE: CTAs that start late; 0: neither
 };
 
 __host__ __device__ inline size_t sg_table_bytes(uint32_t A, uint32_t gtab_len)
@@ -112,7 +112,9 @@ struct CtaShared {
     ScanOrHist u;
     ListShared list[3];
     uint32_t part[4 * 64], elig[3], bad[3], words[4], scalar[5];
-    uint32_t ok;
+    uint32_t ok, lost;                 // a barrier's outcome; 1: this CTA's share is another's
+    uint32_t n_own, pad;               // shares of this CTA: its own and those it has taken over
+    uint16_t own[CS_GRID_MAX_CTAS];
 };
 extern __shared__ __align__(128) unsigned char sg_smem[];
 #define SH (*(CtaShared *)sg_smem)
@@ -123,45 +125,81 @@ static size_t sg_smem_bytes(uint32_t A, uint32_t gtab_len) { return sizeof(CtaSh
 struct Sg {                            // what the passes over the index share
     cs_grid_state *g;
     uint32_t now, a_star, epoch;
+    uint32_t share;                    // whose part of the index
     uint32_t agent, gtab;              // shared-memory addresses of the tables
     bool whole_table;                  // the recency table covers every age before saturation; its last entry is the saturated factor
     bool depth;                        // the walks bring the depths
 };
 
 // ---- grid barrier -----------------------------------------------------------------------------------------------------------------
-// Every CTA is resident (cooperative launch).  Words are used once per launch, in two sets by turns: the last CTA clears the other set after
-// the first barrier, when nobody can be in the launch before any more.
+// The work is cut into gridDim.x shares, share x meant for CTA x.  A barrier counts shares, not CTAs: nobody waits for a CTA that has not
+// started.  A CTA that has waited long at the first barrier takes over shares that nobody has begun, with all that belongs to them until
+// the end of the launch; a CTA that finds its share taken leaves.  So a launch goes on with whatever SMs it gets -- other kernels may hold some
+// for as long as they like -- and from the first barrier on every share is at a running CTA.  (Selects of 1,000,000 entries beside back-to-back
+// compactions: 106 to 118 us each where every CTA had to find a place, 40 so.)
 //
-// All CTAs pass a barrier or none does: a wait that runs out marks the word unless everybody has come, in one step with that look at it, and
-// who comes late finds the mark.
+// A share's CTA adds one to its word when it starts, once in every launch, and so learns the launch's number, and whether the share is still its own;
+// who takes a share over swaps that word for one that carries the launch's mark.
+//
+// All CTAs pass a barrier or none does: a wait that runs out marks the word unless everything is done, in one step with that look at it, and
+// who comes late finds the mark.  The words are used once per launch, in two sets by turns: the CTA with share 0 clears the other set after the first
+// barrier, when the launch before is over and nobody can be in the next one.
 #define SG_GIVEN_UP 0x80000000u
-__device__ __noinline__ bool grid_barrier(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t which)
+enum : uint32_t { SG_FAILED = 0xFFFFFFFEu, SG_PASSED = 0xFFFFFFFFu };
+__device__ __forceinline__ bool share_is_free(u64 taken, uint32_t number) { return (uint32_t)taken == number && (uint32_t)(taken >> 32) != ~number; }
+// done: shares to be counted; take_over: shares may still be without a CTA.  Returns SG_PASSED, SG_FAILED or a share that is this CTA's now.
+__device__ __noinline__ uint32_t grid_barrier(const GridArgs &ga, cs_grid_state *g, uint32_t number, uint32_t which, uint32_t done, bool take_over)
 {
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t *word = g->bar[epoch][which], v = 0, polls = 0;
-        if (ga.give_up == which + 1u) atomicOr(word, SG_GIVEN_UP);
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(word) : "memory");
+    if (threadIdx.x < 32u) {
+        const uint32_t lane = threadIdx.x, G = gridDim.x;
+        uint32_t *word = g->bar[number & 1u][which], v = 0, polls = 0, share = SG_PASSED;
+        if (lane == 0) {
+            if (ga.give_up == which + 1u) atomicOr(word, SG_GIVEN_UP);
+            asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(word), "r"(done) : "memory");
+        }
         for (;;) {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
-            if (v >= gridDim.x) break;                         // (everybody, or the mark)
-            if (++polls > SG_WAIT_LIMIT) atomicCAS(word, v, v | SG_GIVEN_UP);
+            if (lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+            v = __shfl_sync(0xFFFFFFFFu, v, 0);
+            if (v >= G) break;                                 // (everything, or the mark)
+            if (++polls % SG_PATIENCE == 0u && take_over) {
+                for (uint32_t x0 = 0; x0 < G && share == SG_PASSED; x0 += 32u) {
+                    const uint32_t x = x0 + lane;
+                    const u64 taken = x < G ? __ldcg(g->taken + x) : ~0ull;
+                    const uint32_t free = __ballot_sync(0xFFFFFFFFu, x < G && share_is_free(taken, number));
+                    if (!free) continue;
+                    const uint32_t one = __ffs(free) - 1u;
+                    uint32_t mine = 0;
+                    if (lane == one) mine = atomicCAS(g->taken + x, taken, (u64)~number << 32 | number) == taken ? 1u : 0u;
+                    if (__shfl_sync(0xFFFFFFFFu, mine, one)) share = x0 + one;
+                }
+                if (share != SG_PASSED) break;
+            }
+            if (lane == 0 && polls > SG_WAIT_LIMIT) atomicCAS(word, v, v | SG_GIVEN_UP);
             if (polls > 4096u) __nanosleep(256);
         }
-        SH.ok = v & SG_GIVEN_UP ? 0u : 1u;
+        if (lane == 0) {
+            SH.ok = share != SG_PASSED ? share : (v & SG_GIVEN_UP ? SG_FAILED : SG_PASSED);
+            if (share != SG_PASSED) SH.own[SH.n_own++] = (uint16_t)share;
+        }
     }
     __syncthreads();
-    return SH.ok != 0u;
+    return SH.ok;
+}
+// A barrier behind the first one.
+__device__ __forceinline__ bool all_here(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t which)
+{
+    return grid_barrier(ga, g, epoch, which, SH.n_own, false) == SG_PASSED;
 }
 
-// A wait has run out, and every CTA comes here once its own work up to that barrier is done.  The last one leaves empty lists, the status that says
-// why, and nothing that a later call would trip over: no counts in the histograms, nothing remembered, the words of the barriers as they were.
-__device__ __noinline__ void give_up(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, bool first)       // first: it was the launch's first barrier
+// A wait has run out, and every CTA with a share comes here once its own work up to that barrier is done.  The last one leaves empty lists, the status
+// that says why, and nothing that a later call would trip over: no counts in the histograms, nothing remembered.
+__device__ __noinline__ void give_up(const GridArgs &ga, cs_grid_state *g)
 {
     const uint32_t tid = threadIdx.x;
     __threadfence();
     __syncthreads();
-    if (tid == 0) SH.ok = atomicAdd(&g->failed, 1u) == gridDim.x - 1u ? 1u : 0u;
+    if (tid == 0) SH.ok = atomicAdd(&g->failed, SH.n_own) + SH.n_own == gridDim.x ? 1u : 0u;
     __syncthreads();
     if (!SH.ok) return;
     __threadfence();
@@ -175,15 +213,30 @@ __device__ __noinline__ void give_up(const GridArgs &ga, cs_grid_state *g, uint3
             ga.ws[0].sc->sel_T[l] = ~0ull;
         }
     }
-    if (first) {                                               // (its set of words is the next launch's again)
-        for (uint32_t l = 0; l < 3u; ++l) g->count[epoch][l][tid * CS_BCOUNT_STRIDE] = 0;
-        if (tid < 8u) g->bar[epoch][tid][0] = 0;
-        if (tid < 3u) { g->list[epoch][tid].c_scan = 0; g->list[epoch][tid].c_collect = 0; g->list[epoch][tid].eligible = 0; }
-    }
     if (tid == 0) {
         g->failed = 0;
         atomicOr(&ga.ws[0].sc->status, CS_ST_TIMEOUT);
     }
+}
+
+// cs_selftest_select_wait(): a CTA that starts late, once its share is another's (or some tenths of a second have gone by).
+#define SG_LATE 6u
+__device__ __noinline__ void late_start(cs_grid_state *g)
+{
+    if (threadIdx.x == 0) {
+        const uint32_t number = (uint32_t)__ldcg(g->taken + blockIdx.x);
+        for (uint32_t polls = 0; polls < 200000u && share_is_free(__ldcg(g->taken + blockIdx.x), number); ++polls) __nanosleep(256);
+    }
+    __syncthreads();
+}
+
+// The other set of words is the next launch's.
+__device__ __noinline__ void prepare_next_launch(cs_grid_state *g, uint32_t epoch)
+{
+    const uint32_t tid = threadIdx.x, other = epoch ^ 1u;
+    for (uint32_t l = 0; l < 3u; ++l) g->count[other][l][tid * CS_BCOUNT_STRIDE] = 0;
+    if (tid < 8u) g->bar[other][tid][0] = 0;
+    if (tid < 3u) { g->list[other][tid].c_scan = 0; g->list[other][tid].c_collect = 0; g->list[other][tid].eligible = 0; }
 }
 
 // Loads of the tables by shared-memory address.
@@ -230,7 +283,7 @@ __device__ __forceinline__ void quad_ask(const GridArgs &ga, const Sg &s, uint32
 // The first steps of a walk.  (Every thread copies for itself only: no barrier, no wait for anybody else.)
 __device__ __forceinline__ void walk_start(const GridArgs &ga, const Sg &s)
 {
-    const uint32_t q = blockIdx.x * SG_THREADS + threadIdx.x;
+    const uint32_t q = s.share * SG_THREADS + threadIdx.x;
 #pragma unroll
     for (uint32_t i = 0; i < SG_STAGES; ++i) quad_ask(ga, s, q + i * gridDim.x * SG_THREADS, i);
 }
@@ -242,8 +295,8 @@ template <class F>
 __device__ __forceinline__ void walk(const GridArgs &ga, const Sg &s, F f)
 {
     const uint32_t tid = threadIdx.x, n_quads = ga.a.n / 4u, stride = gridDim.x * SG_THREADS, no_sizes = 0x01010101u * ga.a.block_tokens;
-    uint32_t q = blockIdx.x * SG_THREADS + tid, stage = 0;
-    bool tail = (ga.a.n & 3u) != 0u && blockIdx.x == gridDim.x - 1u && tid >= SG_THREADS - 32u;
+    uint32_t q = s.share * SG_THREADS + tid, stage = 0;
+    bool tail = (ga.a.n & 3u) != 0u && s.share == gridDim.x - 1u && tid >= SG_THREADS - 32u;
     for (;;) {
         const bool step = (q & ~31u) < n_quads;                // (whole warps)
         Quad4 Q;
@@ -683,7 +736,7 @@ __device__ __forceinline__ void block_scan4(uint32_t (&v)[4], uint32_t (&total)[
 }
 
 // The keys [8 sub, 8 sub + 8) of a bucket of m keys, ranked within it by the calling warp, four lanes to a key.  The bucket comes through
-// shared memory, 256 keys at a time: one trip, where eight keys per lane and round took one per round.
+// shared memory, SG_KEYS at a time: one trip, where eight keys per lane and round took one per round.
 #define SG_PART 8u
 __device__ __noinline__ void rank_in_bucket(const GridArgs &ga, cs_grid_state *g, uint32_t l, uint32_t b, uint32_t sub, uint32_t m, uint32_t off,
                                             bool sampled)
@@ -726,13 +779,14 @@ __device__ __noinline__ void rank_in_bucket(const GridArgs &ga, cs_grid_state *g
     __syncwarp();
 }
 
-// The lists whose candidates lie in buckets -- by the scan, or (sampled) by the sample's boundaries -- put in order; returns those it could.
-__device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t lists, bool sampled)
+// The lists whose candidates lie in buckets -- by the scan, or (sampled) by the sample's boundaries -- put in order, as far as share `cta` goes;
+// returns those whose buckets can be, the same ones for every share.
+__device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t cta, uint32_t lists, bool sampled)
 {
     ListShared *const list = SH.list;
     FinishShared &F = SH.step.finish;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = blockIdx.x, G = gridDim.x;
-    // ---- one trip: the counts, and the keys of the bucket that is this warp's (bucket x belongs to CTA x % G) ---------------------------------
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x;
+    // ---- one trip: the counts, and the keys of the bucket that is this warp's (bucket x belongs to share x % G) -------------------------------
     const uint32_t my_x = cta + G * warp, my_l = my_x / CS_BUCKETS, my_b = my_x % CS_BUCKETS;
     const bool my_any = my_l < 3u && (lists >> my_l) & 1u && my_b < list[my_l < 3u ? my_l : 0u].nb;
     uint32_t n[3], c_scan = 0, eligible = 0, id[3] = {};
@@ -781,7 +835,7 @@ __device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_st
         F.off[l][tid] = at[l];
         F.cnt[l][tid] = n[l];
         if (n[l] > min(list[l].cap, SG_BUCKET_MAX)) atomicMin(&list[l].bad_at, at[l]);
-        // part x of the whole grid's belongs to CTA x % G
+        // part x of the whole grid's belongs to share x % G
         for (uint32_t x = at[3] + (cta + G - at[3] % G) % G; x < at[3] + parts[l]; x += G)
             if (x / G < SG_MAP) F.map[x / G] = l << 30 | tid << 16 | (x - at[3]);
         at[3] += parts[l];
@@ -846,7 +900,7 @@ __device__ __noinline__ uint32_t order_by_buckets(const GridArgs &ga, cs_grid_st
 
 // A sample of a list's candidates, ranked by all CTAs, for the next call: where its buckets begin (boundaries; too few keys were ranked), and a
 // lower key (bound; too many candidates lay below this one).
-__device__ __noinline__ void sample_for_next(const GridArgs &ga, cs_grid_state *g, uint32_t l, bool boundaries, bool bound)
+__device__ __noinline__ void sample_for_next(const GridArgs &ga, cs_grid_state *g, uint32_t share, uint32_t l, bool boundaries, bool bound)
 {
     const ListShared &L = SH.list[l];
     SampleShared &M = SH.step.sample;
@@ -859,7 +913,7 @@ __device__ __noinline__ void sample_for_next(const GridArgs &ga, cs_grid_state *
     }
     __syncthreads();
     const uint32_t want = (uint32_t)((u64)sg_ahead(ga.k[l]) * S / L.c);
-    for (uint32_t i = blockIdx.x * SG_WARPS + warp; i < S; i += gridDim.x * SG_WARPS) {
+    for (uint32_t i = share * SG_WARPS + warp; i < S; i += gridDim.x * SG_WARPS) {
         uint32_t r = 0;
 #pragma unroll 8
         for (uint32_t q = lane; q < CS_SAMPLE; q += 32u) count_less(r, M.km[q], M.id[q], M.km[i], M.id[i]);
@@ -871,38 +925,46 @@ __device__ __noinline__ void sample_for_next(const GridArgs &ga, cs_grid_state *
         for (uint32_t j = lo + lane; j < L.next_nb && (u64)j * L.step * S / L.c == r; j += 32u) { g->rem_km[l][j] = M.km[i]; g->rem_id[l][j] = M.id[i]; }
         if (lane == 0 && L.end < L.c && (uint32_t)((u64)L.end * S / L.c) == r) { g->rem_km[l][L.next_nb] = M.km[i]; g->rem_id[l][L.next_nb] = M.id[i]; }
     }
-    if (boundaries && blockIdx.x == 0 && tid == 0 && L.end == L.c) { g->rem_km[l][L.next_nb] = ~0ull; g->rem_id[l][L.next_nb] = 0xFFFFFFFFu; }
+    if (boundaries && share == 0 && tid == 0 && L.end == L.c) { g->rem_km[l][L.next_nb] = ~0ull; g->rem_id[l][L.next_nb] = 0xFFFFFFFFu; }
 }
 
 // Lists whose buckets do not hold: a ranked sample, buckets between the samples, keys counted within them.  Two more grid barriers.  The lists
 // share the CTAs up to there: one after the other, every list would take the trips of all its steps.  false: a wait ran out.
-__device__ __noinline__ bool order_by_sample(const GridArgs &ga, cs_grid_state *g, uint32_t epoch, uint32_t lists)
+__device__ __noinline__ bool order_by_sample(const GridArgs &ga, cs_grid_state *g, uint32_t number, uint32_t lists)
 {
     StepShared &S = SH.step;
-    const uint32_t tid = threadIdx.x, cta = blockIdx.x, G = gridDim.x;
-    const uint32_t n_lists = __popc(lists), turn = cta % n_lists, l = __fns(lists, 0u, turn + 1u);      // this CTA's list
-    const uint32_t my_cta = cta / n_lists, my_G = (G - turn + n_lists - 1u) / n_lists;
+    const uint32_t tid = threadIdx.x, G = gridDim.x, n_lists = __popc(lists), epoch = number & 1u;
     uint32_t many = 0;
     for (uint32_t x = 0; x < 3u; ++x)
         if ((lists >> x) & 1u && SH.list[x].c > FEW_MAX) many |= 1u << x;
-    const ListShared &L = SH.list[l];
-    const cs_workspace &ws = ga.ws[l];
-    const NextBuckets N = next_buckets(L.n_out, L.c);
-    if (my_cta == 0) CS_BCOUNT(ws, tid) = 0;
-    __syncthreads();
-    rank_sample(ws, L.c, L.n_out, sg_ahead(ga.k[l]), &g->list[epoch][l].ahead, S.sample.km, S.sample.id, my_cta, my_G, ga.ids[l], [&](uint32_t pos, u64 km, uint32_t id) {
-        if (!ga.speculate) return;
-        if (pos && pos < N.end && pos % N.step == 0u) { g->rem_km[l][pos / N.step] = km; g->rem_id[l][pos / N.step] = id; }
-        if (pos == N.end) { g->rem_km[l][N.nb] = km; g->rem_id[l][N.nb] = id; }
-        if (pos == L.c - 1u && N.end == L.c) { g->rem_km[l][N.nb] = ~0ull; g->rem_id[l][N.nb] = 0xFFFFFFFFu; }
-        if (pos == L.n_out - 1u) remember_bound(ga, g, L, l, list_next_bound(L, ga.k[l], ~0ull, km));
-    });
-    if (my_cta == 0 && tid == 0 && ga.speculate) g->rem_n[l] = N.nb;
+    for (uint32_t o = 0; o < SH.n_own; ++o) {
+        const uint32_t share = SH.own[o], turn = share % n_lists, l = __fns(lists, 0u, turn + 1u);      // the share's list
+        const uint32_t my_cta = share / n_lists, my_G = (G - turn + n_lists - 1u) / n_lists;
+        const ListShared &L = SH.list[l];
+        const cs_workspace &ws = ga.ws[l];
+        const NextBuckets N = next_buckets(L.n_out, L.c);
+        if (my_cta == 0) CS_BCOUNT(ws, tid) = 0;
+        __syncthreads();
+        rank_sample(ws, L.c, L.n_out, sg_ahead(ga.k[l]), &g->list[epoch][l].ahead, S.sample.km, S.sample.id, my_cta, my_G, ga.ids[l], [&](uint32_t pos, u64 km, uint32_t id) {
+            if (!ga.speculate) return;
+            if (pos && pos < N.end && pos % N.step == 0u) { g->rem_km[l][pos / N.step] = km; g->rem_id[l][pos / N.step] = id; }
+            if (pos == N.end) { g->rem_km[l][N.nb] = km; g->rem_id[l][N.nb] = id; }
+            if (pos == L.c - 1u && N.end == L.c) { g->rem_km[l][N.nb] = ~0ull; g->rem_id[l][N.nb] = 0xFFFFFFFFu; }
+            if (pos == L.n_out - 1u) remember_bound(ga, g, L, l, list_next_bound(L, ga.k[l], ~0ull, km));
+        });
+        if (my_cta == 0 && tid == 0 && ga.speculate) g->rem_n[l] = N.nb;
+    }
     if (!many) return true;
-    if (!grid_barrier(ga, g, epoch, 3u)) return false;
-    if ((many >> l) & 1u) {
+    if (!all_here(ga, g, number, 3u)) return false;
+    for (uint32_t o = 0; o < SH.n_own; ++o) {
+        const uint32_t share = SH.own[o], turn = share % n_lists, l = __fns(lists, 0u, turn + 1u);
+        const uint32_t my_cta = share / n_lists, my_G = (G - turn + n_lists - 1u) / n_lists;
+        if (!((many >> l) & 1u)) continue;
+        const ListShared &L = SH.list[l];
+        const NextBuckets N = next_buckets(L.n_out, L.c);
         PlaceShared &Q = S.place;
-        place_candidates(ws, make_uint4(L.c, L.n_out, L.n_elig, 0u), ga.a.max_blocks, ga.a.region_cap_max, Q.s_km, Q.s_id, Q.b_km, Q.b_id, my_cta, my_G, [] {});
+        if (o) __syncthreads();
+        place_candidates(ga.ws[l], make_uint4(L.c, L.n_out, L.n_elig, 0u), ga.a.max_blocks, ga.a.region_cap_max, Q.s_km, Q.s_id, Q.b_km, Q.b_id, my_cta, my_G, [] {});
         if (my_cta == my_G - 1u && ga.speculate) {
             // the next call's boundaries out of the sample
             for (uint32_t j = tid + 1u; j <= N.nb; j += SG_THREADS) {
@@ -915,14 +977,17 @@ __device__ __noinline__ bool order_by_sample(const GridArgs &ga, cs_grid_state *
             }
         }
     }
-    if (!grid_barrier(ga, g, epoch, 4u)) return false;
+    if (!all_here(ga, g, number, 4u)) return false;
     if (tid < 3u && (many >> tid) & 1u) {
         const OrderPlan P = order_plan(SH.list[tid].c, SH.list[tid].n_out, ga.a.max_blocks, ga.a.region_cap_max);
         SH.list[tid].nb = P.nb;
         SH.list[tid].cap = P.cap;
     }
-    __syncthreads();
-    const uint32_t left = many & ~order_by_buckets(ga, g, epoch, many, true);
+    uint32_t left = 0;
+    for (uint32_t o = 0; o < SH.n_own; ++o) {
+        __syncthreads();
+        left = many & ~order_by_buckets(ga, g, epoch, SH.own[o], many, true);
+    }
     // ---- buckets that outgrew their regions, or have too many keys for a warp: every bucket by a CTA
     for (uint32_t x = 0; x < 3u; ++x) {
         if (!((left >> x) & 1u)) continue;
@@ -931,16 +996,62 @@ __device__ __noinline__ bool order_by_sample(const GridArgs &ga, cs_grid_state *
         const OrderPlan P = order_plan(X.c, X.n_out, ga.a.max_blocks, ga.a.region_cap_max);
         const uint32_t n_t = cs_ld_cg_pinned(&CS_BCOUNT(w, tid));
         const u64 ahead = cs_ld_cg_pinned(&g->list[epoch][x].ahead);
-        for (uint32_t b = cta; b < P.nb; b += G) {
-            __syncthreads();
-            if (tid < 3u) SH.words[tid] = 0;
-            __syncthreads();
-            finish_bucket(w, X.c, X.n_out, P, b, n_t, cs_ld_cg_pinned(&CS_BCOUNT(w, b)), x, S.sample.km, S.sample.id, SH.words, SH.words + 1, SH.words + 2, ga.ids[x],
-                          [&](uint32_t pos, u64 km, uint32_t) {
-                              if (ga.speculate && pos == X.n_out - 1u) remember_bound(ga, g, X, x, list_next_bound(X, ga.k[x], ahead, km));
-                          });
+        for (uint32_t o = 0; o < SH.n_own; ++o)
+            for (uint32_t b = SH.own[o]; b < P.nb; b += G) {
+                __syncthreads();
+                if (tid < 3u) SH.words[tid] = 0;
+                __syncthreads();
+                finish_bucket(w, X.c, X.n_out, P, b, n_t, cs_ld_cg_pinned(&CS_BCOUNT(w, b)), x, S.sample.km, S.sample.id, SH.words, SH.words + 1, SH.words + 2, ga.ids[x],
+                              [&](uint32_t pos, u64 km, uint32_t) {
+                                  if (ga.speculate && pos == X.n_out - 1u) remember_bound(ga, g, X, x, list_next_bound(X, ga.k[x], ahead, km));
+                              });
+            }
+    }
+    return true;
+}
+
+// Lists without the candidates they need: a histogram of the full keys, a threshold, another look at the index.  primed: the first tiles of the CTA's own
+// share are on their way.  false: a wait ran out.
+template <int TIERS, bool PF>
+__device__ __noinline__ bool collect_missed(const GridArgs &ga, Sg s, uint32_t number, uint32_t missed, bool primed, bool first)
+{
+    ScanOrHist *const u = &SH.u;
+    const uint32_t tid = threadIdx.x;
+    __syncthreads();                                           // (the tiles' place is the copies' again)
+    for (uint32_t i = tid; i < 3u * CS_HIST_BINS; i += SG_THREADS) u->hist[0][i] = 0;
+    __syncthreads();
+    for (uint32_t o = 0; o < SH.n_own; ++o) {
+        s.share = SH.own[o];                                   // (its own is the first)
+        if (o || !primed) walk_start(ga, s);
+        count_index<TIERS, PF>(ga, s, missed);
+    }
+    __syncthreads();
+    for (uint32_t l = 0; l < 3u; ++l) {
+        if (!((missed >> l) & 1u)) continue;
+        for (uint32_t i = tid; i < CS_HIST_BINS; i += SG_THREADS) {
+            const uint32_t v = u->hist[l][i];
+            if (v) atomicAdd(&ga.ws[l].hist[i], v);
         }
     }
+    if (!all_here(ga, s.g, number, 1u)) return false;
+    uint32_t collect = 0;
+#pragma unroll
+    for (uint32_t l = 0; l < 3u; ++l) {
+        if (!((missed >> l) & 1u)) continue;
+        if (PF && l == 2u) list_threshold<true>(ga, l);
+        else list_threshold<false>(ga, l);
+        if (ga.k[l]) collect |= 1u << l;
+    }
+    for (uint32_t o = 0; collect && o < SH.n_own; ++o) {
+        s.share = SH.own[o];
+        walk_start(ga, s);
+        scan_index<TIERS, PF>(ga, s, collect, 1u);
+    }
+    if (!all_here(ga, s.g, number, 2u)) return false;
+    if (first)                                                 // ready for the next call
+        for (uint32_t l = 0; l < 3u; ++l)
+            if ((missed >> l) & 1u)
+                for (uint32_t i = tid; i < CS_HIST_BINS; i += SG_THREADS) ga.ws[l].hist[i] = 0;
     return true;
 }
 
@@ -958,10 +1069,12 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     float *const gtab = (float *)(agent + a.A);
     cs_grid_state *const g = ws.grid;
     if (tid < 3u) SH.elig[tid] = SH.bad[tid] = 0;
+    if (tid == 0) { SH.n_own = 1u; SH.own[0] = (uint16_t)cta; }
     const float g_sat = cs_recency(a.lambda, a.delta, a.age_sat);
     for (uint32_t i = tid; i <= a.gtab_len; i += n_threads) gtab[i] = i < a.gtab_len ? ws.gtab[i] : g_sat;
     __syncthreads();
     cs_wait_for_predecessor();
+    if (ga.give_up == SG_LATE && cta % 3u) late_start(g);
     // ---- one trip: what is remembered and the tables that change; the first tiles behind it (a small load waits for the megabytes of all SMs
     // when these are asked for first) -------------------------------------------------------------------------------------------------------
     const bool depth = PF && a.anchor;
@@ -972,9 +1085,11 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     for (uint32_t l = 0; l < 3u; ++l)
         if ((ga.want >> l) & 1u) { b_km[l] = cs_ld_cg_pinned(&g->rem_km[l][tid]); b_id[l] = cs_ld_cg_pinned(&g->rem_id[l][tid]); }
     // (one thread per word: 2,368 warps asking for one sector each wait for another)
-    const uint32_t *word = tid == 32u ? &g->epoch : (tid == 33u ? &ws.sc->a_star : (tid == 34u ? &ws.sc->gate : (tid == 35u ? &ws.sc->last_agent : a.now_dev)));
+    u64 taken = 0;
+    if (tid == 64u) taken = atomicAdd(g->taken + cta, 1ull);
+    const uint32_t *word = (tid == 33u ? &ws.sc->a_star : (tid == 34u ? &ws.sc->gate : (tid == 35u ? &ws.sc->last_agent : a.now_dev)));
     uint32_t scalar = a.now;
-    if (tid >= 32u && tid < (a.now_dev ? 37u : 36u)) scalar = cs_ld_cg_pinned(word);
+    if (tid >= 33u && tid < (a.now_dev ? 37u : 36u)) scalar = cs_ld_cg_pinned(word);
 #pragma unroll
     for (uint32_t h = 0; h < 2u; ++h) {                        // (at most 1,024 agents, at least 512 threads)
         const uint32_t i = tid + h * n_threads;
@@ -990,7 +1105,11 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         end_km = cs_ld_cg_pinned(&g->rem_km[tid][CS_BUCKETS]);
         end_id = cs_ld_cg_pinned(&g->rem_id[tid][CS_BUCKETS]);
     }
-    if (tid >= 32u && tid < 37u) SH.scalar[tid - 32u] = scalar;
+    if (tid >= 33u && tid < 37u) SH.scalar[tid - 32u] = scalar;
+    if (tid == 64u) {
+        SH.scalar[0] = (uint32_t)taken;
+        SH.lost = share_is_free(taken, (uint32_t)taken) ? 0u : 1u;
+    }
 #pragma unroll
     for (uint32_t h = 0; h < 2u; ++h)
         if (tid + h * n_threads < a.A) agent[tid + h * n_threads] = t[h];
@@ -1012,10 +1131,10 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         L.spec = 1u;
         L.ranked = 0;
     }
-    Sg s = {g, 0u, 0u, 0u, (uint32_t)__cvta_generic_to_shared(agent), (uint32_t)__cvta_generic_to_shared(gtab), a.gtab_len == a.age_sat, depth};
+    Sg s = {g, 0u, 0u, 0u, cta, (uint32_t)__cvta_generic_to_shared(agent), (uint32_t)__cvta_generic_to_shared(gtab), a.gtab_len == a.age_sat, depth};
     walk_start(ga, s);
     __syncthreads();
-    const uint32_t epoch = SH.scalar[0] & 1u;
+    const uint32_t number = SH.scalar[0], epoch = number & 1u;
     s.epoch = epoch;
     s.a_star = SH.scalar[1];
     s.now = SH.scalar[4];
@@ -1044,62 +1163,39 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     __syncthreads();
     if (tid < 3u && SH.bad[tid]) SH.list[tid].nb = 0;
     __syncthreads();
+    if (SH.lost) return walk_drain();                          // (what it has read besides may be what the others have made of it since)
     bool primed = true;                                        // tiles of a walk that nobody has begun are on their way
-    if (scanned) {
-        scan_index<TIERS, PF>(ga, s, scanned, 0u);
-        primed = false;
-        __syncthreads();
-        if (tid < 3u && SH.elig[tid]) atomicAdd(&g->list[epoch][tid].eligible, SH.elig[tid]);
-    }
-    if (!grid_barrier(ga, g, epoch, 0u)) {
+    uint32_t at_barrier;
+    do {
+        if (scanned) {
+            if (!primed) walk_start(ga, s);
+            primed = false;
+            scan_index<TIERS, PF>(ga, s, scanned, 0u);
+            __syncthreads();
+            if (tid < 3u && SH.elig[tid]) { atomicAdd(&g->list[epoch][tid].eligible, SH.elig[tid]); SH.elig[tid] = 0; }
+        }
+        at_barrier = grid_barrier(ga, g, number, 0u, 1u, true);
+        s.share = at_barrier;                                  // (one more, unless all are done)
+    } while (at_barrier < G);
+    const uint32_t n_own = SH.n_own;
+    bool first = cta == 0;                                     // share 0 is this CTA's
+    for (uint32_t o = 1; o < n_own; ++o) first |= SH.own[o] == 0;
+    if (first) prepare_next_launch(g, epoch);
+    if (at_barrier == SG_FAILED) {
         walk_drain();
-        return give_up(ga, g, epoch, true);
+        return give_up(ga, g);
     }
     cs_release_successor();
-    if (cta == G - 1u) {                                       // the other set of words is the next launch's
-        const uint32_t other = epoch ^ 1u;
-        for (uint32_t l = 0; l < 3u; ++l) g->count[other][l][tid * CS_BCOUNT_STRIDE] = 0;
-        if (tid < 8u) g->bar[other][tid][0] = 0;
-        if (tid < 3u) { g->list[other][tid].c_scan = 0; g->list[other][tid].c_collect = 0; g->list[other][tid].eligible = 0; }
-        if (tid == 0) g->epoch = other;
+    uint32_t quick = scanned ? order_by_buckets(ga, g, epoch, cta, scanned, false) : 0u, missed = open & ~scanned;
+    for (uint32_t o = 1; scanned && o < n_own; ++o) {
+        __syncthreads();
+        quick = order_by_buckets(ga, g, epoch, SH.own[o], scanned, false);
     }
-    uint32_t quick = scanned ? order_by_buckets(ga, g, epoch, scanned, false) : 0u, missed = open & ~scanned;
 #pragma unroll
     for (uint32_t l = 0; l < 3u; ++l)
         if ((scanned >> l) & 1u && !SH.list[l].spec) missed |= 1u << l;
-    // ---- lists without the candidates they need: a histogram of the full keys, a threshold, another look at the index ---------------------
     if (missed) {
-        __syncthreads();                                       // (the tiles' place is the copies' again)
-        if (!primed) walk_start(ga, s);
-        for (uint32_t i = tid; i < 3u * CS_HIST_BINS; i += n_threads) u->hist[0][i] = 0;
-        __syncthreads();
-        count_index<TIERS, PF>(ga, s, missed);
-        __syncthreads();
-        for (uint32_t l = 0; l < 3u; ++l) {
-            if (!((missed >> l) & 1u)) continue;
-            for (uint32_t i = tid; i < CS_HIST_BINS; i += n_threads) {
-                const uint32_t v = u->hist[l][i];
-                if (v) atomicAdd(&ga.ws[l].hist[i], v);
-            }
-        }
-        if (!grid_barrier(ga, g, epoch, 1u)) return give_up(ga, g, epoch, false);
-        uint32_t collect = 0;
-#pragma unroll
-        for (uint32_t l = 0; l < 3u; ++l) {
-            if (!((missed >> l) & 1u)) continue;
-            if (PF && l == 2u) list_threshold<true>(ga, l);
-            else list_threshold<false>(ga, l);
-            if (ga.k[l]) collect |= 1u << l;
-        }
-        if (collect) {
-            walk_start(ga, s);
-            scan_index<TIERS, PF>(ga, s, collect, 1u);
-        }
-        if (!grid_barrier(ga, g, epoch, 2u)) return give_up(ga, g, epoch, false);
-        if (cta == 0)                                          // ready for the next call
-            for (uint32_t l = 0; l < 3u; ++l)
-                if ((missed >> l) & 1u)
-                    for (uint32_t i = tid; i < CS_HIST_BINS; i += n_threads) ga.ws[l].hist[i] = 0;
+        if (!collect_missed<TIERS, PF>(ga, s, number, missed, primed, first)) return give_up(ga, g);
     } else if (primed) {
         walk_drain();                                          // (no list is open)
     }
@@ -1108,8 +1204,9 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     for (uint32_t l = 0; l < 3u; ++l) {
         if (!((ga.want >> l) & 1u)) continue;
         const ListShared &L = SH.list[l];
-        for (uint32_t i = L.n_out + cta * n_threads + tid; i < ga.k[l]; i += G * n_threads) ga.ids[l][i] = CS_ID_NONE;
-        if (cta == 0 && tid == 0) {
+        for (uint32_t o = 0; L.n_out < ga.k[l] && o < n_own; ++o)
+            for (uint32_t i = L.n_out + SH.own[o] * n_threads + tid; i < ga.k[l]; i += G * n_threads) ga.ids[l][i] = CS_ID_NONE;
+        if (first && tid == 0) {
             *ga.n_out[l] = L.n_out;
             count_select(ws, l, L.n_elig, L.n_out);
             count_candidates(ws, l, L.c, L.spec != 0u);
@@ -1117,16 +1214,15 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         if (L.n_out && !((quick >> l) & 1u)) rest |= 1u << l;
         if ((quick >> l) & 1u && ga.speculate) {
             const bool bound = L.c > sg_ahead(ga.k[l]) / 4u * 5u;
-            if (bound || L.refresh) sample_for_next(ga, g, l, L.refresh != 0u, bound);
+            for (uint32_t o = 0; (bound || L.refresh) && o < n_own; ++o) sample_for_next(ga, g, SH.own[o], l, L.refresh != 0u, bound);
         }
     }
-    if (rest && !order_by_sample(ga, g, epoch, rest)) give_up(ga, g, epoch, false);
+    if (rest && !order_by_sample(ga, g, number, rest)) give_up(ga, g);
 }
 
 // ---- host -----------------------------------------------------------------------------------------------------------------------------------
 
-// A device's limits, asked once per process and device: CTAs of the kernels that can be resident at once, 0 when cooperative launches are not
-// to be had.
+// Asked once per process and device: shares of a launch, one per SM; 0 when the kernels' shared memory is not to be had.
 struct GridDevice { int ready, ctas; };
 static std::mutex g_grid_mu;
 static GridDevice g_grid_dev[64];
@@ -1137,15 +1233,12 @@ static int grid_ctas(int device, int sm_count)
     std::lock_guard<std::mutex> lock(g_grid_mu);
     GridDevice &d = g_grid_dev[device];
     if (!d.ready) {
-        int coop = 0;
-        cudaError_t e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
         const int most = (int)sg_smem_bytes(CS_MAX_AGENTS, CS_GTAB_MAX);
-        if (e == cudaSuccess && coop == 1) {
-            for (const auto kernel : {cs_select_grid_kernel<0, true>, cs_select_grid_kernel<1, false>, cs_select_grid_kernel<1, true>,
-                                      cs_select_grid_kernel<2, false>, cs_select_grid_kernel<2, true>})
-                if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-            d.ctas = e == cudaSuccess ? sm_count : 0;
-        }
+        cudaError_t e = cudaSuccess;
+        for (const auto kernel : {cs_select_grid_kernel<0, true>, cs_select_grid_kernel<1, false>, cs_select_grid_kernel<1, true>,
+                                  cs_select_grid_kernel<2, false>, cs_select_grid_kernel<2, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        d.ctas = e == cudaSuccess ? std::min<int>(sm_count, CS_GRID_MAX_CTAS) : 0;
         (void)cudaGetLastError();
         d.ready = 1;
     }
@@ -1182,26 +1275,22 @@ int cs_launch_select_grid(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
     ga.speculate = ctx->no_speculation ? 0u : 1u;
     ga.give_up = ctx->grid_give_up;
     const bool pf = (ga.want & 4u) != 0;
-    const uint32_t G = std::min<uint32_t>(most, std::max<uint32_t>(SG_MIN_CTAS, idx->n_blocks / 512u));
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = CS_USE_PDL;
-    cfg.gridDim = dim3(G);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = CS_USE_PDL;
+    cfg.gridDim = dim3(most);                                  // (the same for every launch of a context: cs_grid_state.taken)
     cfg.blockDim = dim3(SG_THREADS);
     cfg.dynamicSmemBytes = sg_smem_bytes(ga.a.A, ga.a.gtab_len);
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = 1;
     const int tiers = (ga.want & 1u) + ((ga.want >> 1) & 1u);
     const auto kernel = tiers == 2 ? (pf ? cs_select_grid_kernel<2, true> : cs_select_grid_kernel<2, false>)
                                    : (tiers == 1 ? (pf ? cs_select_grid_kernel<1, true> : cs_select_grid_kernel<1, false>) : cs_select_grid_kernel<0, true>);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, ga);
     if (e != cudaSuccess) {
-        // (fewer SMs than the device has may be this process's: nothing has been enqueued)
-        (void)cudaGetLastError();
+        (void)cudaGetLastError();                              // (nothing has been enqueued)
         ctx->grid_refused = 1;
         return CS_ENOTIMPL;
     }

@@ -97,7 +97,30 @@ def test_a_select_that_gives_up_leaves_empty_lists_and_nothing_behind(barrier):
     assert c.get_status() == cs.CS_ST_TIMEOUT
     assert c.get_status() == 0 and ref.get_status() == 0
     with pytest.raises(cs.CacheScoutError):
-        c.selftest_select_wait(6)
+        c.selftest_select_wait(7)
+
+
+@pytest.mark.parametrize("n", [150_003, 1_000_000])
+def test_a_select_goes_on_without_ctas_that_do_not_start(n):
+    """Two CTAs in three of the whole-GPU select start only when the others have taken over their shares.  Lists that are found in the remembered
+    buckets, lists ordered by a sample and lists without a key, in turn with undisturbed calls, all as the launch chain gives them."""
+    cfg, k, kp = synth.CONFIGS["meta1m"], 2500, 2100
+    c, _, _ = warm(cfg, 800, n, r_min=0.02)
+    ref, _, _ = warm(cfg, 800, n, r_min=0.02)
+    ref.set_select_path(cs.CS_SELECT_MULTI)
+    d = cs.DeviceIndex.from_host(synth.make_block_index(cfg, n=n, tier="random"), DEV)
+    la = d.last_access.view(torch.int32)
+    lists = lambda: [torch.full((m,), 7, dtype=torch.int32, device=DEV) for m in (k, 4, k, 4, kp, 4)]
+    for rep in range(12):
+        c.set_select_speculation(rep not in (6, 7))
+        c.selftest_select_wait(6 if rep % 3 else 0)
+        got, want = lists(), lists()
+        c.select_step(d, 100_000 + rep, k, kp, *got)
+        ref.select_step(d, 100_000 + rep, k, kp, *want)
+        assert all(torch.equal(x, y) for x, y in zip(got, want)), rep
+        if rep > 8:
+            la[want[0].long()] = 100_000 + rep - 3
+    assert c.get_status() == ref.get_status() == 0
 
 
 @pytest.mark.parametrize("path", [cs.CS_SELECT_CLUSTER, cs.CS_SELECT_MULTI])

@@ -70,6 +70,7 @@ def test_selects_are_launched_one_by_one_when_their_graph_fails(rt, call, skip):
     """Two lists of a large index, five times.  Whatever the driver refuses of their graph, at whichever call: the call succeeds by
     single launches, no error is left behind, and a graph that failed is not tried again."""
     ctx = make_ctx(rt, n_agents=12, n_chains=4, max_blocks=400_000)
+    cs.cs_set_select_path(ctx, cs.CS_SELECT_MULTI)
     idx = index(300_000)
     rt.fake_fail(call.encode(), skip, 1, OUT_OF_MEMORY)
     by_graph = []

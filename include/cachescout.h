@@ -352,8 +352,7 @@ int cs_import_state(cs_ctx *ctx, const uint32_t *C_in, const uint16_t *cur_in, u
  * Returns CS_EDEVICE_STATUS when the word was non-zero. */
 int cs_get_status(cs_ctx *ctx, uint32_t *device_status, cs_stream_t stream);
 
-/* Number of kernels this context has launched so far (host counter); the copy made by cs_get_model() is not counted.
- * A select of an index above 262,144 entries counts as six whichever way it goes. */
+/* Number of kernels this context has launched so far (host counter); the copy made by cs_get_model() is not counted. */
 int cs_launch_count(cs_ctx *ctx, uint64_t *n_launches);
 
 /* Work counters kept in the workspace by the kernels themselves (the paper reports only hit rate and

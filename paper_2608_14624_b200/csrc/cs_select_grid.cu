@@ -1294,6 +1294,6 @@ int cs_launch_select_grid(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, 
         ctx->grid_refused = 1;
         return CS_ENOTIMPL;
     }
-    ctx->n_launches += idx->n_blocks > CS_SELECT_CLUSTER_MAX_BLOCKS ? (uint64_t)CS_SELECT_STAGES * job : 1u;       // (cs_launch_count())
+    ctx->n_launches++;
     return CS_OK;
 }

@@ -1141,8 +1141,8 @@ def test_survival_from_all_chains(name, n_inv):
     ("meta1m", 262144, 10000, 2000), ("meta1m", 300000, 500, 500), ("meta1m", 1_000_000, 10000, 2000)])
 @pytest.mark.parametrize("path", [cs.CS_SELECT_AUTO, cs.CS_SELECT_MULTI])
 def test_select_step_matches_three_calls_and_oracle(name, n, kv, kp, path):
-    """cs_select_step: one launch of three clusters where the single-launch select applies, three kernel chains
-    side by side elsewhere (300,000 entries, or the multi-launch path forced); lists bit-exact against the oracle,
+    """cs_select_step: one launch of three clusters or one on the whole GPU where these apply, three kernel chains
+    side by side elsewhere (a first call over 300,000 entries, or the multi-launch path forced); lists bit-exact against the oracle,
     and again on a second and third call with a later clock (remembered thresholds in play)."""
     cfg = synth.CONFIGS[name]
     c, o = warm_state(cfg, 800, max(n, 16), r_min=0.02)
@@ -1160,8 +1160,8 @@ def test_select_step_matches_three_calls_and_oracle(name, n, kv, kp, path):
                                             (gp, gpn, kp, o.select_prefetch(idx, now, kp, s32))):
             g = got.cpu().numpy().view(np.uint32)[:k]
             assert H.assert_list_matches(g, int(got_n[0].item()), o_ids, o_n, s64) == 0, (rep, k)
-    fused = path == cs.CS_SELECT_AUTO and n <= 262144
-    assert c.launch_count() - l0 == (3 if fused else 3 * 3 * 6)
+    # the first call of a large index is the chain's, the next two are one launch each for all lists
+    assert c.launch_count() - l0 == (3 * 3 * 6 if path == cs.CS_SELECT_MULTI else (3 if n <= 262144 else 3 * 6 + 1 + 1))
     # a select whose count pointer is NULL is left out
     gh.fill_(7)
     ghn.fill_(7)
@@ -1175,13 +1175,17 @@ def test_select_step_matches_three_calls_and_oracle(name, n, kv, kp, path):
     assert c.get_status() == 0
 
 
-def test_select_step_side_by_side_is_stable_over_many_calls():
-    """The three kernel chains of a step run side by side on three streams with private scratch: over many
-    consecutive calls with a moving clock and a changing index every list must equal the one the same select
-    produces alone (bitwise), and the last call is checked against the oracle."""
+@pytest.mark.parametrize("path", [cs.CS_SELECT_MULTI, cs.CS_SELECT_AUTO])
+def test_select_step_side_by_side_is_stable_over_many_calls(path):
+    """The three kernel chains of a step run side by side on three streams with private scratch (or all lists in one launch): over many
+    consecutive calls with a moving clock and a changing index every list must equal the one that a chain of its own
+    produces (bitwise), and the last call is checked against the oracle."""
     cfg = synth.CONFIGS["meta1m"]
     n, kv, kp = 300_000, 3000, 1500
     c, o = warm_state(cfg, 800, n, r_min=0.02)
+    alone, _ = warm_state(cfg, 800, n, r_min=0.02)
+    c.set_select_path(path)
+    alone.set_select_path(cs.CS_SELECT_MULTI)
     idx = synth.make_block_index(cfg, n=n, tier="random")
     d = cs.DeviceIndex.from_host(idx, DEV)
     i32 = lambda m: torch.full((max(m, 4),), 7, dtype=torch.int32, device=DEV)
@@ -1193,10 +1197,12 @@ def test_select_step_side_by_side_is_stable_over_many_calls():
         now = 100_000 + 3 * it
         if it:
             la[gv[:kv].long().clamp_(min=0)] = now - 3          # the index changes between calls
+        l0 = c.launch_count()
         c.select_step(d, now, kv, kp, gv, gvn, gh, ghn, gp, gpn)
-        c.select_victims(d, now, 0, kv, sv, svn)
-        c.select_victims(d, now, 1, kv, sh, shn)
-        c.select_prefetch(d, now, kp, sp, spn)
+        assert c.launch_count() - l0 == (1 if path == cs.CS_SELECT_AUTO and it else 18)
+        alone.select_victims(d, now, 0, kv, sv, svn)
+        alone.select_victims(d, now, 1, kv, sh, shn)
+        alone.select_prefetch(d, now, kp, sp, spn)
         bad += (gv != sv).sum() + (gh != sh).sum() + (gp != sp).sum() + (gvn != svn).sum() + (ghn != shn).sum() + (gpn != spn).sum()
     assert int(bad.item()) == 0
     idx.last_access[:] = d.last_access.cpu().numpy()
@@ -1208,14 +1214,17 @@ def test_select_step_side_by_side_is_stable_over_many_calls():
     assert c.get_status() == 0
 
 
+@pytest.mark.parametrize("path", [cs.CS_SELECT_MULTI, cs.CS_SELECT_AUTO])
 @pytest.mark.parametrize("wanted", [(0, 1), (0, 2), (1, 2), (0, 1, 2)])
-def test_select_step_graph_takes_new_arguments(wanted):
-    """Large selects side by side, for every two or three of the lists: indexes of different sizes, other list lengths and
-    other buffers on every call, on the null stream, a stream and inside a stream capture.  Each list must equal, bit for
-    bit, the one that the same select gives alone."""
+def test_select_step_graph_takes_new_arguments(wanted, path):
+    """Large selects side by side, as the library's graph of chains or in one launch, for every two or three of the lists: indexes of different
+    sizes, other list lengths and other buffers on every call, on the null stream, a stream and inside a stream capture.  Each list must equal,
+    bit for bit, the one that a chain of its own gives."""
     cfg = synth.CONFIGS["meta1m"]
     c, _ = warm_state(cfg, 800, 400_000, r_min=0.02)
     alone, _ = warm_state(cfg, 800, 400_000, r_min=0.02)
+    c.set_select_path(path)
+    alone.set_select_path(cs.CS_SELECT_MULTI)
     indexes = [cs.DeviceIndex.from_host(synth.make_block_index(cfg, n=n, tier="random"), DEV) for n in (262_145, 400_000, 300_011)]
     side = torch.cuda.Stream()
     empty = lambda m: torch.full((m,), 7, dtype=torch.int32, device=DEV)
@@ -1236,7 +1245,7 @@ def test_select_step_graph_takes_new_arguments(wanted):
             with torch.cuda.graph(g, stream=side):
                 call()
             g.replay()
-        assert c.launch_count() - n0 == 6 * len(wanted)
+        assert c.launch_count() - n0 == (1 if path == cs.CS_SELECT_AUTO and rep else 6 * len(wanted))
         torch.cuda.synchronize()
         for q in wanted:
             ids, cnt = empty(max(k, 4)), empty(4)

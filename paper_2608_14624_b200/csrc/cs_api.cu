@@ -527,8 +527,6 @@ int cs_get_status(cs_ctx *ctx, uint32_t *device_status, cs_stream_t stream)
     cudaError_t e = cudaMemcpyAsync(&st, &ctx->ws.sc->status_read, sizeof(st), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) { ctx->last_cuda_error = (int)e; return CS_ECUDA; }
-    // (a barrier of the whole-GPU select may be what ran out, which then gives no list any more: the launch chain does)
-    if (st & CS_ST_TIMEOUT) ctx->grid_refused = 1;
     *device_status = st;
     return st ? CS_EDEVICE_STATUS : CS_OK;
 }

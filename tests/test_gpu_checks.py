@@ -55,6 +55,25 @@ def test_bounded_wait_runs_out_and_the_context_stays_usable():
         c.selftest_bounded_wait(0)
 
 
+def test_a_transfer_that_ran_out_leaves_the_selects_their_route():
+    """CS_ST_TIMEOUT of the mover's wait, read and cleared: the lists of a large index still come in one launch."""
+    cfg, n, k = synth.CONFIGS["meta1m"], 300_001, 700
+    c, _, _ = warm(cfg, 800, n, r_min=0.02)
+    d = cs.DeviceIndex.from_host(synth.make_block_index(cfg, n=n, tier="random"), DEV)
+    lists = lambda: [torch.full((m,), 7, dtype=torch.int32, device=DEV) for m in (k, 4, k, 4, k, 4)]
+    got = []
+    for rep in range(4):
+        if rep == 3:
+            c.selftest_bounded_wait(1000)
+            assert c.get_status() == cs.CS_ST_TIMEOUT
+        l0 = c.launch_count()
+        got.append(lists())
+        c.select_step(d, 100_000, k, k, *got[-1])
+        assert c.launch_count() - l0 == (18, 1, 1, 1)[rep]
+        assert all(torch.equal(x, y) for x, y in zip(got[0], got[-1]))
+    assert c.get_status() == 0
+
+
 @pytest.mark.parametrize("barrier", [1, 2, 3, 4, 5])
 def test_a_select_that_gives_up_leaves_empty_lists_and_nothing_behind(barrier):
     """The waits at one of the five grid barriers of the whole-GPU select run out, called and replayed from a graph: empty lists, also where

@@ -951,7 +951,8 @@ static int select_route(cs_ctx *ctx, uint32_t n, uint32_t k, uint32_t lists, cud
 {
     if (ctx->select_path == CS_SELECT_MULTI) return ROUTE_CHAIN;
     const bool fits = n <= CS_SELECT_CLUSTER_MAX_BLOCKS, asked = (ctx->lists_asked & lists) == lists;
-    const bool grid = fits ? ctx->select_path != CS_SELECT_CLUSTER && (n > CS_SELECT_GRID_MIN_BLOCKS || (n > CS_SELECT_GRID_LONG_BLOCKS && k >= CS_SELECT_GRID_LONG_LIST))
+    if (ctx->select_path == CS_SELECT_CLUSTER) return fits ? ROUTE_CLUSTER : ROUTE_CHAIN;
+    const bool grid = fits ? n > CS_SELECT_GRID_MIN_BLOCKS || (n > CS_SELECT_GRID_LONG_BLOCKS && k >= CS_SELECT_GRID_LONG_LIST)
                            : n <= CS_SELECT_GRID_MAX_BLOCKS && k <= CS_SELECT_GRID_MAX_LIST;
     if (grid) ctx->lists_asked |= lists;
     if (grid && !asked) {

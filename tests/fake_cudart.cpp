@@ -15,7 +15,7 @@ std::map<const void *, std::string> &kernels()           // (filled by construct
     return names;
 }
 cudaError_t last = cudaSuccess;
-int pointer_device = 0, pointer_type = cudaMemoryTypeDevice, max_clusters = 148;
+int pointer_device = 0, pointer_type = cudaMemoryTypeDevice, max_clusters = 148, capturing = 0;
 size_t handles = 4096;
 
 cudaError_t call(const std::string &name)
@@ -43,10 +43,11 @@ struct { dim3 grid, block; size_t smem; cudaStream_t s; } config;
 
 extern "C" {
 // ---- what the test says and asks ---------------------------------------------------------------------------------
-void fake_reset() { plans.clear(); calls.clear(); last = cudaSuccess; pointer_device = 0; pointer_type = cudaMemoryTypeDevice; max_clusters = 148; }
+void fake_reset() { plans.clear(); calls.clear(); last = cudaSuccess; pointer_device = 0; pointer_type = cudaMemoryTypeDevice; max_clusters = 148; capturing = 0; }
 void fake_fail(const char *name, int skip, int count, int code) { plans[name] = Plan{skip, count, (cudaError_t)code}; }   // count -1: always
 void fake_pointers(int device, int type) { pointer_device = device; pointer_type = type; }
 void fake_clusters(int n) { max_clusters = n; }
+void fake_capturing(int on) { capturing = on; }
 int fake_calls(const char *part)                       // calls whose name contains `part`
 {
     int n = 0;
@@ -105,7 +106,7 @@ cudaError_t cudaStreamDestroy(cudaStream_t) { return call("cudaStreamDestroy"); 
 cudaError_t cudaStreamGetDevice(cudaStream_t, int *d) { *d = 0; return call("cudaStreamGetDevice"); }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, enum cudaStreamCaptureStatus *st)
 {
-    *st = cudaStreamCaptureStatusNone;
+    *st = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
     return call("cudaStreamIsCapturing");
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return call("cudaStreamSynchronize"); }

@@ -93,6 +93,59 @@ def test_selects_are_launched_one_by_one_when_their_graph_fails(rt, call, skip):
     assert calls(rt, "cudaGraphCreate") - (call == "cudaGraphCreate") == calls(rt, "cudaGraphDestroy")
 
 
+def select_kernels(rt):
+    """(cluster, whole-GPU, chain) select launches so far."""
+    return tuple(sum(calls(rt, name) for name in names) for names in (("cs_select_cluster_kernel", "cs_select_step_kernel"), ("cs_select_grid_kernel",), ("cs_sel_",)))
+
+
+CLUSTER, GRID, CHAIN = (1, 0, 0), (0, 1, 0), (0, 0, 6)
+
+
+@pytest.mark.parametrize("path", [cs.CS_SELECT_AUTO, cs.CS_SELECT_CLUSTER, cs.CS_SELECT_MULTI])
+@pytest.mark.parametrize("n,k,later", [(65_536, 4_000, CLUSTER), (65_537, 2_047, CLUSTER), (65_537, 2_048, GRID), (131_072, 100, CLUSTER), (131_073, 100, GRID),
+                                       (262_144, 200_000, GRID), (262_145, 100, GRID), (262_145, 100_000, GRID), (262_145, 100_001, CHAIN), (1 << 25, 100, GRID),
+                                       ((1 << 25) + 1, 100, CHAIN)])
+def test_route_of_a_select(rt, n, k, later, path):
+    """Which kernels a list takes on its first call and from the second one on, on both sides of every line; a captured first call counts as a later one."""
+    first = CLUSTER if n <= 262_144 else CHAIN
+    if path != cs.CS_SELECT_AUTO:
+        first = later = first if path == cs.CS_SELECT_CLUSTER else CHAIN
+    for captured in (0, 1):
+        ctx = make_ctx(rt, n_agents=12, n_chains=4, max_blocks=n + 100)
+        cs.cs_set_select_path(ctx, path)
+        for call in range(4):
+            rt.fake_capturing(captured and call == 0)
+            before, n0 = select_kernels(rt), cs.cs_launch_count(ctx)
+            if call < 3:
+                cs.cs_select_victims(ctx, index(n), 5, 1, k, BUF, BUF, stream=0)
+            else:                                               # (a list that has not been asked for)
+                cs.cs_select_prefetch(ctx, index(n), 5, k, BUF, BUF, stream=0)
+            took = tuple(b - a for a, b in zip(before, select_kernels(rt)))
+            assert took == (later if call in (1, 2) or (captured and call == 0) else first), (captured, call)
+            assert cs.cs_launch_count(ctx) - n0 == sum(took)
+        cs.cs_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,lists,instead", [(200_000, 1, CLUSTER), (200_000, 3, CLUSTER), (300_000, 1, CHAIN), (300_000, 3, (0, 0, 18))])
+@pytest.mark.parametrize("call,skip", [("launch", 0), ("cudaFuncSetAttribute", 0), ("cudaFuncSetAttribute", 4)])
+def test_a_refused_whole_gpu_select_goes_the_other_way(rt, n, lists, instead, call, skip):
+    """The driver refuses the launch or its shared memory: the call succeeds by the cluster or the chain, no error is left behind, and later calls do not
+    ask again."""
+    ctx = make_ctx(rt, n_agents=12, n_chains=4, max_blocks=400_000)
+    select = lambda: (cs.cs_select_step(ctx, index(n), 5, 100, 100, BUF, BUF, BUF, BUF, BUF, BUF, stream=0) if lists == 3 else
+                      cs.cs_select_victims(ctx, index(n), 5, 0, 100, BUF, BUF, stream=0))
+    select()
+    rt.fake_fail(call.encode(), skip, 1, OUT_OF_MEMORY)
+    for _ in range(3):
+        before, graphs, n0 = select_kernels(rt), calls(rt, "cudaGraphLaunch"), cs.cs_launch_count(ctx)
+        select()
+        took = tuple(b - a for a, b in zip(before, select_kernels(rt)))
+        assert took == instead or (calls(rt, "cudaGraphLaunch") == graphs + 1 and took == (0, 0, 0) and instead[2] == 18)
+        assert cs.cs_launch_count(ctx) - n0 == sum(instead)
+        assert rt.cs_last_cuda_error(ctx) == 0 and rt.cudaGetLastError() == 0
+    cs.cs_destroy(ctx)
+
+
 @pytest.mark.parametrize("device,kind,odd,by_kernel", [(0, DEVICE_MEMORY, 0, 8), (1, DEVICE_MEMORY, 0, 0), (0, HOST_MEMORY, 0, 0),
                                                        (0, 0, 0, 0), (0, DEVICE_MEMORY, 1, 0)])
 def test_model_is_exported_by_a_kernel_to_its_own_gpu_only(rt, device, kind, odd, by_kernel):

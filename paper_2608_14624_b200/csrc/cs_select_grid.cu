@@ -1055,10 +1055,31 @@ __device__ __noinline__ bool collect_missed(const GridArgs &ga, Sg s, uint32_t n
     return true;
 }
 
+// Shares that the first barrier has given this CTA besides its own, until there are none left.
+template <int TIERS, bool PF>
+__device__ __noinline__ uint32_t take_over(const GridArgs &ga, Sg s, uint32_t number, uint32_t scanned, uint32_t share)
+{
+    const uint32_t tid = threadIdx.x;
+    while (share < gridDim.x) {
+        s.share = share;
+        if (scanned) {
+            walk_start(ga, s);
+            scan_index<TIERS, PF>(ga, s, scanned, 0u);
+            __syncthreads();
+            if (tid < 3u && SH.elig[tid]) { atomicAdd(&s.g->list[number & 1u][tid].eligible, SH.elig[tid]); SH.elig[tid] = 0; }
+        }
+        share = grid_barrier(ga, s.g, number, 0u, 1u, true);
+    }
+    return share;
+}
+
 // ---- the kernel -------------------------------------------------------------------------------------------------------------------------------
 // TIERS: tiers whose victims are wanted, PF: the prefetch list.
+//
+// Shared memory allows one CTA per SM, so registers are free up to what a compaction's CTAs beside it need (two of 64 threads).  Three lists of 20,000 out of
+// 4,000,000 entries, static index, and a select of 1,000,000 beside back-to-back compactions, us: 64 registers 37 / 36, 80 35 / 31, 96 34 / 28, 124 33 / 73.
 template <int TIERS, bool PF>
-__global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __grid_constant__ GridArgs ga)
+__global__ void __maxnreg__(96) cs_select_grid_kernel(const __grid_constant__ GridArgs ga)
 {
     const uint32_t tid = threadIdx.x, n_threads = SG_THREADS, cta = blockIdx.x, G = gridDim.x;
     const cs_workspace &ws = ga.ws[0];
@@ -1106,10 +1127,7 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         end_id = cs_ld_cg_pinned(&g->rem_id[tid][CS_BUCKETS]);
     }
     if (tid >= 33u && tid < 37u) SH.scalar[tid - 32u] = scalar;
-    if (tid == 64u) {
-        SH.scalar[0] = (uint32_t)taken;
-        SH.lost = share_is_free(taken, (uint32_t)taken) ? 0u : 1u;
-    }
+    // (the share's word comes back last: it is put down further below)
 #pragma unroll
     for (uint32_t h = 0; h < 2u; ++h)
         if (tid + h * n_threads < a.A) agent[tid + h * n_threads] = t[h];
@@ -1134,8 +1152,6 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
     Sg s = {g, 0u, 0u, 0u, cta, (uint32_t)__cvta_generic_to_shared(agent), (uint32_t)__cvta_generic_to_shared(gtab), a.gtab_len == a.age_sat, depth};
     walk_start(ga, s);
     __syncthreads();
-    const uint32_t number = SH.scalar[0], epoch = number & 1u;
-    s.epoch = epoch;
     s.a_star = SH.scalar[1];
     s.now = SH.scalar[4];
     // Blocks age as the clock goes on, and those that leave the index are replaced by those that reach their age: what is remembered stands for
@@ -1145,7 +1161,6 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
         if ((ga.want >> l) & 1u) u->s.b_km[l][tid] = moved_key(b_km[l], s.now - SH.list[l].then, l == 2u);
     if (tid < 3u) {
         ListShared &L = SH.list[tid];
-        L.epoch = epoch;
         L.now = s.now;
         u->s.b_km[tid][CS_BUCKETS] = moved_key(u->s.b_km[tid][CS_BUCKETS], s.now - L.then, tid == 2u);
         if (L.moves) L.bound = moved_key(L.bound, s.now - L.then, tid == 2u);
@@ -1162,21 +1177,23 @@ __global__ void __launch_bounds__(SG_THREADS, 2) cs_select_grid_kernel(const __g
             SH.bad[l] = 1u;
     __syncthreads();
     if (tid < 3u && SH.bad[tid]) SH.list[tid].nb = 0;
+    if (tid == 64u) {
+        SH.scalar[0] = (uint32_t)taken;
+        SH.lost = share_is_free(taken, (uint32_t)taken) ? 0u : 1u;
+    }
     __syncthreads();
+    const uint32_t number = SH.scalar[0], epoch = number & 1u;
+    s.epoch = epoch;
+    if (tid < 3u) SH.list[tid].epoch = epoch;
     if (SH.lost) return walk_drain();                          // (what it has read besides may be what the others have made of it since)
-    bool primed = true;                                        // tiles of a walk that nobody has begun are on their way
-    uint32_t at_barrier;
-    do {
-        if (scanned) {
-            if (!primed) walk_start(ga, s);
-            primed = false;
-            scan_index<TIERS, PF>(ga, s, scanned, 0u);
-            __syncthreads();
-            if (tid < 3u && SH.elig[tid]) { atomicAdd(&g->list[epoch][tid].eligible, SH.elig[tid]); SH.elig[tid] = 0; }
-        }
-        at_barrier = grid_barrier(ga, g, number, 0u, 1u, true);
-        s.share = at_barrier;                                  // (one more, unless all are done)
-    } while (at_barrier < G);
+    const bool primed = !scanned;                              // the first tiles of a walk that nobody has begun are on their way
+    if (scanned) {
+        scan_index<TIERS, PF>(ga, s, scanned, 0u);
+        __syncthreads();
+        if (tid < 3u && SH.elig[tid]) { atomicAdd(&g->list[epoch][tid].eligible, SH.elig[tid]); SH.elig[tid] = 0; }
+    }
+    uint32_t at_barrier = grid_barrier(ga, g, number, 0u, 1u, true);
+    if (at_barrier < G) at_barrier = take_over<TIERS, PF>(ga, s, number, scanned, at_barrier);
     const uint32_t n_own = SH.n_own;
     bool first = cta == 0;                                     // share 0 is this CTA's
     for (uint32_t o = 1; o < n_own; ++o) first |= SH.own[o] == 0;

@@ -472,7 +472,7 @@ int cs_use_survival_table(cs_ctx *ctx, const float *fsurv);
 
 /* Implementation of the two select calls: CS_SELECT_AUTO (= the single-launch cluster kernel for small
  * indexes, one launch on the whole GPU for all lists of large ones from a list's second call on, the
- * multi-launch path for the largest and for longer lists than 100,000 ids), CS_SELECT_CLUSTER (the cluster
+ * multi-launch path for the largest and for longer lists than 50,000 ids), CS_SELECT_CLUSTER (the cluster
  * kernel up to 262,144 entries, the multi-launch path above), CS_SELECT_MULTI (fast pass / histogram / collect / sample /
  * place / finish as six grid-wide launches).  All give the same lists. */
 #define CS_SELECT_AUTO 0u

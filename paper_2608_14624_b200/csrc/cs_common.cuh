@@ -30,7 +30,7 @@ struct cs_nvtx_range {
 #define CS_SELECT_GRID_LONG_BLOCKS (1u << 16)      // with a list of CS_SELECT_GRID_LONG_LIST ids or more
 #define CS_SELECT_GRID_LONG_LIST 2048u
 #define CS_SELECT_GRID_MAX_BLOCKS (1u << 25)
-#define CS_SELECT_GRID_MAX_LIST 100000u
+#define CS_SELECT_GRID_MAX_LIST 50000u
 
 #define CS_CONCURRENT_MAX_BLOCKS (1u << 22)        // up to this index size every select of a step has full-size scratch of its own
 

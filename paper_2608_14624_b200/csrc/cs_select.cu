@@ -937,13 +937,15 @@ static int launch_stage(cs_ctx *ctx, SelectChain &c, int stage, cs_select_graph 
 }
 
 // The route of selects over n entries, the longest list k: a cluster per list, one launch on the whole GPU for all of them, or a launch chain
-// per list.  Both sides of the lines, us per call: three lists and the refresh before them, back to back in a graph (static index), and the
-// three lists alone where every list's entries have left the index before the next call (moving).
-//   cluster / whole GPU  static 80,000 entries, k = 256 19.0 / 18.2, 131,072 22.1 / 20, 262,000 27.4 / 18.2; 131,072, k = 4,000 41.0 / 24.6,
-//                        262,000, k = 16,000 69.3 / 35.9; moving 80,000, k = 256 27.6 / 37.0, 131,072, k = 4,000 45.1 / 50.3
-//   chain / whole GPU    static 300,000, k = 256 28.6 / 20.6, 1,000,000, k = 10,000 48.3 / 30.8, 4,000,000, k = 20,000 75.9 / 49; moving
-//                        44.9 / 29.9, 52.6 / 33.8, 85.9 / 75.8; a remembered key that does not hold, 4,000,000, k = 1,359 70 / 66; one list 1,000,000, k = 10,000 29.2 / 13.5, 32,000,000 73.7 / 70.4, 64,000,000
-//                        114.3 / 119.5; 300,000, k = 75,000 63.8 / 39.7, 1,000,000, k = 142,857 87 / 89
+// per list.  Both sides of the lines, mean us per call replayed from a graph, an index that does not change but for the clock (static) / one whose victims
+// are used again and whose prefetched entries are gone for eight calls (moving); v: one list of k, vhp: three.
+//   cluster / whole GPU   80,000, k = 256, vhp 19.0 / 18.2 (and the refresh) and 27.6 / 37.0, 140,000 30.7 / 18.5 and 31.0 / 29.7; 80,000, k = 4,000, vhp 39.1 / 22.4 and 39.8 / 42.7,
+//                         131,072, k = 4,000 43.3 / 20.6 and 42.5 / 35.2, 262,144, k = 16,000 73.5 / 25.8 and 76.2 / 51.0
+//   chain / whole GPU     300,000, k = 256, vhp 33.2 / 21.4 and 40.2 / 30.2; 1,000,000, k = 10,000, v 33.3 / 22 and 34.3 / 35.9; 4,000,000, k = 20,000, vhp 66.5 / 34.3
+//                         and 108 / 87; 16,000,000, k = 10,000, v 55.9 / 45 and 70 / 75.5; 32,000,000 73.7 / 70.4, 64,000,000 114.3 / 119.5 (static).
+//                         Long lists, v: 1,000,000, k = 30,000 moving 46.1 / 50.3, k = 100,000 70.0 / 47.1 and 78 / 106; 300,000, k = 75,000 67.6 / 60.6 and 71.7 / 91
+// Where victims leave by the thousand, entries of one call are tied but for their ids and swell single buckets, and the list goes on to the ranked
+// sample; the lines lie where the two kinds of index together are no longer faster.
 // A list's first call finds nothing remembered and has four passes more: it takes the route that the list would have without this one
 // (1,000,000 entries, two lists: 114 us, 123 in one launch).
 enum { ROUTE_CLUSTER, ROUTE_GRID, ROUTE_CHAIN };

@@ -103,7 +103,7 @@ CLUSTER, GRID, CHAIN = (1, 0, 0), (0, 1, 0), (0, 0, 6)
 
 @pytest.mark.parametrize("path", [cs.CS_SELECT_AUTO, cs.CS_SELECT_CLUSTER, cs.CS_SELECT_MULTI])
 @pytest.mark.parametrize("n,k,later", [(65_536, 4_000, CLUSTER), (65_537, 2_047, CLUSTER), (65_537, 2_048, GRID), (131_072, 100, CLUSTER), (131_073, 100, GRID),
-                                       (262_144, 200_000, GRID), (262_145, 100, GRID), (262_145, 100_000, GRID), (262_145, 100_001, CHAIN), (1 << 25, 100, GRID),
+                                       (262_144, 200_000, GRID), (262_145, 100, GRID), (262_145, 50_000, GRID), (262_145, 50_001, CHAIN), (1 << 25, 100, GRID),
                                        ((1 << 25) + 1, 100, CHAIN)])
 def test_route_of_a_select(rt, n, k, later, path):
     """Which kernels a list takes on its first call and from the second one on, on both sides of every line; a captured first call counts as a later one."""

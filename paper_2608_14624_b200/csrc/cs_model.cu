@@ -1061,8 +1061,8 @@ cs_exact_survival_kernel(cs_workspace ws, uint32_t A, uint32_t a0_arg, uint32_t 
 // The differences lose nothing that p has: every term of f_n is at most p, so what f_n is off by, before it goes on, is at most n roundings of p,
 // and it goes on as e_n = delta_n - sum e_t d_{n-t}, which the renewal equation sums to at most twice the deltas' sum.
 //
-// (Against extended precision, matrices of 4 to 256 agents, dense, sparse, nearly a chain, and of entries from 1e-9 to 1: both ways are within
-// 1.5e-15 of p, and after the rounding to fp32 the largest errors are the same to three digits, 6e-8.)
+// (Against extended precision, matrices of 4 to 256 agents, dense, sparse, nearly a chain, agents that mostly follow themselves, and of entries from 1e-12
+// to 1: relative to p, the way above is within 3e-15 and this one within 1e-14, and after the rounding to fp32 the largest errors are the same to three digits, 6e-8.)
 //
 // Clusters as above, but a warp multiplies 16 rows by a slice of the agents with matrix instructions (m16n8k8; rows of the new w by the agents summed
 // over, times 8 targets), so that few slices are left to add up and the vectors are read from shared memory once for 16 rows.  Bound by the fp64 pipe
@@ -1088,7 +1088,8 @@ __device__ __forceinline__ void mma_f64(double (&c)[4], double a0, double a1, do
     asm("mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3]) : "d"(a0), "d"(a1), "d"(a2), "d"(a3), "d"(b0), "d"(b1));
 }
-// A probability of the matrix (0, or 2^-32 to 1) times 2^-896: a float's bits in a double's place, which costs no conversion.  The vectors that it is
+// A probability of the matrix times 2^-896: a float's bits in a double's place, which costs no conversion and is exact for every finite float, denormal ones
+// too (the smoothing keeps entries above 0, about eps / n of a row).  The vectors that it is
 // multiplied with are kept times 2^896.  (A product of 64 rows, 256 agents and 8 targets 0.3 us less.)
 #define XS_UP 0x1p896
 #define XS_DOWN 0x1p-896

@@ -17,9 +17,8 @@
 // ranking 2; beyond that by the scan's instructions (about 200 per 128 entries; 64,000,000 entries at 119 us are 4.8 TB/s, where the chain's scan,
 // which compares last_access alone for most entries, has 5.0).  Loads are asynchronous copies by each thread for itself, three steps of four
 // entries ahead: bulk copies into a ring, with a producer warp, took 187 to 330 us for 64,000,000 entries, two steps at a time 10 % longer,
-// four steps 2 % and 22 KiB of shared memory, which keeps the CTA off SMs where a compaction's runs.  Before and after, us per call, a refresh and its
-// lists back to back in a graph: 300,000 entries, three lists of 256 to 384 28.6 / 18.6; 1,000,000, lists of 10,000 and 2,000 (256 agents, 64
-// events) 47 / 38; 4,000,000, three lists of up to 20,000 76 / 50; one list of 10,000: 1,000,000 29.2 / 13.5, 16,000,000 49.1 / 39.4.
+// four steps 2 % and 22 KiB of shared memory, which keeps the CTA off SMs where a compaction's runs.  Times beside those of the routes that it
+// replaces stand at select_route() (cs_select.cu).
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
@@ -34,7 +33,8 @@
 #define SG_BUCKET_WARP 96u             // largest bucket that one warp ranks, three keys per lane
 #define SG_KEYS 128u                   // keys that a warp holds at a time
 #define SG_BUCKET_MAX 1024u            // largest bucket that is counted.  (Index that moves, 1,000,000 entries, lists of 10,000 and 2,000: 256 keys 49 us,
-                                       // 512 49, this 39; three lists 57, 41, 41)
+                                       // 512 49, this 39; three lists 57, 41, 41.  Larger ones divided among the CTAs by a sample of their own, so that
+                                       // nearly no list goes on to the ranked sample: as fast or slower, 36 to 43 us for one list of 10,000, 50 to 65 for one of 30,000)
 #define SG_MAP 512u                    // parts of larger buckets per CTA
 #define SG_WAIT_LIMIT (1u << 23)       // polls of a grid barrier (seconds)
 #define SG_PATIENCE 64u                // polls (about 50 us) between two looks for shares that nobody has begun

@@ -8,7 +8,7 @@
 //              of eight keys.  Whoever places every step-th key stores it as a boundary for the next call: exact quantiles of this call's
 //              order, up to 2.25 lists from its beginning, because a list's entries are usually gone by then.
 //
-// The boundaries decide nothing but the sizes of the buckets.  Where they do not hold -- a bucket of more than 1,024 keys, too few
+// The boundaries decide nothing but the sizes of the buckets.  Where they do not hold -- a bucket of more than SG_BUCKET_MAX keys, too few
 // keys below the last boundary, the first calls -- the candidates are ordered by a ranked sample instead (cs_select_buckets.cuh; two more
 // barriers), and where the remembered key does not, a histogram and a collect pass come first (two more).  Both are remembered as scores and
 // ages: their last_access moves on with the clock.
@@ -32,8 +32,9 @@
 #define SG_STEP 24u                    // keys of a bucket aimed at, as long as CS_BUCKETS buckets hold the list
 #define SG_BUCKET_WARP 96u             // largest bucket that one warp ranks, three keys per lane
 #define SG_KEYS 128u                   // keys that a warp holds at a time
-#define SG_BUCKET_MAX 1024u            // largest bucket that is counted.  (Index that moves, 1,000,000 entries, lists of 10,000 and 2,000: 256 keys 49 us,
-                                       // 512 49, this 39; three lists 57, 41, 41.  Larger ones divided among the CTAs by a sample of their own, so that
+#define SG_BUCKET_MAX 1536u            // largest bucket that is counted.  (Index that moves, 1,000,000 entries, lists of 10,000 and 2,000, bench.py's metadata-scale loop
+                                       // replayed from a graph: 1,024 keys 49.3 us, this 46.2, 2,048 45.2, 3,072 44.8; but where a list of 2,000 has come to lie in one
+                                       // bucket, which the sample then ranks without a barrier more, 45.0, 44.6, 49.3, 48.9.  Larger ones divided among the CTAs by a sample of their own, so that
                                        // nearly no list goes on to the ranked sample: as fast or slower, 36 to 43 us for one list of 10,000, 50 to 65 for one of 30,000)
 #define SG_MAP 512u                    // parts of larger buckets per CTA
 #define SG_WAIT_LIMIT (1u << 23)       // polls of a grid barrier (seconds)

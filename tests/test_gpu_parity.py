@@ -1322,6 +1322,42 @@ def test_select_on_the_whole_gpu(n, kind):
         assert H.assert_list_matches(got.cpu().numpy().view(np.uint32)[:k], int(got_n[0].item()), o_ids, o_n, s64) == 0
 
 
+# Keys that come to lie between two remembered boundaries, beside the 24 or so of that bucket: what parts of a warp count, the last such size and the next
+# (1,536 keys), more than that, more than a bucket's region holds.
+@pytest.mark.parametrize("m", [90, 1000, 1500, 1511, 1512, 1513, 1537, 3000, 20_000])
+def test_a_bucket_of_many_keys(m):
+    """m entries of each tier take the score and the age of a victim in the middle of the list, in the GPU tier with three last_accesses, in the host tier tied but
+    for their ids.  Three lists against the launch chain, bit for bit."""
+    cfg, n, k = synth.CONFIGS["meta1m"], 303_107, 2500
+    c, _ = warm_state(cfg, 800, n, r_min=0.02)
+    chain, _ = warm_state(cfg, 800, n, r_min=0.02)
+    chain.set_select_path(cs.CS_SELECT_MULTI)
+    idx = synth.make_block_index(cfg, n=n, tier="random")
+    idx.flags[:] = synth.FLAG_VALID
+    idx.flags[: n // 2] |= synth.FLAG_TIER_HOST
+    idx.ref_count[:] = 0
+    idx.n_tokens[:] = cfg.block_tokens
+    rng = synth.rng_for(cfg, 98)
+    d = cs.DeviceIndex.from_host(idx, DEV)
+    la, agent = d.last_access.view(torch.int32), d.agent.view(torch.int16)
+    for rep in range(5):
+        outs = []
+        for x in (c, chain):
+            outs.append([torch.full((q,), 7, dtype=torch.int32, device=DEV) for q in (k, 4, k, 4, k, 4)])
+            x.select_step(d, 100_000 + rep, k, k, *outs[-1])
+        for got, want in zip(*outs):
+            assert torch.equal(got, want), rep
+        if rep == 2:
+            for q, lo in ((0, n // 2), (1, 0)):
+                mid = int(outs[1][2 * q][k // 2])
+                some = torch.from_numpy(rng.permutation(n // 2)[: m].astype(np.int64) + lo).to(DEV)
+                la[some] = la[mid].clone() + 1
+                agent[some] = agent[mid].clone()
+                if q == 0:
+                    la[some] += torch.from_numpy(rng.integers(0, 3, m).astype(np.int32)).to(DEV)
+    assert c.get_status() == chain.get_status() == 0
+
+
 # What a call of the whole-GPU select can come with, beside the plain ones above.  n: an index of either side of the 262,144 entries up to which every list has
 # scratch of its own in a context for more than 4,194,304.
 OPTIONS = {"slow_decay": dict(params=dict(lam=1e-4)),                     # the recency table ends before saturation

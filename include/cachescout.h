@@ -273,11 +273,12 @@ int cs_prefetch_blocks_staged(cs_ctx *ctx, const cs_kv_pool *host, const cs_kv_p
 /* The selections of a step at once: cs_select_victims(tier 0, k_victims), cs_select_victims(tier 1,
  * k_victims) and cs_select_prefetch(k_prefetch) over the same index and clock, with the same results, run
  * side by side.  A selection whose count pointer is NULL is left out.  For index sizes the single-launch
- * select covers (<= 262,144 entries) they are the thread-block clusters of ONE launch; for larger indexes
- * each is a chain of grid-wide kernels, the first on `stream` and the others on two streams the context owns,
- * forked from and joined back into `stream` with events, so that to the caller everything is ordered on
- * `stream` (beyond 4,194,304 entries the selections run one after the other: private scratch of that size
- * is not reserved).  Arguments as for the single calls. */
+ * select covers (<= 262,144 entries) they are the thread-block clusters of ONE launch; for larger indexes, and
+ * above 131,072 entries from a selection's second call on, they are ONE launch on the whole GPU (cs_set_select_path()).
+ * Where that does not apply, each is a chain of grid-wide kernels, the first on `stream` and the others on two streams the
+ * context owns, forked from and joined back into `stream` with events, so that to the caller everything is ordered on
+ * `stream` (in a context for more than 4,194,304 blocks, selections of more than 262,144 entries run one after the
+ * other: private scratch of that size is not reserved).  Arguments as for the single calls. */
 int cs_select_step(cs_ctx *ctx, const cs_block_index *idx, uint32_t now, uint32_t k_victims, uint32_t k_prefetch,
                    uint32_t *gpu_victims, uint32_t *n_gpu_victims, uint32_t *host_victims, uint32_t *n_host_victims,
                    uint32_t *prefetch_ids, uint32_t *n_prefetch, cs_stream_t stream);
